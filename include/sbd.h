@@ -194,8 +194,8 @@ int sbd_lookup(sbd_handle handle, int spin, const uint64_t *keys_dev, int64_t n,
  *   c_dev     device pointer, [nvec][nA][nB], double for SBD_FP64 and SBD_F32X2,
  *             float for SBD_MIXED, in sorted-string order
  *   sigma_dev device pointer, [nvec][nA][nB] doubles (written, not accumulated)
- * The handle keeps one transposed copy of a vector as work space (allocated
- * on the first call).  c and sigma must not overlap.
+ * The handle's work vector and sigma itself hold transposed intermediates
+ * while the product runs.  c and sigma must not overlap.
  */
 int sbd_sigma(sbd_handle handle, const void *c_dev, double *sigma_dev, int nvec, sbd_precision prec,
               void *stream);
@@ -279,12 +279,13 @@ int sbd_sort_strings_noalloc(const uint64_t *keys_dev, int64_t n, int norb, int 
  *   c_dev[i]     device pointer, handle i's [nA][nB] vector (float for
  *                SBD_MIXED, double for SBD_FP64), sorted-string order
  *   sigma_dev[i] device pointer, [nA][nB] doubles, written
- *   rows_per_item rows of C staged per work item: 1, 2, or for SBD_MIXED 4 or 8
- *                (8: one column half at a time); 0 picks the largest that fits
- *                shared memory for every instance
- * Each output element is computed by the same arithmetic as sbd_sigma with
- * the same rows per item (sbd_sigma takes 8 rows over column halves for
- * SBD_MIXED where they fit, else the largest that fits).  Enqueued on `stream`
+ *   rows_per_item rows of C staged per work item of the two-operand alpha-beta
+ *                pass: 1, 2, or for SBD_MIXED 4 or 8 (8: only where the
+ *                column-stationary pass runs instead); 0 picks the largest that
+ *                fits shared memory for every instance
+ * Each output element is computed by the same arithmetic as sbd_sigma (in the
+ * two-operand pass: with the same rows per item; sbd_sigma takes the largest
+ * that fits).  Enqueued on `stream`
  * (the handles' work buffers are used), then synchronised.
  */
 int sbd_sigma_batched(int n, const sbd_handle *handles, const void *const *c_dev, double *const *sigma_dev,

@@ -53,6 +53,40 @@ struct DevStatus {
 // ---------------------------------------------------------------------------
 // per-spin tables, all device memory
 
+// Same-spin excitation lists of one string set as the row passes read them (range_rows.cuh).  The
+// targets are cut into ng ranges of w strings (the part of C that a CTA stages at a time).  The
+// strings are dealt to kParts parts (part = string mod kParts); inside a range the parts follow each
+// other, and inside a part the lists descend in length and are taken kListGroup at a time.  Such a
+// group is what a warp walks side by side, so its lists are padded to the longest of them and stored
+// interleaved, block by block: a warp's load of one block of all its lists is one contiguous piece.
+// Padding entries have value zero and repeat the list's first target.
+constexpr int kParts = 16;
+constexpr int kRangeDoubles = 4;  // entries of one list in a block of doubles
+constexpr int kRangeSingles = 2;  // and in a block of singles
+constexpr int kListGroup = 8;     // lists of a group
+constexpr int32_t kListHas = 1 << 30;  // the string's list has entries in this range
+struct RangeLists {
+    int w = 0, ng = 0;
+    int32_t *zi = nullptr;                     // [ng*groups*8] string | kListHas, or -1 (no string)
+    uint32_t *qd = nullptr, *qs = nullptr;     // [ng*groups + 1] first block of a group's doubles, singles
+    uint16_t *dt = nullptr;                    // doubles: target inside the range
+    float *dv32 = nullptr;                     // and matrix element, in the three arithmetics
+    double *dv64 = nullptr;
+    float2 *dvx2 = nullptr;
+    uint32_t *sm = nullptr;  // singles: target inside the range | orbital pair << 16 | phase -1 << 31
+    float *sv32 = nullptr;
+    double *sv64 = nullptr;
+    float2 *svx2 = nullptr;
+    double *jg = nullptr;  // [npair][n] J_i[rs] = sum_{k in string i} (rs|kk), pair r(r-1)/2 + s
+};
+// first group of part p (p = kParts: groups of a range) for n strings
+__host__ __device__ __forceinline__ int64_t part_group(int64_t n, int p)
+{
+    const int64_t a = n / kParts, rest = n % kParts;  // parts below `rest` hold a + 1 strings, the others a
+    const int64_t big = a / kListGroup + 1, small = (a + kListGroup - 1) / kListGroup;
+    return p < rest ? p * big : rest * big + (p - rest) * small;
+}
+
 struct SpinTables {
     int nel = 0;                 // electrons of this spin
     int64_t n = 0;               // |S|
@@ -73,24 +107,13 @@ struct SpinTables {
     int64_t sig_ns = 0, sig_nd = 0;
     uint32_t *s_pk_sig = nullptr;
     double *s_v64_sig = nullptr;
-    int32_t *d_j_sig = nullptr;
+    int32_t *d_j_sig = nullptr;  // the doubles are made with the first block plan
     double *d_v64_sig = nullptr;
     uint2 *s_pkv32 = nullptr;  // (s_pk_sig, FP32 value bits), for the mixed sigma
     uint2 *d_jv32 = nullptr;   // (d_j_sig, FP32 value bits), for the mixed sigma
     float2 *s_vx2 = nullptr;   // s_v64_sig as FP32 pairs (hi, lo), for the FP32-pair sigma
     float2 *d_vx2 = nullptr;   // d_v64_sig as FP32 pairs
-    // Mixed-sigma lists split at the middle of the string set (half = (n + 1) / 2): virtual list
-    // 2i holds the entries of source i with target < half, list 2i + 1 those with target >= half,
-    // each padded to kListPad and in sigma order, for row passes that stage one column half at a
-    // time (8 rows instead of 4 in the same shared memory).
-    int64_t half = 0;
-    int64_t *hs_ptr = nullptr, *hd_ptr = nullptr;  // [2n + 1]
-    uint2 *hs = nullptr;  // (packed single, FP32 value bits)
-    // doubles as two arrays with the same entry index: FP32 values, and targets relative to the
-    // list's column half (0 for the lower half, `half` for the upper), which fit 16 bits: the split
-    // lists are built only for half <= 65536 (six bytes per entry instead of eight)
-    float *hdv = nullptr;
-    uint16_t *hdt = nullptr;
+    RangeLists rl;  // same-spin lists of the row passes
     // Source-major singles for the column-stationary alpha-beta pass.  The canonical singles list
     // of each string is cut into items of at most kSrcItem entries (strings in ascending order,
     // each string's items consecutive, then inside each slice of 32 items the full ones first and
@@ -205,6 +228,9 @@ void sort_validate_into(const uint64_t *in, int64_t n, int norb, int nel, uint64
 
 // tables.cu
 void build_tables(Ctx &c, int spin);
+void build_range_lists(Ctx &c, int spin);
+// doubles of one spin in sigma order, for block plans
+void build_sig_doubles(Ctx &c, SpinTables &t);
 void build_diagonal(Ctx &c);
 void to_float(const double *in, float *out, int64_t n, cudaStream_t s);
 

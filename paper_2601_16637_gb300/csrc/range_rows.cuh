@@ -1,0 +1,471 @@
+// Row passes of the sigma product: same-spin excitation lists against ranges of C staged in shared
+// memory (see RangeLists for the lists).
+//
+// The pass computes, for `nrow` independent rows (the strings of the other spin) and every string i
+// of the list spin,
+//   Y[i][r] (+)= sum_{j in doubles(i)} H(i,j) X[j][r]
+//              + sum_{j in singles(i), pair rs, phase t} [H(i,j) + t J_r[rs]] X[j][r],
+// with the rows contiguous in X and Y: the alpha pass reads C and adds into sigma as they are, the
+// beta pass reads the transpose of C and writes the transpose of its part of sigma.
+//
+// What bounds it and why it is laid out this way: every multiply-add takes one operand of C from
+// shared memory, and what a load brings into registers passes at 128 bytes per SM clock, whether the
+// bytes differ between the lanes or not.  In FP32 the pass is bound by that, in FP64 by the FP64 pipe.
+// A CTA stages 128 bytes of every string j of a range: 32 rows in FP32, 16 in FP64 or FP32 pairs.
+// Four lanes walk one list together, each owning two 16-byte chunks of the staged line (8 rows in
+// FP32), so that a list entry, 6 bytes in FP32, feeds 8 multiply-adds; with eight lanes and one chunk
+// each, the entries took 27 % of the bytes instead of 16 %.  Chunk c holds rows c, c + 8, ...; the two
+// lists that share a 128-bit phase read their chunks in opposite order, so the phase covers all 32
+// banks whatever strings they read.  Every lane works on every entry (on the FP64 pipe an idle lane
+// costs as much as a busy one), no sum crosses lanes, and the four lanes' loads and stores of Y are
+// contiguous without asking anything of its alignment or row length.
+//
+// Measured, beta + alpha pass of one product (CUDA events, before: whole rows of C staged, one list
+// per eight lanes and one entry per lane): 1.0e8 determinants, FP32 25.1 -> 18.5 ms; 3.6e7
+// determinants (norb 29), FP32 7.0 -> 5.5, FP64 64.2 -> 50.5, FP32 pairs 20.8 -> 14.7 ms; 2.5e7
+// determinants at norb 58, FP32 about 12 -> 6.8 ms.  The FP32 pass keeps the L1/shared pipe 87 % busy.
+// Steps tried on the way (FP32, 3.6e7 determinants): an octet per list with separate lists 6.0 ms,
+// with interleaved lists 6.2 (padding costs more than the contiguous loads save while every octet
+// still reads 24 bytes of entries per 64 of C), four lanes per list 5.5.
+#pragma once
+
+#include "common.cuh"
+#include "pair.cuh"
+
+namespace sbd {
+
+constexpr int kRangeThreads = 1024;
+constexpr int kRangeRowBytes = 128;
+
+// The table of J_r[rs] of the staged rows sits in shared memory while it leaves at least half of it
+// to the ranges (norb <= 42); above that the few singles read J from global memory, because shorter
+// ranges would mean more passes over Y.
+__host__ __device__ inline size_t range_j_bytes(int norb) { return (size_t)(norb * (norb - 1) / 2 + 1) * kRangeRowBytes; }
+__host__ __device__ inline size_t range_smem(int optin) { return ((size_t)optin - 1024) / kRangeRowBytes * kRangeRowBytes; }
+__host__ __device__ inline bool range_j_staged(int optin, int norb) { return 2 * range_j_bytes(norb) <= range_smem(optin); }
+// most strings of one range
+inline int range_width_max(int optin, int norb)
+{
+    const size_t room = range_smem(optin) - (range_j_staged(optin, norb) ? range_j_bytes(norb) : 0);
+    return (int)(room / kRangeRowBytes);
+}
+
+// list value type of an arithmetic
+template <typename T>
+struct RangeVal {
+    using type = T;
+};
+template <>
+struct RangeVal<F2> {
+    using type = float2;
+};
+// element type of the vectors (the pair arithmetic reads FP64 vectors)
+template <typename T>
+struct RangeIn {
+    using type = T;
+};
+template <>
+struct RangeIn<F2> {
+    using type = double;
+};
+
+template <typename T>
+struct RangeArgs {
+    const typename RangeIn<T>::type *X;  // [n][nrow]
+    double *Y;                           // [n][nrow]
+    int64_t n, nrow;
+    int accumulate;  // add to Y (0: the first range writes)
+    float *rowmax;   // FP32 only, optional: [nrow] max_j |X[j][r]|
+    int npair, jstaged, w, ng;
+    int q;             // batched launches: pieces a row block is cut into (a divisor of kParts)
+    const double *jg;  // [npair][nrow]
+    const int32_t *zi;
+    const uint32_t *qd, *qs;
+    const uint16_t *dt;
+    const typename RangeVal<T>::type *dv;
+    const uint32_t *sm;
+    const typename RangeVal<T>::type *sv;
+};
+
+template <typename T>
+constexpr int kRangeRows = kRangeRowBytes / (int)sizeof(T);
+
+
+// Packed FP32 arithmetic on two rows at a time: the same roundings as two scalar operations in half
+// the instructions (the pass issues in 73 % of the cycles with scalar ones).
+__device__ __forceinline__ uint64_t pk_fma(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t pk_mul(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t pk_add(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t pk_dup(float v)
+{
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(v));
+    return d;
+}
+__device__ __forceinline__ uint64_t pk_pair(float a, float b)
+{
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ float pk_get(uint64_t p, int i)
+{
+    return __uint_as_float(i ? (unsigned)(p >> 32) : (unsigned)p);
+}
+// x - y as one rounded operation per half
+__device__ __forceinline__ uint64_t pk_sub(uint64_t x, uint64_t y) { return pk_fma(y, pk_dup(-1.f), x); }
+
+// The sums of one lane: two chunks (h = 0, 1) of a staged line.  A chunk's 16 bytes are two words:
+// two packed pairs of rows (FP32), two FP64 rows, or the high and the low parts of two pair rows.
+template <typename T>
+struct RangeAcc;
+
+template <>
+struct RangeAcc<float> {
+    static constexpr int kRowsPerChunk = 4;
+    using Val = float;
+    uint64_t blk[4], acc[4], sum[4];
+    float v[4];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = sum[i] = 0ull;
+    }
+    static __device__ __forceinline__ void load(const float *p, float (&v)[4])
+    {
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
+        v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+    }
+    // entry u of a block; the block's products are summed by themselves, and the blocks on two
+    // levels (eight blocks, then all): short chains keep the rounding error of a long list down
+    __device__ __forceinline__ void mac(int u, float v, const ulonglong2 (&x)[2])
+    {
+        const uint64_t vv = pk_dup(v);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            blk[2 * h] = u == 0 ? pk_mul(vv, x[h].x) : pk_fma(vv, x[h].x, blk[2 * h]);
+            blk[2 * h + 1] = u == 0 ? pk_mul(vv, x[h].y) : pk_fma(vv, x[h].y, blk[2 * h + 1]);
+        }
+    }
+    __device__ __forceinline__ void end_block(unsigned count)
+    {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = pk_add(acc[i], blk[i]);
+        if ((count & 7u) == 0u) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sum[i] = pk_add(sum[i], acc[i]), acc[i] = 0ull;
+        }
+    }
+    // (v + sg*j) x
+    __device__ __forceinline__ void single(float v, float sg, const ulonglong2 (&j)[2], const ulonglong2 (&x)[2])
+    {
+        const uint64_t vv = pk_dup(v), ss = pk_dup(sg);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            acc[2 * h] = pk_fma(pk_fma(ss, j[h].x, vv), x[h].x, acc[2 * h]);
+            acc[2 * h + 1] = pk_fma(pk_fma(ss, j[h].y, vv), x[h].y, acc[2 * h + 1]);
+        }
+    }
+    __device__ __forceinline__ double value(int h, int i) const
+    {
+        return (double)(pk_get(acc[2 * h + i / 2], i & 1) + pk_get(sum[2 * h + i / 2], i & 1));
+    }
+    static __device__ __forceinline__ void store(unsigned char *line, int row, double x)
+    {
+        reinterpret_cast<float *>(line)[(row & 7) * 4 + (row >> 3)] = (float)x;
+    }
+    static __device__ __forceinline__ ulonglong2 chunk(const double (&x)[4])
+    {
+        return make_ulonglong2(pk_pair((float)x[0], (float)x[1]), pk_pair((float)x[2], (float)x[3]));
+    }
+};
+
+template <>
+struct RangeAcc<double> {
+    static constexpr int kRowsPerChunk = 2;
+    using Val = double;
+    double acc[4];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = 0.0;
+    }
+    static __device__ __forceinline__ void load(const double *p, double (&v)[4])
+    {
+        const double2 a = __ldg(reinterpret_cast<const double2 *>(p)), b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
+        v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+    }
+    __device__ __forceinline__ void mac(int, double v, const ulonglong2 (&x)[2])
+    {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            acc[2 * h] = fma(v, __longlong_as_double((long long)x[h].x), acc[2 * h]);
+            acc[2 * h + 1] = fma(v, __longlong_as_double((long long)x[h].y), acc[2 * h + 1]);
+        }
+    }
+    __device__ __forceinline__ void end_block(unsigned) {}
+    __device__ __forceinline__ void single(double v, float sg, const ulonglong2 (&j)[2], const ulonglong2 (&x)[2])
+    {
+        const uint64_t flip = sg < 0.f ? 0x8000000000000000ull : 0ull;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            acc[2 * h] = fma(v + __longlong_as_double((long long)(j[h].x ^ flip)),
+                             __longlong_as_double((long long)x[h].x), acc[2 * h]);
+            acc[2 * h + 1] = fma(v + __longlong_as_double((long long)(j[h].y ^ flip)),
+                                 __longlong_as_double((long long)x[h].y), acc[2 * h + 1]);
+        }
+    }
+    __device__ __forceinline__ double value(int h, int i) const { return acc[2 * h + i]; }
+    static __device__ __forceinline__ void store(unsigned char *line, int row, double x)
+    {
+        reinterpret_cast<double *>(line)[(row & 7) * 2 + (row >> 3)] = x;
+    }
+    static __device__ __forceinline__ ulonglong2 chunk(const double (&x)[2])
+    {
+        return make_ulonglong2((uint64_t)__double_as_longlong(x[0]), (uint64_t)__double_as_longlong(x[1]));
+    }
+};
+
+template <>
+struct RangeAcc<F2> {
+    static constexpr int kRowsPerChunk = 2;
+    using Val = float2;
+    uint64_t hi[2], lo[2];
+    __device__ __forceinline__ void zero() { hi[0] = hi[1] = lo[0] = lo[1] = 0ull; }
+    static __device__ __forceinline__ void load(const float2 *p, float2 (&v)[4])
+    {
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(p)), b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
+        v[0] = make_float2(a.x, a.y), v[1] = make_float2(a.z, a.w);
+        v[2] = make_float2(b.x, b.y), v[3] = make_float2(b.z, b.w);
+    }
+    // f2_mac on two rows; vn = -a.hi b.hi saves negating the product for its error term
+    __device__ __forceinline__ void mac2(int h, uint64_t ah, uint64_t an, uint64_t al, ulonglong2 b)
+    {
+        const uint64_t pn = pk_mul(an, b.x);
+        uint64_t e = pk_fma(ah, b.x, pn);
+        e = pk_fma(ah, b.y, e);
+        e = pk_fma(al, b.x, e);
+        const uint64_t s = pk_sub(hi[h], pn);
+        const uint64_t bb = pk_sub(s, hi[h]);
+        const uint64_t t = pk_sub(pk_sub(hi[h], pk_sub(s, bb)), pk_add(pn, bb));
+        hi[h] = s;
+        lo[h] = pk_add(lo[h], pk_add(t, e));
+    }
+    __device__ __forceinline__ void mac(int, float2 v, const ulonglong2 (&x)[2])
+    {
+        const uint64_t ah = pk_dup(v.x), an = pk_dup(-v.x), al = pk_dup(v.y);
+        mac2(0, ah, an, al, x[0]);
+        mac2(1, ah, an, al, x[1]);
+    }
+    // the gathered low parts go back below the rounding of the high part: left to grow, each further
+    // sum would round at their size
+    __device__ __forceinline__ void end_block(unsigned)
+    {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint64_t s = pk_add(hi[h], lo[h]);
+            lo[h] = pk_sub(lo[h], pk_sub(s, hi[h]));
+            hi[h] = s;
+        }
+    }
+    __device__ __forceinline__ void single(float2 v, float sg, const ulonglong2 (&j)[2], const ulonglong2 (&x)[2])
+    {
+        const uint64_t ss = pk_dup(sg), sn = pk_dup(-sg);
+        mac(0, v, x);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) mac2(h, pk_mul(ss, j[h].x), pk_mul(sn, j[h].x), pk_mul(ss, j[h].y), x[h]);
+        end_block(0);
+    }
+    __device__ __forceinline__ double value(int h, int i) const
+    {
+        return (double)pk_get(hi[h], i) + (double)pk_get(lo[h], i);
+    }
+    static __device__ __forceinline__ void store(unsigned char *line, int row, double x)
+    {
+        const F2 s = f2_split(x);
+        float *f = reinterpret_cast<float *>(line) + (row & 7) * 4 + (row >> 3);
+        f[0] = s.hi;
+        f[2] = s.lo;
+    }
+    static __device__ __forceinline__ ulonglong2 chunk(const double (&x)[2])
+    {
+        const F2 a = f2_split(x[0]), b = f2_split(x[1]);
+        return make_ulonglong2(pk_pair(a.hi, b.hi), pk_pair(a.lo, b.lo));
+    }
+};
+
+// Rows row0 .. row0 + kRangeRows - 1, output strings of the parts [p0, p1).
+template <typename T>
+__device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, int p0, int p1, unsigned char *smem)
+{
+    using Acc = RangeAcc<T>;
+    using In = typename RangeIn<T>::type;
+    constexpr int ROWS = kRangeRows<T>, RPC = Acc::kRowsPerChunk, LPW = 32 / ROWS;  // LPW: lines a warp stages at once
+    constexpr int kWarps = kRangeThreads / 32;
+    unsigned char *Js = smem + (size_t)a.w * kRangeRowBytes;  // [npair + 1] lines behind the w staged lines
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lst = lane >> 2, l = lane & 3;  // list of the group, lane of the list
+    const int nr = (int)min((int64_t)ROWS, a.nrow - row0);
+    const int sr = lane & (ROWS - 1), sub = lane / ROWS;  // staging: row and line of the lane
+    const bool srow = sr < nr;
+    // the lane's chunks of a line and its first rows in them
+    const int c0 = l + 4 * (lst & 1), c1 = c0 ^ 4;
+    unsigned rmax = 0u;
+    __shared__ unsigned rmax_s[ROWS];
+    __shared__ unsigned next_s;
+    __syncthreads();  // the previous rows are finished with shared memory
+    if (threadIdx.x < ROWS) rmax_s[threadIdx.x] = 0u;
+    if (a.jstaged) {
+        for (int p = warp * LPW + sub; p <= a.npair; p += kWarps * LPW)
+            Acc::store(Js + (size_t)p * kRangeRowBytes, sr,
+                       p < a.npair && srow ? __ldg(a.jg + (int64_t)p * a.nrow + row0 + sr) : 0.0);
+    }
+    const int64_t groups = part_group(a.n, kParts);
+    const unsigned q0 = (unsigned)part_group(a.n, p0), q1 = (unsigned)part_group(a.n, p1);
+    for (int g = 0; g < a.ng; ++g) {
+        if (g) __syncthreads();  // every warp is finished with the previous range
+        if (threadIdx.x == 0) next_s = q0 + kWarps;
+        const int64_t j0 = (int64_t)g * a.w;
+        const int wj = (int)min((int64_t)a.w, a.n - j0);
+        const In *src = a.X + j0 * a.nrow + row0 + sr;
+        for (int jb = warp * LPW + sub; jb < wj; jb += 8 * kWarps * LPW) {
+            In v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int j = jb + u * kWarps * LPW;
+                v[u] = (j < wj && srow) ? src[(int64_t)j * a.nrow] : In(0);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int j = jb + u * kWarps * LPW;
+                if (j < wj) Acc::store(smem + (size_t)j * kRangeRowBytes, sr, (double)v[u]);
+                if constexpr (sizeof(T) == 4) rmax = max(rmax, __float_as_uint(fabsf(v[u])));
+            }
+        }
+        __syncthreads();
+        const unsigned char *x0 = smem + c0 * 16, *x1 = smem + c1 * 16;
+        const bool add = g > 0 || a.accumulate;
+        const int32_t *zi_g = a.zi + (int64_t)g * groups * kListGroup + lst;
+        const uint32_t *qd_g = a.qd + (int64_t)g * groups, *qs_g = a.qs + (int64_t)g * groups;
+        // the groups of lists are taken from a counter: their lengths differ, and the range ends with a barrier
+        unsigned q = q0 + warp;
+        int zi = -1;
+        uint32_t db = 0, de = 0, sb = 0, se = 0;
+        if (q < q1) zi = zi_g[(int64_t)q * kListGroup], db = qd_g[q], de = qd_g[q + 1], sb = qs_g[q], se = qs_g[q + 1];
+        while (q < q1) {  // uniform over the warp
+            unsigned qn = 0;
+            if (lane == 0) qn = atomicAdd(&next_s, 1u);
+            qn = __shfl_sync(0xffffffffu, qn, 0);
+            int zi_n = -1;
+            uint32_t db_n = 0, de_n = 0, sb_n = 0, se_n = 0;  // the next group's bounds
+            if (qn < q1)
+                zi_n = zi_g[(int64_t)qn * kListGroup], db_n = qd_g[qn], de_n = qd_g[qn + 1], sb_n = qs_g[qn], se_n = qs_g[qn + 1];
+            if (!add || db < de || sb < se) {
+                Acc acc;
+                acc.zero();
+                for (uint32_t b = sb; b < se; ++b) {
+                    const size_t at = (size_t)b * kListGroup + lst;
+                    const uint2 m2 = __ldg(reinterpret_cast<const uint2 *>(a.sm) + at);
+                    const uint32_t m[2] = {m2.x, m2.y};
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const typename Acc::Val v = __ldg(a.sv + at * 2 + u);
+                        const uint32_t jo = (m[u] & 0xffffu) * kRangeRowBytes;
+                        const int pr = (int)((m[u] >> 16) & 0x7fffu);
+                        const ulonglong2 x[2] = {*reinterpret_cast<const ulonglong2 *>(x0 + jo),
+                                                 *reinterpret_cast<const ulonglong2 *>(x1 + jo)};
+                        ulonglong2 jv[2];
+                        if (a.jstaged) {
+                            jv[0] = *reinterpret_cast<const ulonglong2 *>(Js + pr * kRangeRowBytes + c0 * 16);
+                            jv[1] = *reinterpret_cast<const ulonglong2 *>(Js + pr * kRangeRowBytes + c1 * 16);
+                        } else {
+                            double t[2][RPC];
+#pragma unroll
+                            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                                for (int i = 0; i < RPC; ++i) {
+                                    const int r = (h ? c1 : c0) + 8 * i;
+                                    t[h][i] = pr < a.npair && r < nr ? __ldg(a.jg + (int64_t)pr * a.nrow + row0 + r) : 0.0;
+                                }
+                            jv[0] = Acc::chunk(t[0]);
+                            jv[1] = Acc::chunk(t[1]);
+                        }
+                        acc.single(v, (m[u] >> 31) ? -1.f : 1.f, jv, x);
+                    }
+                }
+                // doubles, a block of four entries at a time; the next block is loaded before this one is used
+                if (db < de) {
+                    typename Acc::Val v[4];
+                    const uint2 *tp = reinterpret_cast<const uint2 *>(a.dt) + (size_t)db * kListGroup + lst;
+                    const typename Acc::Val *vp = a.dv + ((size_t)db * kListGroup + lst) * 4;
+                    uint2 t4 = __ldg(tp);
+                    Acc::load(vp, v);
+                    const unsigned nb = de - db;
+                    for (unsigned b = 1; b <= nb; ++b) {
+                        const uint2 t = t4;
+                        const typename Acc::Val c[4] = {v[0], v[1], v[2], v[3]};
+                        tp += kListGroup;
+                        vp += kListGroup * 4;
+                        if (b < nb) {
+                            t4 = __ldg(tp);
+                            Acc::load(vp, v);
+                        }
+                        const uint32_t j[4] = {t.x & 0xffffu, t.x >> 16, t.y & 0xffffu, t.y >> 16};
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const uint32_t jo = j[u] * kRangeRowBytes;
+                            const ulonglong2 x[2] = {*reinterpret_cast<const ulonglong2 *>(x0 + jo),
+                                                     *reinterpret_cast<const ulonglong2 *>(x1 + jo)};
+                            acc.mac(u, c[u], x);
+                        }
+                        acc.end_block(b);
+                    }
+                }
+                if (zi >= 0 && (!add || (zi & kListHas))) {  // the string's sum changes Y
+                    double *y = a.Y + (int64_t)(zi & ~kListHas) * a.nrow + row0;
+                    double yo[2][RPC];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int i = 0; i < RPC; ++i) {
+                            const int r = (h ? c1 : c0) + 8 * i;
+                            yo[h][i] = add && r < nr ? y[r] : 0.0;
+                        }
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int i = 0; i < RPC; ++i) {
+                            const int r = (h ? c1 : c0) + 8 * i;
+                            if (r < nr) y[r] = (zi & kListHas) ? yo[h][i] + acc.value(h, i) : 0.0;
+                        }
+                }
+            }
+            q = qn;
+            zi = zi_n, db = db_n, de = de_n, sb = sb_n, se = se_n;
+        }
+    }
+    if constexpr (sizeof(T) == 4) {
+        if (a.rowmax && p0 == 0) {  // uniform over the CTA
+            atomicMax(rmax_s + sr, rmax);
+            __syncthreads();
+            if (threadIdx.x < nr) a.rowmax[row0 + threadIdx.x] = __uint_as_float(rmax_s[threadIdx.x]);
+        }
+    }
+}
+
+}  // namespace sbd

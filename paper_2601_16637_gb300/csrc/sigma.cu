@@ -14,18 +14,19 @@
 //     + sum_{ja in doubles(ia)} Ha(ia,ja) c(ja,ib)
 //     + sum_{ja in singles(ia), code pq, phase u} [Ha(ia,ja) + u J_ib[pq]] c(ja,ib)
 //     + sum_{ja in singles(ia)} sum_{jb in singles(ib)} u t (pq|rs) c(ja,jb)
-// The first three lines are a gather inside row ia of C ("beta pass"), the
-// next two the same gather inside column ib, run on the transpose C^T
-// ("alpha pass", same kernel), and the last line is the alpha-beta pass.
+// The second and third line are a gather inside row ia of C ("beta pass"), the next two the same
+// gather inside column ib ("alpha pass", same kernel: range_rows.cuh), and the last line is the
+// alpha-beta pass.  The beta pass runs on the transpose of C and leaves its result transposed; the
+// pass that transposes it back adds the diagonal term.
 //
-// Every output element is owned by one thread group in each pass and each
-// pass adds into it in program order, so results are deterministic.  Rows of
-// C are staged in shared memory, R rows interleaved per column so one vector
-// load fetches the same column of all R rows; the inner gathers then hit
-// shared memory only.  The lists are the padded sigma copies: each lane of an
-// 8-lane group fetches 4 entries with 16-byte loads, and the next column's
-// list bounds are prefetched.  The phase of a single is folded into the
-// shared-memory coefficient tables, which are indexed by 2*code + (phase<0).
+// Every output element is owned by one thread group in each pass and each pass adds into it in
+// program order, so results are deterministic.
+//
+// Row-block products (alpha-row sharding) and the two-operand alpha-beta pass stage whole rows of C
+// in shared memory, R rows interleaved per column so one vector load fetches the same column of all
+// R rows; each lane of an 8-lane group fetches 4 entries of the padded sigma copies of the lists with
+// 16-byte loads, and the next column's list bounds are prefetched.  The phase of a single is folded
+// into the shared-memory coefficient tables, which are indexed by 2*code + (phase<0).
 // Precision T = double (FP64), float (mixed: FP32 amplitudes, integrals,
 // products and per-list sums, each list sum and the diagonal term accumulated
 // into the FP64 output), or F2 (FP64-accurate arithmetic on the FP32 pipe:
@@ -40,6 +41,7 @@
 
 #include "common.cuh"
 #include "pair.cuh"
+#include "range_rows.cuh"
 
 namespace sbd {
 
@@ -273,18 +275,11 @@ struct RowArgs {
     int accumulate;
     const double *hd;    // optional diagonal, indexed like Y
     const double *xd64;  // optional FP64 amplitudes [nrow][ncol] for the diagonal term
-    float *rowmax;       // optional (FP32 only): rowmax[r] = max_c |X[r][c]| of every row of the pass
     const uint64_t *row_strings;
     int norb;
     const double *eri;  // FP64 integrals, for the J vectors of the staged rows
     const int64_t *s_ptr, *d_ptr;
     Lists<T> lists;
-    // mixed passes over column halves (row_halves): the column spin's lists split at `half`
-    const int64_t *hls_ptr, *hld_ptr;  // singles, doubles: [2n + 1]
-    const uint2 *hls;                  // (packed single, FP32 value bits)
-    const float *hldv;                 // doubles: FP32 values
-    const uint16_t *hldt;              // doubles: targets relative to their column half
-    int64_t half;
 };
 
 // Gather pass over rows of X: each CTA stages R consecutive rows, then every
@@ -306,35 +301,12 @@ __device__ __forceinline__ void row_group(const RowArgs<T> &a, int64_t r0, unsig
     {
         const int nr = (int)min((int64_t)R, a.nrow - r0);
         __syncthreads();
-        // row maxima (FP32 pass only): largest |x| as the bit pattern of a non-negative float, so a
-        // NaN amplitude leaves a NaN maximum
-        unsigned rmax[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) rmax[r] = 0u;
-        constexpr bool kMax = std::is_same<T, float>::value;
         if (STAGED) {
             for (int64_t c = tid; c < a.ncol; c += kThreads) {
                 T v[R];
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[r] = r < nr ? conv<T>(a.X[(r0 + r) * a.ncol + c]) : T(0);
                 VecIO<T, R>::st(Xs + c * R, v);
-                if constexpr (kMax) {
-#pragma unroll
-                    for (int r = 0; r < R; ++r) rmax[r] = max(rmax[r], __float_as_uint(fabsf(v[r])));
-                }
-            }
-        } else if constexpr (kMax) {
-            if (a.rowmax)
-                for (int64_t c = tid; c < a.ncol; c += kThreads) rmax[0] = max(rmax[0], __float_as_uint(fabsf(a.X[r0 * a.ncol + c])));
-        }
-        __shared__ unsigned red_max[kMax ? R : 1][kMax ? kThreads / 32 : 1];
-        if constexpr (kMax) {
-            if (a.rowmax) {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const unsigned w = __reduce_max_sync(0xffffffffu, rmax[r]);
-                    if (lane == 0) red_max[r][warp] = w;
-                }
             }
         }
         // sign-folded J table: row key = 2*code + neg holds (neg ? -1 : 1) * J_r[code]; code 0 rows
@@ -355,14 +327,6 @@ __device__ __forceinline__ void row_group(const RowArgs<T> &a, int64_t r0, unsig
             VecIO<T, R>::st(Js + (size_t)key * R, v);
         }
         __syncthreads();
-        if constexpr (kMax) {
-            if (a.rowmax && tid < nr) {
-                unsigned m = 0u;
-                for (int w = 0; w < kThreads / 32; ++w) m = max(m, red_max[tid][w]);
-                a.rowmax[r0 + tid] = __uint_as_float(m);
-            }
-        }
-
         int64_t cb = (int64_t)warp * kGroupsPerWarp;
         int64_t nxt_s0 = 0, nxt_s1 = 0, nxt_d0 = 0, nxt_d1 = 0;
         if (cb + gi < a.ncol_out) {
@@ -469,168 +433,20 @@ __global__ void __launch_bounds__(Threads<T>::value) row_pass_kernel(const RowAr
     for (int64_t r0 = (int64_t)blockIdx.x * R; r0 < a.nrow; r0 += (int64_t)gridDim.x * R) row_group<T, R, STAGED>(a, r0, smem);
 }
 
-// Mixed-precision gather pass over 8 rows, one column half at a time.  With 4 rows the whole row
-// range fits shared memory; staging 8 rows of one half ([0, half) or [half, ncol)) in the same space
-// lets every excitation-list entry, loaded once from L2, feed 8 multiply-adds instead of 4.  Each
-// output column sums its entries with targets in the staged half (the split lists of the column
-// spin), writes that half's sum (with the diagonal term), and adds the other half's sum after the
-// second staging.  The 8 rows are kept as two 4-row interleaved arrays, so a 16-byte gather per
-// array has the bank pattern of the 4-row pass; the coefficient table of the singles likewise.
-constexpr int kHalfRows = 8;
-
-__host__ __device__ inline size_t halves_smem(int64_t half, int norb)
-{
-    return (size_t)32 * half + (size_t)64 * norb * norb;
-}
-
-__device__ __forceinline__ void row_halves(const RowArgs<float> &a, int64_t r0, unsigned char *smem)
-{
-    constexpr int kThreads = Threads<float>::value;
-    const int n2 = a.norb * a.norb;
-    const int64_t hw = a.half;  // rows of the staged arrays: the lower half is the wider one
-    float *Xa = reinterpret_cast<float *>(smem);                   // [hw][4]  rows 0-3
-    float *Xb = Xa + 4 * hw;                                        // [hw][4]  rows 4-7
-    float *Ja = Xb + 4 * hw;                                        // [2 n2][4]
-    float *Jb = Ja + 8 * n2;                                        // [2 n2][4]
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int gi = lane / kGroup, lig = lane % kGroup;
-    const int64_t ngroups = (kThreads / 32) * kGroupsPerWarp;
-    const int nr = (int)min((int64_t)kHalfRows, a.nrow - r0);
-    unsigned rmax[kHalfRows];
-#pragma unroll
-    for (int r = 0; r < kHalfRows; ++r) rmax[r] = 0u;
-    __shared__ unsigned red_h[kHalfRows];
-    __syncthreads();  // the previous row group is finished with shared memory
-    if (tid < kHalfRows) red_h[tid] = 0u;
-    // sign-folded J table of the 8 rows (row key = 2*code + neg; code 0 rows zero)
-    for (int key = tid; key < 2 * n2; key += kThreads) {
-        const int code = key >> 1;
-        float v[kHalfRows];
-#pragma unroll
-        for (int r = 0; r < kHalfRows; ++r) {
-            double sj = 0.0;
-            if (r < nr && code != 0)
-                for (uint64_t m = a.row_strings[r0 + r]; m; m &= m - 1ull) {
-                    const int k = __ffsll((long long)m) - 1;
-                    sj += __ldg(a.eri + (size_t)code * n2 + (size_t)k * (a.norb + 1));
-                }
-            v[r] = (float)((key & 1) ? -sj : sj);
-        }
-        *reinterpret_cast<float4 *>(Ja + (size_t)key * 4) = make_float4(v[0], v[1], v[2], v[3]);
-        *reinterpret_cast<float4 *>(Jb + (size_t)key * 4) = make_float4(v[4], v[5], v[6], v[7]);
-    }
-    for (int h = 0; h < 2; ++h) {
-        const int64_t c0 = h ? a.half : 0, c1 = h ? a.ncol : a.half;
-        if (h) __syncthreads();  // every column is finished with the first half
-        for (int64_t c = c0 + tid; c < c1; c += kThreads) {
-            float v[kHalfRows];
-#pragma unroll
-            for (int r = 0; r < kHalfRows; ++r) v[r] = r < nr ? a.X[(r0 + r) * a.ncol + c] : 0.f;
-            *reinterpret_cast<float4 *>(Xa + (c - c0) * 4) = make_float4(v[0], v[1], v[2], v[3]);
-            *reinterpret_cast<float4 *>(Xb + (c - c0) * 4) = make_float4(v[4], v[5], v[6], v[7]);
-#pragma unroll
-            for (int r = 0; r < kHalfRows; ++r) rmax[r] = max(rmax[r], __float_as_uint(fabsf(v[r])));
-        }
-        __syncthreads();
-        for (int64_t cb = (int64_t)warp * kGroupsPerWarp; cb < a.ncol_out; cb += ngroups) {
-            const int64_t c = cb + gi;
-            const bool valid = c < a.ncol_out;
-            float acc[kHalfRows];
-#pragma unroll
-            for (int r = 0; r < kHalfRows; ++r) acc[r] = 0.f;
-            if (valid) {
-                const int64_t s0 = a.hls_ptr[2 * c + h], s1 = a.hls_ptr[2 * c + h + 1];
-                const int64_t d0 = a.hld_ptr[2 * c + h], d1 = a.hld_ptr[2 * c + h + 1];
-                const int ls = (int)(s1 - s0), ld = (int)(d1 - d0);
-                for (int cb2 = 0; cb2 < ls; cb2 += kGroup * kListPad) {
-                    const int lc = min(kGroup * kListPad, ls - cb2);
-                    if (kListPad * lig >= lc) break;
-                    int64_t e0, e1;
-                    list_slots(s0, cb2, lc, lig, e0, e1);
-                    const uint4 p0 = __ldg(reinterpret_cast<const uint4 *>(a.hls + e0));
-                    const uint4 p1 = __ldg(reinterpret_cast<const uint4 *>(a.hls + e1));
-                    const uint32_t pk[4] = {p0.x, p0.z, p1.x, p1.z};
-                    const float vv[4] = {__uint_as_float(p0.y), __uint_as_float(p0.w), __uint_as_float(p1.y),
-                                         __uint_as_float(p1.w)};
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int64_t jl = (pk[u] ? (int64_t)pk_j(pk[u]) - c0 : 0);
-                        const float4 xa = *reinterpret_cast<const float4 *>(Xa + jl * 4);
-                        const float4 xb = *reinterpret_cast<const float4 *>(Xb + jl * 4);
-                        const float4 ja = *reinterpret_cast<const float4 *>(Ja + (size_t)pk_key(pk[u]) * 4);
-                        const float4 jb = *reinterpret_cast<const float4 *>(Jb + (size_t)pk_key(pk[u]) * 4);
-                        acc[0] += (vv[u] + ja.x) * xa.x;
-                        acc[1] += (vv[u] + ja.y) * xa.y;
-                        acc[2] += (vv[u] + ja.z) * xa.z;
-                        acc[3] += (vv[u] + ja.w) * xa.w;
-                        acc[4] += (vv[u] + jb.x) * xb.x;
-                        acc[5] += (vv[u] + jb.y) * xb.y;
-                        acc[6] += (vv[u] + jb.z) * xb.z;
-                        acc[7] += (vv[u] + jb.w) * xb.w;
-                    }
-                }
-                for (int cb2 = 0; cb2 < ld; cb2 += kGroup * kListPad) {
-                    const int lc = min(kGroup * kListPad, ld - cb2);
-                    if (kListPad * lig >= lc) break;
-                    int64_t e0, e1;
-                    list_slots(d0, cb2, lc, lig, e0, e1);
-                    // entries e0 .. e0 + 3: four values (16 bytes) and four 16-bit targets (8 bytes)
-                    const float4 v4 = __ldg(reinterpret_cast<const float4 *>(a.hldv + e0));
-                    const uint2 t4 = __ldg(reinterpret_cast<const uint2 *>(a.hldt + e0));
-                    const uint32_t jj[4] = {t4.x & 0xFFFFu, t4.x >> 16, t4.y & 0xFFFFu, t4.y >> 16};
-                    const float vv[4] = {v4.x, v4.y, v4.z, v4.w};
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        // targets are relative to the staged half; padding entries: target 0, value 0
-                        const int64_t jl = (int64_t)jj[u];
-                        const float4 xa = *reinterpret_cast<const float4 *>(Xa + jl * 4);
-                        const float4 xb = *reinterpret_cast<const float4 *>(Xb + jl * 4);
-                        acc[0] += vv[u] * xa.x;
-                        acc[1] += vv[u] * xa.y;
-                        acc[2] += vv[u] * xa.z;
-                        acc[3] += vv[u] * xa.w;
-                        acc[4] += vv[u] * xb.x;
-                        acc[5] += vv[u] * xb.y;
-                        acc[6] += vv[u] * xb.z;
-                        acc[7] += vv[u] * xb.w;
-                    }
-                }
-            }
-#pragma unroll
-            for (int off = kGroup / 2; off > 0; off >>= 1)
-#pragma unroll
-                for (int r = 0; r < kHalfRows; ++r) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], off, kGroup);
-            if (valid && lig < nr) {
-                double out = (double)pick<kHalfRows>(acc, lig);
-                const int64_t idx = (r0 + lig) * a.y_rs + c * a.y_cs;
-                if (h == 0) {
-                    if (a.hd) {
-                        const double xc = a.xd64 ? a.xd64[(r0 + lig) * a.ncol + c] : (double)a.X[(r0 + lig) * a.ncol + c];
-                        out += a.hd[idx] * xc;
-                    }
-                    a.Y[idx] = a.accumulate ? a.Y[idx] + out : out;
-                } else {
-                    a.Y[idx] += out;
-                }
-            }
-        }
-    }
-    if (a.rowmax) {  // uniform
-#pragma unroll
-        for (int r = 0; r < kHalfRows; ++r) {
-            const unsigned w = __reduce_max_sync(0xffffffffu, rmax[r]);
-            if (lane == 0) atomicMax(red_h + r, w);
-        }
-        __syncthreads();
-        if (tid < nr) a.rowmax[r0 + tid] = __uint_as_float(red_h[tid]);
-    }
-}
-
-__global__ void __launch_bounds__(Threads<float>::value) row_halves_kernel(const RowArgs<float> a)
+// Row passes of whole instances (range_rows.cuh).  A unit is (row block, part): a CTA takes a run of
+// consecutive units, so that all CTAs get the same number (+-1) and a row block's staging is shared
+// by the units of a run.
+template <typename T>
+__global__ void __launch_bounds__(kRangeThreads, 1) range_rows_kernel(const RangeArgs<T> a, int64_t units)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    for (int64_t r0 = (int64_t)blockIdx.x * kHalfRows; r0 < a.nrow; r0 += (int64_t)gridDim.x * kHalfRows)
-        row_halves(a, r0, smem);
+    int64_t u = units * blockIdx.x / gridDim.x;
+    const int64_t end = units * (blockIdx.x + 1) / gridDim.x;
+    while (u < end) {
+        const int p0 = (int)(u % kParts), p1 = (int)min((int64_t)kParts, p0 + (end - u));
+        range_rows<T>(a, u / kParts * kRangeRows<T>, p0, p1, smem);
+        u += p1 - p0;
+    }
 }
 
 template <typename T>
@@ -1088,6 +904,37 @@ __global__ void transpose_kernel(const T *__restrict__ in, T *__restrict__ out, 
     }
 }
 
+// One 32 x 32 tile of sigma[r][c] = st[c][r] + hd[r][c] x[r][c]: the beta pass' transposed result
+// and the diagonal term (x: the FP64 amplitudes where the caller has them)
+template <typename E>
+__device__ __forceinline__ void untranspose_tile(double (&tile)[32][33], const double *__restrict__ st,
+                                                 const double *__restrict__ hd, const E *__restrict__ x,
+                                                 const double *__restrict__ x64, double *__restrict__ sigma,
+                                                 int64_t rows, int64_t cols, int64_t by, int64_t bx)
+{
+    for (int j = threadIdx.y; j < 32; j += 8) {
+        const int64_t c = bx + j, r = by + threadIdx.x;
+        if (r < rows && c < cols) tile[j][threadIdx.x] = st[c * rows + r];
+    }
+    __syncthreads();
+    for (int j = threadIdx.y; j < 32; j += 8) {
+        const int64_t r = by + j, c = bx + threadIdx.x;
+        if (r < rows && c < cols) {
+            const int64_t i = r * cols + c;
+            sigma[i] = tile[threadIdx.x][j] + hd[i] * (x64 ? x64[i] : (double)x[i]);
+        }
+    }
+}
+
+template <typename E>
+__global__ void untranspose_kernel(const double *__restrict__ st, const double *__restrict__ hd,
+                                   const E *__restrict__ x, const double *__restrict__ x64, double *__restrict__ sigma,
+                                   int64_t rows, int64_t cols)
+{
+    __shared__ double tile[32][33];
+    untranspose_tile<E>(tile, st, hd, x, x64, sigma, rows, cols, (int64_t)blockIdx.y * 32, (int64_t)blockIdx.x * 32);
+}
+
 struct PassCfg {
     int R = 1;
     bool staged = false;
@@ -1168,6 +1015,7 @@ void launch_ab_src(const AbSrcArgs &a, int num_sms, cudaStream_t s)
 template <typename T>
 void set_attrs(int optin)
 {
+    SBD_CUDA(cudaFuncSetAttribute(range_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
     if constexpr (sizeof(T) == 4) {
         SBD_CUDA(cudaFuncSetAttribute(row_pass_kernel<T, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
         SBD_CUDA(cudaFuncSetAttribute(ab_pass_kernel<T, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
@@ -1180,18 +1028,13 @@ void set_attrs(int optin)
     SBD_CUDA(cudaFuncSetAttribute(ab_pass_kernel<T, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
 }
 
-// the mixed 8-row pass over column halves applies when its staged half and tables fit
-bool halves_fit(const RowArgs<float> &a, size_t limit)
+template <typename T>
+void launch_range(const Ctx &c, const RangeArgs<T> &a, cudaStream_t s)
 {
-    return a.hls_ptr && a.ncol_out == a.ncol && a.half > 0 && halves_smem(a.half, a.norb) <= limit;
-}
-
-void launch_halves(const RowArgs<float> &a, cudaStream_t s)
-{
-    const int64_t groups = (a.nrow + kHalfRows - 1) / kHalfRows;
-    const int grid = (int)(groups < 65535 ? groups : 65535);
-    row_halves_kernel<<<grid, Threads<float>::value, halves_smem(a.half, a.norb), s>>>(a);
-    SBD_LAUNCH("row_halves_kernel");
+    const int64_t units = (a.nrow + kRangeRows<T> - 1) / kRangeRows<T> * kParts;
+    const int grid = (int)std::min<int64_t>(units, c.num_sms);
+    range_rows_kernel<T><<<grid, kRangeThreads, range_smem(c.smem_optin), s>>>(a, units);
+    SBD_LAUNCH("range_rows_kernel");
 }
 
 template <typename T>
@@ -1270,58 +1113,11 @@ void timed(Ctx &c, int slot, cudaStream_t s, F &&launch)
     c.pending.push_back({slot, a, b});
 }
 
-// Arguments of the three gather passes of one instance: beta pass on C, alpha pass on its
-// transpose Ct, alpha-beta pass on C (the single-instance and the batched launches share them).
+// Arguments of the two-operand alpha-beta pass.
 template <typename T>
-void make_args(const Ctx &c, const typename In<T>::type *C, double *S, const double *c64,
-               const typename In<T>::type *Ct, RowArgs<T> &rb, RowArgs<T> &ra, AbArgs<T> &ab)
+void make_ab_args(const Ctx &c, const typename In<T>::type *C, double *S, AbArgs<T> &ab)
 {
     const SpinTables &ta = c.sp[0], &tb = c.sp[1];
-    rb = RowArgs<T>{};
-    rb.X = C;
-    rb.nrow = c.nA;
-    rb.ncol = c.nB;
-    rb.ncol_out = c.nB;
-    rb.Y = S;
-    rb.y_rs = c.nB;
-    rb.y_cs = 1;
-    rb.accumulate = 0;
-    rb.hd = c.hd;
-    rb.xd64 = c64;
-    rb.row_strings = ta.strings;
-    rb.norb = c.norb;
-    rb.eri = c.eri64;
-    rb.s_ptr = tb.sig_s_ptr;
-    rb.d_ptr = tb.sig_d_ptr;
-    rb.lists = lists_of<T>(tb);
-    rb.hls_ptr = tb.hs_ptr;
-    rb.hld_ptr = tb.hd_ptr;
-    rb.hls = tb.hs;
-    rb.hldv = tb.hdv;
-    rb.hldt = tb.hdt;
-    rb.half = tb.half;
-
-    ra = rb;
-    ra.X = Ct;
-    ra.nrow = c.nB;
-    ra.ncol = c.nA;
-    ra.ncol_out = c.nA;
-    ra.y_rs = 1;
-    ra.y_cs = c.nB;
-    ra.accumulate = 1;
-    ra.hd = nullptr;
-    ra.xd64 = nullptr;
-    ra.row_strings = tb.strings;
-    ra.s_ptr = ta.sig_s_ptr;
-    ra.d_ptr = ta.sig_d_ptr;
-    ra.lists = lists_of<T>(ta);
-    ra.hls_ptr = ta.hs_ptr;
-    ra.hld_ptr = ta.hd_ptr;
-    ra.hls = ta.hs;
-    ra.hldv = ta.hdv;
-    ra.hldt = ta.hdt;
-    ra.half = ta.half;
-
     ab = AbArgs<T>{};
     ab.C = C;
     ab.S = S;
@@ -1337,42 +1133,75 @@ void make_args(const Ctx &c, const typename In<T>::type *C, double *S, const dou
 }
 
 template <typename T>
+const typename RangeVal<T>::type *range_vals(const float *v32, const double *v64, const float2 *vx2)
+{
+    if constexpr (kIsF2<T>) return vx2;
+    else if constexpr (sizeof(T) == 4) return v32;
+    else return v64;
+}
+
+// Row pass over the lists of spin `ls` of a handle: X and Y have that spin's strings as rows of
+// the other spin's length.
+template <typename T>
+RangeArgs<T> range_args(const Ctx &c, int ls, const typename In<T>::type *X, double *Y, int accumulate)
+{
+    const SpinTables &t = c.sp[ls], &o = c.sp[1 - ls];
+    const RangeLists &r = t.rl;
+    RangeArgs<T> a{};
+    a.X = X;
+    a.Y = Y;
+    a.n = t.n;
+    a.nrow = o.n;
+    a.accumulate = accumulate;
+    a.npair = npairs(c.norb);
+    a.jstaged = range_j_staged(c.smem_optin, c.norb);
+    a.w = r.w;
+    a.ng = r.ng;
+    a.q = 1;
+    a.jg = o.rl.jg;
+    a.zi = r.zi;
+    a.qd = r.qd;
+    a.qs = r.qs;
+    a.dt = r.dt;
+    a.sm = r.sm;
+    a.dv = range_vals<T>(r.dv32, r.dv64, r.dvx2);
+    a.sv = range_vals<T>(r.sv32, r.sv64, r.svx2);
+    return a;
+}
+
+// The transposed copy of C is kept in the output buffer until the beta pass has read it, and the
+// beta pass' transposed result in the handle's work vector, so the row passes need no memory of
+// their own.
+template <typename T>
 void apply(Ctx &c, const typename In<T>::type *C, double *S, const double *c64, cudaStream_t s)
 {
     using E = typename In<T>::type;
     const int n2 = c.norb * c.norb;
-    const int rmax = kRowsMax<T>;
     const size_t lim = smem_limit(c);
     const int base = kSlotBase<T>;
-    E *Ct = static_cast<E *>(c.work_t);
+    E *Ct = reinterpret_cast<E *>(S);
+    double *St = static_cast<double *>(c.work_t);
     // the mixed alpha-beta pass takes the row maxima of C from the beta pass
     const bool src = std::is_same<T, float>::value && src_fits(c);
     timed(c, base + 0, s, [&] { transpose<E>(C, Ct, c.nA, c.nB, s); });
-    RowArgs<T> rb, ra;
-    AbArgs<T> ab;
-    make_args<T>(c, C, S, c64, Ct, rb, ra, ab);
+    RangeArgs<T> rb = range_args<T>(c, 1, Ct, St, 0), ra = range_args<T>(c, 0, C, S, 1);
     if (src) rb.rowmax = c.rowmax;
-    if constexpr (std::is_same<T, float>::value) {
-        // 8 rows over column halves where they fit, else 4 rows over the whole row
-        timed(c, base + 1, s, [&] {
-            if (halves_fit(rb, lim)) launch_halves(rb, s);
-            else launch_row<T>(rb, choose(c.nB, n2, sizeof(T), rmax, lim), s);
-        });
-        timed(c, base + 2, s, [&] {
-            if (halves_fit(ra, lim)) launch_halves(ra, s);
-            else launch_row<T>(ra, choose(c.nA, n2, sizeof(T), rmax, lim), s);
-        });
-    } else {
-        timed(c, base + 1, s, [&] { launch_row<T>(rb, choose(c.nB, n2, sizeof(T), rmax, lim), s); });
-        timed(c, base + 2, s, [&] { launch_row<T>(ra, choose(c.nA, n2, sizeof(T), rmax, lim), s); });
-    }
+    timed(c, base + 1, s, [&] {
+        launch_range<T>(c, rb, s);
+        const dim3 grid((unsigned)((c.nB + 31) / 32), (unsigned)((c.nA + 31) / 32));
+        untranspose_kernel<E><<<grid, dim3(32, 8), 0, s>>>(St, c.hd, C, c64, S, c.nA, c.nB);
+        SBD_LAUNCH("untranspose_kernel");
+    });
+    timed(c, base + 2, s, [&] { launch_range<T>(c, ra, s); });
     if constexpr (std::is_same<T, float>::value) {
         if (src) {
             timed(c, base + 3, s, [&] { launch_ab_src(src_args(c, C, S, c.rowmax), c.num_sms, s); });
             return;
         }
     }
-    timed(c, base + 3, s, [&] { launch_ab<T>(ab, choose(c.nB, n2, sizeof(T), rmax, lim), s); });
+    AbArgs<T> ab;
+    make_ab_args<T>(c, C, S, ab);
+    timed(c, base + 3, s, [&] { launch_ab<T>(ab, choose(c.nB, n2, sizeof(T), kRowsMax<T>, lim), s); });
 }
 
 // ---------------------------------------------------------------------------
@@ -1383,8 +1212,11 @@ void apply(Ctx &c, const typename In<T>::type *C, double *S, const double *c64, 
 
 template <typename T>
 struct TDesc {
-    const T *in;
-    T *out;
+    const T *x;         // amplitudes [rows][cols]
+    const double *x64;  // FP64 amplitudes for the diagonal term, or null
+    double *y;          // sigma; holds the transposed amplitudes until the beta pass has read them
+    double *st;         // the beta pass' transposed result
+    const double *hd;
     int64_t rows, cols;
 };
 
@@ -1408,8 +1240,8 @@ Layout layout_for(int m)
     L.off_a = take(sizeof(int64_t) * (m + 1));
     L.off_ab = take(sizeof(int64_t) * (m + 1));
     L.td = take(sizeof(TDesc<typename In<T>::type>) * m);
-    L.rb = take(sizeof(RowArgs<T>) * m);
-    L.ra = take(sizeof(RowArgs<T>) * m);
+    L.rb = take(sizeof(RangeArgs<T>) * m);
+    L.ra = take(sizeof(RangeArgs<T>) * m);
     L.ab = take(sizeof(AbArgs<T>) * m);
     L.src = take(sizeof(AbSrcArgs) * m);
     L.total = o;
@@ -1428,10 +1260,12 @@ __device__ __forceinline__ int find_slot(const int64_t *off, int n, int64_t item
     return lo;
 }
 
-template <typename T>
+// BACK 0: the transposed amplitudes of every slot; 1: sigma = the beta pass' result transposed back
+// plus the diagonal term
+template <typename T, bool BACK>
 __global__ void transpose_batch_kernel(const int *pn, const int64_t *off, const TDesc<T> *td)
 {
-    __shared__ T tile[32][33];
+    __shared__ double tile[32][33];
     const int n = *pn;
     const int64_t total = off[n];
     for (int64_t it = blockIdx.x; it < total; it += gridDim.x) {
@@ -1440,14 +1274,19 @@ __global__ void transpose_batch_kernel(const int *pn, const int64_t *off, const 
         const int64_t lt = it - off[sl], tx = (d.cols + 31) / 32;
         const int64_t by = (lt / tx) * 32, bx = (lt % tx) * 32;
         __syncthreads();
-        for (int j = threadIdx.y; j < 32; j += 8) {
-            const int64_t r = by + j, c = bx + threadIdx.x;
-            if (r < d.rows && c < d.cols) tile[j][threadIdx.x] = d.in[r * d.cols + c];
-        }
-        __syncthreads();
-        for (int j = threadIdx.y; j < 32; j += 8) {
-            const int64_t c = bx + j, r = by + threadIdx.x;
-            if (r < d.rows && c < d.cols) d.out[c * d.rows + r] = tile[threadIdx.x][j];
+        if constexpr (BACK) {
+            untranspose_tile<T>(tile, d.st, d.hd, d.x, d.x64, d.y, d.rows, d.cols, by, bx);
+        } else {
+            T *out = reinterpret_cast<T *>(d.y);
+            for (int j = threadIdx.y; j < 32; j += 8) {
+                const int64_t r = by + j, c = bx + threadIdx.x;
+                if (r < d.rows && c < d.cols) tile[j][threadIdx.x] = (double)d.x[r * d.cols + c];
+            }
+            __syncthreads();
+            for (int j = threadIdx.y; j < 32; j += 8) {
+                const int64_t c = bx + j, r = by + threadIdx.x;
+                if (r < d.rows && c < d.cols) out[c * d.rows + r] = (T)tile[threadIdx.x][j];
+            }
         }
     }
 }
@@ -1485,14 +1324,17 @@ __device__ __forceinline__ void item_loop(const int *pn, const int64_t *off, con
     }
 }
 
-template <typename T, int R>
-__global__ void __launch_bounds__(Threads<T>::value) row_batch_kernel(const int *pn, const int64_t *off,
-                                                                      const RowArgs<T> *args,
+template <typename T>
+__global__ void __launch_bounds__(kRangeThreads, 1) range_batch_kernel(const int *pn, const int64_t *off,
+                                                                      const RangeArgs<T> *args,
                                                                       unsigned long long *counter)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ RowArgs<T> sa;
-    item_loop(pn, off, args, counter, sa, [&](int64_t li) { row_group<T, R, true>(sa, li * R, smem); });
+    __shared__ RangeArgs<T> sa;
+    item_loop(pn, off, args, counter, sa, [&](int64_t li) {
+        const int per = kParts / sa.q, p0 = (int)(li % sa.q) * per;
+        range_rows<T>(sa, li / sa.q * kRangeRows<T>, p0, p0 + per, smem);
+    });
 }
 
 template <typename T, int R>
@@ -1515,18 +1357,12 @@ __global__ void __launch_bounds__(kSrcThreads, 1) ab_src_batch_kernel(const int 
     item_loop(pn, off, args, counter, sa, [&](int64_t li) { src_row<RS>(sa, li, smem); });
 }
 
-__global__ void __launch_bounds__(Threads<float>::value) row_halves_batch_kernel(const int *pn, const int64_t *off,
-                                                                               const RowArgs<float> *args,
-                                                                               unsigned long long *counter)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ RowArgs<float> sa;
-    item_loop(pn, off, args, counter, sa, [&](int64_t li) { row_halves(sa, li * kHalfRows, smem); });
-}
+constexpr int kHalfRows = 8;  // the largest rows-per-item setting (mixed)
 
 size_t batch_smem(size_t elem, int R, int max_strings, int max_norb)
 {
-    if (R == kHalfRows) return halves_smem((max_strings + 1) / 2, max_norb);
+    // 8 rows: the limit that this setting has always had (8 rows of one column half and their J tables)
+    if (R == kHalfRows) return (size_t)32 * ((max_strings + 1) / 2) + (size_t)64 * max_norb * max_norb;
     return round16((size_t)max_strings * R * elem) + (size_t)2 * max_norb * max_norb * R * elem;
 }
 
@@ -1534,8 +1370,8 @@ size_t batch_smem(size_t elem, int R, int max_strings, int max_norb)
 
 struct SigmaBatch {
     sbd_precision prec = SBD_MIXED;
-    int max_slots = 0, R = 1, device = 0, grid_pass = 0, grid_t = 0, grid_src = 0;
-    size_t smem = 0;
+    int max_slots = 0, R = 1, device = 0, grid_range = 0, grid_ab = 0, grid_t = 0, grid_src = 0;
+    size_t smem = 0, range_smem = 0;  // alpha-beta pass, row passes
     bool src = false;     // mixed: the column-stationary alpha-beta pass (when its table and accumulator fit)
     int src_rs = 0;       // its W row stride for the largest slot (8 or 4 float4)
     size_t src_smem = 0;
@@ -1556,15 +1392,23 @@ void batch_set(SigmaBatch *b, const SigmaSlot *slots, int n)
     int64_t *oa = reinterpret_cast<int64_t *>(h + L.off_a), *oab = reinterpret_cast<int64_t *>(h + L.off_ab);
     using E = typename In<T>::type;
     TDesc<E> *td = reinterpret_cast<TDesc<E> *>(h + L.td);
-    RowArgs<T> *rb = reinterpret_cast<RowArgs<T> *>(h + L.rb), *ra = reinterpret_cast<RowArgs<T> *>(h + L.ra);
+    RangeArgs<T> *rb = reinterpret_cast<RangeArgs<T> *>(h + L.rb), *ra = reinterpret_cast<RangeArgs<T> *>(h + L.ra);
     AbArgs<T> *ab = reinterpret_cast<AbArgs<T> *>(h + L.ab);
     ot[0] = ob[0] = oa[0] = oab[0] = 0;
+    // row blocks are cut into q pieces, enough for about eight work items per CTA
+    int64_t blocks = 0;
+    for (int i = 0; i < n; ++i) blocks += (std::min(slots[i].c->nA, slots[i].c->nB) + kRangeRows<T> - 1) / kRangeRows<T>;
+    int q = 1;
+    while (q < kParts && blocks * q < (int64_t)8 * b->grid_range) q *= 2;
     for (int i = 0; i < n; ++i) {
         const SigmaSlot &sl = slots[i];
         const Ctx &c = *sl.c;
         const E *x = static_cast<const E *>(sl.x);
-        E *xt = static_cast<E *>(sl.xt);
-        make_args<T>(c, x, sl.y, sl.x64, xt, rb[i], ra[i], ab[i]);
+        double *st = static_cast<double *>(sl.xt);
+        rb[i] = range_args<T>(c, 1, reinterpret_cast<const E *>(sl.y), st, 0);
+        ra[i] = range_args<T>(c, 0, x, sl.y, 1);
+        rb[i].q = ra[i].q = q;
+        make_ab_args<T>(c, x, sl.y, ab[i]);
         if constexpr (std::is_same<T, float>::value) {
             if (b->src) {
                 rb[i].rowmax = c.rowmax;
@@ -1573,10 +1417,10 @@ void batch_set(SigmaBatch *b, const SigmaSlot *slots, int n)
                 reinterpret_cast<AbSrcArgs *>(h + L.src)[i] = sa;
             }
         }
-        td[i] = TDesc<E>{x, xt, c.nA, c.nB};
+        td[i] = TDesc<E>{x, sl.x64, sl.y, st, c.hd, c.nA, c.nB};
         ot[i + 1] = ot[i] + ((c.nA + 31) / 32) * ((c.nB + 31) / 32);
-        ob[i + 1] = ob[i] + (c.nA + b->R - 1) / b->R;
-        oa[i + 1] = oa[i] + (c.nB + b->R - 1) / b->R;
+        ob[i + 1] = ob[i] + (c.nA + kRangeRows<T> - 1) / kRangeRows<T> * q;
+        oa[i + 1] = oa[i] + (c.nB + kRangeRows<T> - 1) / kRangeRows<T> * q;
         oab[i + 1] = oab[i] + c.nA;
     }
 }
@@ -1584,33 +1428,23 @@ void batch_set(SigmaBatch *b, const SigmaSlot *slots, int n)
 template <typename T, int R>
 void batch_launch_r(SigmaBatch *b, cudaStream_t s)
 {
-    constexpr int kThreads = Threads<T>::value;
     const Layout &L = b->L;
     unsigned char *d = b->dev;
     const int *pn = reinterpret_cast<const int *>(d + L.n);
     using E = typename In<T>::type;
-    transpose_batch_kernel<E><<<b->grid_t, dim3(32, 8), 0, s>>>(pn, reinterpret_cast<const int64_t *>(d + L.off_t),
-                                                                reinterpret_cast<const TDesc<E> *>(d + L.td));
+    const int64_t *off_t = reinterpret_cast<const int64_t *>(d + L.off_t);
+    const TDesc<E> *td = reinterpret_cast<const TDesc<E> *>(d + L.td);
+    transpose_batch_kernel<E, false><<<b->grid_t, dim3(32, 8), 0, s>>>(pn, off_t, td);
     SBD_LAUNCH("transpose_batch_kernel");
-    if constexpr (R == kHalfRows) {
-        row_halves_batch_kernel<<<b->grid_pass, kThreads, b->smem, s>>>(
-            pn, reinterpret_cast<const int64_t *>(d + L.off_b), reinterpret_cast<const RowArgs<float> *>(d + L.rb),
-            b->counters);
-        SBD_LAUNCH("row_halves_batch_kernel");
-        row_halves_batch_kernel<<<b->grid_pass, kThreads, b->smem, s>>>(
-            pn, reinterpret_cast<const int64_t *>(d + L.off_a), reinterpret_cast<const RowArgs<float> *>(d + L.ra),
-            b->counters + 1);
-        SBD_LAUNCH("row_halves_batch_kernel");
-    } else {
-        row_batch_kernel<T, R><<<b->grid_pass, kThreads, b->smem, s>>>(
-            pn, reinterpret_cast<const int64_t *>(d + L.off_b), reinterpret_cast<const RowArgs<T> *>(d + L.rb),
-            b->counters);
-        SBD_LAUNCH("row_batch_kernel");
-        row_batch_kernel<T, R><<<b->grid_pass, kThreads, b->smem, s>>>(
-            pn, reinterpret_cast<const int64_t *>(d + L.off_a), reinterpret_cast<const RowArgs<T> *>(d + L.ra),
-            b->counters + 1);
-        SBD_LAUNCH("row_batch_kernel");
-    }
+    range_batch_kernel<T><<<b->grid_range, kRangeThreads, b->range_smem, s>>>(
+        pn, reinterpret_cast<const int64_t *>(d + L.off_b), reinterpret_cast<const RangeArgs<T> *>(d + L.rb), b->counters);
+    SBD_LAUNCH("range_batch_kernel");
+    transpose_batch_kernel<E, true><<<b->grid_t, dim3(32, 8), 0, s>>>(pn, off_t, td);
+    SBD_LAUNCH("transpose_batch_kernel");
+    range_batch_kernel<T><<<b->grid_range, kRangeThreads, b->range_smem, s>>>(
+        pn, reinterpret_cast<const int64_t *>(d + L.off_a), reinterpret_cast<const RangeArgs<T> *>(d + L.ra),
+        b->counters + 1);
+    SBD_LAUNCH("range_batch_kernel");
     if (std::is_same<T, float>::value && b->src) {
         const int64_t *off_ab = reinterpret_cast<const int64_t *>(d + L.off_ab);
         const AbSrcArgs *src_args_d = reinterpret_cast<const AbSrcArgs *>(d + L.src);
@@ -1622,7 +1456,7 @@ void batch_launch_r(SigmaBatch *b, cudaStream_t s)
         return;
     }
     if constexpr (R != kHalfRows) {  // 8 rows per item only come with the column-stationary pass
-        ab_batch_kernel<T, R><<<b->grid_pass, kThreads, b->smem, s>>>(
+        ab_batch_kernel<T, R><<<b->grid_ab, Threads<T>::value, b->smem, s>>>(
             pn, reinterpret_cast<const int64_t *>(d + L.off_ab), reinterpret_cast<const AbArgs<T> *>(d + L.ab),
             b->counters + 2);
         SBD_LAUNCH("ab_batch_kernel");
@@ -1632,22 +1466,18 @@ void batch_launch_r(SigmaBatch *b, cudaStream_t s)
 template <typename T, int R>
 void batch_attrs(SigmaBatch *b)
 {
-    constexpr int kThreads = Threads<T>::value;
-    int occ_row = 0, occ_ab = 1 << 20;
-    if constexpr (R == kHalfRows) {
-        SBD_CUDA(cudaFuncSetAttribute(row_halves_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)b->smem));
-        SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_row, row_halves_batch_kernel, kThreads, b->smem));
-    } else {
-        SBD_CUDA(cudaFuncSetAttribute(row_batch_kernel<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
-        SBD_CUDA(cudaFuncSetAttribute(ab_batch_kernel<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
-        SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_row, row_batch_kernel<T, R>, kThreads, b->smem));
-        SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_ab, ab_batch_kernel<T, R>, kThreads, b->smem));
-    }
-    const int occ = std::max(1, std::min(occ_row, occ_ab));
     int sms = 0;
     SBD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
-    b->grid_pass = sms * occ;
+    SBD_CUDA(cudaFuncSetAttribute(range_batch_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)b->range_smem));
+    b->grid_range = sms;
+    if constexpr (R != kHalfRows) {
+        int occ_ab = 0;
+        SBD_CUDA(cudaFuncSetAttribute(ab_batch_kernel<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
+        SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_ab, ab_batch_kernel<T, R>, Threads<T>::value,
+                                                               b->smem));
+        b->grid_ab = sms * std::max(1, occ_ab);
+    }
     b->grid_t = sms * 8;
     if (b->src) {
         int occ_src = 0;
@@ -1678,7 +1508,6 @@ void sigma_prepare(Ctx &c)
     set_attrs<F2>(lim);
     SBD_CUDA(cudaFuncSetAttribute(ab_src_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
     SBD_CUDA(cudaFuncSetAttribute(ab_src_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-    SBD_CUDA(cudaFuncSetAttribute(row_halves_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
     // max |(pq|rs)| of the FP32 integrals, for the fixed-point scale of the alpha-beta pass
     const int64_t n4 = (int64_t)c.norb * c.norb * c.norb * c.norb;
     unsigned *m = reinterpret_cast<unsigned *>(c.dstat);  // status words are free after create
@@ -1729,6 +1558,12 @@ SigmaBatch *sigma_batch_create(int max_slots, sbd_precision prec, int R, int max
     b->R = R;
     b->device = device;
     b->smem = smem;
+    int optin = 0;
+    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess) {
+        delete b;
+        fail(SBD_ERR_CUDA, "batched sigma: the device does not report its shared memory");
+    }
+    b->range_smem = range_smem(optin);
     b->src_rs = max_norb >= 2 ? src_rs(npairs(max_norb), max_strings, sigma_batch_smem_limit(device)) : 0;
     b->src_smem = b->src_rs ? src_smem(npairs(max_norb), max_strings, b->src_rs) : 0;
     b->src = prec == SBD_MIXED && b->src_rs > 0;
@@ -1794,7 +1629,7 @@ void sigma_batch_launch(SigmaBatch *b, cudaStream_t s)
     }
 }
 
-int64_t sigma_batch_launches(const SigmaBatch *) { return 4; }
+int64_t sigma_batch_launches(const SigmaBatch *) { return 5; }
 
 void sigma_batch_destroy(SigmaBatch *b)
 {
@@ -1824,21 +1659,28 @@ void apply_block(BlockPlan &p, const typename In<T>::type *Cb, double *S, cudaSt
     transpose<E>(Cb, Ct, nj, c.nB, s, src ? p.rowmax : nullptr);
     // beta pass: the output rows inside the block
     const int64_t lo = std::max(p.r0, p.j0), hi = std::min(p.r1, p.j1);
-    RowArgs<T> rb, ra;
-    AbArgs<T> ab;
-    make_args<T>(c, Cb, S, nullptr, Ct, rb, ra, ab);
+    RowArgs<T> row{};
+    row.norb = c.norb;
+    row.eri = c.eri64;
+    row.accumulate = 1;
     if (lo < hi) {
-        RowArgs<T> b = rb;
+        RowArgs<T> b = row;
         b.X = Cb + (lo - p.j0) * c.nB;
         b.nrow = hi - lo;
+        b.ncol = b.ncol_out = c.nB;
         b.Y = S + (lo - p.r0) * c.nB;
-        b.accumulate = 1;
+        b.y_rs = c.nB;
+        b.y_cs = 1;
         b.hd = c.hd + lo * c.nB;
         b.xd64 = x64 ? x64 + (lo - p.r0) * c.nB : nullptr;
         b.row_strings = ta.strings + lo;
+        b.s_ptr = tb.sig_s_ptr;
+        b.d_ptr = tb.sig_d_ptr;
+        b.lists = lists_of<T>(tb);
         launch_row<T>(b, choose(c.nB, n2, sizeof(T), rmax, lim), s);
     }
     // alpha pass: rows of the transposed block, output columns r0..r1, lists restricted to the block
+    RowArgs<T> ra = row;
     ra.X = Ct;
     ra.nrow = c.nB;
     ra.ncol = nj;
@@ -1846,7 +1688,7 @@ void apply_block(BlockPlan &p, const typename In<T>::type *Cb, double *S, cudaSt
     ra.Y = S;
     ra.y_rs = 1;
     ra.y_cs = c.nB;
-    ra.accumulate = 1;
+    ra.row_strings = tb.strings;
     ra.s_ptr = p.sig_s_ptr;
     ra.d_ptr = p.sig_d_ptr;
     if constexpr (kIsF2<T>) ra.lists = Lists<F2>{p.s_pk_sig, p.s_vx2, p.d_j_sig, p.d_vx2};
@@ -1864,12 +1706,11 @@ void apply_block(BlockPlan &p, const typename In<T>::type *Cb, double *S, cudaSt
             return;
         }
     }
-    ab.C = Cb;
-    ab.S = S;
+    AbArgs<T> ab;
+    make_ab_args<T>(c, Cb, S, ab);
     ab.nA = nr;
     ab.as_ptr = p.s_ptr;
     ab.as_pk = p.s_pk;
-    (void)tb;
     launch_ab<T>(ab, choose(c.nB, n2, sizeof(T), rmax, lim), s);
 }
 

@@ -25,6 +25,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "range_rows.cuh"
 
 namespace sbd {
 
@@ -518,46 +519,175 @@ __global__ void src_slice_order_kernel(const uint32_t *__restrict__ item_in, con
     }
 }
 
-// Split of each source list at target `half`: ptr2[2i] = start of list i, ptr2[2i+1] = its first
-// entry with target >= half (targets ascend in the canonical lists), ptr2[2n] = end of the last list
-__global__ void half_split_kernel(const int64_t *__restrict__ ptr, const int32_t *__restrict__ tgt, int64_t n,
-                                  int64_t half, int64_t *ptr2)
+// ---- range lists of the row passes (RangeLists) --------------------------------
+
+// first entry of [lo, hi) with target >= key (targets ascend)
+__device__ __forceinline__ int64_t first_at_least(const int32_t *__restrict__ tgt, int64_t lo, int64_t hi, int64_t key)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t lo = ptr[i], hi = ptr[i + 1];
-        ptr2[2 * i] = lo;
-        while (lo < hi) {
-            const int64_t mid = (lo + hi) / 2;
-            if (tgt[mid] < half) lo = mid + 1;
-            else hi = mid;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) / 2;
+        if (tgt[mid] < key) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// cnt[g*n + i] = blocks of `pad` entries that string i's list needs for the targets of range g
+__global__ void range_count_kernel(const int64_t *__restrict__ ptr, const int32_t *__restrict__ tgt, int64_t n, int w,
+                                   int ng, int pad, uint32_t *cnt)
+{
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n * ng; x += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t g = x / n, i = x - g * n;
+        const int64_t lo = first_at_least(tgt, ptr[i], ptr[i + 1], g * w);
+        const int64_t hi = first_at_least(tgt, lo, ptr[i + 1], (g + 1) * w);
+        cnt[x] = (uint32_t)((hi - lo + pad - 1) / pad);
+    }
+}
+
+// One CTA per (range, part): counting sort of the part's strings by descending doubles blocks (cd, by
+// string) into zi.  (The order of equal lengths is left to the atomics: a list's sum does not depend
+// on its position.)
+constexpr int kOrderKeys = 1024;
+__global__ void __launch_bounds__(256) range_order_kernel(int64_t n, const uint32_t *__restrict__ cd,
+                                                          int32_t *zi)
+{
+    __shared__ unsigned hist[kOrderKeys];
+    __shared__ unsigned wsum[8];
+    const int64_t g = blockIdx.x / kParts, p = blockIdx.x % kParts;
+    const int tid = threadIdx.x;
+    for (int k = tid; k < kOrderKeys; k += 256) hist[k] = 0u;
+    __syncthreads();
+    for (int64_t i = p + (int64_t)kParts * tid; i < n; i += (int64_t)kParts * 256)
+        atomicAdd(hist + (kOrderKeys - 1 - min(cd[g * n + i], (unsigned)kOrderKeys - 1u)), 1u);
+    __syncthreads();
+    // exclusive prefix over the keys, four per thread
+    unsigned v[4], s = 0u;
+    for (int k = 0; k < 4; ++k) v[k] = hist[4 * tid + k], s += v[k];
+    unsigned x = s;
+    for (int off = 1; off < 32; off <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, x, off);
+        if ((tid & 31) >= off) x += y;
+    }
+    if ((tid & 31) == 31) wsum[tid >> 5] = x;
+    __syncthreads();
+    unsigned run = x - s;
+    for (int q = 0; q < (tid >> 5); ++q) run += wsum[q];
+    for (int k = 0; k < 4; ++k) {
+        hist[4 * tid + k] = run;
+        run += v[k];
+    }
+    __syncthreads();
+    const int64_t nq = part_group(n, kParts);
+    const int64_t z0 = kListGroup * (g * nq + part_group(n, (int)p));
+    const int64_t z1 = kListGroup * (g * nq + part_group(n, (int)p + 1));
+    for (int64_t i = p + (int64_t)kParts * tid; i < n; i += (int64_t)kParts * 256)
+        zi[z0 + atomicAdd(hist + (kOrderKeys - 1 - min(cd[g * n + i], (unsigned)kOrderKeys - 1u)), 1u)] = (int32_t)i;
+    for (int64_t z = z0 + (n - p + kParts - 1) / kParts + tid; z < z1; z += 256) zi[z] = -1;
+}
+
+// Blocks of each group (the longest of its lists), and the kListHas mark of its strings
+__global__ void range_group_kernel(int64_t n, int64_t groups, int64_t total, const uint32_t *__restrict__ cd,
+                                  const uint32_t *__restrict__ cs, int32_t *zi, int64_t *nd, int64_t *ns)
+{
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t g = q / groups;
+        uint32_t md = 0, ms = 0;
+        for (int o = 0; o < kListGroup; ++o) {
+            const int32_t i = zi[kListGroup * q + o];
+            if (i < 0) continue;
+            const uint32_t d = cd[g * n + i], s = cs[g * n + i];
+            md = max(md, d);
+            ms = max(ms, s);
+            if (d | s) zi[kListGroup * q + o] = i | kListHas;
         }
-        ptr2[2 * i + 1] = lo;
-        if (i == n - 1) ptr2[2 * n] = ptr[n];
+        nd[q] = md;
+        ns[q] = ms;
     }
 }
 
-// Doubles of the half-split lists: val[o] = FP32 of v[perm[o]], tgt[o] = its target relative to
-// the column half it lies in (target - half for targets >= half); zeros for padding
-__global__ void gather_half_doubles_kernel(const int64_t *__restrict__ perm, int64_t m,
-                                           const int32_t *__restrict__ j, const double *__restrict__ v,
-                                           int64_t half, float *val, uint16_t *tgt)
+// x = hi + lo with hi the FP32 rounding of x and lo the FP32 rounding of the remainder
+__device__ __forceinline__ float2 split2(double x)
 {
-    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < m; o += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t e = perm[o];
-        const int64_t jj = e >= 0 ? (int64_t)j[e] : 0;
-        val[o] = e >= 0 ? __double2float_rn(v[e]) : 0.f;
-        tgt[o] = (uint16_t)(jj >= half ? jj - half : jj);
+    const float hi = __double2float_rn(x);
+    return make_float2(hi, __double2float_rn(x - (double)hi));
+}
+
+// One warp per list (group q, place o): copies its entries (KIND 1 singles, 2 doubles) to their blocks.
+template <int KIND>
+__global__ void range_fill_kernel(const int64_t *__restrict__ ptr, const int32_t *__restrict__ tgt,
+                                  const uint32_t *__restrict__ pk, const double *__restrict__ val, int64_t groups,
+                                  int norb, RangeLists r)
+{
+    constexpr int B = KIND == 1 ? kRangeSingles : kRangeDoubles;
+    const uint32_t *qp = KIND == 1 ? r.qs : r.qd;
+    const int lane = threadIdx.x & 31;
+    const int64_t lists = kListGroup * groups * r.ng;
+    for (int64_t z = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; z < lists;
+         z += (int64_t)gridDim.x * blockDim.x / 32) {
+        const int64_t q = z / kListGroup, g = q / groups;
+        const int o = (int)(z % kListGroup);
+        const int64_t b0 = qp[q];
+        const int len = (int)(qp[q + 1] - qp[q]) * B;
+        int64_t lo = 0, hi = 0;
+        if (r.zi[z] >= 0 && len > 0) {
+            const int64_t i = r.zi[z] & ~kListHas;
+            lo = first_at_least(tgt, ptr[i], ptr[i + 1], g * r.w);
+            hi = first_at_least(tgt, lo, ptr[i + 1], (g + 1) * r.w);
+        }
+        for (int x = lane; x < len; x += 32) {
+            const int64_t e = lo + x, at = ((b0 + x / B) * kListGroup + o) * B + x % B;
+            const bool real = e < hi;
+            const uint32_t t = hi > lo ? (uint32_t)(tgt[real ? e : lo] - g * r.w) : 0u;
+            const double v = real ? val[e] : 0.0;
+            if constexpr (KIND == 1) {
+                // padding: value 0 and pair index npair, whose row of the coefficient table is zero
+                uint32_t m = t | ((uint32_t)(norb * (norb - 1) / 2) << 16);
+                if (real) {
+                    const uint32_t key = pk[e] >> kPackKeyShift;
+                    const int p = (int)(key >> 1) / norb, s = (int)(key >> 1) % norb;
+                    const int mx = max(p, s), mn = min(p, s);
+                    m = t | ((uint32_t)(mx * (mx - 1) / 2 + mn) << 16) | ((key & 1u) << 31);
+                }
+                r.sm[at] = m;
+                r.sv32[at] = __double2float_rn(v);
+                r.sv64[at] = v;
+                r.svx2[at] = split2(v);
+            } else {
+                r.dt[at] = (uint16_t)t;
+                r.dv32[at] = __double2float_rn(v);
+                r.dv64[at] = v;
+                r.dvx2[at] = split2(v);
+            }
+        }
     }
 }
 
-// out[o] = (key[perm[o]], FP32 of val[perm[o]]), zeros for padding
-__global__ void gather_pair_kernel(const int64_t *__restrict__ perm, int64_t m, const uint32_t *__restrict__ key,
-                                   const double *__restrict__ val, uint2 *out)
+// jg[pair][i] = sum_{k in string i} (rs|kk)
+__global__ void pair_j_kernel(const uint64_t *__restrict__ S, int64_t n, int norb, const double *__restrict__ eri,
+                              double *jg)
 {
-    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < m; o += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t e = perm[o];
-        out[o] = e >= 0 ? make_uint2(key[e], __float_as_uint(__double2float_rn(val[e]))) : make_uint2(0u, 0u);
+    const int npair = norb * (norb - 1) / 2;
+    const int64_t n2 = (int64_t)norb * norb;
+    int r = 1, s = 0;
+    for (int x = 0; x < (int)blockIdx.y; ++x)
+        if (++s == r) ++r, s = 0;
+    for (int x = blockIdx.y; x < npair; x += gridDim.y) {
+        const double *row = eri + ((int64_t)r * norb + s) * n2;
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+            double v = 0.0;
+            for (uint64_t m = S[i]; m; m &= m - 1ull) v += __ldg(row + (int64_t)(__ffsll((long long)m) - 1) * (norb + 1));
+            jg[(int64_t)x * n + i] = v;
+        }
+        for (int k = 0; k < (int)gridDim.y; ++k)
+            if (++s == r) ++r, s = 0;
     }
+}
+
+// out[i] = in[i] (a scan of block counts that fits 32 bits)
+__global__ void narrow_kernel(const int64_t *__restrict__ in, uint32_t *out, int64_t n)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = (uint32_t)in[i];
 }
 
 // Order of the entries inside the items of each slice: in round i every lane of the warp adds the
@@ -742,25 +872,17 @@ void build_tables(Ctx &c, int spin)
     }
     // sigma copies: padded, bank-aware order
     t.sig_s_ptr = dalloc_n<int64_t>(c, n + 1);
-    t.sig_d_ptr = dalloc_n<int64_t>(c, n + 1);
     padded_count_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(t.s_ptr, n, cnt);
-    padded_count_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(t.d_ptr, n, cnt + n);
     SBD_LAUNCH("padded_count_kernel");
     scan_kernel<<<1, 1024, 0, c.stream>>>(cnt, n, t.sig_s_ptr);
-    scan_kernel<<<1, 1024, 0, c.stream>>>(cnt + n, n, t.sig_d_ptr);
     SBD_LAUNCH("scan_kernel(sigma lists)");
     SBD_CUDA(cudaMemcpyAsync(&t.sig_ns, t.sig_s_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
-    SBD_CUDA(cudaMemcpyAsync(&t.sig_nd, t.sig_d_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
     SBD_CUDA(cudaStreamSynchronize(c.stream));
     t.s_pk_sig = dalloc_n<uint32_t>(c, t.sig_ns);
     t.s_v64_sig = dalloc_n<double>(c, t.sig_ns);
     t.s_pkv32 = dalloc_n<uint2>(c, t.sig_ns);
-    t.d_j_sig = dalloc_n<int32_t>(c, t.sig_nd);
-    t.d_v64_sig = dalloc_n<double>(c, t.sig_nd);
-    t.d_jv32 = dalloc_n<uint2>(c, t.sig_nd);
     t.s_vx2 = dalloc_n<float2>(c, t.sig_ns);
-    t.d_vx2 = dalloc_n<float2>(c, t.sig_nd);
-    int64_t *perm = dalloc_n<int64_t>(c, (size_t)std::max<int64_t>(std::max(t.sig_ns, t.sig_nd), 1));
+    int64_t *perm = dalloc_n<int64_t>(c, (size_t)std::max<int64_t>(t.sig_ns, 1));
     const int ob = blocks_for(n, 128);
     if (t.sig_ns) {
         sigma_order_kernel<<<ob, 128, 0, c.stream>>>(t.s_ptr, t.sig_s_ptr, n, t.s_j, t.s_pk, perm);
@@ -774,67 +896,7 @@ void build_tables(Ctx &c, int spin)
         split_kernel<<<gb, 256, 0, c.stream>>>(t.s_v64_sig, t.s_vx2, t.sig_ns);
         SBD_LAUNCH("split_kernel(singles)");
     }
-    if (t.sig_nd) {
-        sigma_order_kernel<<<ob, 128, 0, c.stream>>>(t.d_ptr, t.sig_d_ptr, n, t.d_j, nullptr, perm);
-        SBD_LAUNCH("sigma_order_kernel(doubles)");
-        const int gb = blocks_for(t.sig_nd, 256, 16384);
-        gather_kernel<int32_t><<<gb, 256, 0, c.stream>>>(t.d_j, perm, t.d_j_sig, t.sig_nd);
-        gather_kernel<double><<<gb, 256, 0, c.stream>>>(t.d_v64, perm, t.d_v64_sig, t.sig_nd);
-        SBD_LAUNCH("gather_kernel(doubles)");
-        pair_kernel<<<gb, 256, 0, c.stream>>>(reinterpret_cast<const uint32_t *>(t.d_j_sig), t.d_v64_sig, t.d_jv32,
-                                               t.sig_nd);
-        SBD_LAUNCH("pair_kernel(doubles)");
-        split_kernel<<<gb, 256, 0, c.stream>>>(t.d_v64_sig, t.d_vx2, t.sig_nd);
-        SBD_LAUNCH("split_kernel(doubles)");
-    }
     dfree(c, perm);
-    // mixed-sigma lists split at the middle of the set (row passes over column halves); their
-    // 16-bit doubles targets need half <= 65536 (the staged halves fit shared memory only far below)
-    if ((n + 1) / 2 <= 65536) {
-        t.half = (n + 1) / 2;
-        int64_t *ptr2 = dalloc_n<int64_t>(c, 2 * (size_t)n + 1);
-        int64_t *cnt2 = dalloc_n<int64_t>(c, 2 * (size_t)n);
-        for (int kind = 0; kind < 2; ++kind) {
-            const int64_t *ptr = kind == 0 ? t.s_ptr : t.d_ptr;
-            const int32_t *tgt = kind == 0 ? t.s_j : t.d_j;
-            int64_t *&hptr = kind == 0 ? t.hs_ptr : t.hd_ptr;
-            half_split_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(ptr, tgt, n, t.half, ptr2);
-            SBD_LAUNCH("half_split_kernel");
-            hptr = dalloc_n<int64_t>(c, 2 * (size_t)n + 1);
-            padded_count_kernel<<<blocks_for(2 * n, 256), 256, 0, c.stream>>>(ptr2, 2 * n, cnt2);
-            SBD_LAUNCH("padded_count_kernel(halves)");
-            scan_kernel<<<1, 1024, 0, c.stream>>>(cnt2, 2 * n, hptr);
-            SBD_LAUNCH("scan_kernel(halves)");
-            int64_t m = 0;
-            SBD_CUDA(cudaMemcpyAsync(&m, hptr + 2 * n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
-            SBD_CUDA(cudaStreamSynchronize(c.stream));
-            const size_t mm = (size_t)std::max<int64_t>(m, 1);
-            if (kind == 0) {
-                t.hs = dalloc_n<uint2>(c, mm);
-            } else {
-                t.hdv = dalloc_n<float>(c, mm);
-                t.hdt = dalloc_n<uint16_t>(c, mm);
-            }
-            if (m) {
-                int64_t *hperm = dalloc_n<int64_t>(c, (size_t)m);
-                sigma_order_kernel<<<blocks_for(2 * n, 128), 128, 0, c.stream>>>(ptr2, hptr, 2 * n, tgt,
-                                                                                  kind == 0 ? t.s_pk : nullptr, hperm);
-                SBD_LAUNCH("sigma_order_kernel(halves)");
-                if (kind == 0) {
-                    gather_pair_kernel<<<blocks_for(m, 256, 16384), 256, 0, c.stream>>>(hperm, m, t.s_pk, t.s_v64,
-                                                                                         t.hs);
-                    SBD_LAUNCH("gather_pair_kernel(halves)");
-                } else {
-                    gather_half_doubles_kernel<<<blocks_for(m, 256, 16384), 256, 0, c.stream>>>(
-                        hperm, m, t.d_j, t.d_v64, t.half, t.hdv, t.hdt);
-                    SBD_LAUNCH("gather_half_doubles_kernel");
-                }
-                dfree(c, hperm);
-            }
-        }
-        dfree(c, cnt2);
-        dfree(c, ptr2);
-    }
     // source-major singles: items of at most kSrcItem singles, 32 items per slice
     {
         int64_t *ioff = dalloc_n<int64_t>(c, n + 1);
@@ -872,6 +934,103 @@ void build_tables(Ctx &c, int spin)
     ediag_kernel<<<blocks_for(n, 128), 128, 0, c.stream>>>(t.strings, n, norb, c.h64, c.eri64, t.ediag);
     SBD_LAUNCH("ediag_kernel");
     dfree(c, cnt);
+}
+
+void build_sig_doubles(Ctx &c, SpinTables &t)
+{
+    const int64_t n = t.n;
+    int64_t *cnt = dalloc_n<int64_t>(c, (size_t)n);
+    t.sig_d_ptr = dalloc_n<int64_t>(c, n + 1);
+    padded_count_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(t.d_ptr, n, cnt);
+    SBD_LAUNCH("padded_count_kernel(doubles)");
+    scan_kernel<<<1, 1024, 0, c.stream>>>(cnt, n, t.sig_d_ptr);
+    SBD_LAUNCH("scan_kernel(doubles)");
+    SBD_CUDA(cudaMemcpyAsync(&t.sig_nd, t.sig_d_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
+    SBD_CUDA(cudaStreamSynchronize(c.stream));
+    t.d_j_sig = dalloc_n<int32_t>(c, t.sig_nd);
+    t.d_v64_sig = dalloc_n<double>(c, t.sig_nd);
+    t.d_jv32 = dalloc_n<uint2>(c, t.sig_nd);
+    t.d_vx2 = dalloc_n<float2>(c, t.sig_nd);
+    if (t.sig_nd) {
+        int64_t *perm = dalloc_n<int64_t>(c, (size_t)t.sig_nd);
+        sigma_order_kernel<<<blocks_for(n, 128), 128, 0, c.stream>>>(t.d_ptr, t.sig_d_ptr, n, t.d_j, nullptr, perm);
+        SBD_LAUNCH("sigma_order_kernel(doubles)");
+        const int gb = blocks_for(t.sig_nd, 256, 16384);
+        gather_kernel<int32_t><<<gb, 256, 0, c.stream>>>(t.d_j, perm, t.d_j_sig, t.sig_nd);
+        gather_kernel<double><<<gb, 256, 0, c.stream>>>(t.d_v64, perm, t.d_v64_sig, t.sig_nd);
+        SBD_LAUNCH("gather_kernel(doubles)");
+        pair_kernel<<<gb, 256, 0, c.stream>>>(reinterpret_cast<const uint32_t *>(t.d_j_sig), t.d_v64_sig, t.d_jv32,
+                                               t.sig_nd);
+        SBD_LAUNCH("pair_kernel(doubles)");
+        split_kernel<<<gb, 256, 0, c.stream>>>(t.d_v64_sig, t.d_vx2, t.sig_nd);
+        SBD_LAUNCH("split_kernel(doubles)");
+        dfree(c, perm);
+    }
+    dfree(c, cnt);
+}
+
+void build_range_lists(Ctx &c, int spin)
+{
+    SpinTables &t = c.sp[spin];
+    RangeLists &r = t.rl;
+    const int64_t n = t.n;
+    const int wmax = range_width_max(c.smem_optin, c.norb);
+    r.ng = (int)((n + wmax - 1) / wmax);
+    r.w = (int)((n + r.ng - 1) / r.ng);
+    const int64_t groups = part_group(n, kParts), nq = groups * r.ng;
+    uint32_t *cd = dalloc_n<uint32_t>(c, (size_t)(n * r.ng)), *cs = dalloc_n<uint32_t>(c, (size_t)(n * r.ng));
+    int64_t *cnt = dalloc_n<int64_t>(c, 2 * (size_t)nq);
+    int64_t *scan = dalloc_n<int64_t>(c, (size_t)nq + 1);
+    r.zi = dalloc_n<int32_t>(c, kListGroup * (size_t)nq);
+    r.qd = dalloc_n<uint32_t>(c, (size_t)nq + 1);
+    r.qs = dalloc_n<uint32_t>(c, (size_t)nq + 1);
+    const int cb = blocks_for(n * r.ng, 256, 16384), qb = blocks_for(nq + 1, 256, 16384);
+    range_count_kernel<<<cb, 256, 0, c.stream>>>(t.d_ptr, t.d_j, n, r.w, r.ng, kRangeDoubles, cd);
+    range_count_kernel<<<cb, 256, 0, c.stream>>>(t.s_ptr, t.s_j, n, r.w, r.ng, kRangeSingles, cs);
+    SBD_LAUNCH("range_count_kernel");
+    range_order_kernel<<<r.ng * kParts, 256, 0, c.stream>>>(n, cd, r.zi);
+    SBD_LAUNCH("range_order_kernel");
+    range_group_kernel<<<qb, 256, 0, c.stream>>>(n, groups, nq, cd, cs, r.zi, cnt, cnt + nq);
+    SBD_LAUNCH("range_group_kernel");
+    int64_t total[2] = {0, 0};
+    for (int kind = 0; kind < 2; ++kind) {
+        scan_kernel<<<1, 1024, 0, c.stream>>>(kind == 0 ? cnt + nq : cnt, nq, scan);
+        SBD_LAUNCH("scan_kernel(range lists)");
+        narrow_kernel<<<qb, 256, 0, c.stream>>>(scan, kind == 0 ? r.qs : r.qd, nq + 1);
+        SBD_LAUNCH("narrow_kernel");
+        SBD_CUDA(cudaMemcpyAsync(&total[kind], scan + nq, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
+    }
+    SBD_CUDA(cudaStreamSynchronize(c.stream));
+    const size_t ms = (size_t)total[0] * kListGroup * kRangeSingles, md = (size_t)total[1] * kListGroup * kRangeDoubles;
+    if (total[0] > 0xffffffffLL || total[1] > 0xffffffffLL) fail(SBD_ERR_UNSUPPORTED, "excitation lists too large");
+    r.sm = dalloc_n<uint32_t>(c, ms);
+    r.sv32 = dalloc_n<float>(c, ms);
+    r.sv64 = dalloc_n<double>(c, ms);
+    r.svx2 = dalloc_n<float2>(c, ms);
+    r.dt = dalloc_n<uint16_t>(c, md);
+    r.dv32 = dalloc_n<float>(c, md);
+    r.dv64 = dalloc_n<double>(c, md);
+    r.dvx2 = dalloc_n<float2>(c, md);
+    const int fb = blocks_for(nq * kListGroup * 32, 256, 16384);
+    if (ms) {
+        range_fill_kernel<1><<<fb, 256, 0, c.stream>>>(t.s_ptr, t.s_j, t.s_pk, t.s_v64, groups, c.norb, r);
+        SBD_LAUNCH("range_fill_kernel(singles)");
+    }
+    if (md) {
+        range_fill_kernel<2><<<fb, 256, 0, c.stream>>>(t.d_ptr, t.d_j, nullptr, t.d_v64, groups, c.norb, r);
+        SBD_LAUNCH("range_fill_kernel(doubles)");
+    }
+    const int npair = c.norb * (c.norb - 1) / 2;
+    r.jg = dalloc_n<double>(c, (size_t)npair * n);
+    if (npair) {
+        const dim3 jb((unsigned)blocks_for(n, 256, 1024), (unsigned)std::min(npair, 256));
+        pair_j_kernel<<<jb, 256, 0, c.stream>>>(t.strings, n, c.norb, c.eri64, r.jg);
+        SBD_LAUNCH("pair_j_kernel");
+    }
+    dfree(c, cd);
+    dfree(c, cs);
+    dfree(c, cnt);
+    dfree(c, scan);
 }
 
 void build_diagonal(Ctx &c)
