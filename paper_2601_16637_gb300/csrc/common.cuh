@@ -100,19 +100,29 @@ struct SpinTables {
     // packed single: target j (bits 0-17) | code p*norb+q (bits 18-29) | phase -1 (bit 30)
     uint32_t *s_pk = nullptr;
     double *s_v64 = nullptr, *d_v64 = nullptr;   // same-spin matrix elements
-    // Sigma copies of the lists: the same entries per source, each list padded with zero entries
-    // to a multiple of kListPad and reordered so that the 8 entries one 128-bit shared-memory
-    // phase gathers have distinct targets modulo 8 where possible (kBankGroups).
+    // Sigma copies of the lists, made with the first block plan (which restricts them): the same
+    // entries per source, each list padded with zero entries to a multiple of kListPad and reordered so
+    // that the 8 entries one 128-bit shared-memory phase gathers have distinct targets modulo 8 where
+    // possible (kBankGroups).
     int64_t *sig_s_ptr = nullptr, *sig_d_ptr = nullptr;  // [n+1], padded CSR offsets
     int64_t sig_ns = 0, sig_nd = 0;
     uint32_t *s_pk_sig = nullptr;
     double *s_v64_sig = nullptr;
-    int32_t *d_j_sig = nullptr;  // the doubles are made with the first block plan
+    int32_t *d_j_sig = nullptr;
     double *d_v64_sig = nullptr;
     uint2 *s_pkv32 = nullptr;  // (s_pk_sig, FP32 value bits), for the mixed sigma
     uint2 *d_jv32 = nullptr;   // (d_j_sig, FP32 value bits), for the mixed sigma
     float2 *s_vx2 = nullptr;   // s_v64_sig as FP32 pairs (hi, lo), for the FP32-pair sigma
     float2 *d_vx2 = nullptr;   // d_v64_sig as FP32 pairs
+    // Singles for the two-operand alpha-beta pass, one lane per string: the strings in descending order
+    // of their number of singles (ties ascending), cut into slices of 32; a slice holds as many steps as
+    // its longest list, entry t of lane l at sl_ent[(sl_off[slice] + t)*32 + l].  An entry is the target
+    // (bits 0-17) and the coefficient row 2*pair + (phase < 0) at bits 18-29; padding repeats the list's
+    // first target with row 2*npair, which is zero.  Inside a list the entries are ordered so that the 8
+    // lanes of a 128-bit phase read distinct targets and rows modulo 8 where they can.
+    int32_t *sl_col = nullptr;   // [slices*32] string, -1: none or no singles
+    uint32_t *sl_off = nullptr;  // [slices + 1]
+    uint32_t *sl_ent = nullptr;
     RangeLists rl;  // same-spin lists of the row passes
     // Source-major singles for the column-stationary alpha-beta pass.  The canonical singles list
     // of each string is cut into items of at most kSrcItem entries (strings in ascending order,
@@ -229,8 +239,8 @@ void sort_validate_into(const uint64_t *in, int64_t n, int norb, int nel, uint64
 // tables.cu
 void build_tables(Ctx &c, int spin);
 void build_range_lists(Ctx &c, int spin);
-// doubles of one spin in sigma order, for block plans
-void build_sig_doubles(Ctx &c, SpinTables &t);
+// sigma copies of one spin's lists, for block plans
+void build_sig_lists(Ctx &c, SpinTables &t);
 void build_diagonal(Ctx &c);
 void to_float(const double *in, float *out, int64_t n, cudaStream_t s);
 

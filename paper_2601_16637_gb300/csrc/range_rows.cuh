@@ -130,6 +130,28 @@ __device__ __forceinline__ float pk_get(uint64_t p, int i)
 // x - y as one rounded operation per half
 __device__ __forceinline__ uint64_t pk_sub(uint64_t x, uint64_t y) { return pk_fma(y, pk_dup(-1.f), x); }
 
+// f2_mac on two pairs at once: (hi, lo) += (ah + al) * (b.x + b.y), an = -ah (which saves negating the
+// product for its error term)
+__device__ __forceinline__ void pk_f2_mac(uint64_t &hi, uint64_t &lo, uint64_t ah, uint64_t an, uint64_t al, ulonglong2 b)
+{
+    const uint64_t pn = pk_mul(an, b.x);
+    uint64_t e = pk_fma(ah, b.x, pn);
+    e = pk_fma(ah, b.y, e);
+    e = pk_fma(al, b.x, e);
+    const uint64_t s = pk_sub(hi, pn);
+    const uint64_t bb = pk_sub(s, hi);
+    const uint64_t t = pk_sub(pk_sub(hi, pk_sub(s, bb)), pk_add(pn, bb));
+    hi = s;
+    lo = pk_add(lo, pk_add(t, e));
+}
+// the gathered low parts back below the rounding of the high parts
+__device__ __forceinline__ void pk_f2_renorm(uint64_t &hi, uint64_t &lo)
+{
+    const uint64_t s = pk_add(hi, lo);
+    lo = pk_sub(lo, pk_sub(s, hi));
+    hi = s;
+}
+
 // The sums of one lane: two chunks (h = 0, 1) of a staged line.  A chunk's 16 bytes are two words:
 // two packed pairs of rows (FP32), two FP64 rows, or the high and the low parts of two pair rows.
 template <typename T>
@@ -253,18 +275,9 @@ struct RangeAcc<F2> {
         v[0] = make_float2(a.x, a.y), v[1] = make_float2(a.z, a.w);
         v[2] = make_float2(b.x, b.y), v[3] = make_float2(b.z, b.w);
     }
-    // f2_mac on two rows; vn = -a.hi b.hi saves negating the product for its error term
     __device__ __forceinline__ void mac2(int h, uint64_t ah, uint64_t an, uint64_t al, ulonglong2 b)
     {
-        const uint64_t pn = pk_mul(an, b.x);
-        uint64_t e = pk_fma(ah, b.x, pn);
-        e = pk_fma(ah, b.y, e);
-        e = pk_fma(al, b.x, e);
-        const uint64_t s = pk_sub(hi[h], pn);
-        const uint64_t bb = pk_sub(s, hi[h]);
-        const uint64_t t = pk_sub(pk_sub(hi[h], pk_sub(s, bb)), pk_add(pn, bb));
-        hi[h] = s;
-        lo[h] = pk_add(lo[h], pk_add(t, e));
+        pk_f2_mac(hi[h], lo[h], ah, an, al, b);
     }
     __device__ __forceinline__ void mac(int, float2 v, const ulonglong2 (&x)[2])
     {
@@ -276,12 +289,8 @@ struct RangeAcc<F2> {
     // sum would round at their size
     __device__ __forceinline__ void end_block(unsigned)
     {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint64_t s = pk_add(hi[h], lo[h]);
-            lo[h] = pk_sub(lo[h], pk_sub(s, hi[h]));
-            hi[h] = s;
-        }
+        pk_f2_renorm(hi[0], lo[0]);
+        pk_f2_renorm(hi[1], lo[1]);
     }
     __device__ __forceinline__ void single(float2 v, float sg, const ulonglong2 (&j)[2], const ulonglong2 (&x)[2])
     {

@@ -458,135 +458,196 @@ struct AbArgs {
     const typename In<T>::type *eri;  // (pq|rs) as a [norb^2][norb^2] matrix
     const int64_t *as_ptr;
     const uint32_t *as_pk;
-    const int64_t *bs_ptr;
-    const uint32_t *bs_pk;
+    const int32_t *sl_col;  // beta singles in slices (SpinTables::sl_*)
+    const uint32_t *sl_off, *sl_ent;
 };
 
-// Alpha-beta pass: CTA per output row ia.  The alpha single excitations of
-// ia are taken R at a time: their rows C[ja,:] are staged interleaved and
-// W[rs][k] = u_k (p_k q_k|rs) is tabulated; each output column ib then
-// runs over its beta singles (jb, rs, t): acc += t * sum_k W[rs][k] C[ja_k, jb],
-// and adds acc to s(ia, ib) with a fire-and-forget reduction (the same thread
-// owns (ia, ib) for every group of this row, so the adds land in program order).
+// R elements of one staged column or coefficient row, and a lane's sum over its entries.
+template <typename T, int R>
+struct AbVec {
+    T v[R];
+    __device__ static void st(T *p, const T (&v)[R]) { VecIO<T, R>::st(p, v); }
+    __device__ __forceinline__ void ld(const T *p) { VecIO<T, R>::ld(p, v); }
+};
+// two pairs as (hi, hi, lo, lo): the packed arithmetic takes both at once
+template <>
+struct AbVec<F2, 2> {
+    ulonglong2 v;
+    __device__ static void st(F2 *p, const F2 (&x)[2])
+    {
+        *reinterpret_cast<float4 *>(p) = make_float4(x[0].hi, x[1].hi, x[0].lo, x[1].lo);
+    }
+    __device__ __forceinline__ void ld(const F2 *p) { v = *reinterpret_cast<const ulonglong2 *>(p); }
+};
+
+template <typename T, int R>
+struct AbSum {  // FP64: one chain per row k
+    T s[R];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int k = 0; k < R; ++k) s[k] = T(0);
+    }
+    __device__ __forceinline__ void mac(const AbVec<T, R> &w, const AbVec<T, R> &c)
+    {
+#pragma unroll
+        for (int k = 0; k < R; ++k) s[k] = fma(w.v[k], c.v[k], s[k]);
+    }
+    __device__ __forceinline__ void end_block() {}
+    __device__ __forceinline__ double value() const
+    {
+        double t = (double)s[0];
+#pragma unroll
+        for (int k = 1; k < R; ++k) t += (double)s[k];
+        return t;
+    }
+};
+template <int R>
+struct AbSum<float, R> {  // FP32: a short chain per block of entries
+    float s, blk;
+    __device__ __forceinline__ void zero() { s = blk = 0.f; }
+    __device__ __forceinline__ void mac(const AbVec<float, R> &w, const AbVec<float, R> &c)
+    {
+#pragma unroll
+        for (int k = 0; k < R; ++k) blk = fmaf(w.v[k], c.v[k], blk);
+    }
+    __device__ __forceinline__ void end_block()
+    {
+        s += blk;
+        blk = 0.f;
+    }
+    __device__ __forceinline__ double value() const { return (double)s; }
+};
+template <>
+struct AbSum<F2, 1> {
+    F2 s;
+    __device__ __forceinline__ void zero() { s = F2(0.f); }
+    __device__ __forceinline__ void mac(const AbVec<F2, 1> &w, const AbVec<F2, 1> &c) { f2_mac(s, w.v[0], c.v[0]); }
+    __device__ __forceinline__ void end_block()
+    {
+        const float h = __fadd_rn(s.hi, s.lo);
+        s.lo = __fsub_rn(s.lo, __fsub_rn(h, s.hi));
+        s.hi = h;
+    }
+    __device__ __forceinline__ double value() const { return f2_value(s); }
+};
+template <>
+struct AbSum<F2, 2> {
+    uint64_t hi, lo;
+    __device__ __forceinline__ void zero() { hi = lo = 0ull; }
+    __device__ __forceinline__ void mac(const AbVec<F2, 2> &w, const AbVec<F2, 2> &c)
+    {
+        pk_f2_mac(hi, lo, w.v.x, pk_mul(w.v.x, pk_dup(-1.f)), w.v.y, c.v);
+    }
+    __device__ __forceinline__ void end_block() { pk_f2_renorm(hi, lo); }
+    __device__ __forceinline__ double value() const
+    {
+        return ((double)pk_get(hi, 0) + (double)pk_get(lo, 0)) + ((double)pk_get(hi, 1) + (double)pk_get(lo, 1));
+    }
+};
+
+// Two-operand alpha-beta pass: CTA per output row ia.  The alpha singles of ia are taken R at a
+// time: their rows C[ja,:] are staged interleaved, W[2*pair + neg][k] = +-u_k (p_k q_k|rs) is
+// tabulated, and every lane walks the beta singles of one output column ib (slices of 32 columns
+// with lists of nearly equal length, so that the lanes of a warp stay busy: on the FP64 pipe an idle
+// lane costs as much as a busy one): acc += sum_k W[rs][k] C[ja_k, jb], added to s(ia, ib) with a
+// fire-and-forget reduction.  Warps take the slices from a counter, longest lists first (dealt out in
+// a fixed pattern, the warp with the longest list held up the barrier of every group).  A column is
+// added to once per group, and the groups are separated by a barrier, so its adds land in order.
+//
+// Bound by the FP64 pipe (FP64) or by the two 16-byte gathers per entry (pairs: L1/shared pipe 72 %,
+// 45 % of the gather wavefronts are bank conflicts left by the ordering of the entries).  Measured
+// against eight lanes per column (each column's list padded to 32 slots), 3.6e7 determinants, norb 29:
+// FP64 84.1 -> 33.7 ms, pairs 33.1 -> 18.9 ms; with the slices dealt out in a fixed pattern 36.6 and
+// 21.4 ms.
 template <typename T, int R, bool STAGED>
 __device__ __forceinline__ void ab_row(const AbArgs<T> &a, int64_t ia, unsigned char *smem)
 {
-    constexpr int kThreads = Threads<T>::value;
-    const int n2 = a.norb * a.norb;
+    constexpr int kThreads = Threads<T>::value, kWarps = kThreads / 32;
+    const int n2 = a.norb * a.norb, nkey = a.norb * (a.norb - 1);
     const size_t cs_bytes = STAGED ? round16((size_t)a.nB * R * sizeof(T)) : 0;
     T *Cs = reinterpret_cast<T *>(smem);
-    T *Ws = reinterpret_cast<T *>(smem + cs_bytes);
+    T *Ws = reinterpret_cast<T *>(smem + cs_bytes);  // [nkey + 1][R]
+    __shared__ int next_s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int gi = lane / kGroup, lig = lane % kGroup;
-    const int64_t ngroups = (kThreads / 32) * kGroupsPerWarp;
-    {
-        const int64_t e0 = a.as_ptr[ia];
-        const int K = (int)(a.as_ptr[ia + 1] - e0);
-        for (int k0 = 0; k0 < K; k0 += R) {
-            const int kr = min(R, K - k0);
-            int64_t ja[R];
-            int pq[R];
-            T u[R];
+    const int64_t e0 = a.as_ptr[ia], nsl = (a.nB + 31) / 32;
+    const int K = (int)(a.as_ptr[ia + 1] - e0);
+    for (int k0 = 0; k0 < K; k0 += R) {
+        const int kr = min(R, K - k0);
+        int64_t ja[R];
+        int pq[R];
+        double u[R];
 #pragma unroll
-            for (int k = 0; k < R; ++k) {
-                const bool ok = k < kr;
-                const uint32_t pk = ok ? a.as_pk[e0 + k0 + k] : 0u;
-                ja[k] = pk_j(pk);
-                pq[k] = pk_code(pk);
-                u[k] = ok ? (pk_neg(pk) ? T(-1) : T(1)) : T(0);
-            }
-            __syncthreads();
-            if (STAGED) {
-                for (int64_t c = tid; c < a.nB; c += kThreads) {
-                    T v[R];
-#pragma unroll
-                    for (int k = 0; k < R; ++k) v[k] = k < kr ? conv<T>(a.C[ja[k] * a.nB + c]) : T(0);
-                    VecIO<T, R>::st(Cs + c * R, v);
-                }
-            }
-            // sign-folded W: row key = 2*rs + t holds (t ? -1 : 1) * u_k (p_k q_k|rs); rs = 0 rows zero
-            for (int key = tid; key < 2 * n2; key += kThreads) {
-                const int code = key >> 1;
+        for (int k = 0; k < R; ++k) {
+            const bool ok = k < kr;
+            const uint32_t pk = ok ? a.as_pk[e0 + k0 + k] : 0u;
+            ja[k] = pk_j(pk);
+            pq[k] = pk_code(pk);
+            u[k] = ok ? (pk_neg(pk) ? -1.0 : 1.0) : 0.0;
+        }
+        __syncthreads();
+        if (tid == 0) next_s = kWarps;
+        if (STAGED) {
+            for (int64_t c = tid; c < a.nB; c += kThreads) {
                 T v[R];
-                if constexpr (kIsF2<T>) {
-                    const double sg = (key & 1) ? -1.0 : 1.0;
 #pragma unroll
-                    for (int k = 0; k < R; ++k)
-                        v[k] = code ? f2_split(sg * (double)u[k].hi * __ldg(a.eri + (size_t)pq[k] * n2 + code)) : T(0);
-                } else {
-                    const T sg = (key & 1) ? T(-1) : T(1);
-#pragma unroll
-                    for (int k = 0; k < R; ++k) v[k] = code ? sg * u[k] * __ldg(a.eri + (size_t)pq[k] * n2 + code) : T(0);
-                }
-                VecIO<T, R>::st(Ws + (size_t)key * R, v);
+                for (int k = 0; k < R; ++k) v[k] = k < kr ? conv<T>(a.C[ja[k] * a.nB + c]) : T(0);
+                AbVec<T, R>::st(Cs + c * R, v);
             }
-            __syncthreads();
-
-            int64_t cb = (int64_t)warp * kGroupsPerWarp;
-            int64_t nxt0 = 0, nxt1 = 0;
-            if (cb + gi < a.nB) {
-                nxt0 = a.bs_ptr[cb + gi];
-                nxt1 = a.bs_ptr[cb + gi + 1];
-            }
-            for (; cb < a.nB; cb += ngroups) {
-                const int64_t ib = cb + gi;
-                const bool valid = ib < a.nB;
-                const int64_t b0 = nxt0, b1 = nxt1;
-                if (ib + ngroups < a.nB) {
-                    nxt0 = a.bs_ptr[ib + ngroups];
-                    nxt1 = a.bs_ptr[ib + ngroups + 1];
-                }
-                T acc = T(0);
-                if (valid) {
-                    const int lb = (int)(b1 - b0);
-                    for (int cb = 0; cb < lb; cb += kGroup * kListPad) {
-                        const int lc = min(kGroup * kListPad, lb - cb);
-                        if (kListPad * lig >= lc) break;
-                        int64_t e0, e1;
-                        list_slots(b0, cb, lc, lig, e0, e1);
-                        const uint2 pa = __ldg(reinterpret_cast<const uint2 *>(a.bs_pk + e0));
-                        const uint2 pb = __ldg(reinterpret_cast<const uint2 *>(a.bs_pk + e1));
-                        const uint32_t pk[4] = {pa.x, pa.y, pb.x, pb.y};
-                        T part[4];
+        }
+        for (int key = tid; key <= nkey; key += kThreads) {
+            const int pair = key >> 1;
+            int r = (int)((1.f + sqrtf(8.f * (float)pair + 1.f)) * 0.5f);
+            if (r * (r - 1) / 2 > pair) --r;
+            if (r * (r + 1) / 2 <= pair) ++r;
+            const int rs = r * a.norb + (pair - r * (r - 1) / 2);
+            const double sg = (key & 1) ? -1.0 : 1.0;
+            T v[R];
 #pragma unroll
-                        for (int t = 0; t < 4; ++t) {
-                            T cv[R], wv[R];
-                            if (STAGED) VecIO<T, R>::ld(Cs + (size_t)pk_j(pk[t]) * R, cv);
-                            else cv[0] = conv<T>(a.C[ja[0] * a.nB + pk_j(pk[t])]);
-                            VecIO<T, R>::ld(Ws + (size_t)pk_key(pk[t]) * R, wv);
-                            if constexpr (kIsF2<T>) {
+            for (int k = 0; k < R; ++k)
+                v[k] = key < nkey ? conv<T>((typename In<T>::type)(sg * u[k]) * __ldg(a.eri + (size_t)pq[k] * n2 + rs)) : T(0);
+            AbVec<T, R>::st(Ws + (size_t)key * R, v);
+        }
+        __syncthreads();
+        int64_t sl = warp;
+        while (sl < nsl) {
+            const uint32_t o0 = a.sl_off[sl];
+            const int len = (int)(a.sl_off[sl + 1] - o0);
+            if (len == 0) break;  // the lists descend: nothing follows
+            int nsl_next = 0;
+            if (lane == 0) nsl_next = atomicAdd(&next_s, 1);
+            nsl_next = __shfl_sync(0xffffffffu, nsl_next, 0);
+            const int col = a.sl_col[sl * 32 + lane];
+            const uint32_t *ent = a.sl_ent + (size_t)o0 * 32 + lane;
+            AbSum<T, R> acc;
+            acc.zero();
+            uint32_t nx[4];
 #pragma unroll
-                                for (int k = 0; k < R; ++k) f2_mac(acc, wv[k], cv[k]);
-                            } else if constexpr (sizeof(T) == 4) {
-                                // FP32: one short chain per entry keeps the four entries independent
-                                part[t] = wv[0] * cv[0];
+            for (int i = 0; i < 4; ++i) nx[i] = i < len ? __ldg(ent + 32 * i) : 0u;
+            for (int t = 0; t < len; t += 4) {
+                uint32_t e[4];
 #pragma unroll
-                                for (int k = 1; k < R; ++k) part[t] = fma(wv[k], cv[k], part[t]);
-                            } else {
-                                // FP64 is bound by the FP64 pipe: a single chain needs the fewest operations
+                for (int i = 0; i < 4; ++i) e[i] = nx[i];
+                ent += 128;
 #pragma unroll
-                                for (int k = 0; k < R; ++k) acc = fma(wv[k], cv[k], acc);
-                            }
+                for (int i = 0; i < 4; ++i) nx[i] = t + 4 + i < len ? __ldg(ent + 32 * i) : 0u;
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (t + i < len) {
+                        AbVec<T, R> c, w;
+                        const int jb = pk_j(e[i]);
+                        if constexpr (STAGED) {
+                            c.ld(Cs + (size_t)jb * R);
+                        } else {
+                            c.v[0] = conv<T>(a.C[ja[0] * a.nB + jb]);
                         }
-                        if constexpr (sizeof(T) == 4) acc += (part[0] + part[1]) + (part[2] + part[3]);
+                        w.ld(Ws + (size_t)(e[i] >> kPackKeyShift) * R);
+                        acc.mac(w, c);
                     }
-                }
-                double total;
-                if constexpr (kIsF2<T>) {
-#pragma unroll
-                    for (int off = kGroup / 2; off > 0; off >>= 1) {
-                        const F2 o(__shfl_xor_sync(0xffffffffu, acc.hi, off, kGroup),
-                                   __shfl_xor_sync(0xffffffffu, acc.lo, off, kGroup));
-                        acc = f2_add(acc, o);
-                    }
-                    total = f2_value(acc);
-                } else {
-#pragma unroll
-                    for (int off = kGroup / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off, kGroup);
-                    total = (double)acc;
-                }
-                if (valid && lig == 0) atomicAdd(a.S + ia * a.nB + ib, total);
+                acc.end_block();
             }
+            if (col >= 0) atomicAdd(a.S + ia * a.nB + col, acc.value());
+            sl = nsl_next;
         }
     }
 }
@@ -1128,8 +1189,9 @@ void make_ab_args(const Ctx &c, const typename In<T>::type *C, double *S, AbArgs
     ab.eri = sizeof(E) == 4 ? (const E *)(const void *)c.eri32 : (const E *)(const void *)c.eri64;
     ab.as_ptr = ta.s_ptr;      // canonical alpha lists: exact counts for the row groups
     ab.as_pk = ta.s_pk;
-    ab.bs_ptr = tb.sig_s_ptr;  // padded beta lists for 16-byte loads
-    ab.bs_pk = tb.s_pk_sig;
+    ab.sl_col = tb.sl_col;
+    ab.sl_off = tb.sl_off;
+    ab.sl_ent = tb.sl_ent;
 }
 
 template <typename T>

@@ -683,6 +683,86 @@ __global__ void pair_j_kernel(const uint64_t *__restrict__ S, int64_t n, int nor
     }
 }
 
+// ---- slices of the two-operand alpha-beta pass -----------------------------------
+
+// sort key of string i: descending number of singles in the low 16 bits, i above
+__global__ void slice_key_kernel(const int64_t *__restrict__ ptr, int64_t n, uint64_t *keys)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        keys[i] = ((uint64_t)i << 16) | (uint64_t)(0xffff - min((int64_t)0xffff, ptr[i + 1] - ptr[i]));
+}
+
+// strings of the slices, and each slice's steps (its first list is the longest)
+__global__ void slice_col_kernel(const uint64_t *__restrict__ keys, int64_t n, int64_t nsl, int32_t *col, int64_t *len)
+{
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < 32 * nsl; x += (int64_t)gridDim.x * blockDim.x) {
+        const uint64_t k = x < n ? keys[x] : 0xffffull;
+        const int64_t l = 0xffff - (int64_t)(k & 0xffffull);
+        col[x] = l > 0 ? (int32_t)(k >> 16) : -1;
+        if ((x & 31) == 0) len[x / 32] = l;
+    }
+}
+
+__global__ void slice_fill_kernel(const int64_t *__restrict__ ptr, const uint32_t *__restrict__ pk, int norb, int64_t nsl,
+                                  const int32_t *__restrict__ col, const uint32_t *__restrict__ off, uint32_t *ent)
+{
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < 32 * nsl; x += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t s = x / 32;
+        const int lane = (int)(x % 32), steps = (int)(off[s + 1] - off[s]);
+        const int64_t b = col[x] >= 0 ? ptr[col[x]] : 0, e = col[x] >= 0 ? ptr[col[x] + 1] : 0;
+        const uint32_t zero = (uint32_t)(norb * (norb - 1)) << kPackKeyShift;
+        for (int t = 0; t < steps; ++t) {
+            uint32_t v = (b < e ? pk[b] & kPackJMask : 0u) | zero;
+            if (b + t < e) {
+                const uint32_t w = pk[b + t], key = w >> kPackKeyShift;
+                const int p = (int)(key >> 1) / norb, q = (int)(key >> 1) % norb;
+                const int r = max(p, q), m = min(p, q);
+                v = (w & kPackJMask) | ((2u * (uint32_t)(r * (r - 1) / 2 + m) + (key & 1u)) << kPackKeyShift);
+            }
+            ent[((int64_t)off[s] + t) * 32 + lane] = v;
+        }
+    }
+}
+
+// Order inside the lists of one 128-bit phase (8 lanes of a slice, one thread): step by step, each lane
+// takes from its next kSliceWindow entries the one whose target and coefficient row, modulo 8, no
+// earlier lane of the step has taken (both, else one, else the first).
+constexpr int kSliceWindow = 16;
+__global__ void slice_order_kernel(const int64_t *__restrict__ ptr, int64_t nsl, const int32_t *__restrict__ col,
+                                   const uint32_t *__restrict__ off, uint32_t *ent)
+{
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < 4 * nsl; x += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t s = x / 4;
+        uint32_t *e = ent + (int64_t)off[s] * 32 + 8 * (x % 4);
+        int len[8], most = 0;
+#pragma unroll
+        for (int l = 0; l < 8; ++l) {
+            const int32_t i = col[s * 32 + 8 * (x % 4) + l];
+            len[l] = i >= 0 ? (int)(ptr[i + 1] - ptr[i]) : 0;
+            most = max(most, len[l]);
+        }
+        for (int t = 0; t < most; ++t) {
+            unsigned used_j = 0u, used_k = 0u;
+#pragma unroll
+            for (int l = 0; l < 8; ++l) {
+                if (t >= len[l]) continue;
+                int best = t, score = -1;
+                for (int y = t; y < min(t + kSliceWindow, len[l]); ++y) {
+                    const uint32_t v = e[32 * y + l];
+                    const int f = (int)!((used_j >> (v & 7u)) & 1u) + (int)!((used_k >> ((v >> kPackKeyShift) & 7u)) & 1u);
+                    if (f > score) best = y, score = f;
+                    if (f == 2) break;
+                }
+                const uint32_t v = e[32 * best + l];
+                e[32 * best + l] = e[32 * t + l];
+                e[32 * t + l] = v;
+                used_j |= 1u << (v & 7u);
+                used_k |= 1u << ((v >> kPackKeyShift) & 7u);
+            }
+        }
+    }
+}
+
 // out[i] = in[i] (a scan of block counts that fits 32 bits)
 __global__ void narrow_kernel(const int64_t *__restrict__ in, uint32_t *out, int64_t n)
 {
@@ -870,33 +950,6 @@ void build_tables(Ctx &c, int spin)
                                                                   c.h64, c.eri64, o);
         SBD_LAUNCH("enum_kernel(fill)");
     }
-    // sigma copies: padded, bank-aware order
-    t.sig_s_ptr = dalloc_n<int64_t>(c, n + 1);
-    padded_count_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(t.s_ptr, n, cnt);
-    SBD_LAUNCH("padded_count_kernel");
-    scan_kernel<<<1, 1024, 0, c.stream>>>(cnt, n, t.sig_s_ptr);
-    SBD_LAUNCH("scan_kernel(sigma lists)");
-    SBD_CUDA(cudaMemcpyAsync(&t.sig_ns, t.sig_s_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
-    SBD_CUDA(cudaStreamSynchronize(c.stream));
-    t.s_pk_sig = dalloc_n<uint32_t>(c, t.sig_ns);
-    t.s_v64_sig = dalloc_n<double>(c, t.sig_ns);
-    t.s_pkv32 = dalloc_n<uint2>(c, t.sig_ns);
-    t.s_vx2 = dalloc_n<float2>(c, t.sig_ns);
-    int64_t *perm = dalloc_n<int64_t>(c, (size_t)std::max<int64_t>(t.sig_ns, 1));
-    const int ob = blocks_for(n, 128);
-    if (t.sig_ns) {
-        sigma_order_kernel<<<ob, 128, 0, c.stream>>>(t.s_ptr, t.sig_s_ptr, n, t.s_j, t.s_pk, perm);
-        SBD_LAUNCH("sigma_order_kernel(singles)");
-        const int gb = blocks_for(t.sig_ns, 256, 16384);
-        gather_kernel<uint32_t><<<gb, 256, 0, c.stream>>>(t.s_pk, perm, t.s_pk_sig, t.sig_ns);
-        gather_kernel<double><<<gb, 256, 0, c.stream>>>(t.s_v64, perm, t.s_v64_sig, t.sig_ns);
-        SBD_LAUNCH("gather_kernel(singles)");
-        pair_kernel<<<gb, 256, 0, c.stream>>>(t.s_pk_sig, t.s_v64_sig, t.s_pkv32, t.sig_ns);
-        SBD_LAUNCH("pair_kernel(singles)");
-        split_kernel<<<gb, 256, 0, c.stream>>>(t.s_v64_sig, t.s_vx2, t.sig_ns);
-        SBD_LAUNCH("split_kernel(singles)");
-    }
-    dfree(c, perm);
     // source-major singles: items of at most kSrcItem singles, 32 items per slice
     {
         int64_t *ioff = dalloc_n<int64_t>(c, n + 1);
@@ -936,24 +989,45 @@ void build_tables(Ctx &c, int spin)
     dfree(c, cnt);
 }
 
-void build_sig_doubles(Ctx &c, SpinTables &t)
+void build_sig_lists(Ctx &c, SpinTables &t)
 {
     const int64_t n = t.n;
-    int64_t *cnt = dalloc_n<int64_t>(c, (size_t)n);
-    t.sig_d_ptr = dalloc_n<int64_t>(c, n + 1);
-    padded_count_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(t.d_ptr, n, cnt);
-    SBD_LAUNCH("padded_count_kernel(doubles)");
-    scan_kernel<<<1, 1024, 0, c.stream>>>(cnt, n, t.sig_d_ptr);
-    SBD_LAUNCH("scan_kernel(doubles)");
-    SBD_CUDA(cudaMemcpyAsync(&t.sig_nd, t.sig_d_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
+    int64_t *cnt = dalloc_n<int64_t>(c, 2 * (size_t)n);
+    t.sig_s_ptr = dalloc_n<int64_t>(c, n + 1);
+    int64_t *d_ptr = dalloc_n<int64_t>(c, n + 1);
+    padded_count_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(t.s_ptr, n, cnt);
+    padded_count_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(t.d_ptr, n, cnt + n);
+    SBD_LAUNCH("padded_count_kernel");
+    scan_kernel<<<1, 1024, 0, c.stream>>>(cnt, n, t.sig_s_ptr);
+    scan_kernel<<<1, 1024, 0, c.stream>>>(cnt + n, n, d_ptr);
+    SBD_LAUNCH("scan_kernel(sigma lists)");
+    SBD_CUDA(cudaMemcpyAsync(&t.sig_ns, t.sig_s_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
+    SBD_CUDA(cudaMemcpyAsync(&t.sig_nd, d_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
     SBD_CUDA(cudaStreamSynchronize(c.stream));
+    t.s_pk_sig = dalloc_n<uint32_t>(c, t.sig_ns);
+    t.s_v64_sig = dalloc_n<double>(c, t.sig_ns);
+    t.s_pkv32 = dalloc_n<uint2>(c, t.sig_ns);
+    t.s_vx2 = dalloc_n<float2>(c, t.sig_ns);
     t.d_j_sig = dalloc_n<int32_t>(c, t.sig_nd);
     t.d_v64_sig = dalloc_n<double>(c, t.sig_nd);
     t.d_jv32 = dalloc_n<uint2>(c, t.sig_nd);
     t.d_vx2 = dalloc_n<float2>(c, t.sig_nd);
+    int64_t *perm = dalloc_n<int64_t>(c, (size_t)std::max<int64_t>(std::max(t.sig_ns, t.sig_nd), 1));
+    const int ob = blocks_for(n, 128);
+    if (t.sig_ns) {
+        sigma_order_kernel<<<ob, 128, 0, c.stream>>>(t.s_ptr, t.sig_s_ptr, n, t.s_j, t.s_pk, perm);
+        SBD_LAUNCH("sigma_order_kernel(singles)");
+        const int gb = blocks_for(t.sig_ns, 256, 16384);
+        gather_kernel<uint32_t><<<gb, 256, 0, c.stream>>>(t.s_pk, perm, t.s_pk_sig, t.sig_ns);
+        gather_kernel<double><<<gb, 256, 0, c.stream>>>(t.s_v64, perm, t.s_v64_sig, t.sig_ns);
+        SBD_LAUNCH("gather_kernel(singles)");
+        pair_kernel<<<gb, 256, 0, c.stream>>>(t.s_pk_sig, t.s_v64_sig, t.s_pkv32, t.sig_ns);
+        SBD_LAUNCH("pair_kernel(singles)");
+        split_kernel<<<gb, 256, 0, c.stream>>>(t.s_v64_sig, t.s_vx2, t.sig_ns);
+        SBD_LAUNCH("split_kernel(singles)");
+    }
     if (t.sig_nd) {
-        int64_t *perm = dalloc_n<int64_t>(c, (size_t)t.sig_nd);
-        sigma_order_kernel<<<blocks_for(n, 128), 128, 0, c.stream>>>(t.d_ptr, t.sig_d_ptr, n, t.d_j, nullptr, perm);
+        sigma_order_kernel<<<ob, 128, 0, c.stream>>>(t.d_ptr, d_ptr, n, t.d_j, nullptr, perm);
         SBD_LAUNCH("sigma_order_kernel(doubles)");
         const int gb = blocks_for(t.sig_nd, 256, 16384);
         gather_kernel<int32_t><<<gb, 256, 0, c.stream>>>(t.d_j, perm, t.d_j_sig, t.sig_nd);
@@ -964,9 +1038,43 @@ void build_sig_doubles(Ctx &c, SpinTables &t)
         SBD_LAUNCH("pair_kernel(doubles)");
         split_kernel<<<gb, 256, 0, c.stream>>>(t.d_v64_sig, t.d_vx2, t.sig_nd);
         SBD_LAUNCH("split_kernel(doubles)");
-        dfree(c, perm);
     }
+    dfree(c, perm);
     dfree(c, cnt);
+    t.sig_d_ptr = d_ptr;  // set last: marks the copies as complete
+}
+
+// Slices of the two-operand alpha-beta pass (SpinTables::sl_*).
+static void build_slices(Ctx &c, SpinTables &t)
+{
+    const int64_t n = t.n, nsl = (n + 31) / 32;
+    uint64_t *keys = dalloc_n<uint64_t>(c, (size_t)n);
+    int64_t *len = dalloc_n<int64_t>(c, (size_t)nsl), *off = dalloc_n<int64_t>(c, (size_t)nsl + 1);
+    t.sl_col = dalloc_n<int32_t>(c, 32 * (size_t)nsl);
+    t.sl_off = dalloc_n<uint32_t>(c, (size_t)nsl + 1);
+    slice_key_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(t.s_ptr, n, keys);
+    SBD_LAUNCH("slice_key_kernel");
+    radix_sort_strings(c, keys, n, 16);  // stable, by the low 16 bits: descending length
+    slice_col_kernel<<<blocks_for(32 * nsl, 256), 256, 0, c.stream>>>(keys, n, nsl, t.sl_col, len);
+    SBD_LAUNCH("slice_col_kernel");
+    scan_kernel<<<1, 1024, 0, c.stream>>>(len, nsl, off);
+    SBD_LAUNCH("scan_kernel(slices)");
+    narrow_kernel<<<blocks_for(nsl + 1, 256), 256, 0, c.stream>>>(off, t.sl_off, nsl + 1);
+    SBD_LAUNCH("narrow_kernel(slices)");
+    int64_t steps = 0;
+    SBD_CUDA(cudaMemcpyAsync(&steps, off + nsl, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
+    SBD_CUDA(cudaStreamSynchronize(c.stream));
+    t.sl_ent = dalloc_n<uint32_t>(c, 32 * (size_t)steps);
+    if (steps) {
+        slice_fill_kernel<<<blocks_for(32 * nsl, 128, 65535), 128, 0, c.stream>>>(t.s_ptr, t.s_pk, c.norb, nsl, t.sl_col,
+                                                                                t.sl_off, t.sl_ent);
+        SBD_LAUNCH("slice_fill_kernel");
+        slice_order_kernel<<<blocks_for(4 * nsl, 32, 65535), 32, 0, c.stream>>>(t.s_ptr, nsl, t.sl_col, t.sl_off, t.sl_ent);
+        SBD_LAUNCH("slice_order_kernel");
+    }
+    dfree(c, keys);
+    dfree(c, len);
+    dfree(c, off);
 }
 
 void build_range_lists(Ctx &c, int spin)
@@ -1020,6 +1128,7 @@ void build_range_lists(Ctx &c, int spin)
         range_fill_kernel<2><<<fb, 256, 0, c.stream>>>(t.d_ptr, t.d_j, nullptr, t.d_v64, groups, c.norb, r);
         SBD_LAUNCH("range_fill_kernel(doubles)");
     }
+    build_slices(c, t);
     const int npair = c.norb * (c.norb - 1) / 2;
     r.jg = dalloc_n<double>(c, (size_t)npair * n);
     if (npair) {
