@@ -152,19 +152,23 @@ __global__ void __launch_bounds__(kBlas) mdot_pair_partial(const double *__restr
 }
 
 // out1[a*st1] (and out2[a*st2] when given) = sum_b partial[b][a] for a < k;
-// slot kDotMax (the norm) goes to *norm2 when given.  Fixed summation order.
-__global__ void mdot_final(const double *partial, int nblocks, int k, double *out1, int64_t st1, double *out2,
-                           int64_t st2, double *norm2)
+// slot kDotMax (the norm) goes to *norm2 when given.  One block per output (block k: the norm), every
+// thread a strided share of the blocks, then a tree: a fixed summation order.  (One thread per output
+// summed up to 608 values one after the other: 51 us of every pass over the basis.)
+constexpr int kFinal = 128;
+__global__ void __launch_bounds__(kFinal) mdot_final(const double *partial, int nblocks, int k, double *out1, int64_t st1,
+                                                     double *out2, int64_t st2, double *norm2)
 {
-    const int a = threadIdx.x;
+    __shared__ double red[kFinal / 32];
+    const int a = blockIdx.x, slot = a < k ? a : kDotMax;
+    double s = 0.0;
+    for (int b = threadIdx.x; b < nblocks; b += kFinal) s += partial[b * kPart + slot];
+    s = block_sum(s, red);
+    if (threadIdx.x != 0) return;
     if (a < k) {
-        double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += partial[b * kPart + a];
         out1[a * st1] = s;
         if (out2) out2[a * st2] = s;
-    } else if (a == kDotMax && norm2) {
-        double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += partial[b * kPart + kDotMax];
+    } else {
         *norm2 = s;
     }
 }
@@ -441,11 +445,14 @@ __global__ void precond_kernel(const double *__restrict__ u, const double *__res
     }
 }
 
-// dst = src * s (dst may equal src)
-__global__ void scale_kernel(const double *src, double *dst, double s, int64_t N)
+// dst = src * s (dst may equal src); f32 (optional): the FP32 rounding of dst
+__global__ void scale_kernel(const double *src, double *dst, double s, int64_t N, float *f32)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
-        dst[i] = src[i] * s;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+        const double v = src[i] * s;
+        dst[i] = v;
+        if (f32) f32[i] = __double2float_rn(v);
+    }
 }
 
 __global__ void set_kernel(double *x, int64_t idx, double v) { x[idx] = v; }
@@ -522,7 +529,7 @@ __global__ void argmaxabs_partial(const double *__restrict__ x, int64_t N, doubl
     }
 }
 
-__global__ void jacobi_kernel(const double *__restrict__ T, int ldt, int k, double *evals, double *Y, int ldy)
+__global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const double *__restrict__ T, int ldt, int k, double *evals, double *Y, int ldy)
 {
     extern __shared__ double js[];
     jacobi_eig(T, ldt, k, evals, Y, ldy, js);
@@ -544,7 +551,7 @@ struct Work {
     double *dscal = nullptr;    // kMaxSub + 1 doubles: local dot products before the sum over ranks
     double *pv = nullptr;
     int64_t *pi = nullptr;
-    std::vector<double> hpart;
+    double *dtheta = nullptr;   // [kMaxSub] Ritz values, then [kRitzMax] sums of residual squares
     Work(Ctx &cc, int64_t n, int64_t o, ShardCtx *shard)
         : c(cc), s(cc.stream), N(n), off(o), sh(shard), grid(blas_grid(cc, n)) {}
 
@@ -624,7 +631,7 @@ struct Work {
                 if (pr) launch_mdot<false, true>(Xa, ldx, kb, y);
                 else launch_mdot<false, false>(Xa, ldx, kb, y);
             }
-            mdot_final<<<1, kDotMax + 1, 0, s>>>(partial, grid, kb, out1 + a0 * st1, st1,
+            mdot_final<<<kb + (nrm ? 1 : 0), kFinal, 0, s>>>(partial, grid, kb, out1 + a0 * st1, st1,
                                                  out2 ? out2 + a0 * st2 : nullptr, st2, nrm ? norm2 : nullptr);
             SBD_LAUNCH("mdot_final");
             if (k <= a0 + kDotMax) break;
@@ -637,7 +644,7 @@ struct Work {
             if (pair) maxpy_kernel<true, true><<<grid, kBlas, 0, s>>>(X, ldx, k, coef, y, N, partial);
             else maxpy_kernel<true, false><<<grid, kBlas, 0, s>>>(X, ldx, k, coef, y, N, partial);
             SBD_LAUNCH("maxpy_kernel");
-            mdot_final<<<1, kDotMax + 1, 0, s>>>(partial, grid, 0, nullptr, 0, nullptr, 0, norm2);
+            mdot_final<<<1, kFinal, 0, s>>>(partial, grid, 0, nullptr, 0, nullptr, 0, norm2);
             SBD_LAUNCH("mdot_final");
             globalize(norm2, 1, 1);
         } else {
@@ -687,12 +694,13 @@ struct Work {
     // With one root, FP32 pairs, one process and k <= kDotMax, the same pass also leaves the first
     // Gram-Schmidt projections V^T tc and tc . tc in partial2 (returns true; see proj_dots).
     bool ritz(const double *V, const double *W, int64_t ld, int k, const double *Y, int ldy, int m, double *U,
-              double *HU, const double *theta, const double *hd, double delta, double *tc, double *rn_host)
+              double *HU, const double *theta, const double *hd, double delta, double *tc, double *rn_host,
+              double *th_host)
     {
         const bool fuse = pair && m == 1 && k >= 1 && k <= kDotMax && (!sh || sh->world == 1) && partial2;
         if (!fuse) {
             launch_combine<true>(V, W, ld, k, Y, ldy, m, U, HU, ld, theta, hd, delta, tc);
-            reduce_norms(m, rn_host);
+            reduce_norms(m, rn_host, 0, k, th_host);
             return false;
         }
         // every block of the fused pass resident at once: a grid-strided block left for a second
@@ -701,7 +709,7 @@ struct Work {
         else if (k <= 16) launch_ritz_dots<16>(V, W, ld, k, Y, U, HU, theta, hd, delta, tc);
         else if (k <= 24) launch_ritz_dots<24>(V, W, ld, k, Y, U, HU, theta, hd, delta, tc);
         else launch_ritz_dots<kDotMax>(V, W, ld, k, Y, U, HU, theta, hd, delta, tc);
-        reduce_norms(m, rn_host, rgrid);
+        reduce_norms(m, rn_host, rgrid, k, th_host);
         return true;
     }
     int rgrid = 0;  // blocks of the last fused Ritz pass (partial sums in partial, partial2)
@@ -721,21 +729,23 @@ struct Work {
     // partial2; valid while X, k and tc are those of that pass
     void proj_dots(int k, double *coef, double *norm2)
     {
-        mdot_final<<<1, kDotMax + 1, 0, s>>>(partial2, rgrid, k, coef, 1, nullptr, 0, norm2);
+        mdot_final<<<k + 1, kFinal, 0, s>>>(partial2, rgrid, k, coef, 1, nullptr, 0, norm2);
         SBD_LAUNCH("mdot_final");
     }
-    // nb: blocks that wrote partial (0: the BLAS grid)
-    void reduce_norms(int m, double *rn_host, int nb = 0)
+    // rn_host[j] = sqrt(sum_b partial[b][j]), j < m; nb: blocks that wrote partial (0: the BLAS grid);
+    // with th_host, also the k Ritz values, in the same copy
+    void reduce_norms(int m, double *rn_host, int nb = 0, int k = 0, double *th_host = nullptr)
     {
-        if (nb <= 0) nb = grid;
-        hpart.assign((size_t)nb * kPart, 0.0);
-        SBD_CUDA(cudaMemcpyAsync(hpart.data(), partial, sizeof(double) * nb * kPart, cudaMemcpyDeviceToHost, s));
+        mdot_final<<<m, kFinal, 0, s>>>(partial, nb > 0 ? nb : grid, m, dtheta + kMaxSub, 1, nullptr, 0, nullptr);
+        SBD_LAUNCH("mdot_final");
+        double h[kMaxSub + kRitzMax];
+        const int h0 = th_host ? 0 : kMaxSub;
+        SBD_CUDA(cudaMemcpyAsync(h + h0, dtheta + h0, sizeof(double) * (kMaxSub + m - h0), cudaMemcpyDeviceToHost, s));
         SBD_CUDA(cudaStreamSynchronize(s));
-        std::vector<double> acc((size_t)m, 0.0);
-        for (int j = 0; j < m; ++j)
-            for (int b = 0; b < nb; ++b) acc[j] += hpart[(size_t)b * kPart + j];
-        allreduce(acc.data(), m);
-        for (int j = 0; j < m; ++j) rn_host[j] = sqrt(acc[j]);
+        if (th_host) std::copy(h, h + k, th_host);
+        std::copy(h + kMaxSub, h + kMaxSub + m, rn_host);
+        allreduce(rn_host, m);
+        for (int j = 0; j < m; ++j) rn_host[j] = sqrt(rn_host[j]);
     }
     // residual norms ||HU_j - theta_j U_j||, j < m (theta on device)
     void resid_norms(const double *U, const double *HU, int64_t ld, int m, const double *theta, double *out_host)
@@ -744,9 +754,9 @@ struct Work {
         SBD_LAUNCH("resid_partial");
         reduce_norms(m, out_host);
     }
-    void scale(const double *src, double *dst, double f)
+    void scale(const double *src, double *dst, double f, float *f32 = nullptr)
     {
-        scale_kernel<<<grid, kBlas, 0, s>>>(src, dst, f, N);
+        scale_kernel<<<grid, kBlas, 0, s>>>(src, dst, f, N, f32);
         SBD_LAUNCH("scale_kernel");
     }
     // global index of the smallest entry not in excl (global indices); ties: lowest index
@@ -873,7 +883,7 @@ int davidson(Ctx &c, int nroots, double tol, sbd_precision prec, double *energie
     sbd_report r{};
     r.status = SBD_OK;
     SBD_CUDA(cudaFuncSetAttribute(jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)(2 * sizeof(double) * kMaxSub * kMaxSub)));
+                                  (int)jacobi_smem(kMaxSub)));
     SBD_CUDA(cudaFuncSetAttribute(ritz_dots_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   ritz_dots_smem<16>()));
     SBD_CUDA(cudaFuncSetAttribute(ritz_dots_kernel<24>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -900,7 +910,9 @@ int davidson(Ctx &c, int nroots, double tol, sbd_precision prec, double *energie
         float *c32 = mixed ? (float *)grab((size_t)N * sizeof(float)) : nullptr;
         double *T = (double *)grab(sizeof(double) * kMaxSub * kMaxSub);
         double *Y = (double *)grab(sizeof(double) * kMaxSub * kMaxSub);
-        double *theta = (double *)grab(sizeof(double) * kMaxSub);
+        double *theta = (double *)grab(sizeof(double) * (kMaxSub + kRitzMax));
+        w.dtheta = theta;
+        SBD_CUDA(cudaMemsetAsync(theta, 0, sizeof(double) * (kMaxSub + kRitzMax), w.s));
         double *coef = (double *)grab(sizeof(double) * kMaxSub);
         double *dscr = (double *)grab(sizeof(double) * kMaxSub);
         int64_t *dexcl = (int64_t *)grab(sizeof(int64_t) * (kRitzMax + 1));
@@ -916,11 +928,23 @@ int davidson(Ctx &c, int nroots, double tol, sbd_precision prec, double *energie
 
         // exact[a]: W column a came from the FP64 sigma (always, in FP64 mode)
         std::vector<char> exact(kMaxSub, mixed ? 0 : 1);
+        bool pending = false;  // ev0, ev1 bracket products whose time has not been read
+        auto harvest_sigma = [&]() {
+            if (!pending) return;
+            SBD_CUDA(cudaEventSynchronize(ev1));
+            float ms = 0.f;
+            SBD_CUDA(cudaEventElapsedTime(&ms, ev0, ev1));
+            sigma_ms += ms;
+            pending = false;
+        };
+        int c32_of = -1;  // the basis vector whose FP32 copy c32 already holds
         auto sigma_cols = [&](int b0, int nb, bool fp64) {
+            harvest_sigma();
             SBD_CUDA(cudaEventRecord(ev0, w.s));
             for (int b = b0; b < b0 + nb; ++b) {
                 if (!fp64) {
-                    to_float(V + b * ld, c32, N, w.s);
+                    if (c32_of != b) to_float(V + b * ld, c32, N, w.s);
+                    c32_of = b;
                     if (shard) ring_sigma(*shard, c, c32, W + b * ld, SBD_MIXED, w.s, V + b * ld);
                     else sigma_apply(c, c32, W + b * ld, SBD_MIXED, w.s, V + b * ld);
                     r.sigma_mixed++;
@@ -932,10 +956,8 @@ int davidson(Ctx &c, int nroots, double tol, sbd_precision prec, double *energie
                 exact[b] = fp64;
             }
             SBD_CUDA(cudaEventRecord(ev1, w.s));
-            SBD_CUDA(cudaEventSynchronize(ev1));
-            float ms = 0.f;
-            SBD_CUDA(cudaEventElapsedTime(&ms, ev0, ev1));
-            sigma_ms += ms;
+            pending = true;
+            c32_of = -1;
         };
         // column b of T (and its mirror row) against V[0..kk): T[a][b] = V[a].W[b].  Where one of
         // the pair has an FP64-exact W column and the other does not, the exact one is used,
@@ -984,13 +1006,12 @@ int davidson(Ctx &c, int nroots, double tol, sbd_precision prec, double *energie
         int iter = 0;
         while (true) {
             // 2b-2c. Rayleigh-Ritz
-            jacobi_kernel<<<1, 256, 2 * sizeof(double) * k * k, w.s>>>(T, kMaxSub, k, theta, Y, kMaxSub);
+            jacobi_kernel<<<1, kJacobiThreads, jacobi_smem(k), w.s>>>(T, kMaxSub, k, theta, Y, kMaxSub);
             SBD_LAUNCH("jacobi_kernel");
             // 2d + 2f. Ritz vectors, residual norms and the preconditioned corrections in one pass
             // proj_ok: V, k and TC still those of the fused pass (cleared by a refinement or a restart)
-            bool proj_ok = w.ritz(V, W, ld, k, Y, kMaxSub, nroots, U, HU, theta, hd, delta, TC, rn.data());
-            SBD_CUDA(cudaMemcpyAsync(th.data(), theta, sizeof(double) * k, cudaMemcpyDeviceToHost, w.s));
-            SBD_CUDA(cudaStreamSynchronize(w.s));
+            bool proj_ok = w.ritz(V, W, ld, k, Y, kMaxSub, nroots, U, HU, theta, hd, delta, TC, rn.data(), th.data());
+            harvest_sigma();
             k_ritz = k;
             harvest_timing(c);
             double rmax = *std::max_element(rn.begin(), rn.end());
@@ -1096,7 +1117,8 @@ int davidson(Ctx &c, int nroots, double tol, sbd_precision prec, double *energie
                 }
                 const double n0 = sqrt(nn[0]), n1 = sqrt(nn[1]);
                 if (!(n1 > 1e-10 * n0) || !std::isfinite(n1)) continue;
-                w.scale(t, V + k * ld, 1.0 / n1);
+                w.scale(t, V + k * ld, 1.0 / n1, c32);
+                if (mixed) c32_of = k;  // several new vectors: the last one's copy stays
                 ++k;
             }
             if (k == k_old) {
@@ -1108,6 +1130,7 @@ int davidson(Ctx &c, int nroots, double tol, sbd_precision prec, double *energie
             sigma_cols(k_old, k - k_old, !mixed);
             for (int b = k_old; b < k; ++b) extend_T(b, b + 1);
         }
+        harvest_sigma();
         r.iterations = iter;
         r.seconds_sigma = sigma_ms * 1e-3;
         // sign convention: the largest-magnitude component of each vector is positive

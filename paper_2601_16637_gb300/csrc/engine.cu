@@ -702,7 +702,7 @@ void sbd_engine_s::init()
     SBD_CUDA(cudaMalloc(&small_scratch, sizeof(double) * grid_vec));
     SBD_CUDA(cudaMalloc(&small_idx, sizeof(int64_t) * grid_vec));
     SBD_CUDA(cudaFuncSetAttribute(e_jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)(2 * sizeof(double) * kEMaxSub * kEMaxSub)));
+                                  (int)jacobi_smem(kEMaxSub)));
     const int ms = std::max(opt.max_strings, 1);
     // FP64-accurate sigma for the checks (FP32 pairs): the largest rows per item that fits
     for (int R : {2, 1})
@@ -994,7 +994,7 @@ void sbd_engine_s::capture()
     // graph A: Rayleigh-Ritz and the corrections
     int64_t l0 = begin();
     SBD_CUDA(cudaMemcpyAsync(dstage, hstage, stage_bytes, cudaMemcpyHostToDevice, stream));
-    e_jacobi_kernel<<<nsl, 256, 2 * sizeof(double) * kEMaxSub * kEMaxSub, stream>>>(hd, sd);
+    e_jacobi_kernel<<<nsl, kJacobiThreads, jacobi_smem(kEMaxSub), stream>>>(hd, sd);
     SBD_LAUNCH("e_jacobi_kernel");
     e_ritz_kernel<<<gv, kEThreads, 0, stream>>>(hd, sd, cs, co, partial);
     SBD_LAUNCH("e_ritz_kernel");
