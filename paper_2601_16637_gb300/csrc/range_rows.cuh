@@ -21,12 +21,13 @@
 // contiguous without asking anything of its alignment or row length.
 //
 // Measured, beta + alpha pass of one product (CUDA events, before: whole rows of C staged, one list
-// per eight lanes and one entry per lane): 1.0e8 determinants, FP32 25.1 -> 18.5 ms; 3.6e7
-// determinants (norb 29), FP32 7.0 -> 5.5, FP64 64.2 -> 50.5, FP32 pairs 20.8 -> 14.7 ms; 2.5e7
-// determinants at norb 58, FP32 about 12 -> 6.8 ms.  The FP32 pass keeps the L1/shared pipe 87 % busy.
-// Steps tried on the way (FP32, 3.6e7 determinants): an octet per list with separate lists 6.0 ms,
-// with interleaved lists 6.2 (padding costs more than the contiguous loads save while every octet
-// still reads 24 bytes of entries per 64 of C), four lanes per list 5.5.
+// per eight lanes and one entry per lane): 1.0e8 determinants, FP32 25.1 -> 17.6 ms; 3.6e7
+// determinants (norb 29), FP32 7.0 -> 5.0, FP64 64.2 -> 49.8, FP32 pairs 20.8 -> 14.5 ms; 2.5e7
+// determinants at norb 58, FP32 about 12 -> 6.4 ms.
+// Steps on the way (FP32, 3.6e7 determinants): an octet per list with separate lists 6.0 ms, with
+// interleaved lists 6.2 (padding costs more than the contiguous loads save while every octet still
+// reads 24 bytes of entries per 64 of C), four lanes per list 5.5; 24 warps with 80 registers instead
+// of 32 with 64 (which spilled) 5.1, 16 warps 5.9; entries loaded two blocks ahead 5.0.
 #pragma once
 
 #include "common.cuh"
@@ -34,7 +35,7 @@
 
 namespace sbd {
 
-constexpr int kRangeThreads = 1024;
+constexpr int kRangeThreads = 768;
 constexpr int kRangeRowBytes = 128;
 
 // The table of J_r[rs] of the staged rows sits in shared memory while it leaves at least half of it
@@ -326,6 +327,8 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
     using In = typename RangeIn<T>::type;
     constexpr int ROWS = kRangeRows<T>, RPC = Acc::kRowsPerChunk, LPW = 32 / ROWS;  // LPW: lines a warp stages at once
     constexpr int kWarps = kRangeThreads / 32;
+    // the FP64-accurate arithmetics have no registers left for a second block (pairs: 7.3 -> 7.9 ms)
+    constexpr int kAhead = sizeof(T) == 4 ? 2 : 1;
     unsigned char *Js = smem + (size_t)a.w * kRangeRowBytes;  // [npair + 1] lines behind the w staged lines
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lst = lane >> 2, l = lane & 3;  // list of the group, lane of the list
@@ -345,10 +348,17 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
                        p < a.npair && srow ? __ldg(a.jg + (int64_t)p * a.nrow + row0 + sr) : 0.0);
     }
     const int64_t groups = part_group(a.n, kParts);
-    const unsigned q0 = (unsigned)part_group(a.n, p0), q1 = (unsigned)part_group(a.n, p1);
+    // Groups are taken from a counter (their lengths differ, and the range ends with a barrier) in the
+    // order: the first (longest) of every part, the second of every part, ...
+    const unsigned np = p1 - p0, most = (unsigned)(part_group(a.n, p0 + 1) - part_group(a.n, p0)) * np;
+    auto group_of = [&](unsigned i, unsigned &q) {  // the i-th to be taken; false where a part has one less
+        const unsigned gi = i / np, p = p0 + (i - gi * np);
+        q = (unsigned)part_group(a.n, (int)p) + gi;
+        return i < most && q < (unsigned)part_group(a.n, (int)p + 1);
+    };
     for (int g = 0; g < a.ng; ++g) {
         if (g) __syncthreads();  // every warp is finished with the previous range
-        if (threadIdx.x == 0) next_s = q0 + kWarps;
+        if (threadIdx.x == 0) next_s = kWarps;
         const int64_t j0 = (int64_t)g * a.w;
         const int wj = (int)min((int64_t)a.w, a.n - j0);
         const In *src = a.X + j0 * a.nrow + row0 + sr;
@@ -371,19 +381,17 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
         const bool add = g > 0 || a.accumulate;
         const int32_t *zi_g = a.zi + (int64_t)g * groups * kListGroup + lst;
         const uint32_t *qd_g = a.qd + (int64_t)g * groups, *qs_g = a.qs + (int64_t)g * groups;
-        // the groups of lists are taken from a counter: their lengths differ, and the range ends with a barrier
-        unsigned q = q0 + warp;
+        unsigned i = warp, q = 0;
         int zi = -1;
         uint32_t db = 0, de = 0, sb = 0, se = 0;
-        if (q < q1) zi = zi_g[(int64_t)q * kListGroup], db = qd_g[q], de = qd_g[q + 1], sb = qs_g[q], se = qs_g[q + 1];
-        while (q < q1) {  // uniform over the warp
-            unsigned qn = 0;
-            if (lane == 0) qn = atomicAdd(&next_s, 1u);
-            qn = __shfl_sync(0xffffffffu, qn, 0);
+        if (group_of(i, q)) zi = zi_g[(int64_t)q * kListGroup], db = qd_g[q], de = qd_g[q + 1], sb = qs_g[q], se = qs_g[q + 1];
+        while (i < most) {  // uniform over the warp
+            if (lane == 0) i = atomicAdd(&next_s, 1u);
+            i = __shfl_sync(0xffffffffu, i, 0);
             int zi_n = -1;
             uint32_t db_n = 0, de_n = 0, sb_n = 0, se_n = 0;  // the next group's bounds
-            if (qn < q1)
-                zi_n = zi_g[(int64_t)qn * kListGroup], db_n = qd_g[qn], de_n = qd_g[qn + 1], sb_n = qs_g[qn], se_n = qs_g[qn + 1];
+            if (group_of(i, q))
+                zi_n = zi_g[(int64_t)q * kListGroup], db_n = qd_g[q], de_n = qd_g[q + 1], sb_n = qs_g[q], se_n = qs_g[q + 1];
             if (!add || db < de || sb < se) {
                 Acc acc;
                 acc.zero();
@@ -417,32 +425,41 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
                         acc.single(v, (m[u] >> 31) ? -1.f : 1.f, jv, x);
                     }
                 }
-                // doubles, a block of four entries at a time; the next block is loaded before this one is used
+                // doubles, a block of four entries at a time, loaded kAhead blocks ahead
                 if (db < de) {
-                    typename Acc::Val v[4];
+                    typename Acc::Val v[kAhead][4];
+                    uint2 t4[kAhead];
                     const uint2 *tp = reinterpret_cast<const uint2 *>(a.dt) + (size_t)db * kListGroup + lst;
                     const typename Acc::Val *vp = a.dv + ((size_t)db * kListGroup + lst) * 4;
-                    uint2 t4 = __ldg(tp);
-                    Acc::load(vp, v);
                     const unsigned nb = de - db;
-                    for (unsigned b = 1; b <= nb; ++b) {
-                        const uint2 t = t4;
-                        const typename Acc::Val c[4] = {v[0], v[1], v[2], v[3]};
-                        tp += kListGroup;
-                        vp += kListGroup * 4;
-                        if (b < nb) {
-                            t4 = __ldg(tp);
-                            Acc::load(vp, v);
-                        }
-                        const uint32_t j[4] = {t.x & 0xffffu, t.x >> 16, t.y & 0xffffu, t.y >> 16};
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const uint32_t jo = j[u] * kRangeRowBytes;
-                            const ulonglong2 x[2] = {*reinterpret_cast<const ulonglong2 *>(x0 + jo),
-                                                     *reinterpret_cast<const ulonglong2 *>(x1 + jo)};
-                            acc.mac(u, c[u], x);
+                    for (int s = 0; s < kAhead; ++s)
+                        if (s < nb) {
+                            t4[s] = __ldg(tp + s * kListGroup);
+                            Acc::load(vp + s * kListGroup * 4, v[s]);
                         }
-                        acc.end_block(b);
+                    for (unsigned b = 0; b < nb; b += kAhead) {
+#pragma unroll
+                        for (int s = 0; s < kAhead; ++s) {
+                            if (b + s >= nb) break;
+                            const uint2 t = t4[s];
+                            const typename Acc::Val c[4] = {v[s][0], v[s][1], v[s][2], v[s][3]};
+                            if (b + s + kAhead < nb) {
+                                t4[s] = __ldg(tp + (s + kAhead) * kListGroup);
+                                Acc::load(vp + (s + kAhead) * kListGroup * 4, v[s]);
+                            }
+                            const uint32_t j[4] = {t.x & 0xffffu, t.x >> 16, t.y & 0xffffu, t.y >> 16};
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const uint32_t jo = j[u] * kRangeRowBytes;
+                                const ulonglong2 x[2] = {*reinterpret_cast<const ulonglong2 *>(x0 + jo),
+                                                         *reinterpret_cast<const ulonglong2 *>(x1 + jo)};
+                                acc.mac(u, c[u], x);
+                            }
+                            acc.end_block(b + s + 1);
+                        }
+                        tp += kAhead * kListGroup;
+                        vp += kAhead * kListGroup * 4;
                     }
                 }
                 if (zi >= 0 && (!add || (zi & kListHas))) {  // the string's sum changes Y
@@ -464,7 +481,6 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
                         }
                 }
             }
-            q = qn;
             zi = zi_n, db = db_n, de = de_n, sb = sb_n, se = se_n;
         }
     }
