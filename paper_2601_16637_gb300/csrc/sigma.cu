@@ -711,6 +711,7 @@ struct AbSrcArgs {
     float bound;              // maxdeg_beta * max |(pq|rs)|
     int maxdeg;               // maxdeg_beta: most singles of a beta string
     int rs;                   // W row stride in float4: 8 (chunks of up to 32 alpha singles) or 4 (up to 16)
+    const int32_t *row_order; // rows by descending number of alpha singles, -1 where there is none; may be null
 };
 
 // shared memory of one CTA: W [npair][rs] float4, accumulator [nB] u64, pair -> rs code.  rs = 4
@@ -933,7 +934,14 @@ template <int RS>
 __global__ void __launch_bounds__(kSrcThreads, 1) ab_src_kernel(const AbSrcArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    for (int64_t ia = blockIdx.x; ia < a.nA; ia += gridDim.x) src_row<RS>(a, ia, smem);
+    // A row costs as much as it has alpha singles (none to several times the mean).  The rows are dealt
+    // out in descending order, back and forth over the CTAs, which evens out their sums; in ascending
+    // order of the strings the last CTA ended a tenth later than the mean.
+    for (int64_t i = 0; i * gridDim.x < a.nA; ++i) {
+        const int64_t x = i * gridDim.x + ((i & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+        const int64_t ia = x >= a.nA ? -1 : a.row_order ? a.row_order[x] : x;
+        if (ia >= 0) src_row<RS>(a, ia, smem);
+    }
 }
 
 // out[c][r] = in[r][c]; with rowmax (FP32 only, zeroed beforehand): rowmax[r] = max_c |in[r][c]|,
@@ -1062,6 +1070,7 @@ AbSrcArgs src_args(const Ctx &c, const float *C, double *S, const float *rowmax)
     a.bound = (float)((double)tb.src_maxdeg * (double)c.eri_absmax);
     a.maxdeg = tb.src_maxdeg;
     a.rs = src_rs_of(c);
+    a.row_order = ta.sl_col;
     return a;
 }
 
@@ -1764,6 +1773,7 @@ void apply_block(BlockPlan &p, const typename In<T>::type *Cb, double *S, cudaSt
             a.nA = nr;
             a.as_ptr = p.s_ptr;
             a.as_pk = p.s_pk;
+            a.row_order = nullptr;
             launch_ab_src(a, c.num_sms, s);
             return;
         }
