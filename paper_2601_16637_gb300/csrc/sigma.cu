@@ -673,11 +673,11 @@ __global__ void __launch_bounds__(Threads<T>::value) ab_pass_kernel(const AbArgs
 // 4 bytes per FMA) and adds the FP32 dot product to the row accumulator of ib.
 //
 // Bank conflicts: a W row is 128 bytes (eight 16-byte chunks).  With KC = 32 lane l reads chunk
-// (step + l) mod 8 at each step, so the 8 lanes of a 128-bit phase hit 8 distinct bank groups
+// step xor (l mod 8) at each step, so the 8 lanes of a 128-bit phase hit 8 distinct bank groups
 // whatever rows they read; with KC = 16 (8) each row holds 2 (4) copies and lanes read their own
-// copy, rotated within it.  The lane's registers hold the amplitudes in the same rotated order.
+// copy, permuted within it.  The lane's registers hold the amplitudes in the same permuted order.
 // For large norb the rows are 64 bytes (RS = 4 chunks, KC <= 16): with KC = 16 a row holds one
-// copy, the rotation spreads lanes l and l + 4 of a phase over the same four chunks, and two of
+// copy, lanes l and l + 4 of a phase read the same four chunks, and two of
 // them conflict when their rows lie in the same half of the 128-byte bank window.
 //
 // Determinism: each FP32 dot product is rounded once onto a fixed-point grid with one scale 2^e per
@@ -728,27 +728,39 @@ __host__ __device__ inline int src_rs(int npair, int64_t nB, size_t limit)
     return src_smem(npair, nB, 8) <= limit ? 8 : (src_smem(npair, nB, 4) <= limit ? 4 : 0);
 }
 
-// adds t * f to element ib of the row accumulator (words lo[ib], hi[ib]; see above)
-__device__ __forceinline__ void src_add(unsigned *acc_lo, unsigned *acc_hi, uint32_t e, float f, float scale,
-                                        int lbits)
+// adds t * f to element ib of the row accumulator (words lo[ib], hi[ib]; see above).  scale_hi =
+// scale 2^-L and two_l = 2^L: |f| scale_hi is cut into its whole part (hi) and the rest, scaled back
+// and rounded to an integer (lo); both steps are exact in FP32 but for that one rounding, so the value
+// is the nearest grid point, as a conversion of f scale to a 64-bit integer gives (which runs on the
+// FP64 pipe: 37 % of its cycles).
+__device__ __forceinline__ void src_add(unsigned *acc_lo, unsigned *acc_hi, uint32_t e, float f, float scale_hi,
+                                        float two_l, int lbits)
 {
-    long long v = __float2ll_rn(f * scale);
-    if ((e >> kSrcNegBit) & 1u) v = -v;
+    const float x = fabsf(f) * scale_hi;
+    unsigned hi = __float2uint_rz(x);
+    unsigned lo = __float2uint_rn((x - __uint2float_rz(hi)) * two_l);
+    const unsigned neg = ((__float_as_uint(f) >> 31) ^ (e >> kSrcNegBit)) & 1u;
+    if (neg) {  // -(hi 2^L + lo) with the low word in [0, 2^L]
+        const unsigned some = lo != 0u ? 1u : 0u;
+        hi = 0u - hi - some;
+        lo = (some << lbits) - lo;
+    }
     const int ib = (int)(e & kPackJMask);
-    atomicAdd(acc_lo + ib, (unsigned)v & ((1u << lbits) - 1u));
-    atomicAdd(acc_hi + ib, (unsigned)(int)(v >> lbits));
+    atomicAdd(acc_lo + ib, lo);
+    atomicAdd(acc_hi + ib, hi);
 }
 
 template <int KC, int RS>
 __device__ __forceinline__ void src_chunk(const AbSrcArgs &a, const float4 *__restrict__ Wt, unsigned *acc_lo,
-                                          unsigned *acc_hi, const int *ja_s, int kc, float scale, int lbits,
-                                          int *ctr)
+                                          unsigned *acc_hi, const int *ja_s, int kc, float scale_hi, float two_l,
+                                          int lbits, int *ctr)
 {
     static_assert(KC / 4 <= RS, "a W row holds at least one copy of the chunk");
     constexpr int CPW = KC / 4;  // 16-byte chunks per copy of a W row
     const int lane = threadIdx.x & 31;
     const int rot = lane & (CPW - 1);
-    const int base = ((lane / CPW) & (RS / CPW - 1)) * CPW;  // first chunk of this lane's copy
+    const uint32_t first = (uint32_t)(((lane / CPW) & (RS / CPW - 1)) * CPW + rot) * 16u;  // this lane's copy, chunk rot
+    const unsigned char *Wb = reinterpret_cast<const unsigned char *>(Wt);
     const int nsl = (int)((a.src_nitem + 31) >> 5);
     while (true) {
         int sl = 0;
@@ -765,52 +777,52 @@ __device__ __forceinline__ void src_chunk(const AbSrcArgs &a, const float4 *__re
 #pragma unroll
         for (int i = 0; i < kSrcItem; ++i) e[i] = i < cnt ? __ldg(ent + 32 * i) : 0u;
         // amplitudes of the chunk's alpha singles at column jb (consecutive lanes: consecutive or equal
-        // columns), then rotated by `rot` chunks so that register chunk s holds amplitude chunk
-        // (s + rot) mod CPW
-        float cv[KC];
+        // columns), two to a word, then permuted so that register chunk s holds amplitude chunk s xor rot
+        uint64_t cv[KC / 2];
 #pragma unroll
         for (int k4 = 0; k4 < KC; k4 += 4) {
             const int4 j4 = *reinterpret_cast<const int4 *>(ja_s + k4);  // one broadcast load per 4 rows
             const int jr[4] = {j4.x, j4.y, j4.z, j4.w};
+            float v[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                cv[k4 + i] = (cnt > 0 && k4 + i < kc) ? __ldg(a.C + (int64_t)jr[i] * a.nB + jb) : 0.f;
+                v[i] = (cnt > 0 && k4 + i < kc) ? __ldg(a.C + (int64_t)jr[i] * a.nB + jb) : 0.f;
+            cv[k4 / 2] = pk_pair(v[0], v[1]);
+            cv[k4 / 2 + 1] = pk_pair(v[2], v[3]);
         }
 #pragma unroll
         for (int b = 1; b < CPW; b <<= 1) {
-            if (rot & b) {
-                float tmp[KC];
+            const bool swap = rot & b;
 #pragma unroll
-                for (int s = 0; s < CPW; ++s)
+            for (int s = 0; s < CPW; ++s)
+                if (!(s & b)) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) tmp[4 * s + i] = cv[4 * ((s + b) % CPW) + i];
-#pragma unroll
-                for (int k = 0; k < KC; ++k) cv[k] = tmp[k];
-            }
+                    for (int i = 0; i < 2; ++i) {
+                        const uint64_t x = cv[2 * s + i], y = cv[2 * (s ^ b) + i];
+                        cv[2 * s + i] = swap ? y : x;
+                        cv[2 * (s ^ b) + i] = swap ? x : y;
+                    }
+                }
         }
 #pragma unroll
         for (int i = 0; i < kSrcItem; i += 2) {  // two singles per round for independent chains
             if (i < cnt) {
                 const bool two = i + 1 < cnt;
-                const float4 *w0 = Wt + ((e[i] >> kSrcPairShift) & 0x7ffu) * RS + base;
-                const float4 *w1 = Wt + ((e[i + 1] >> kSrcPairShift) & 0x7ffu) * RS + base;
-                float f0 = 0.f, f1 = 0.f;
+                const uint32_t o0 = ((e[i] >> kSrcPairShift) & 0x7ffu) * (RS * 16u) + first;
+                const uint32_t o1 = ((e[i + 1] >> kSrcPairShift) & 0x7ffu) * (RS * 16u) + first;
+                uint64_t f0 = 0ull, f1 = 0ull;
 #pragma unroll
-                for (int s = 0; s < CPW; ++s) {
-                    const int q = (s + rot) & (CPW - 1);
-                    const float4 x0 = w0[q];
-                    const float4 x1 = two ? w1[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    f0 = fmaf(x0.x, cv[4 * s], f0);
-                    f1 = fmaf(x1.x, cv[4 * s], f1);
-                    f0 = fmaf(x0.y, cv[4 * s + 1], f0);
-                    f1 = fmaf(x1.y, cv[4 * s + 1], f1);
-                    f0 = fmaf(x0.z, cv[4 * s + 2], f0);
-                    f1 = fmaf(x1.z, cv[4 * s + 2], f1);
-                    f0 = fmaf(x0.w, cv[4 * s + 3], f0);
-                    f1 = fmaf(x1.w, cv[4 * s + 3], f1);
+                for (int s = 0; s < CPW; ++s) {  // chunk s xor rot of the row: 8 lanes, 8 bank groups
+                    const ulonglong2 x0 = *reinterpret_cast<const ulonglong2 *>(Wb + (o0 ^ (s * 16u)));
+                    const ulonglong2 x1 = two ? *reinterpret_cast<const ulonglong2 *>(Wb + (o1 ^ (s * 16u)))
+                                              : make_ulonglong2(0ull, 0ull);
+                    f0 = pk_fma(x0.x, cv[2 * s], f0);
+                    f1 = pk_fma(x1.x, cv[2 * s], f1);
+                    f0 = pk_fma(x0.y, cv[2 * s + 1], f0);
+                    f1 = pk_fma(x1.y, cv[2 * s + 1], f1);
                 }
-                src_add(acc_lo, acc_hi, e[i], f0, scale, lbits);
-                if (two) src_add(acc_lo, acc_hi, e[i + 1], f1, scale, lbits);
+                src_add(acc_lo, acc_hi, e[i], pk_get(f0, 0) + pk_get(f0, 1), scale_hi, two_l, lbits);
+                if (two) src_add(acc_lo, acc_hi, e[i + 1], pk_get(f1, 0) + pk_get(f1, 1), scale_hi, two_l, lbits);
             }
         }
     }
@@ -823,17 +835,20 @@ __device__ __forceinline__ void src_build_w(const AbSrcArgs &a, float4 *Wt, cons
 {
     constexpr int CPW = KC / 4;
     const int n2 = a.norb * a.norb;
-    for (int idx = threadIdx.x; idx < a.npair * RS; idx += blockDim.x) {
-        const int p = idx / a.npair, x = idx - p * a.npair;
-        const int c = p & (CPW - 1);
-        const int rs = rs_of[x];
-        float v[4];
+    const int p = threadIdx.x % RS, c = p & (CPW - 1);  // RS divides the block size
+    float u[4];
+    const float *row[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int k = 4 * c + i;
-            v[i] = k < kc ? u_s[k] * __ldg(a.eri + (size_t)pq_s[k] * n2 + rs) : 0.f;
-        }
-        Wt[(size_t)x * RS + p] = make_float4(v[0], v[1], v[2], v[3]);
+    for (int i = 0; i < 4; ++i) {
+        const int k = 4 * c + i;
+        u[i] = k < kc ? u_s[k] : 0.f;
+        row[i] = a.eri + (size_t)(k < kc ? pq_s[k] : 0) * n2;
+    }
+#pragma unroll 4
+    for (int x = threadIdx.x / RS; x < a.npair; x += blockDim.x / RS) {
+        const int rs = rs_of[x];
+        Wt[(size_t)x * RS + p] = make_float4(u[0] * __ldg(row[0] + rs), u[1] * __ldg(row[1] + rs),
+                                             u[2] * __ldg(row[2] + rs), u[3] * __ldg(row[3] + rs));
     }
 }
 
@@ -880,7 +895,7 @@ __device__ __forceinline__ void src_row(const AbSrcArgs &a, int64_t ia, unsigned
                 const int lbits = max(1, 32 - (64 - __clzll(m)));
                 int e = 30 + lbits - ilogb(bnd) - 1;  // bnd < 2^(ilogb+1), so bnd * 2^e < 2^(30+lbits)
                 e = max(-120, min(120, e));
-                s_scale = ldexpf(1.f, e);
+                s_scale = ldexpf(1.f, e - lbits);
                 s_inv = ldexp(1.0, -e);
                 s_lbits = lbits;
                 s_state = 1;
@@ -894,8 +909,8 @@ __device__ __forceinline__ void src_row(const AbSrcArgs &a, int64_t ia, unsigned
         for (int64_t ib = tid; ib < a.nB; ib += blockDim.x) a.S[ia * a.nB + ib] = __longlong_as_double(0x7ff8000000000000ll);
         return;
     }
-    const float scale = s_scale;
     const int lbits = s_lbits;
+    const float two_l = __uint_as_float((unsigned)(127 + lbits) << 23), scale_hi = s_scale;
     for (int k0 = 0; k0 < K; k0 += KMAX) {
         const int kc = min(KMAX, K - k0);
         __syncthreads();  // the previous chunk is finished with W and the chunk arrays
@@ -910,22 +925,32 @@ __device__ __forceinline__ void src_row(const AbSrcArgs &a, int64_t ia, unsigned
         if (kc <= 8) {
             src_build_w<8, RS>(a, Wt, rs_of, pq_s, u_s, kc);
             __syncthreads();
-            src_chunk<8, RS>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale, lbits, &ctr);
+            src_chunk<8, RS>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale_hi, two_l, lbits, &ctr);
         } else if (RS == 4 || kc <= 16) {
             src_build_w<16, RS>(a, Wt, rs_of, pq_s, u_s, kc);
             __syncthreads();
-            src_chunk<16, RS>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale, lbits, &ctr);
+            src_chunk<16, RS>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale_hi, two_l, lbits, &ctr);
         } else {
             src_build_w<(RS == 8 ? 32 : 16), RS>(a, Wt, rs_of, pq_s, u_s, kc);
             __syncthreads();
-            src_chunk<(RS == 8 ? 32 : 16), RS>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale, lbits, &ctr);
+            src_chunk<(RS == 8 ? 32 : 16), RS>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale_hi, two_l, lbits, &ctr);
         }
     }
     __syncthreads();
     const double inv = s_inv;
-    for (int64_t ib = tid; ib < a.nB; ib += blockDim.x) {
-        const long long v = (long long)(int)acc_hi[ib] * (1ll << lbits) + (long long)acc_lo[ib];
-        a.S[ia * a.nB + ib] += (double)v * inv;
+    double *s = a.S + ia * a.nB;
+    for (int64_t b = tid; b < a.nB; b += 4 * (int64_t)blockDim.x) {  // four loads of sigma in flight
+        double y[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) y[u] = b + u * blockDim.x < a.nB ? s[b + u * blockDim.x] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t ib = b + u * blockDim.x;
+            if (ib < a.nB) {
+                const long long v = (long long)(int)acc_hi[ib] * (1ll << lbits) + (long long)acc_lo[ib];
+                s[ib] = y[u] + (double)v * inv;
+            }
+        }
     }
 }
 
@@ -1074,11 +1099,22 @@ AbSrcArgs src_args(const Ctx &c, const float *C, double *S, const float *rowmax)
     return a;
 }
 
-void launch_ab_src(const AbSrcArgs &a, int num_sms, cudaStream_t s)
+// CTAs that share an SM: two of half the threads where both fit and have a few rows each.  Between its
+// rows and chunks a CTA tabulates W and adds its sums to sigma while its gathers idle, and the other's
+// rows fill that (one product at norb 20, 1,703 x 2,381 strings: one CTA 1.52 ms, two 1.46, four 1.56;
+// norb 24, 300 strings: one 88 us, two 92 us).
+int src_ctas(size_t smem, int sm_bytes, int64_t rows, int num_sms)
 {
-    const int grid = (int)std::min<int64_t>(a.nA, (int64_t)num_sms);
-    if (a.rs == 8) ab_src_kernel<8><<<grid, kSrcThreads, src_smem(a.npair, a.nB, 8), s>>>(a);
-    else ab_src_kernel<4><<<grid, kSrcThreads, src_smem(a.npair, a.nB, 4), s>>>(a);
+    return 2 * (smem + 2048) <= (size_t)sm_bytes && rows >= 4 * (int64_t)num_sms ? 2 : 1;
+}
+
+void launch_ab_src(const AbSrcArgs &a, const Ctx &c, cudaStream_t s)
+{
+    const size_t smem = src_smem(a.npair, a.nB, a.rs);
+    const int f = src_ctas(smem, c.smem_optin, a.nA, c.num_sms);
+    const int grid = (int)std::min<int64_t>(a.nA, (int64_t)c.num_sms * f);
+    if (a.rs == 8) ab_src_kernel<8><<<grid, kSrcThreads / f, smem, s>>>(a);
+    else ab_src_kernel<4><<<grid, kSrcThreads / f, smem, s>>>(a);
     SBD_LAUNCH("ab_src_kernel");
 }
 
@@ -1266,7 +1302,7 @@ void apply(Ctx &c, const typename In<T>::type *C, double *S, const double *c64, 
     timed(c, base + 2, s, [&] { launch_range<T>(c, ra, s); });
     if constexpr (std::is_same<T, float>::value) {
         if (src) {
-            timed(c, base + 3, s, [&] { launch_ab_src(src_args(c, C, S, c.rowmax), c.num_sms, s); });
+            timed(c, base + 3, s, [&] { launch_ab_src(src_args(c, C, S, c.rowmax), c, s); });
             return;
         }
     }
@@ -1446,6 +1482,7 @@ struct SigmaBatch {
     bool src = false;     // mixed: the column-stationary alpha-beta pass (when its table and accumulator fit)
     int src_rs = 0;       // its W row stride for the largest slot (8 or 4 float4)
     size_t src_smem = 0;
+    int src_threads = 0;
     Layout L{};
     unsigned char *dev = nullptr, *host = nullptr;
     unsigned long long *counters = nullptr;  // [3]: beta, alpha, alpha-beta
@@ -1520,9 +1557,9 @@ void batch_launch_r(SigmaBatch *b, cudaStream_t s)
         const int64_t *off_ab = reinterpret_cast<const int64_t *>(d + L.off_ab);
         const AbSrcArgs *src_args_d = reinterpret_cast<const AbSrcArgs *>(d + L.src);
         if (b->src_rs == 8)
-            ab_src_batch_kernel<8><<<b->grid_src, kSrcThreads, b->src_smem, s>>>(pn, off_ab, src_args_d, b->counters + 2);
+            ab_src_batch_kernel<8><<<b->grid_src, b->src_threads, b->src_smem, s>>>(pn, off_ab, src_args_d, b->counters + 2);
         else
-            ab_src_batch_kernel<4><<<b->grid_src, kSrcThreads, b->src_smem, s>>>(pn, off_ab, src_args_d, b->counters + 2);
+            ab_src_batch_kernel<4><<<b->grid_src, b->src_threads, b->src_smem, s>>>(pn, off_ab, src_args_d, b->counters + 2);
         SBD_LAUNCH("ab_src_batch_kernel");
         return;
     }
@@ -1551,16 +1588,18 @@ void batch_attrs(SigmaBatch *b)
     }
     b->grid_t = sms * 8;
     if (b->src) {
-        int occ_src = 0;
+        int occ_src = 0, optin = 0;
+        SBD_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device));
+        b->src_threads = kSrcThreads / src_ctas(b->src_smem, optin, INT64_MAX, sms);
         if (b->src_rs == 8) {
             SBD_CUDA(cudaFuncSetAttribute(ab_src_batch_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)b->src_smem));
-            SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_src, ab_src_batch_kernel<8>, kSrcThreads,
+            SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_src, ab_src_batch_kernel<8>, b->src_threads,
                                                                    b->src_smem));
         } else {
             SBD_CUDA(cudaFuncSetAttribute(ab_src_batch_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)b->src_smem));
-            SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_src, ab_src_batch_kernel<4>, kSrcThreads,
+            SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_src, ab_src_batch_kernel<4>, b->src_threads,
                                                                    b->src_smem));
         }
         b->grid_src = sms * std::max(1, occ_src);
@@ -1774,7 +1813,7 @@ void apply_block(BlockPlan &p, const typename In<T>::type *Cb, double *S, cudaSt
             a.as_ptr = p.s_ptr;
             a.as_pk = p.s_pk;
             a.row_order = nullptr;
-            launch_ab_src(a, c.num_sms, s);
+            launch_ab_src(a, c, s);
             return;
         }
     }
