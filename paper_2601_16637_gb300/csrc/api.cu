@@ -353,7 +353,7 @@ int sbd_create(sbd_handle *out, int norb, int nalpha, int nbeta, const double *h
             same = st.differ == 0;
         }
         build_tables(c, 0);
-        build_range_lists(c, 0);
+        build_range_lists(c, 0, same);
         if (same) {
             uint64_t *own = c.sp[1].strings;
             c.sp[1] = c.sp[0];
@@ -361,8 +361,9 @@ int sbd_create(sbd_handle *out, int norb, int nalpha, int nbeta, const double *h
             c.sp[1].alias = true;
         } else {
             build_tables(c, 1);
-            build_range_lists(c, 1);
+            build_range_lists(c, 1, true);
         }
+        build_src_lists(c, 1);
         build_diagonal(c);
         c.work_t = dalloc(c, (size_t)c.N * sizeof(double));
         sigma_prepare(c);

@@ -37,6 +37,7 @@ constexpr int64_t kMaxStringsPerSpin = (int64_t)1 << kPackJBits;
 constexpr int kSrcPairShift = 18;  // source-major singles: orbital-pair index at bits 18-28
 constexpr int kSrcNegBit = 29;     // and the phase at bit 29
 constexpr int kSrcItem = 8;        // source-major singles per work item
+constexpr int kSrcParts = 8;      // most parts the orbital pairs of the alpha-beta pass are cut into
 constexpr int kBankGroups = 8;     // 16-byte bank groups of shared memory (32 banks x 4 bytes)
 constexpr int kListPad = 4;        // sigma lists are padded to multiples of 4 entries (16-byte loads)
 
@@ -100,7 +101,8 @@ struct SpinTables {
     // packed single: target j (bits 0-17) | code p*norb+q (bits 18-29) | phase -1 (bit 30)
     uint32_t *s_pk = nullptr;
     double *s_v64 = nullptr, *d_v64 = nullptr;   // same-spin matrix elements
-    // Sigma copies of the lists, made with the first block plan (which restricts them): the same
+    // Sigma copies of the lists, made with the first block plan (which restricts them) or for an engine
+    // job (the FP32 ones): the same
     // entries per source, each list padded with zero entries to a multiple of kListPad and reordered so
     // that the 8 entries one 128-bit shared-memory phase gathers have distinct targets modulo 8 where
     // possible (kBankGroups).
@@ -114,6 +116,16 @@ struct SpinTables {
     uint2 *d_jv32 = nullptr;   // (d_j_sig, FP32 value bits), for the mixed sigma
     float2 *s_vx2 = nullptr;   // s_v64_sig as FP32 pairs (hi, lo), for the FP32-pair sigma
     float2 *d_vx2 = nullptr;   // d_v64_sig as FP32 pairs
+    // Engine jobs: the mixed row passes' lists split at the middle of the string set (half = (n + 1) / 2):
+    // virtual list 2i holds the entries of source i with target < half, list 2i + 1 those with target
+    // >= half, each padded to kListPad and in sigma order.
+    int64_t half = 0;
+    int64_t *hs_ptr = nullptr, *hd_ptr = nullptr;  // [2n + 1]
+    uint2 *hs = nullptr;  // (packed single, FP32 value bits)
+    // doubles as two arrays with the same entry index: FP32 values, and targets relative to the
+    // list's column half, which fit 16 bits: the split lists are built only for half <= 65536
+    float *hdv = nullptr;
+    uint16_t *hdt = nullptr;
     // Singles for the two-operand alpha-beta pass, one lane per string: the strings in descending order
     // of their number of singles (ties ascending), cut into slices of 32; a slice holds as many steps as
     // its longest list, entry t of lane l at sl_ent[(sl_off[slice] + t)*32 + l].  An entry is the target
@@ -124,16 +136,21 @@ struct SpinTables {
     uint32_t *sl_off = nullptr;  // [slices + 1]
     uint32_t *sl_ent = nullptr;
     RangeLists rl;  // same-spin lists of the row passes
-    // Source-major singles for the column-stationary alpha-beta pass.  The canonical singles list
-    // of each string is cut into items of at most kSrcItem entries (strings in ascending order,
+    // Source-major singles for the column-stationary alpha-beta pass, of the spin that is the beta spin
+    // of the pass.  The orbital pairs {p, q} are cut into src_parts ranges of src_width pairs (one where
+    // the pass' table of all pairs fits shared memory).  For each part, the canonical singles list
+    // of each string, restricted to the part's pairs, is cut into items of at most kSrcItem entries
+    // (strings in ascending order,
     // each string's items consecutive, then inside each slice of 32 items the full ones first and
     // the partial ones by decreasing length), so that the lanes of a warp, one item each, walk
-    // lists of nearly equal length; item t = string | entries << 18 (src_item[t]); entry i of item t is
+    // lists of nearly equal length; part h has the slices [src_slice[h], src_slice[h + 1]);
+    // item t = string | entries << 18 (src_item[t]); entry i of item t is
     // src_ent[(t / 32) * 32 * kSrcItem + 32 * i + t % 32] (coalesced for the 32 items of a warp):
-    // target (bits 0-17) | index of the unordered orbital pair {p, q} (bits 18-28) | phase -1 (bit 29).
+    // target (bits 0-17) | index of the pair inside its part (bits 18-28) | phase -1 (bit 29).
     uint32_t *src_item = nullptr;
     uint32_t *src_ent = nullptr;
-    int64_t src_nitem = 0;
+    int src_parts = 0, src_width = 0;  // 0: the pass does not fit for this many strings
+    int src_slice[kSrcParts + 1] = {0};
     int src_maxdeg = 0;          // largest singles count of a string
     double *ediag = nullptr;     // [n] same-spin diagonal energies
     bool alias = false;          // storage owned by the other spin (A == B)
@@ -238,14 +255,22 @@ void sort_validate_into(const uint64_t *in, int64_t n, int norb, int nel, uint64
 
 // tables.cu
 void build_tables(Ctx &c, int spin);
-void build_range_lists(Ctx &c, int spin);
-// sigma copies of one spin's lists, for block plans
-void build_sig_lists(Ctx &c, SpinTables &t);
+// beta: also what the alpha-beta passes read of their beta spin
+void build_range_lists(Ctx &c, int spin, bool beta);
+// sigma copies of one spin's lists, for block plans and (only the FP32 ones) engine jobs
+void build_sig_lists(Ctx &c, SpinTables &t, bool fp32_only = false);
+// lists of the engine's mixed row passes with `rows` rows per item (0: any); drops what such a job
+// does not read
+void build_engine_lists(Ctx &c, int rows);
 void build_diagonal(Ctx &c);
 void to_float(const double *in, float *out, int64_t n, cudaStream_t s);
 
 // sigma.cu
 void sigma_prepare(Ctx &c);
+// parts the orbital pairs are cut into by the column-stationary alpha-beta pass for n beta strings
+// (0: does not fit), within the shared memory of the device
+int src_parts(int norb, int64_t n, int smem_optin);
+void build_src_lists(Ctx &c, int spin);
 
 // ---------------------------------------------------------------------------
 // row-block sigma for alpha-row sharding (shard.cu, sigma.cu)
@@ -292,7 +317,9 @@ struct SigmaBatch;
 // Device descriptors for up to max_slots instances whose string sets have at most max_strings
 // entries per spin and norb <= max_norb; R = rows staged per work item (1, 2, or for the mixed
 // precision 4, or 8 over column halves).
-SigmaBatch *sigma_batch_create(int max_slots, sbd_precision prec, int R, int max_strings, int max_norb, int device);
+// rows: mixed row passes over whole staged rows, R per work item (the handles need build_engine_lists)
+SigmaBatch *sigma_batch_create(int max_slots, sbd_precision prec, int R, int max_strings, int max_norb, int device,
+                               bool rows = false);
 // Shared memory one work item needs with R staged rows; compare with sigma_batch_smem_limit().
 size_t sigma_batch_smem(sbd_precision prec, int R, int max_strings, int max_norb);
 size_t sigma_batch_smem_limit(int device);

@@ -712,7 +712,7 @@ void sbd_engine_s::init()
         }
     if (!sb64) fail(SBD_ERR_UNSUPPORTED, "engine: max_strings/max_norb too large for the FP64 sigma staging");
     if (opt.rows_per_item) {
-        sb32 = sigma_batch_create(opt.max_slots, SBD_MIXED, opt.rows_per_item, ms, opt.max_norb, device);
+        sb32 = sigma_batch_create(opt.max_slots, SBD_MIXED, opt.rows_per_item, ms, opt.max_norb, device, true);
         rows_per_item = opt.rows_per_item;
     }
 }
@@ -817,6 +817,16 @@ bool sbd_engine_s::admit_one()
         if (opt.hbm_budget_bytes) o.hbm_budget_bytes = opt.hbm_budget_bytes - bytes_in_use - basis_bytes(N);
         int rc = sbd_create(&s.handle, j->norb, j->na, j->nb, j->h.data(), j->eri.data(), j->A.data(), nA,
                             j->B.data(), nB, &o, (void *)stream);
+        if (rc == SBD_OK) {
+            try {
+                build_engine_lists(ctx_of(s.handle), rows_per_item);
+            } catch (const Error &e) {
+                set_thread_error(e.msg);
+                rc = e.code;
+                sbd_destroy(s.handle);
+                s.handle = nullptr;
+            }
+        }
         if (rc == SBD_ERR_OVER_BUDGET && bytes_in_use > 0) {
             // the estimate was too low: wait at the head of the queue until running jobs free memory
             s = Slot{};
@@ -1079,7 +1089,7 @@ void sbd_engine_s::autotune()
     for (int ci = 0; ci < 4; ++ci) {
         const int R = cand[ci];
         if (!sigma_batch_fits(SBD_MIXED, R, ms, opt.max_norb, device)) continue;
-        SigmaBatch *sb = sigma_batch_create(opt.max_slots, SBD_MIXED, R, ms, opt.max_norb, device);
+        SigmaBatch *sb = sigma_batch_create(opt.max_slots, SBD_MIXED, R, ms, opt.max_norb, device, true);
         float t = INFINITY;
         for (int rep = 0; rep < 3; ++rep) {
             sigma_batch_set(sb, list.data(), (int)list.size());
@@ -1092,17 +1102,18 @@ void sbd_engine_s::autotune()
             if (rep > 0) t = std::min(t, ms_t);  // the first run warms up
         }
         tune_ms[ci] = t;
-        if (t < best) {
-            best = t;
-            best_r = R;
-        }
         sigma_batch_destroy(sb);
+        // fewer rows per item read the lists more often: once a candidate is slower than the one before
+        // it, so are the rest (they took two thirds of the tuning)
+        if (!(t < best)) break;
+        best = t;
+        best_r = R;
     }
     (void)cudaEventDestroy(a);
     (void)cudaEventDestroy(b);
     if (!best_r) fail(SBD_ERR_UNSUPPORTED, "engine: no sigma configuration fits shared memory");
     rows_per_item = best_r;
-    sb32 = sigma_batch_create(opt.max_slots, SBD_MIXED, best_r, ms, opt.max_norb, device);
+    sb32 = sigma_batch_create(opt.max_slots, SBD_MIXED, best_r, ms, opt.max_norb, device, true);
 }
 
 int sbd_engine_s::step()

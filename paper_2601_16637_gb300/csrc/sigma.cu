@@ -275,11 +275,18 @@ struct RowArgs {
     int accumulate;
     const double *hd;    // optional diagonal, indexed like Y
     const double *xd64;  // optional FP64 amplitudes [nrow][ncol] for the diagonal term
+    float *rowmax;       // optional (FP32 only): rowmax[r] = max_c |X[r][c]| of every row of the pass
     const uint64_t *row_strings;
     int norb;
     const double *eri;  // FP64 integrals, for the J vectors of the staged rows
     const int64_t *s_ptr, *d_ptr;
     Lists<T> lists;
+    // mixed passes over column halves (row_halves): the column spin's lists split at `half`
+    const int64_t *hls_ptr, *hld_ptr;  // singles, doubles: [2n + 1]
+    const uint2 *hls;                  // (packed single, FP32 value bits)
+    const float *hldv;                 // doubles: FP32 values
+    const uint16_t *hldt;              // doubles: targets relative to their column half
+    int64_t half;
 };
 
 // Gather pass over rows of X: each CTA stages R consecutive rows, then every
@@ -301,12 +308,35 @@ __device__ __forceinline__ void row_group(const RowArgs<T> &a, int64_t r0, unsig
     {
         const int nr = (int)min((int64_t)R, a.nrow - r0);
         __syncthreads();
+        // row maxima (FP32 pass only): largest |x| as the bit pattern of a non-negative float, so a
+        // NaN amplitude leaves a NaN maximum
+        unsigned rmax[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) rmax[r] = 0u;
+        constexpr bool kMax = std::is_same<T, float>::value;
         if (STAGED) {
             for (int64_t c = tid; c < a.ncol; c += kThreads) {
                 T v[R];
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[r] = r < nr ? conv<T>(a.X[(r0 + r) * a.ncol + c]) : T(0);
                 VecIO<T, R>::st(Xs + c * R, v);
+                if constexpr (kMax) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) rmax[r] = max(rmax[r], __float_as_uint(fabsf(v[r])));
+                }
+            }
+        } else if constexpr (kMax) {
+            if (a.rowmax)
+                for (int64_t c = tid; c < a.ncol; c += kThreads) rmax[0] = max(rmax[0], __float_as_uint(fabsf(a.X[r0 * a.ncol + c])));
+        }
+        __shared__ unsigned red_max[kMax ? R : 1][kMax ? kThreads / 32 : 1];
+        if constexpr (kMax) {
+            if (a.rowmax) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const unsigned w = __reduce_max_sync(0xffffffffu, rmax[r]);
+                    if (lane == 0) red_max[r][warp] = w;
+                }
             }
         }
         // sign-folded J table: row key = 2*code + neg holds (neg ? -1 : 1) * J_r[code]; code 0 rows
@@ -327,6 +357,14 @@ __device__ __forceinline__ void row_group(const RowArgs<T> &a, int64_t r0, unsig
             VecIO<T, R>::st(Js + (size_t)key * R, v);
         }
         __syncthreads();
+        if constexpr (kMax) {
+            if (a.rowmax && tid < nr) {
+                unsigned m = 0u;
+                for (int w = 0; w < kThreads / 32; ++w) m = max(m, red_max[tid][w]);
+                a.rowmax[r0 + tid] = __uint_as_float(m);
+            }
+        }
+
         int64_t cb = (int64_t)warp * kGroupsPerWarp;
         int64_t nxt_s0 = 0, nxt_s1 = 0, nxt_d0 = 0, nxt_d1 = 0;
         if (cb + gi < a.ncol_out) {
@@ -431,6 +469,163 @@ __global__ void __launch_bounds__(Threads<T>::value) row_pass_kernel(const RowAr
 {
     extern __shared__ __align__(16) unsigned char smem[];
     for (int64_t r0 = (int64_t)blockIdx.x * R; r0 < a.nrow; r0 += (int64_t)gridDim.x * R) row_group<T, R, STAGED>(a, r0, smem);
+}
+
+// Mixed-precision gather pass over 8 rows, one column half at a time (the engine's 8-row setting).  With 4 rows the whole row
+// range fits shared memory; staging 8 rows of one half ([0, half) or [half, ncol)) in the same space
+// lets every excitation-list entry, loaded once from L2, feed 8 multiply-adds instead of 4.  Each
+// output column sums its entries with targets in the staged half (the split lists of the column
+// spin), writes that half's sum (with the diagonal term), and adds the other half's sum after the
+// second staging.  The 8 rows are kept as two 4-row interleaved arrays, so a 16-byte gather per
+// array has the bank pattern of the 4-row pass; the coefficient table of the singles likewise.
+constexpr int kHalfRows = 8;
+
+__host__ __device__ inline size_t halves_smem(int64_t half, int norb)
+{
+    return (size_t)32 * half + (size_t)64 * norb * norb;
+}
+
+__device__ __forceinline__ void row_halves(const RowArgs<float> &a, int64_t r0, unsigned char *smem)
+{
+    constexpr int kThreads = Threads<float>::value;
+    const int n2 = a.norb * a.norb;
+    const int64_t hw = a.half;  // rows of the staged arrays: the lower half is the wider one
+    float *Xa = reinterpret_cast<float *>(smem);                   // [hw][4]  rows 0-3
+    float *Xb = Xa + 4 * hw;                                        // [hw][4]  rows 4-7
+    float *Ja = Xb + 4 * hw;                                        // [2 n2][4]
+    float *Jb = Ja + 8 * n2;                                        // [2 n2][4]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int gi = lane / kGroup, lig = lane % kGroup;
+    const int64_t ngroups = (kThreads / 32) * kGroupsPerWarp;
+    const int nr = (int)min((int64_t)kHalfRows, a.nrow - r0);
+    unsigned rmax[kHalfRows];
+#pragma unroll
+    for (int r = 0; r < kHalfRows; ++r) rmax[r] = 0u;
+    __shared__ unsigned red_h[kHalfRows];
+    __syncthreads();  // the previous row group is finished with shared memory
+    if (tid < kHalfRows) red_h[tid] = 0u;
+    // sign-folded J table of the 8 rows (row key = 2*code + neg; code 0 rows zero)
+    for (int key = tid; key < 2 * n2; key += kThreads) {
+        const int code = key >> 1;
+        float v[kHalfRows];
+#pragma unroll
+        for (int r = 0; r < kHalfRows; ++r) {
+            double sj = 0.0;
+            if (r < nr && code != 0)
+                for (uint64_t m = a.row_strings[r0 + r]; m; m &= m - 1ull) {
+                    const int k = __ffsll((long long)m) - 1;
+                    sj += __ldg(a.eri + (size_t)code * n2 + (size_t)k * (a.norb + 1));
+                }
+            v[r] = (float)((key & 1) ? -sj : sj);
+        }
+        *reinterpret_cast<float4 *>(Ja + (size_t)key * 4) = make_float4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<float4 *>(Jb + (size_t)key * 4) = make_float4(v[4], v[5], v[6], v[7]);
+    }
+    for (int h = 0; h < 2; ++h) {
+        const int64_t c0 = h ? a.half : 0, c1 = h ? a.ncol : a.half;
+        if (h) __syncthreads();  // every column is finished with the first half
+        for (int64_t c = c0 + tid; c < c1; c += kThreads) {
+            float v[kHalfRows];
+#pragma unroll
+            for (int r = 0; r < kHalfRows; ++r) v[r] = r < nr ? a.X[(r0 + r) * a.ncol + c] : 0.f;
+            *reinterpret_cast<float4 *>(Xa + (c - c0) * 4) = make_float4(v[0], v[1], v[2], v[3]);
+            *reinterpret_cast<float4 *>(Xb + (c - c0) * 4) = make_float4(v[4], v[5], v[6], v[7]);
+#pragma unroll
+            for (int r = 0; r < kHalfRows; ++r) rmax[r] = max(rmax[r], __float_as_uint(fabsf(v[r])));
+        }
+        __syncthreads();
+        for (int64_t cb = (int64_t)warp * kGroupsPerWarp; cb < a.ncol_out; cb += ngroups) {
+            const int64_t c = cb + gi;
+            const bool valid = c < a.ncol_out;
+            float acc[kHalfRows];
+#pragma unroll
+            for (int r = 0; r < kHalfRows; ++r) acc[r] = 0.f;
+            if (valid) {
+                const int64_t s0 = a.hls_ptr[2 * c + h], s1 = a.hls_ptr[2 * c + h + 1];
+                const int64_t d0 = a.hld_ptr[2 * c + h], d1 = a.hld_ptr[2 * c + h + 1];
+                const int ls = (int)(s1 - s0), ld = (int)(d1 - d0);
+                for (int cb2 = 0; cb2 < ls; cb2 += kGroup * kListPad) {
+                    const int lc = min(kGroup * kListPad, ls - cb2);
+                    if (kListPad * lig >= lc) break;
+                    int64_t e0, e1;
+                    list_slots(s0, cb2, lc, lig, e0, e1);
+                    const uint4 p0 = __ldg(reinterpret_cast<const uint4 *>(a.hls + e0));
+                    const uint4 p1 = __ldg(reinterpret_cast<const uint4 *>(a.hls + e1));
+                    const uint32_t pk[4] = {p0.x, p0.z, p1.x, p1.z};
+                    const float vv[4] = {__uint_as_float(p0.y), __uint_as_float(p0.w), __uint_as_float(p1.y),
+                                         __uint_as_float(p1.w)};
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int64_t jl = (pk[u] ? (int64_t)pk_j(pk[u]) - c0 : 0);
+                        const float4 xa = *reinterpret_cast<const float4 *>(Xa + jl * 4);
+                        const float4 xb = *reinterpret_cast<const float4 *>(Xb + jl * 4);
+                        const float4 ja = *reinterpret_cast<const float4 *>(Ja + (size_t)pk_key(pk[u]) * 4);
+                        const float4 jb = *reinterpret_cast<const float4 *>(Jb + (size_t)pk_key(pk[u]) * 4);
+                        acc[0] += (vv[u] + ja.x) * xa.x;
+                        acc[1] += (vv[u] + ja.y) * xa.y;
+                        acc[2] += (vv[u] + ja.z) * xa.z;
+                        acc[3] += (vv[u] + ja.w) * xa.w;
+                        acc[4] += (vv[u] + jb.x) * xb.x;
+                        acc[5] += (vv[u] + jb.y) * xb.y;
+                        acc[6] += (vv[u] + jb.z) * xb.z;
+                        acc[7] += (vv[u] + jb.w) * xb.w;
+                    }
+                }
+                for (int cb2 = 0; cb2 < ld; cb2 += kGroup * kListPad) {
+                    const int lc = min(kGroup * kListPad, ld - cb2);
+                    if (kListPad * lig >= lc) break;
+                    int64_t e0, e1;
+                    list_slots(d0, cb2, lc, lig, e0, e1);
+                    // entries e0 .. e0 + 3: four values (16 bytes) and four 16-bit targets (8 bytes)
+                    const float4 v4 = __ldg(reinterpret_cast<const float4 *>(a.hldv + e0));
+                    const uint2 t4 = __ldg(reinterpret_cast<const uint2 *>(a.hldt + e0));
+                    const uint32_t jj[4] = {t4.x & 0xFFFFu, t4.x >> 16, t4.y & 0xFFFFu, t4.y >> 16};
+                    const float vv[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        // targets are relative to the staged half; padding entries: target 0, value 0
+                        const int64_t jl = (int64_t)jj[u];
+                        const float4 xa = *reinterpret_cast<const float4 *>(Xa + jl * 4);
+                        const float4 xb = *reinterpret_cast<const float4 *>(Xb + jl * 4);
+                        acc[0] += vv[u] * xa.x;
+                        acc[1] += vv[u] * xa.y;
+                        acc[2] += vv[u] * xa.z;
+                        acc[3] += vv[u] * xa.w;
+                        acc[4] += vv[u] * xb.x;
+                        acc[5] += vv[u] * xb.y;
+                        acc[6] += vv[u] * xb.z;
+                        acc[7] += vv[u] * xb.w;
+                    }
+                }
+            }
+#pragma unroll
+            for (int off = kGroup / 2; off > 0; off >>= 1)
+#pragma unroll
+                for (int r = 0; r < kHalfRows; ++r) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], off, kGroup);
+            if (valid && lig < nr) {
+                double out = (double)pick<kHalfRows>(acc, lig);
+                const int64_t idx = (r0 + lig) * a.y_rs + c * a.y_cs;
+                if (h == 0) {
+                    if (a.hd) {
+                        const double xc = a.xd64 ? a.xd64[(r0 + lig) * a.ncol + c] : (double)a.X[(r0 + lig) * a.ncol + c];
+                        out += a.hd[idx] * xc;
+                    }
+                    a.Y[idx] = a.accumulate ? a.Y[idx] + out : out;
+                } else {
+                    a.Y[idx] += out;
+                }
+            }
+        }
+    }
+    if (a.rowmax) {  // uniform
+#pragma unroll
+        for (int r = 0; r < kHalfRows; ++r) {
+            const unsigned w = __reduce_max_sync(0xffffffffu, rmax[r]);
+            if (lane == 0) atomicMax(red_h + r, w);
+        }
+        __syncthreads();
+        if (tid < nr) a.rowmax[r0 + tid] = __uint_as_float(red_h[tid]);
+    }
 }
 
 // Row passes of whole instances (range_rows.cuh).  A unit is (row block, part): a CTA takes a run of
@@ -673,12 +868,15 @@ __global__ void __launch_bounds__(Threads<T>::value) ab_pass_kernel(const AbArgs
 // 4 bytes per FMA) and adds the FP32 dot product to the row accumulator of ib.
 //
 // Bank conflicts: a W row is 128 bytes (eight 16-byte chunks).  With KC = 32 lane l reads chunk
-// step xor (l mod 8) at each step, so the 8 lanes of a 128-bit phase hit 8 distinct bank groups
+// (step + l) mod 8 at each step, so the 8 lanes of a 128-bit phase hit 8 distinct bank groups
 // whatever rows they read; with KC = 16 (8) each row holds 2 (4) copies and lanes read their own
-// copy, permuted within it.  The lane's registers hold the amplitudes in the same permuted order.
-// For large norb the rows are 64 bytes (RS = 4 chunks, KC <= 16): with KC = 16 a row holds one
-// copy, lanes l and l + 4 of a phase read the same four chunks, and two of
-// them conflict when their rows lie in the same half of the 128-byte bank window.
+// copy, rotated within it.  The lane's registers hold the amplitudes in the same order.
+// Where the rows of all pairs do not fit beside the row accumulator (norb 58: 1,653 pairs, 211 KB), the
+// pairs are cut into parts: the table holds one part's rows at a time and the beta singles come part by
+// part, so a column's amplitudes are loaded once per part.  (Rows of 64 bytes for chunks of at most 16
+// alpha singles, the layout before, had two lanes of a phase in the same bank group half of the time
+// and added to the accumulator twice as often: norb 58, 5,000 strings,
+// 11.4 -> 8.5 ms; 15,000 strings 164 -> 109 ms.)
 //
 // Determinism: each FP32 dot product is rounded once onto a fixed-point grid with one scale 2^e per
 // output row and added as an integer, and integer addition is exact and order independent, so the
@@ -706,26 +904,26 @@ struct AbSrcArgs {
     const uint32_t *as_pk;
     const uint32_t *src_item; // beta singles, source-major items (string | entries << 18)
     const uint32_t *src_ent;
-    int64_t src_nitem;
+    int parts, width;         // parts of the orbital pairs, pairs of a part
+    int slice[kSrcParts + 1]; // slices of 32 items of each part
     const float *rowmax;      // [nA] max |C(ja, :)|
     float bound;              // maxdeg_beta * max |(pq|rs)|
     int maxdeg;               // maxdeg_beta: most singles of a beta string
-    int rs;                   // W row stride in float4: 8 (chunks of up to 32 alpha singles) or 4 (up to 16)
     const int32_t *row_order; // rows by descending number of alpha singles, -1 where there is none; may be null
 };
 
-// shared memory of one CTA: W [npair][rs] float4, accumulator [nB] u64, pair -> rs code.  rs = 4
-// (64-byte W rows, chunks of at most 16 alpha singles) is the layout for large norb, where the
-// 128-byte rows and the row accumulator do not fit together (norb 58: 1,653 pairs, 211 KB of rows)
-__host__ __device__ constexpr size_t src_w_bytes(int npair, int rs) { return (size_t)npair * rs * 16; }
-__host__ __device__ inline size_t src_smem(int npair, int64_t nB, int rs)
+// shared memory of one CTA: W [width][8] float4, accumulator [nB] u64, pair -> rs code
+__host__ __device__ constexpr size_t src_w_bytes(int width) { return (size_t)width * 128; }
+__host__ __device__ inline size_t src_smem(int npair, int width, int64_t nB)
 {
-    return src_w_bytes(npair, rs) + (size_t)nB * 8 + round16((size_t)npair * 2);
+    return src_w_bytes(width) + (size_t)nB * 8 + round16((size_t)npair * 2);
 }
-// the W row stride that fits `limit` bytes (8 preferred), 0 if neither does
-__host__ __device__ inline int src_rs(int npair, int64_t nB, size_t limit)
+// the fewest parts whose table fits `limit` bytes, 0 if kSrcParts do not
+inline int src_parts_for(int npair, int64_t nB, size_t limit)
 {
-    return src_smem(npair, nB, 8) <= limit ? 8 : (src_smem(npair, nB, 4) <= limit ? 4 : 0);
+    for (int h = 1; h <= kSrcParts; ++h)
+        if (src_smem(npair, (npair + h - 1) / h, nB) <= limit) return h;
+    return 0;
 }
 
 // adds t * f to element ib of the row accumulator (words lo[ib], hi[ib]; see above).  scale_hi =
@@ -750,90 +948,146 @@ __device__ __forceinline__ void src_add(unsigned *acc_lo, unsigned *acc_hi, uint
     atomicAdd(acc_hi + ib, hi);
 }
 
-template <int KC, int RS>
+// PACKED: two multiply-adds per instruction (even and odd alpha singles in two sums), chunk step xor
+// lane instead of (step + lane) mod CPW.  The engine keeps the one chain per dot product that its jobs
+// have always summed in: the result of a job stopped by its iteration cap depends on the rounding of
+// its products to 1e-9 of the energy.
+template <int KC, bool PACKED>
 __device__ __forceinline__ void src_chunk(const AbSrcArgs &a, const float4 *__restrict__ Wt, unsigned *acc_lo,
                                           unsigned *acc_hi, const int *ja_s, int kc, float scale_hi, float two_l,
-                                          int lbits, int *ctr)
+                                          int lbits, int sl1, int *ctr)
 {
-    static_assert(KC / 4 <= RS, "a W row holds at least one copy of the chunk");
+    constexpr int RS = 8;  // 16-byte chunks of a W row
     constexpr int CPW = KC / 4;  // 16-byte chunks per copy of a W row
     const int lane = threadIdx.x & 31;
     const int rot = lane & (CPW - 1);
-    const uint32_t first = (uint32_t)(((lane / CPW) & (RS / CPW - 1)) * CPW + rot) * 16u;  // this lane's copy, chunk rot
+    const int base = ((lane / CPW) & (RS / CPW - 1)) * CPW;  // first chunk of this lane's copy
+    const uint32_t first = (uint32_t)(base + rot) * 16u;
     const unsigned char *Wb = reinterpret_cast<const unsigned char *>(Wt);
-    const int nsl = (int)((a.src_nitem + 31) >> 5);
     while (true) {
         int sl = 0;
         if (lane == 0) sl = atomicAdd(ctr, 1);
         sl = __shfl_sync(0xffffffffu, sl, 0);
-        if (sl >= nsl) break;
+        if (sl >= sl1) break;
         // one item per lane: a string jb (column of C) and at most kSrcItem of its singles
         const int64_t t = (int64_t)sl * 32 + lane;
-        const uint32_t info = t < a.src_nitem ? __ldg(a.src_item + t) : 0u;
+        const uint32_t info = __ldg(a.src_item + t);
         const int64_t jb = info & kPackJMask;
         const int cnt = (int)(info >> kSrcPairShift);
         const uint32_t *ent = a.src_ent + (int64_t)sl * 32 * kSrcItem + lane;
         uint32_t e[kSrcItem];
 #pragma unroll
         for (int i = 0; i < kSrcItem; ++i) e[i] = i < cnt ? __ldg(ent + 32 * i) : 0u;
-        // amplitudes of the chunk's alpha singles at column jb (consecutive lanes: consecutive or equal
-        // columns), two to a word, then permuted so that register chunk s holds amplitude chunk s xor rot
-        uint64_t cv[KC / 2];
+        if constexpr (PACKED) {
+            // amplitudes of the chunk's alpha singles at column jb (consecutive lanes: consecutive or equal
+            // columns), two to a word, then permuted so that register chunk s holds amplitude chunk s xor rot
+            uint64_t cv[KC / 2];
 #pragma unroll
-        for (int k4 = 0; k4 < KC; k4 += 4) {
-            const int4 j4 = *reinterpret_cast<const int4 *>(ja_s + k4);  // one broadcast load per 4 rows
-            const int jr[4] = {j4.x, j4.y, j4.z, j4.w};
-            float v[4];
+            for (int k4 = 0; k4 < KC; k4 += 4) {
+                const int4 j4 = *reinterpret_cast<const int4 *>(ja_s + k4);  // one broadcast load per 4 rows
+                const int jr[4] = {j4.x, j4.y, j4.z, j4.w};
+                float v[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                v[i] = (cnt > 0 && k4 + i < kc) ? __ldg(a.C + (int64_t)jr[i] * a.nB + jb) : 0.f;
-            cv[k4 / 2] = pk_pair(v[0], v[1]);
-            cv[k4 / 2 + 1] = pk_pair(v[2], v[3]);
-        }
+                for (int i = 0; i < 4; ++i)
+                    v[i] = (cnt > 0 && k4 + i < kc) ? __ldg(a.C + (int64_t)jr[i] * a.nB + jb) : 0.f;
+                cv[k4 / 2] = pk_pair(v[0], v[1]);
+                cv[k4 / 2 + 1] = pk_pair(v[2], v[3]);
+            }
 #pragma unroll
-        for (int b = 1; b < CPW; b <<= 1) {
-            const bool swap = rot & b;
+            for (int b = 1; b < CPW; b <<= 1) {
+                const bool swap = rot & b;
 #pragma unroll
-            for (int s = 0; s < CPW; ++s)
-                if (!(s & b)) {
+                for (int s = 0; s < CPW; ++s)
+                    if (!(s & b)) {
 #pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        const uint64_t x = cv[2 * s + i], y = cv[2 * (s ^ b) + i];
-                        cv[2 * s + i] = swap ? y : x;
-                        cv[2 * (s ^ b) + i] = swap ? x : y;
+                        for (int i = 0; i < 2; ++i) {
+                            const uint64_t x = cv[2 * s + i], y = cv[2 * (s ^ b) + i];
+                            cv[2 * s + i] = swap ? y : x;
+                            cv[2 * (s ^ b) + i] = swap ? x : y;
+                        }
                     }
-                }
-        }
+            }
 #pragma unroll
-        for (int i = 0; i < kSrcItem; i += 2) {  // two singles per round for independent chains
-            if (i < cnt) {
-                const bool two = i + 1 < cnt;
-                const uint32_t o0 = ((e[i] >> kSrcPairShift) & 0x7ffu) * (RS * 16u) + first;
-                const uint32_t o1 = ((e[i + 1] >> kSrcPairShift) & 0x7ffu) * (RS * 16u) + first;
-                uint64_t f0 = 0ull, f1 = 0ull;
+            for (int i = 0; i < kSrcItem; i += 2) {  // two singles per round for independent chains
+                if (i < cnt) {
+                    const bool two = i + 1 < cnt;
+                    const uint32_t o0 = ((e[i] >> kSrcPairShift) & 0x7ffu) * (RS * 16u) + first;
+                    const uint32_t o1 = ((e[i + 1] >> kSrcPairShift) & 0x7ffu) * (RS * 16u) + first;
+                    uint64_t f0 = 0ull, f1 = 0ull;
 #pragma unroll
-                for (int s = 0; s < CPW; ++s) {  // chunk s xor rot of the row: 8 lanes, 8 bank groups
-                    const ulonglong2 x0 = *reinterpret_cast<const ulonglong2 *>(Wb + (o0 ^ (s * 16u)));
-                    const ulonglong2 x1 = two ? *reinterpret_cast<const ulonglong2 *>(Wb + (o1 ^ (s * 16u)))
-                                              : make_ulonglong2(0ull, 0ull);
-                    f0 = pk_fma(x0.x, cv[2 * s], f0);
-                    f1 = pk_fma(x1.x, cv[2 * s], f1);
-                    f0 = pk_fma(x0.y, cv[2 * s + 1], f0);
-                    f1 = pk_fma(x1.y, cv[2 * s + 1], f1);
+                    for (int s = 0; s < CPW; ++s) {  // chunk s xor rot of the row: 8 lanes, 8 bank groups
+                        const ulonglong2 x0 = *reinterpret_cast<const ulonglong2 *>(Wb + (o0 ^ (s * 16u)));
+                        const ulonglong2 x1 = two ? *reinterpret_cast<const ulonglong2 *>(Wb + (o1 ^ (s * 16u)))
+                                                  : make_ulonglong2(0ull, 0ull);
+                        f0 = pk_fma(x0.x, cv[2 * s], f0);
+                        f1 = pk_fma(x1.x, cv[2 * s], f1);
+                        f0 = pk_fma(x0.y, cv[2 * s + 1], f0);
+                        f1 = pk_fma(x1.y, cv[2 * s + 1], f1);
+                    }
+                    src_add(acc_lo, acc_hi, e[i], pk_get(f0, 0) + pk_get(f0, 1), scale_hi, two_l, lbits);
+                    if (two) src_add(acc_lo, acc_hi, e[i + 1], pk_get(f1, 0) + pk_get(f1, 1), scale_hi, two_l, lbits);
                 }
-                src_add(acc_lo, acc_hi, e[i], pk_get(f0, 0) + pk_get(f0, 1), scale_hi, two_l, lbits);
-                if (two) src_add(acc_lo, acc_hi, e[i + 1], pk_get(f1, 0) + pk_get(f1, 1), scale_hi, two_l, lbits);
+            }
+        } else {
+            // amplitudes of the chunk's alpha singles at column jb (consecutive lanes: consecutive or equal
+            // columns), then rotated by `rot` chunks so that register chunk s holds amplitude chunk
+            // (s + rot) mod CPW
+            float cv[KC];
+#pragma unroll
+            for (int k4 = 0; k4 < KC; k4 += 4) {
+                const int4 j4 = *reinterpret_cast<const int4 *>(ja_s + k4);  // one broadcast load per 4 rows
+                const int jr[4] = {j4.x, j4.y, j4.z, j4.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    cv[k4 + i] = (cnt > 0 && k4 + i < kc) ? __ldg(a.C + (int64_t)jr[i] * a.nB + jb) : 0.f;
+            }
+#pragma unroll
+            for (int b = 1; b < CPW; b <<= 1) {
+                if (rot & b) {
+                    float tmp[KC];
+#pragma unroll
+                    for (int s = 0; s < CPW; ++s)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) tmp[4 * s + i] = cv[4 * ((s + b) % CPW) + i];
+#pragma unroll
+                    for (int k = 0; k < KC; ++k) cv[k] = tmp[k];
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < kSrcItem; i += 2) {  // two singles per round for independent chains
+                if (i < cnt) {
+                    const bool two = i + 1 < cnt;
+                    const float4 *w0 = Wt + ((e[i] >> kSrcPairShift) & 0x7ffu) * RS + base;
+                    const float4 *w1 = Wt + ((e[i + 1] >> kSrcPairShift) & 0x7ffu) * RS + base;
+                    float f0 = 0.f, f1 = 0.f;
+#pragma unroll
+                    for (int s = 0; s < CPW; ++s) {
+                        const int q = (s + rot) & (CPW - 1);
+                        const float4 x0 = w0[q];
+                        const float4 x1 = two ? w1[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        f0 = fmaf(x0.x, cv[4 * s], f0);
+                        f1 = fmaf(x1.x, cv[4 * s], f1);
+                        f0 = fmaf(x0.y, cv[4 * s + 1], f0);
+                        f1 = fmaf(x1.y, cv[4 * s + 1], f1);
+                        f0 = fmaf(x0.z, cv[4 * s + 2], f0);
+                        f1 = fmaf(x1.z, cv[4 * s + 2], f1);
+                        f0 = fmaf(x0.w, cv[4 * s + 3], f0);
+                        f1 = fmaf(x1.w, cv[4 * s + 3], f1);
+                    }
+                    src_add(acc_lo, acc_hi, e[i], f0, scale_hi, two_l, lbits);
+                    if (two) src_add(acc_lo, acc_hi, e[i + 1], f1, scale_hi, two_l, lbits);
+                }
             }
         }
     }
 }
 
 // W[x][position p] for the chunk's alpha singles, position p holding amplitude chunk p mod CPW
-template <int KC, int RS>
-__device__ __forceinline__ void src_build_w(const AbSrcArgs &a, float4 *Wt, const int16_t *rs_of,
+template <int KC>
+__device__ __forceinline__ void src_build_w(const AbSrcArgs &a, float4 *Wt, const int16_t *rs_of, int width,
                                             const int *pq_s, const float *u_s, int kc)
 {
-    constexpr int CPW = KC / 4;
+    constexpr int CPW = KC / 4, RS = 8;
     const int n2 = a.norb * a.norb;
     const int p = threadIdx.x % RS, c = p & (CPW - 1);  // RS divides the block size
     float u[4];
@@ -845,21 +1099,21 @@ __device__ __forceinline__ void src_build_w(const AbSrcArgs &a, float4 *Wt, cons
         row[i] = a.eri + (size_t)(k < kc ? pq_s[k] : 0) * n2;
     }
 #pragma unroll 4
-    for (int x = threadIdx.x / RS; x < a.npair; x += blockDim.x / RS) {
+    for (int x = threadIdx.x / RS; x < width; x += blockDim.x / RS) {
         const int rs = rs_of[x];
         Wt[(size_t)x * RS + p] = make_float4(u[0] * __ldg(row[0] + rs), u[1] * __ldg(row[1] + rs),
                                              u[2] * __ldg(row[2] + rs), u[3] * __ldg(row[3] + rs));
     }
 }
 
-template <int RS>
+template <bool PACKED>
 __device__ __forceinline__ void src_row(const AbSrcArgs &a, int64_t ia, unsigned char *smem)
 {
-    constexpr int KMAX = RS * 4;  // alpha singles per chunk
+    constexpr int KMAX = 32;  // alpha singles per chunk
     float4 *Wt = reinterpret_cast<float4 *>(smem);
-    unsigned *acc_lo = reinterpret_cast<unsigned *>(smem + src_w_bytes(a.npair, RS));
+    unsigned *acc_lo = reinterpret_cast<unsigned *>(smem + src_w_bytes(a.width));
     unsigned *acc_hi = acc_lo + a.nB;
-    const int16_t *rs_of = reinterpret_cast<const int16_t *>(smem + src_w_bytes(a.npair, RS) + (size_t)a.nB * 8);
+    const int16_t *rs_of = reinterpret_cast<const int16_t *>(smem + src_w_bytes(a.width) + (size_t)a.nB * 8);
     __shared__ __align__(16) int ja_s[32];
     __shared__ int pq_s[32];
     __shared__ float u_s[32];
@@ -874,7 +1128,7 @@ __device__ __forceinline__ void src_row(const AbSrcArgs &a, int64_t ia, unsigned
     __syncthreads();  // the previous row is finished with shared memory
     for (int64_t ib = tid; ib < a.nB; ib += blockDim.x) acc_lo[ib] = acc_hi[ib] = 0u;
     {
-        int16_t *rs_w = reinterpret_cast<int16_t *>(smem + src_w_bytes(a.npair, RS) + (size_t)a.nB * 8);
+        int16_t *rs_w = reinterpret_cast<int16_t *>(smem + src_w_bytes(a.width) + (size_t)a.nB * 8);
         for (int r = 1; r < a.norb; ++r)
             for (int s = tid; s < r; s += blockDim.x) rs_w[r * (r - 1) / 2 + s] = (int16_t)(r * a.norb + s);
     }
@@ -920,20 +1174,19 @@ __device__ __forceinline__ void src_row(const AbSrcArgs &a, int64_t ia, unsigned
             pq_s[tid] = (int)(pk >> (kPackKeyShift + 1));
             u_s[tid] = ((pk >> kPackKeyShift) & 1u) ? -1.f : 1.f;
         }
-        if (tid == 0) ctr = 0;
-        __syncthreads();
-        if (kc <= 8) {
-            src_build_w<8, RS>(a, Wt, rs_of, pq_s, u_s, kc);
+        for (int h = 0; h < a.parts; ++h) {
+            const int p0 = h * a.width, width = min(a.width, a.npair - p0);
+            if (h) __syncthreads();  // the previous part is finished with W
+            if (tid == 0) ctr = a.slice[h];
             __syncthreads();
-            src_chunk<8, RS>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale_hi, two_l, lbits, &ctr);
-        } else if (RS == 4 || kc <= 16) {
-            src_build_w<16, RS>(a, Wt, rs_of, pq_s, u_s, kc);
+            if (kc <= 8) src_build_w<8>(a, Wt, rs_of + p0, width, pq_s, u_s, kc);
+            else if (kc <= 16) src_build_w<16>(a, Wt, rs_of + p0, width, pq_s, u_s, kc);
+            else src_build_w<32>(a, Wt, rs_of + p0, width, pq_s, u_s, kc);
             __syncthreads();
-            src_chunk<16, RS>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale_hi, two_l, lbits, &ctr);
-        } else {
-            src_build_w<(RS == 8 ? 32 : 16), RS>(a, Wt, rs_of, pq_s, u_s, kc);
-            __syncthreads();
-            src_chunk<(RS == 8 ? 32 : 16), RS>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale_hi, two_l, lbits, &ctr);
+            const int sl1 = a.slice[h + 1];
+            if (kc <= 8) src_chunk<8, PACKED>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale_hi, two_l, lbits, sl1, &ctr);
+            else if (kc <= 16) src_chunk<16, PACKED>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale_hi, two_l, lbits, sl1, &ctr);
+            else src_chunk<32, PACKED>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale_hi, two_l, lbits, sl1, &ctr);
         }
     }
     __syncthreads();
@@ -954,8 +1207,6 @@ __device__ __forceinline__ void src_row(const AbSrcArgs &a, int64_t ia, unsigned
     }
 }
 
-// one instance per W row stride (the host launches the one a.rs names)
-template <int RS>
 __global__ void __launch_bounds__(kSrcThreads, 1) ab_src_kernel(const AbSrcArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -965,7 +1216,7 @@ __global__ void __launch_bounds__(kSrcThreads, 1) ab_src_kernel(const AbSrcArgs 
     for (int64_t i = 0; i * gridDim.x < a.nA; ++i) {
         const int64_t x = i * gridDim.x + ((i & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
         const int64_t ia = x >= a.nA ? -1 : a.row_order ? a.row_order[x] : x;
-        if (ia >= 0) src_row<RS>(a, ia, smem);
+        if (ia >= 0) src_row<true>(a, ia, smem);
     }
 }
 
@@ -1067,13 +1318,8 @@ __global__ void absmax_kernel(const float *__restrict__ x, int64_t n, unsigned *
 
 int npairs(int norb) { return norb * (norb - 1) / 2; }
 
-// the column-stationary alpha-beta pass applies when its W table (128- or 64-byte rows) and row
-// accumulator fit
-int src_rs_of(const Ctx &c)
-{
-    return (c.norb >= 2 && c.sp[1].src_ent) ? src_rs(npairs(c.norb), c.nB, smem_limit(c)) : 0;
-}
-bool src_fits(const Ctx &c) { return src_rs_of(c) > 0; }
+// the column-stationary alpha-beta pass applies when a part of its W table and the row accumulator fit
+bool src_fits(const Ctx &c) { return c.norb >= 2 && c.sp[1].src_parts > 0; }
 
 AbSrcArgs src_args(const Ctx &c, const float *C, double *S, const float *rowmax)
 {
@@ -1090,11 +1336,12 @@ AbSrcArgs src_args(const Ctx &c, const float *C, double *S, const float *rowmax)
     a.as_pk = ta.s_pk;
     a.src_item = tb.src_item;
     a.src_ent = tb.src_ent;
-    a.src_nitem = tb.src_nitem;
+    a.parts = tb.src_parts;
+    a.width = tb.src_width;
+    std::copy(tb.src_slice, tb.src_slice + kSrcParts + 1, a.slice);
     a.rowmax = rowmax;
     a.bound = (float)((double)tb.src_maxdeg * (double)c.eri_absmax);
     a.maxdeg = tb.src_maxdeg;
-    a.rs = src_rs_of(c);
     a.row_order = ta.sl_col;
     return a;
 }
@@ -1110,11 +1357,10 @@ int src_ctas(size_t smem, int sm_bytes, int64_t rows, int num_sms)
 
 void launch_ab_src(const AbSrcArgs &a, const Ctx &c, cudaStream_t s)
 {
-    const size_t smem = src_smem(a.npair, a.nB, a.rs);
+    const size_t smem = src_smem(a.npair, a.width, a.nB);
     const int f = src_ctas(smem, c.smem_optin, a.nA, c.num_sms);
     const int grid = (int)std::min<int64_t>(a.nA, (int64_t)c.num_sms * f);
-    if (a.rs == 8) ab_src_kernel<8><<<grid, kSrcThreads / f, smem, s>>>(a);
-    else ab_src_kernel<4><<<grid, kSrcThreads / f, smem, s>>>(a);
+    ab_src_kernel<<<grid, kSrcThreads / f, smem, s>>>(a);
     SBD_LAUNCH("ab_src_kernel");
 }
 
@@ -1239,6 +1485,47 @@ void make_ab_args(const Ctx &c, const typename In<T>::type *C, double *S, AbArgs
     ab.sl_ent = tb.sl_ent;
 }
 
+// Arguments of the engine's mixed row passes: beta pass on C, alpha pass on its transpose Ct.
+void make_row_args(const Ctx &c, const float *C, double *S, const double *c64, const float *Ct, RowArgs<float> &rb,
+                   RowArgs<float> &ra)
+{
+    const SpinTables &ta = c.sp[0], &tb = c.sp[1];
+    auto lists = [](RowArgs<float> &r, const SpinTables &t) {
+        r.s_ptr = t.sig_s_ptr;
+        r.d_ptr = t.sig_d_ptr;
+        r.lists = lists_of<float>(t);
+        r.hls_ptr = t.hs_ptr;
+        r.hld_ptr = t.hd_ptr;
+        r.hls = t.hs;
+        r.hldv = t.hdv;
+        r.hldt = t.hdt;
+        r.half = t.half;
+    };
+    rb = RowArgs<float>{};
+    rb.norb = c.norb;
+    rb.eri = c.eri64;
+    ra = rb;
+    rb.X = C;
+    rb.nrow = c.nA;
+    rb.ncol = rb.ncol_out = c.nB;
+    rb.Y = S;
+    rb.y_rs = c.nB;
+    rb.y_cs = 1;
+    rb.hd = c.hd;
+    rb.xd64 = c64;
+    rb.row_strings = ta.strings;
+    lists(rb, tb);
+    ra.X = Ct;
+    ra.nrow = c.nB;
+    ra.ncol = ra.ncol_out = c.nA;
+    ra.Y = S;
+    ra.y_rs = 1;
+    ra.y_cs = c.nB;
+    ra.accumulate = 1;
+    ra.row_strings = tb.strings;
+    lists(ra, ta);
+}
+
 template <typename T>
 const typename RangeVal<T>::type *range_vals(const float *v32, const double *v64, const float2 *vx2)
 {
@@ -1347,8 +1634,8 @@ Layout layout_for(int m)
     L.off_a = take(sizeof(int64_t) * (m + 1));
     L.off_ab = take(sizeof(int64_t) * (m + 1));
     L.td = take(sizeof(TDesc<typename In<T>::type>) * m);
-    L.rb = take(sizeof(RangeArgs<T>) * m);
-    L.ra = take(sizeof(RangeArgs<T>) * m);
+    L.rb = take(std::max(sizeof(RangeArgs<T>), sizeof(RowArgs<T>)) * m);
+    L.ra = take(std::max(sizeof(RangeArgs<T>), sizeof(RowArgs<T>)) * m);
     L.ab = take(sizeof(AbArgs<T>) * m);
     L.src = take(sizeof(AbSrcArgs) * m);
     L.total = o;
@@ -1431,6 +1718,26 @@ __device__ __forceinline__ void item_loop(const int *pn, const int64_t *off, con
     }
 }
 
+// The engine's mixed row passes: whole rows of C staged, R at a time (8: one column half at a time)
+template <typename T, int R>
+__global__ void __launch_bounds__(Threads<T>::value) row_batch_kernel(const int *pn, const int64_t *off,
+                                                                      const RowArgs<T> *args,
+                                                                      unsigned long long *counter)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ RowArgs<T> sa;
+    item_loop(pn, off, args, counter, sa, [&](int64_t li) { row_group<T, R, true>(sa, li * R, smem); });
+}
+
+__global__ void __launch_bounds__(Threads<float>::value) row_halves_batch_kernel(const int *pn, const int64_t *off,
+                                                                               const RowArgs<float> *args,
+                                                                               unsigned long long *counter)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ RowArgs<float> sa;
+    item_loop(pn, off, args, counter, sa, [&](int64_t li) { row_halves(sa, li * kHalfRows, smem); });
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kRangeThreads, 1) range_batch_kernel(const int *pn, const int64_t *off,
                                                                       const RangeArgs<T> *args,
@@ -1454,22 +1761,19 @@ __global__ void __launch_bounds__(Threads<T>::value) ab_batch_kernel(const int *
     item_loop(pn, off, args, counter, sa, [&](int64_t li) { ab_row<T, R, true>(sa, li, smem); });
 }
 
-template <int RS>
+template <bool PACKED>
 __global__ void __launch_bounds__(kSrcThreads, 1) ab_src_batch_kernel(const int *pn, const int64_t *off,
                                                                       const AbSrcArgs *args,
                                                                       unsigned long long *counter)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ AbSrcArgs sa;
-    item_loop(pn, off, args, counter, sa, [&](int64_t li) { src_row<RS>(sa, li, smem); });
+    item_loop(pn, off, args, counter, sa, [&](int64_t li) { src_row<PACKED>(sa, li, smem); });
 }
-
-constexpr int kHalfRows = 8;  // the largest rows-per-item setting (mixed)
 
 size_t batch_smem(size_t elem, int R, int max_strings, int max_norb)
 {
-    // 8 rows: the limit that this setting has always had (8 rows of one column half and their J tables)
-    if (R == kHalfRows) return (size_t)32 * ((max_strings + 1) / 2) + (size_t)64 * max_norb * max_norb;
+    if (R == kHalfRows) return halves_smem((max_strings + 1) / 2, max_norb);
     return round16((size_t)max_strings * R * elem) + (size_t)2 * max_norb * max_norb * R * elem;
 }
 
@@ -1479,8 +1783,9 @@ struct SigmaBatch {
     sbd_precision prec = SBD_MIXED;
     int max_slots = 0, R = 1, device = 0, grid_range = 0, grid_ab = 0, grid_t = 0, grid_src = 0;
     size_t smem = 0, range_smem = 0;  // alpha-beta pass, row passes
+    bool rows = false;    // the row passes over whole staged rows (engine, mixed)
+    int grid_rows = 0;
     bool src = false;     // mixed: the column-stationary alpha-beta pass (when its table and accumulator fit)
-    int src_rs = 0;       // its W row stride for the largest slot (8 or 4 float4)
     size_t src_smem = 0;
     int src_threads = 0;
     Layout L{};
@@ -1513,22 +1818,29 @@ void batch_set(SigmaBatch *b, const SigmaSlot *slots, int n)
         const Ctx &c = *sl.c;
         const E *x = static_cast<const E *>(sl.x);
         double *st = static_cast<double *>(sl.xt);
-        rb[i] = range_args<T>(c, 1, reinterpret_cast<const E *>(sl.y), st, 0);
-        ra[i] = range_args<T>(c, 0, x, sl.y, 1);
-        rb[i].q = ra[i].q = q;
         make_ab_args<T>(c, x, sl.y, ab[i]);
-        if constexpr (std::is_same<T, float>::value) {
-            if (b->src) {
-                rb[i].rowmax = c.rowmax;
-                AbSrcArgs sa = src_args(c, x, sl.y, c.rowmax);
-                sa.rs = b->src_rs;  // every slot in the layout the batch's shared memory was sized for
-                reinterpret_cast<AbSrcArgs *>(h + L.src)[i] = sa;
-            }
-        }
         td[i] = TDesc<E>{x, sl.x64, sl.y, st, c.hd, c.nA, c.nB};
-        ot[i + 1] = ot[i] + ((c.nA + 31) / 32) * ((c.nB + 31) / 32);
         ob[i + 1] = ob[i] + (c.nA + kRangeRows<T> - 1) / kRangeRows<T> * q;
         oa[i + 1] = oa[i] + (c.nB + kRangeRows<T> - 1) / kRangeRows<T> * q;
+        float *rowmax = nullptr;
+        if constexpr (std::is_same<T, float>::value) rowmax = b->src ? c.rowmax : nullptr;
+        if (std::is_same<T, float>::value && b->rows) {
+            RowArgs<float> *wb = reinterpret_cast<RowArgs<float> *>(h + L.rb), *wa = reinterpret_cast<RowArgs<float> *>(h + L.ra);
+            make_row_args(c, static_cast<const float *>(sl.x), sl.y, sl.x64, static_cast<const float *>(sl.xt), wb[i], wa[i]);
+            wb[i].rowmax = rowmax;
+            td[i].y = st;  // the transposed amplitudes stay in the work vector
+            ob[i + 1] = ob[i] + (c.nA + b->R - 1) / b->R;
+            oa[i + 1] = oa[i] + (c.nB + b->R - 1) / b->R;
+        } else {
+            rb[i] = range_args<T>(c, 1, reinterpret_cast<const E *>(sl.y), st, 0);
+            ra[i] = range_args<T>(c, 0, x, sl.y, 1);
+            rb[i].q = ra[i].q = q;
+            rb[i].rowmax = rowmax;
+        }
+        if constexpr (std::is_same<T, float>::value) {
+            if (b->src) reinterpret_cast<AbSrcArgs *>(h + L.src)[i] = src_args(c, x, sl.y, c.rowmax);
+        }
+        ot[i + 1] = ot[i] + ((c.nA + 31) / 32) * ((c.nB + 31) / 32);
         oab[i + 1] = oab[i] + c.nA;
     }
 }
@@ -1544,22 +1856,41 @@ void batch_launch_r(SigmaBatch *b, cudaStream_t s)
     const TDesc<E> *td = reinterpret_cast<const TDesc<E> *>(d + L.td);
     transpose_batch_kernel<E, false><<<b->grid_t, dim3(32, 8), 0, s>>>(pn, off_t, td);
     SBD_LAUNCH("transpose_batch_kernel");
-    range_batch_kernel<T><<<b->grid_range, kRangeThreads, b->range_smem, s>>>(
-        pn, reinterpret_cast<const int64_t *>(d + L.off_b), reinterpret_cast<const RangeArgs<T> *>(d + L.rb), b->counters);
-    SBD_LAUNCH("range_batch_kernel");
-    transpose_batch_kernel<E, true><<<b->grid_t, dim3(32, 8), 0, s>>>(pn, off_t, td);
-    SBD_LAUNCH("transpose_batch_kernel");
-    range_batch_kernel<T><<<b->grid_range, kRangeThreads, b->range_smem, s>>>(
-        pn, reinterpret_cast<const int64_t *>(d + L.off_a), reinterpret_cast<const RangeArgs<T> *>(d + L.ra),
-        b->counters + 1);
-    SBD_LAUNCH("range_batch_kernel");
+    const int64_t *off_b = reinterpret_cast<const int64_t *>(d + L.off_b), *off_a = reinterpret_cast<const int64_t *>(d + L.off_a);
+    if (std::is_same<T, float>::value && b->rows) {
+        if constexpr (std::is_same<T, float>::value) {
+            const RowArgs<float> *wb = reinterpret_cast<const RowArgs<float> *>(d + L.rb);
+            const RowArgs<float> *wa = reinterpret_cast<const RowArgs<float> *>(d + L.ra);
+            constexpr int kThreads = Threads<float>::value;
+            if constexpr (R == kHalfRows) {
+                row_halves_batch_kernel<<<b->grid_rows, kThreads, b->smem, s>>>(pn, off_b, wb, b->counters);
+                SBD_LAUNCH("row_halves_batch_kernel");
+                row_halves_batch_kernel<<<b->grid_rows, kThreads, b->smem, s>>>(pn, off_a, wa, b->counters + 1);
+                SBD_LAUNCH("row_halves_batch_kernel");
+            } else {
+                row_batch_kernel<float, R><<<b->grid_rows, kThreads, b->smem, s>>>(pn, off_b, wb, b->counters);
+                SBD_LAUNCH("row_batch_kernel");
+                row_batch_kernel<float, R><<<b->grid_rows, kThreads, b->smem, s>>>(pn, off_a, wa, b->counters + 1);
+                SBD_LAUNCH("row_batch_kernel");
+            }
+        }
+    } else {
+        range_batch_kernel<T><<<b->grid_range, kRangeThreads, b->range_smem, s>>>(
+            pn, off_b, reinterpret_cast<const RangeArgs<T> *>(d + L.rb), b->counters);
+        SBD_LAUNCH("range_batch_kernel");
+        transpose_batch_kernel<E, true><<<b->grid_t, dim3(32, 8), 0, s>>>(pn, off_t, td);
+        SBD_LAUNCH("transpose_batch_kernel");
+        range_batch_kernel<T><<<b->grid_range, kRangeThreads, b->range_smem, s>>>(
+            pn, off_a, reinterpret_cast<const RangeArgs<T> *>(d + L.ra), b->counters + 1);
+        SBD_LAUNCH("range_batch_kernel");
+    }
     if (std::is_same<T, float>::value && b->src) {
         const int64_t *off_ab = reinterpret_cast<const int64_t *>(d + L.off_ab);
         const AbSrcArgs *src_args_d = reinterpret_cast<const AbSrcArgs *>(d + L.src);
-        if (b->src_rs == 8)
-            ab_src_batch_kernel<8><<<b->grid_src, b->src_threads, b->src_smem, s>>>(pn, off_ab, src_args_d, b->counters + 2);
+        if (b->rows)
+            ab_src_batch_kernel<false><<<b->grid_src, b->src_threads, b->src_smem, s>>>(pn, off_ab, src_args_d, b->counters + 2);
         else
-            ab_src_batch_kernel<4><<<b->grid_src, b->src_threads, b->src_smem, s>>>(pn, off_ab, src_args_d, b->counters + 2);
+            ab_src_batch_kernel<true><<<b->grid_src, b->src_threads, b->src_smem, s>>>(pn, off_ab, src_args_d, b->counters + 2);
         SBD_LAUNCH("ab_src_batch_kernel");
         return;
     }
@@ -1579,6 +1910,23 @@ void batch_attrs(SigmaBatch *b)
     SBD_CUDA(cudaFuncSetAttribute(range_batch_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)b->range_smem));
     b->grid_range = sms;
+    if constexpr (std::is_same<T, float>::value) {
+        if (b->rows) {
+            int occ = 0;
+            if constexpr (R == kHalfRows) {
+                SBD_CUDA(cudaFuncSetAttribute(row_halves_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)b->smem));
+                SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, row_halves_batch_kernel, Threads<T>::value,
+                                                                       b->smem));
+            } else {
+                SBD_CUDA(cudaFuncSetAttribute(row_batch_kernel<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)b->smem));
+                SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, row_batch_kernel<T, R>, Threads<T>::value,
+                                                                       b->smem));
+            }
+            b->grid_rows = sms * std::max(1, occ);
+        }
+    }
     if constexpr (R != kHalfRows) {
         int occ_ab = 0;
         SBD_CUDA(cudaFuncSetAttribute(ab_batch_kernel<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
@@ -1591,22 +1939,19 @@ void batch_attrs(SigmaBatch *b)
         int occ_src = 0, optin = 0;
         SBD_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device));
         b->src_threads = kSrcThreads / src_ctas(b->src_smem, optin, INT64_MAX, sms);
-        if (b->src_rs == 8) {
-            SBD_CUDA(cudaFuncSetAttribute(ab_src_batch_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)b->src_smem));
-            SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_src, ab_src_batch_kernel<8>, b->src_threads,
-                                                                   b->src_smem));
-        } else {
-            SBD_CUDA(cudaFuncSetAttribute(ab_src_batch_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)b->src_smem));
-            SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_src, ab_src_batch_kernel<4>, b->src_threads,
-                                                                   b->src_smem));
-        }
+        auto *kernel = b->rows ? ab_src_batch_kernel<false> : ab_src_batch_kernel<true>;
+        SBD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->src_smem));
+        SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_src, kernel, b->src_threads, b->src_smem));
         b->grid_src = sms * std::max(1, occ_src);
     }
 }
 
 }  // namespace
+
+int src_parts(int norb, int64_t n, int smem_optin)
+{
+    return norb >= 2 ? src_parts_for(npairs(norb), n, (size_t)smem_optin - 1024) : 0;
+}
 
 void sigma_prepare(Ctx &c)
 {
@@ -1616,8 +1961,7 @@ void sigma_prepare(Ctx &c)
     set_attrs<double>(lim);
     set_attrs<float>(lim);
     set_attrs<F2>(lim);
-    SBD_CUDA(cudaFuncSetAttribute(ab_src_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-    SBD_CUDA(cudaFuncSetAttribute(ab_src_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+    SBD_CUDA(cudaFuncSetAttribute(ab_src_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
     // max |(pq|rs)| of the FP32 integrals, for the fixed-point scale of the alpha-beta pass
     const int64_t n4 = (int64_t)c.norb * c.norb * c.norb * c.norb;
     unsigned *m = reinterpret_cast<unsigned *>(c.dstat);  // status words are free after create
@@ -1641,7 +1985,7 @@ bool sigma_batch_fits(sbd_precision prec, int R, int max_strings, int max_norb, 
     const size_t lim = sigma_batch_smem_limit(device);
     if (R == kHalfRows)
         return prec == SBD_MIXED && max_norb >= 2 && sigma_batch_smem(prec, R, max_strings, max_norb) <= lim &&
-               src_rs(npairs(max_norb), max_strings, lim) > 0;
+               (size_t)64 * npairs(max_norb) + (size_t)8 * max_strings + round16((size_t)2 * npairs(max_norb)) <= lim;
     if (R == 4 && prec != SBD_MIXED) return false;
     return sigma_batch_smem(prec, R, max_strings, max_norb) <= lim;
 }
@@ -1653,7 +1997,8 @@ size_t sigma_batch_smem_limit(int device)
     return (size_t)optin - 1024;  // headroom for the kernels' static shared memory
 }
 
-SigmaBatch *sigma_batch_create(int max_slots, sbd_precision prec, int R, int max_strings, int max_norb, int device)
+SigmaBatch *sigma_batch_create(int max_slots, sbd_precision prec, int R, int max_strings, int max_norb, int device,
+                               bool rows)
 {
     if (max_slots < 1) fail(SBD_ERR_INVALID_ARG, "batched sigma needs at least one slot");
     if (!(R == 1 || R == 2 || ((R == 4 || R == kHalfRows) && prec == SBD_MIXED)) || prec < SBD_FP64 ||
@@ -1666,6 +2011,7 @@ SigmaBatch *sigma_batch_create(int max_slots, sbd_precision prec, int R, int max
     b->prec = prec;
     b->max_slots = max_slots;
     b->R = R;
+    b->rows = rows && prec == SBD_MIXED;
     b->device = device;
     b->smem = smem;
     int optin = 0;
@@ -1674,9 +2020,11 @@ SigmaBatch *sigma_batch_create(int max_slots, sbd_precision prec, int R, int max
         fail(SBD_ERR_CUDA, "batched sigma: the device does not report its shared memory");
     }
     b->range_smem = range_smem(optin);
-    b->src_rs = max_norb >= 2 ? src_rs(npairs(max_norb), max_strings, sigma_batch_smem_limit(device)) : 0;
-    b->src_smem = b->src_rs ? src_smem(npairs(max_norb), max_strings, b->src_rs) : 0;
-    b->src = prec == SBD_MIXED && b->src_rs > 0;
+    const size_t lim = sigma_batch_smem_limit(device);
+    const int mp = npairs(max_norb), h = max_norb >= 2 ? src_parts_for(mp, max_strings, lim) : 0;
+    // one part for the largest instance is one part for all; else a smaller one may take up to the limit
+    b->src_smem = h == 1 ? src_smem(mp, mp, max_strings) : lim;
+    b->src = prec == SBD_MIXED && h > 0;
     if (R == kHalfRows && !b->src) {
         delete b;
         fail(SBD_ERR_UNSUPPORTED, "batched sigma: 8 rows per item need the column-stationary alpha-beta pass, "

@@ -156,26 +156,68 @@ __global__ void pairs_count_kernel(const uint64_t *__restrict__ S, int64_t n, in
     }
 }
 
-__global__ void pairs_fill_kernel(const uint64_t *__restrict__ S, int64_t n, int norb,
-                                  const double *__restrict__ h, const double *__restrict__ eri, TableOut o)
+// A warp collects its hits in shared memory and works them out 32 at a time: one or two hits in a
+// window of 32 strings would leave the warp waiting for their integrals with the other lanes idle
+// (580 us at 10,000 strings of norb 29).
+constexpr int kFillWarps = 8;
+__global__ void __launch_bounds__(32 * kFillWarps) pairs_fill_kernel(const uint64_t *__restrict__ S, int64_t n, int norb,
+                                                                     const double *__restrict__ h,
+                                                                     const double *__restrict__ eri, TableOut o)
 {
-    const int lane = threadIdx.x & 31;
+    __shared__ int32_t queue[kFillWarps][2][64];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const int64_t nw = (int64_t)gridDim.x * (blockDim.x / 32);
-    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; i < n; i += nw) {
+    int32_t *qs = queue[wib][0], *qd = queue[wib][1];
+    const int64_t nw = (int64_t)gridDim.x * kFillWarps;
+    for (int64_t i = blockIdx.x * (int64_t)kFillWarps + wib; i < n; i += nw) {
         const uint64_t si = S[i];
         int64_t ps = o.s_ptr[i], pd = o.d_ptr[i];
+        int cs = 0, cd = 0;  // hits waiting
+        auto flush_s = [&](int m) {
+            if (lane < m) {
+                const int32_t j = qs[lane];
+                store_single(o, ps + lane, make_single(si, __ldg(S + j), j, norb, h, eri), norb);
+            }
+            ps += m;
+        };
+        auto flush_d = [&](int m) {
+            if (lane < m) {
+                const int32_t j = qd[lane];
+                store_double(o, pd + lane, make_double(si, __ldg(S + j), j, norb, eri));
+            }
+            pd += m;
+        };
         for (int64_t j0 = 0; j0 < n; j0 += 32) {
             const int64_t j = j0 + lane;
             const uint64_t sj = j < n ? __ldg(S + j) : si;
             const int pc = __popcll(si ^ sj);
             const unsigned bs = __ballot_sync(0xffffffffu, pc == 2);
             const unsigned bd = __ballot_sync(0xffffffffu, pc == 4);
-            if (pc == 2) store_single(o, ps + __popc(bs & lt), make_single(si, sj, (int32_t)j, norb, h, eri), norb);
-            if (pc == 4) store_double(o, pd + __popc(bd & lt), make_double(si, sj, (int32_t)j, norb, eri));
-            ps += __popc(bs);
-            pd += __popc(bd);
+            if (pc == 2) qs[cs + __popc(bs & lt)] = (int32_t)j;
+            if (pc == 4) qd[cd + __popc(bd & lt)] = (int32_t)j;
+            cs += __popc(bs);
+            cd += __popc(bd);
+            __syncwarp();
+            if (cs >= 32) {  // uniform
+                flush_s(32);
+                cs -= 32;
+                const int32_t r = qs[32 + lane];
+                __syncwarp();
+                qs[lane] = r;
+                __syncwarp();
+            }
+            if (cd >= 32) {
+                flush_d(32);
+                cd -= 32;
+                const int32_t r = qd[32 + lane];
+                __syncwarp();
+                qd[lane] = r;
+                __syncwarp();
+            }
         }
+        flush_s(cs);
+        flush_d(cd);
+        __syncwarp();  // the next string's hits reuse the queues
     }
 }
 
@@ -374,61 +416,74 @@ __device__ __forceinline__ int slot_of(int q, int Lp)
 // first (both sides, then one), and among those the residues most frequent among the untaken
 // entries, since the busiest residue classes bound the number of conflict-free phases.  Lists longer
 // than kJointMax keep the target-only order.
+// The picks follow one another; a warp scores a list's entries at once (one thread per list: up to 1.3 ms
+// for a few thousand strings).
 constexpr int kJointMax = 1024;
-__device__ bool joint_order(int64_t b, int64_t e, int64_t sb, int Lp, const int32_t *__restrict__ j_src,
-                            const uint32_t *__restrict__ pk, int64_t *perm)
+__global__ void joint_order_kernel(const int64_t *__restrict__ ptr, const int64_t *__restrict__ sig_ptr, int64_t n,
+                                   const int32_t *__restrict__ j_src, const uint32_t *__restrict__ pk, int64_t *perm)
 {
-    const int L = (int)(e - b);
-    if (L > kJointMax) return false;
-    uint32_t taken[kJointMax / 32];
-    for (int w = 0; w < (L + 31) / 32; ++w) taken[w] = 0u;
-    int cj[kBankGroups] = {0, 0, 0, 0, 0, 0, 0, 0}, ck[kBankGroups] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int x = 0; x < L; ++x) {
-        ++cj[j_src[b + x] & (kBankGroups - 1)];
-        ++ck[(pk[b + x] >> kPackKeyShift) & (kBankGroups - 1)];
-    }
-    int q = 0;
-    while (q < L) {
-        const int chunk = q / 32;
-        const int m = min(32, Lp - chunk * 32) / 4;
-        const int phase_end = min(L, q + m - (q - chunk * 32) % m);  // end of the phase q lies in
-        unsigned int usedJ = 0u, usedK = 0u;
-        for (; q < phase_end; ++q) {
-            int best = -1, best_score = -1, brj = 0, brk = 0;
-            for (int x = 0; x < L; ++x) {
-                if (taken[x >> 5] >> (x & 31) & 1u) continue;
-                const int rj = j_src[b + x] & (kBankGroups - 1);
-                const int rk = (pk[b + x] >> kPackKeyShift) & (kBankGroups - 1);
-                const int fresh = (int)!((usedJ >> rj) & 1u) + (int)!((usedK >> rk) & 1u);
-                const int score = fresh * 4096 + cj[rj] + ck[rk];
-                if (score > best_score) {
-                    best_score = score;
-                    best = x;
-                    brj = rj;
-                    brk = rk;
-                }
+    const int lane = threadIdx.x & 31;
+    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; i < n;
+         i += (int64_t)gridDim.x * blockDim.x / 32) {
+        const int64_t b = ptr[i], e = ptr[i + 1], sb = sig_ptr[i];
+        const int L = (int)(e - b), Lp = (int)(sig_ptr[i + 1] - sb);
+        if (L > kJointMax) continue;  // sigma_order_kernel orders these
+        for (int q = lane; q < Lp; q += 32) perm[sb + q] = -1;  // slots no entry lands on stay padding
+        // entry x = lane + 32 y: residues of its target (3 bits) and coefficient row (3 bits), taken when
+        // bit y of `taken` is set; lane r < 8 counts the untaken entries of target residue r, lane 8 + r of
+        // row residue r
+        unsigned taken = 0u;
+        int count = 0;
+        for (int x0 = 0; x0 < L; x0 += 32) {
+            const int x = x0 + lane;
+            const bool in = x < L;
+            const int rj = in ? j_src[b + x] & 7 : -1, rk = in ? (int)(pk[b + x] >> kPackKeyShift) & 7 : -1;
+            for (int r = 0; r < 8; ++r) {
+                const int cj = __popc(__ballot_sync(0xffffffffu, rj == r)), ck = __popc(__ballot_sync(0xffffffffu, rk == r));
+                if (lane == r) count += cj;
+                if (lane == 8 + r) count += ck;
             }
-            taken[best >> 5] |= 1u << (best & 31);
-            usedJ |= 1u << brj;
-            usedK |= 1u << brk;
-            --cj[brj];
-            --ck[brk];
-            perm[sb + slot_of(q, Lp)] = b + best;
+        }
+        __syncwarp();
+        int q = 0;
+        while (q < L) {
+            const int chunk = q / 32;
+            const int m = min(32, Lp - chunk * 32) / 4;
+            const int phase_end = min(L, q + m - (q - chunk * 32) % m);  // end of the phase q lies in
+            unsigned used_j = 0u, used_k = 0u;
+            for (; q < phase_end; ++q) {
+                int best = -1;  // (score << 10 | 1023 - x): the largest score, the first entry among equals
+                for (int x0 = 0, y = 0; x0 < L; x0 += 32, ++y) {
+                    const int x = x0 + lane;
+                    const bool in = x < L && !((taken >> y) & 1u);
+                    const int rj = x < L ? j_src[b + x] & 7 : 0, rk = x < L ? (int)(pk[b + x] >> kPackKeyShift) & 7 : 0;
+                    const int cj = __shfl_sync(0xffffffffu, count, rj), ck = __shfl_sync(0xffffffffu, count, 8 + rk);
+                    const int fresh = (int)!((used_j >> rj) & 1u) + (int)!((used_k >> rk) & 1u);
+                    if (in) best = max(best, ((fresh * 4096 + cj + ck) << 10) | (kJointMax - 1 - x));
+                }
+                best = __reduce_max_sync(0xffffffffu, best);
+                const int x = kJointMax - 1 - (best & (kJointMax - 1));
+                const int rj = j_src[b + x] & 7, rk = (int)(pk[b + x] >> kPackKeyShift) & 7;
+                if ((x & 31) == lane) taken |= 1u << (x >> 5);
+                if (lane == rj || lane == 8 + rk) --count;
+                used_j |= 1u << rj;
+                used_k |= 1u << rk;
+                if (lane == 0) perm[sb + slot_of(q, Lp)] = b + x;
+            }
         }
     }
-    return true;
 }
 
 // perm[sig_ptr[i] + slot] = index of the canonical entry, or -1 for padding.  One thread per source.
-// pk (singles only): packed entries, for the joint target/key order.
+// joint: lists of at most kJointMax entries are joint_order_kernel's.
 __global__ void sigma_order_kernel(const int64_t *__restrict__ ptr, const int64_t *__restrict__ sig_ptr, int64_t n,
-                                   const int32_t *__restrict__ j_src, const uint32_t *__restrict__ pk, int64_t *perm)
+                                   const int32_t *__restrict__ j_src, bool joint, int64_t *perm)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = ptr[i], e = ptr[i + 1], sb = sig_ptr[i], se = sig_ptr[i + 1];
         const int Lp = (int)(se - sb);
+        if (joint && e - b <= kJointMax) continue;
         for (int q = 0; q < Lp; ++q) perm[sb + q] = -1;  // slots no entry lands on stay padding
-        if (pk && joint_order(b, e, sb, Lp, j_src, pk, perm)) continue;
         int count[kBankGroups] = {0, 0, 0, 0, 0, 0, 0, 0};
         for (int64_t x = b; x < e; ++x) ++count[j_src[x] & (kBankGroups - 1)];
         int seen[kBankGroups] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -462,35 +517,48 @@ __global__ void padded_count_kernel(const int64_t *__restrict__ ptr, int64_t n, 
 }
 
 // Source-major singles (column-stationary alpha-beta pass): cnt[i] = items of string i (its singles
-// in pieces of kSrcItem); *maxdeg = largest singles count.
-__global__ void src_count_kernel(const int64_t *__restrict__ ptr, int64_t n, int64_t *cnt, int *maxdeg)
+// with a pair in [p0, p1), in pieces of kSrcItem); *maxdeg = largest singles count.
+// index of the unordered pair of the orbital code of a packed single
+__device__ __forceinline__ int single_pair(uint32_t pk, int norb)
+{
+    const int code = (int)(pk >> (kPackKeyShift + 1)), p = code / norb, q = code - p * norb;
+    const int r = max(p, q), s = min(p, q);
+    return r * (r - 1) / 2 + s;
+}
+
+__global__ void src_count_kernel(const int64_t *__restrict__ ptr, const uint32_t *__restrict__ pk, int64_t n, int norb,
+                                 int p0, int p1, int64_t *cnt, int *maxdeg)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int d = (int)(ptr[i + 1] - ptr[i]);
+        int d = 0;
+        for (int64_t x = ptr[i]; x < ptr[i + 1]; ++x) {
+            const int pair = single_pair(pk[x], norb);
+            d += pair >= p0 && pair < p1;
+        }
         cnt[i] = (d + kSrcItem - 1) / kSrcItem;
-        atomicMax(maxdeg, d);
+        atomicMax(maxdeg, (int)(ptr[i + 1] - ptr[i]));
     }
 }
 
 // items of string i from item ioff[i] on; each entry keeps the target and phase of the canonical
-// single and replaces its orbital code p*norb+q by the index r(r-1)/2 + s of the pair r = max, s = min
+// single and replaces its orbital code p*norb+q by the index r(r-1)/2 + s - p0 of the pair r = max, s = min
 __global__ void src_fill_kernel(const int64_t *__restrict__ ptr, const uint32_t *__restrict__ pk, int64_t n,
-                                int norb, const int64_t *__restrict__ ioff, uint32_t *item, uint32_t *ent)
+                                int norb, int p0, int p1, const int64_t *__restrict__ ioff, uint32_t *item, uint32_t *ent)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = ptr[i], e = ptr[i + 1];
+        int d = 0;
         for (int64_t x = b; x < e; ++x) {
-            const int64_t t = ioff[i] + (x - b) / kSrcItem;
-            const int slot = (int)((x - b) % kSrcItem);
-            if (slot == 0) item[t] = (uint32_t)i | ((uint32_t)min((int64_t)kSrcItem, e - x) << kSrcPairShift);
             const uint32_t v = pk[x];
-            const int code = (int)(v >> (kPackKeyShift + 1));
-            const int p = code / norb, q = code - p * norb;
-            const int r = max(p, q), s = min(p, q);
-            const uint32_t pair = (uint32_t)(r * (r - 1) / 2 + s);
+            const int pair = single_pair(v, norb);
+            if (pair < p0 || pair >= p1) continue;
+            const int64_t t = ioff[i] + d / kSrcItem;
+            const int slot = d % kSrcItem;
+            ++d;
+            item[t] = (uint32_t)i | ((uint32_t)(slot + 1) << kSrcPairShift);  // the last entry leaves the count
             const uint32_t neg = (v >> kPackKeyShift) & 1u;
             ent[(t / 32) * 32 * kSrcItem + 32 * slot + (t % 32)] =
-                (v & kPackJMask) | (pair << kSrcPairShift) | (neg << kSrcNegBit);
+                (v & kPackJMask) | ((uint32_t)(pair - p0) << kSrcPairShift) | (neg << kSrcNegBit);
         }
     }
 }
@@ -516,6 +584,48 @@ __global__ void src_slice_order_kernel(const uint32_t *__restrict__ item_in, con
         item_out[s * 32 + rank] = it;
         const int64_t base = s * 32 * kSrcItem;
         for (int i = 0; i < kSrcItem; ++i) ent_out[base + 32 * i + rank] = ent_in[base + 32 * i + lane];
+    }
+}
+
+// Split of each source list at target `half`: ptr2[2i] = start of list i, ptr2[2i+1] = its first
+// entry with target >= half (targets ascend in the canonical lists), ptr2[2n] = end of the last list
+__global__ void half_split_kernel(const int64_t *__restrict__ ptr, const int32_t *__restrict__ tgt, int64_t n,
+                                  int64_t half, int64_t *ptr2)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        int64_t lo = ptr[i], hi = ptr[i + 1];
+        ptr2[2 * i] = lo;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) / 2;
+            if (tgt[mid] < half) lo = mid + 1;
+            else hi = mid;
+        }
+        ptr2[2 * i + 1] = lo;
+        if (i == n - 1) ptr2[2 * n] = ptr[n];
+    }
+}
+
+// Doubles of the half-split lists: val[o] = FP32 of v[perm[o]], tgt[o] = its target relative to
+// the column half it lies in (target - half for targets >= half); zeros for padding
+__global__ void gather_half_doubles_kernel(const int64_t *__restrict__ perm, int64_t m,
+                                           const int32_t *__restrict__ j, const double *__restrict__ v,
+                                           int64_t half, float *val, uint16_t *tgt)
+{
+    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < m; o += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = perm[o];
+        const int64_t jj = e >= 0 ? (int64_t)j[e] : 0;
+        val[o] = e >= 0 ? __double2float_rn(v[e]) : 0.f;
+        tgt[o] = (uint16_t)(jj >= half ? jj - half : jj);
+    }
+}
+
+// out[o] = (key[perm[o]], FP32 of val[perm[o]]), zeros for padding
+__global__ void gather_pair_kernel(const int64_t *__restrict__ perm, int64_t m, const uint32_t *__restrict__ key,
+                                   const double *__restrict__ val, uint2 *out)
+{
+    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < m; o += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = perm[o];
+        out[o] = e >= 0 ? make_uint2(key[e], __float_as_uint(__double2float_rn(val[e]))) : make_uint2(0u, 0u);
     }
 }
 
@@ -724,42 +834,50 @@ __global__ void slice_fill_kernel(const int64_t *__restrict__ ptr, const uint32_
     }
 }
 
-// Order inside the lists of one 128-bit phase (8 lanes of a slice, one thread): step by step, each lane
+// Order inside the lists of one 128-bit phase (8 lanes of a slice; one warp): step by step, each list
 // takes from its next kSliceWindow entries the one whose target and coefficient row, modulo 8, no
-// earlier lane of the step has taken (both, else one, else the first).
+// earlier list of the step has taken (both, else one, else the first).  The steps follow one another;
+// the warp looks at a window at once, in shared memory (one thread per phase in global memory: 945 us
+// at 10,000 strings of norb 29, 168 singles in the longest list).
 constexpr int kSliceWindow = 16;
-__global__ void slice_order_kernel(const int64_t *__restrict__ ptr, int64_t nsl, const int32_t *__restrict__ col,
-                                   const uint32_t *__restrict__ off, uint32_t *ent)
+constexpr int kSliceSteps = 1024;  // most singles of a string: 32 * 32
+__global__ void __launch_bounds__(32) slice_order_kernel(const int64_t *__restrict__ ptr, int64_t nsl,
+                                                         const int32_t *__restrict__ col,
+                                                         const uint32_t *__restrict__ off, uint32_t *ent)
 {
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < 4 * nsl; x += (int64_t)gridDim.x * blockDim.x) {
+    __shared__ uint32_t w[kSliceSteps * 8];
+    const int lane = threadIdx.x;
+    for (int64_t x = blockIdx.x; x < 4 * nsl; x += gridDim.x) {
         const int64_t s = x / 4;
         uint32_t *e = ent + (int64_t)off[s] * 32 + 8 * (x % 4);
-        int len[8], most = 0;
-#pragma unroll
-        for (int l = 0; l < 8; ++l) {
-            const int32_t i = col[s * 32 + 8 * (x % 4) + l];
-            len[l] = i >= 0 ? (int)(ptr[i + 1] - ptr[i]) : 0;
-            most = max(most, len[l]);
-        }
+        const int32_t i = lane < 8 ? col[s * 32 + 8 * (x % 4) + lane] : -1;
+        const int len = i >= 0 ? (int)(ptr[i + 1] - ptr[i]) : 0;
+        const int most = __reduce_max_sync(0xffffffffu, len);
+        for (int z = lane; z < most * 8; z += 32) w[z] = e[32 * (z / 8) + z % 8];
+        __syncwarp();
         for (int t = 0; t < most; ++t) {
             unsigned used_j = 0u, used_k = 0u;
-#pragma unroll
             for (int l = 0; l < 8; ++l) {
-                if (t >= len[l]) continue;
-                int best = t, score = -1;
-                for (int y = t; y < min(t + kSliceWindow, len[l]); ++y) {
-                    const uint32_t v = e[32 * y + l];
-                    const int f = (int)!((used_j >> (v & 7u)) & 1u) + (int)!((used_k >> ((v >> kPackKeyShift) & 7u)) & 1u);
-                    if (f > score) best = y, score = f;
-                    if (f == 2) break;
+                const int ll = __shfl_sync(0xffffffffu, len, l);
+                if (t >= ll) continue;
+                const int y = t + lane;
+                const bool in = lane < kSliceWindow && y < ll;
+                const uint32_t v = in ? w[8 * y + l] : 0u;
+                const bool fj = in && !((used_j >> (v & 7u)) & 1u), fk = in && !((used_k >> ((v >> kPackKeyShift) & 7u)) & 1u);
+                const unsigned two = __ballot_sync(0xffffffffu, fj && fk), one = __ballot_sync(0xffffffffu, fj || fk);
+                const int best = two ? __ffs(two) - 1 : one ? __ffs(one) - 1 : 0;
+                const uint32_t take = __shfl_sync(0xffffffffu, v, best), head = __shfl_sync(0xffffffffu, v, 0);
+                if (lane == 0) {
+                    w[8 * (t + best) + l] = head;
+                    w[8 * t + l] = take;
                 }
-                const uint32_t v = e[32 * best + l];
-                e[32 * best + l] = e[32 * t + l];
-                e[32 * t + l] = v;
-                used_j |= 1u << (v & 7u);
-                used_k |= 1u << ((v >> kPackKeyShift) & 7u);
+                __syncwarp();
+                used_j |= 1u << (take & 7u);
+                used_k |= 1u << ((take >> kPackKeyShift) & 7u);
             }
         }
+        for (int z = lane; z < most * 8; z += 32) e[32 * (z / 8) + z % 8] = w[z];
+        __syncwarp();
     }
 }
 
@@ -832,7 +950,10 @@ __global__ void to_float_kernel(const double *in, float *out, int64_t n)
         out[i] = __double2float_rn(in[i]);
 }
 
-// Hd[ia, ib] = E_alpha(ia) + E_beta(ib) + sum_{p in ia, r in ib} (pp|rr)   (Sec. II-E)
+// Hd[ia, ib] = E_alpha(ia) + E_beta(ib) + sum_{p in ia, r in ib} (pp|rr)   (Sec. II-E).  Bound by the FP64
+// pipe, one addition per electron.  (Looking the sum up byte by byte halves the time, but rounds
+// differently: determinants of equal energy then take another order, and a solve that starts from the
+// lowest of them can take another path.)
 __global__ void hdiag_kernel(const uint64_t *__restrict__ A, const uint64_t *__restrict__ B,
                              const double *__restrict__ eA, const double *__restrict__ eB,
                              const double *__restrict__ eri, int norb, int64_t nA, int64_t nB, double *hd)
@@ -950,46 +1071,25 @@ void build_tables(Ctx &c, int spin)
                                                                   c.h64, c.eri64, o);
         SBD_LAUNCH("enum_kernel(fill)");
     }
-    // source-major singles: items of at most kSrcItem singles, 32 items per slice
-    {
-        int64_t *ioff = dalloc_n<int64_t>(c, n + 1);
-        int *dmax = reinterpret_cast<int *>(cnt + n);  // the doubles counts are no longer needed
-        SBD_CUDA(cudaMemsetAsync(dmax, 0, sizeof(int), c.stream));
-        src_count_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(t.s_ptr, n, cnt, dmax);
-        SBD_LAUNCH("src_count_kernel");
-        scan_kernel<<<1, 1024, 0, c.stream>>>(cnt, n, ioff);
-        SBD_LAUNCH("scan_kernel(source-major singles)");
-        SBD_CUDA(cudaMemcpyAsync(&t.src_nitem, ioff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
-        SBD_CUDA(cudaMemcpyAsync(&t.src_maxdeg, dmax, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
-        SBD_CUDA(cudaStreamSynchronize(c.stream));
-        const int64_t nsl = std::max<int64_t>((t.src_nitem + 31) / 32, 1);
-        t.src_item = dalloc_n<uint32_t>(c, (size_t)nsl * 32);
-        t.src_ent = dalloc_n<uint32_t>(c, (size_t)nsl * 32 * kSrcItem);
-        SBD_CUDA(cudaMemsetAsync(t.src_item, 0, (size_t)nsl * 32 * sizeof(uint32_t), c.stream));
-        SBD_CUDA(cudaMemsetAsync(t.src_ent, 0, (size_t)nsl * 32 * kSrcItem * sizeof(uint32_t), c.stream));
-        src_fill_kernel<<<blocks_for(n, 128), 128, 0, c.stream>>>(t.s_ptr, t.s_pk, n, norb, ioff, t.src_item,
-                                                                  t.src_ent);
-        SBD_LAUNCH("src_fill_kernel");
-        dfree(c, ioff);
-        uint32_t *item2 = dalloc_n<uint32_t>(c, (size_t)nsl * 32);
-        uint32_t *ent2 = dalloc_n<uint32_t>(c, (size_t)nsl * 32 * kSrcItem);
-        src_slice_order_kernel<<<blocks_for(nsl * 32, 256), 256, 0, c.stream>>>(t.src_item, t.src_ent, nsl, item2,
-                                                                                ent2);
-        SBD_LAUNCH("src_slice_order_kernel");
-        dfree(c, t.src_item);
-        dfree(c, t.src_ent);
-        t.src_item = item2;
-        t.src_ent = ent2;
-        src_entry_order_kernel<<<blocks_for(nsl, 64), 64, 0, c.stream>>>(t.src_item, t.src_ent, nsl);
-        SBD_LAUNCH("src_entry_order_kernel");
-    }
     t.ediag = dalloc_n<double>(c, n);
     ediag_kernel<<<blocks_for(n, 128), 128, 0, c.stream>>>(t.strings, n, norb, c.h64, c.eri64, t.ediag);
     SBD_LAUNCH("ediag_kernel");
     dfree(c, cnt);
 }
 
-void build_sig_lists(Ctx &c, SpinTables &t)
+// sigma order of n lists; pk (singles only): packed entries, for the joint target/row order
+static void order_lists(Ctx &c, const int64_t *ptr, const int64_t *sig_ptr, int64_t n, const int32_t *j,
+                        const uint32_t *pk, int64_t *perm)
+{
+    if (pk) {
+        joint_order_kernel<<<blocks_for(n, 4, 65535), 128, 0, c.stream>>>(ptr, sig_ptr, n, j, pk, perm);
+        SBD_LAUNCH("joint_order_kernel");
+    }
+    sigma_order_kernel<<<blocks_for(n, 128), 128, 0, c.stream>>>(ptr, sig_ptr, n, j, pk != nullptr, perm);
+    SBD_LAUNCH("sigma_order_kernel");
+}
+
+void build_sig_lists(Ctx &c, SpinTables &t, bool fp32_only)
 {
     const int64_t n = t.n;
     int64_t *cnt = dalloc_n<int64_t>(c, 2 * (size_t)n);
@@ -1013,9 +1113,8 @@ void build_sig_lists(Ctx &c, SpinTables &t)
     t.d_jv32 = dalloc_n<uint2>(c, t.sig_nd);
     t.d_vx2 = dalloc_n<float2>(c, t.sig_nd);
     int64_t *perm = dalloc_n<int64_t>(c, (size_t)std::max<int64_t>(std::max(t.sig_ns, t.sig_nd), 1));
-    const int ob = blocks_for(n, 128);
     if (t.sig_ns) {
-        sigma_order_kernel<<<ob, 128, 0, c.stream>>>(t.s_ptr, t.sig_s_ptr, n, t.s_j, t.s_pk, perm);
+        order_lists(c, t.s_ptr, t.sig_s_ptr, n, t.s_j, t.s_pk, perm);
         SBD_LAUNCH("sigma_order_kernel(singles)");
         const int gb = blocks_for(t.sig_ns, 256, 16384);
         gather_kernel<uint32_t><<<gb, 256, 0, c.stream>>>(t.s_pk, perm, t.s_pk_sig, t.sig_ns);
@@ -1027,7 +1126,7 @@ void build_sig_lists(Ctx &c, SpinTables &t)
         SBD_LAUNCH("split_kernel(singles)");
     }
     if (t.sig_nd) {
-        sigma_order_kernel<<<ob, 128, 0, c.stream>>>(t.d_ptr, d_ptr, n, t.d_j, nullptr, perm);
+        order_lists(c, t.d_ptr, d_ptr, n, t.d_j, nullptr, perm);
         SBD_LAUNCH("sigma_order_kernel(doubles)");
         const int gb = blocks_for(t.sig_nd, 256, 16384);
         gather_kernel<int32_t><<<gb, 256, 0, c.stream>>>(t.d_j, perm, t.d_j_sig, t.sig_nd);
@@ -1041,11 +1140,151 @@ void build_sig_lists(Ctx &c, SpinTables &t)
     }
     dfree(c, perm);
     dfree(c, cnt);
+    if (fp32_only) {
+        for (void *q : {(void *)t.s_pk_sig, (void *)t.s_v64_sig, (void *)t.s_vx2, (void *)t.d_j_sig, (void *)t.d_v64_sig,
+                        (void *)t.d_vx2})
+            dfree(c, q);
+        t.s_pk_sig = nullptr;
+        t.s_v64_sig = t.d_v64_sig = nullptr;
+        t.s_vx2 = t.d_vx2 = nullptr;
+        t.d_j_sig = nullptr;
+    }
     t.sig_d_ptr = d_ptr;  // set last: marks the copies as complete
 }
 
-// Slices of the two-operand alpha-beta pass (SpinTables::sl_*).
-static void build_slices(Ctx &c, SpinTables &t)
+// Lists split at the middle of the string set
+static void build_half_lists(Ctx &c, SpinTables &t)
+{
+    const int64_t n = t.n;
+    // mixed-sigma lists split at the middle of the set (row passes over column halves); their
+    // 16-bit doubles targets need half <= 65536 (the staged halves fit shared memory only far below)
+    if ((n + 1) / 2 <= 65536) {
+        t.half = (n + 1) / 2;
+        int64_t *ptr2 = dalloc_n<int64_t>(c, 2 * (size_t)n + 1);
+        int64_t *cnt2 = dalloc_n<int64_t>(c, 2 * (size_t)n);
+        for (int kind = 0; kind < 2; ++kind) {
+            const int64_t *ptr = kind == 0 ? t.s_ptr : t.d_ptr;
+            const int32_t *tgt = kind == 0 ? t.s_j : t.d_j;
+            int64_t *&hptr = kind == 0 ? t.hs_ptr : t.hd_ptr;
+            half_split_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(ptr, tgt, n, t.half, ptr2);
+            SBD_LAUNCH("half_split_kernel");
+            hptr = dalloc_n<int64_t>(c, 2 * (size_t)n + 1);
+            padded_count_kernel<<<blocks_for(2 * n, 256), 256, 0, c.stream>>>(ptr2, 2 * n, cnt2);
+            SBD_LAUNCH("padded_count_kernel(halves)");
+            scan_kernel<<<1, 1024, 0, c.stream>>>(cnt2, 2 * n, hptr);
+            SBD_LAUNCH("scan_kernel(halves)");
+            int64_t m = 0;
+            SBD_CUDA(cudaMemcpyAsync(&m, hptr + 2 * n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
+            SBD_CUDA(cudaStreamSynchronize(c.stream));
+            const size_t mm = (size_t)std::max<int64_t>(m, 1);
+            if (kind == 0) {
+                t.hs = dalloc_n<uint2>(c, mm);
+            } else {
+                t.hdv = dalloc_n<float>(c, mm);
+                t.hdt = dalloc_n<uint16_t>(c, mm);
+            }
+            if (m) {
+                int64_t *hperm = dalloc_n<int64_t>(c, (size_t)m);
+                order_lists(c, ptr2, hptr, 2 * n, tgt, kind == 0 ? t.s_pk : nullptr, hperm);
+                SBD_LAUNCH("sigma_order_kernel(halves)");
+                if (kind == 0) {
+                    gather_pair_kernel<<<blocks_for(m, 256, 16384), 256, 0, c.stream>>>(hperm, m, t.s_pk, t.s_v64,
+                                                                                         t.hs);
+                    SBD_LAUNCH("gather_pair_kernel(halves)");
+                } else {
+                    gather_half_doubles_kernel<<<blocks_for(m, 256, 16384), 256, 0, c.stream>>>(
+                        hperm, m, t.d_j, t.d_v64, t.half, t.hdv, t.hdt);
+                    SBD_LAUNCH("gather_half_doubles_kernel");
+                }
+                dfree(c, hperm);
+            }
+        }
+        dfree(c, cnt2);
+        dfree(c, ptr2);
+    }
+}
+
+void build_engine_lists(Ctx &c, int rows)
+{
+    for (int spin = 0; spin < 2; ++spin) {
+        SpinTables &t = c.sp[spin];
+        if (t.alias) {
+            const SpinTables o = c.sp[0];
+            uint64_t *own = t.strings;
+            const int parts = t.src_parts, width = t.src_width, deg = t.src_maxdeg;
+            uint32_t *item = t.src_item, *ent = t.src_ent;
+            int slice[kSrcParts + 1];
+            std::copy(t.src_slice, t.src_slice + kSrcParts + 1, slice);
+            t = o;
+            t.strings = own;
+            t.alias = true;
+            t.src_parts = parts, t.src_width = width, t.src_maxdeg = deg;
+            t.src_item = item, t.src_ent = ent;
+            std::copy(slice, slice + kSrcParts + 1, t.src_slice);
+            continue;
+        }
+        // the FP32 and FP64 elements of the range lists: the engine's products are these lists' and pairs
+        for (void *q : {(void *)t.rl.dv32, (void *)t.rl.dv64, (void *)t.rl.sv32, (void *)t.rl.sv64}) dfree(c, q);
+        t.rl.dv32 = t.rl.sv32 = nullptr;
+        t.rl.dv64 = t.rl.sv64 = nullptr;
+        if (rows == 0 || rows == 8) build_half_lists(c, t);
+        if (rows != 8) build_sig_lists(c, t, true);
+    }
+    SBD_CUDA(cudaStreamSynchronize(c.stream));
+}
+
+void build_src_lists(Ctx &c, int spin)
+{
+    SpinTables &t = c.sp[spin];
+    const int64_t n = t.n;
+    const int norb = c.norb, npair = norb * (norb - 1) / 2;
+    t.src_parts = src_parts(norb, n, c.smem_optin);
+    const int parts = std::max(t.src_parts, 1);
+    t.src_width = std::max(1, (npair + parts - 1) / parts);
+    int64_t *cnt = dalloc_n<int64_t>(c, (size_t)n);
+    int64_t *ioff = dalloc_n<int64_t>(c, (size_t)parts * (n + 1));
+    int *dmax = dalloc_n<int>(c, 1);
+    SBD_CUDA(cudaMemsetAsync(dmax, 0, sizeof(int), c.stream));
+    int64_t items[kSrcParts] = {0};
+    for (int h = 0; h < parts; ++h) {
+        src_count_kernel<<<blocks_for(n, 128), 128, 0, c.stream>>>(t.s_ptr, t.s_pk, n, norb, h * t.src_width,
+                                                                   (h + 1) * t.src_width, cnt, dmax);
+        SBD_LAUNCH("src_count_kernel");
+        scan_kernel<<<1, 1024, 0, c.stream>>>(cnt, n, ioff + h * (n + 1));
+        SBD_LAUNCH("scan_kernel(source-major singles)");
+        SBD_CUDA(cudaMemcpyAsync(&items[h], ioff + h * (n + 1) + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
+    }
+    SBD_CUDA(cudaMemcpyAsync(&t.src_maxdeg, dmax, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
+    SBD_CUDA(cudaStreamSynchronize(c.stream));
+    t.src_slice[0] = 0;
+    for (int h = 0; h < parts; ++h) t.src_slice[h + 1] = t.src_slice[h] + (int)((items[h] + 31) / 32);
+    const int64_t nsl = std::max(t.src_slice[parts], 1);
+    uint32_t *item = dalloc_n<uint32_t>(c, (size_t)nsl * 32), *ent = dalloc_n<uint32_t>(c, (size_t)nsl * 32 * kSrcItem);
+    t.src_item = dalloc_n<uint32_t>(c, (size_t)nsl * 32);
+    t.src_ent = dalloc_n<uint32_t>(c, (size_t)nsl * 32 * kSrcItem);
+    SBD_CUDA(cudaMemsetAsync(item, 0, (size_t)nsl * 32 * sizeof(uint32_t), c.stream));
+    SBD_CUDA(cudaMemsetAsync(ent, 0, (size_t)nsl * 32 * kSrcItem * sizeof(uint32_t), c.stream));
+    for (int h = 0; h < parts; ++h) {
+        const size_t s0 = (size_t)t.src_slice[h] * 32;
+        src_fill_kernel<<<blocks_for(n, 128), 128, 0, c.stream>>>(t.s_ptr, t.s_pk, n, norb, h * t.src_width,
+                                                                  (h + 1) * t.src_width, ioff + h * (n + 1), item + s0,
+                                                                  ent + s0 * kSrcItem);
+        SBD_LAUNCH("src_fill_kernel");
+    }
+    src_slice_order_kernel<<<blocks_for(nsl * 32, 256), 256, 0, c.stream>>>(item, ent, nsl, t.src_item, t.src_ent);
+    SBD_LAUNCH("src_slice_order_kernel");
+    src_entry_order_kernel<<<blocks_for(nsl, 64), 64, 0, c.stream>>>(t.src_item, t.src_ent, nsl);
+    SBD_LAUNCH("src_entry_order_kernel");
+    dfree(c, item);
+    dfree(c, ent);
+    dfree(c, cnt);
+    dfree(c, ioff);
+    dfree(c, dmax);
+}
+
+// Slices of the two-operand alpha-beta pass (SpinTables::sl_*); without `entries`, only the order of the
+// strings (in which the column-stationary pass takes its rows).
+static void build_slices(Ctx &c, SpinTables &t, bool entries)
 {
     const int64_t n = t.n, nsl = (n + 31) / 32;
     uint64_t *keys = dalloc_n<uint64_t>(c, (size_t)n);
@@ -1057,6 +1296,12 @@ static void build_slices(Ctx &c, SpinTables &t)
     radix_sort_strings(c, keys, n, 16);  // stable, by the low 16 bits: descending length
     slice_col_kernel<<<blocks_for(32 * nsl, 256), 256, 0, c.stream>>>(keys, n, nsl, t.sl_col, len);
     SBD_LAUNCH("slice_col_kernel");
+    if (!entries) {
+        dfree(c, keys);
+        dfree(c, len);
+        dfree(c, off);
+        return;
+    }
     scan_kernel<<<1, 1024, 0, c.stream>>>(len, nsl, off);
     SBD_LAUNCH("scan_kernel(slices)");
     narrow_kernel<<<blocks_for(nsl + 1, 256), 256, 0, c.stream>>>(off, t.sl_off, nsl + 1);
@@ -1069,7 +1314,7 @@ static void build_slices(Ctx &c, SpinTables &t)
         slice_fill_kernel<<<blocks_for(32 * nsl, 128, 65535), 128, 0, c.stream>>>(t.s_ptr, t.s_pk, c.norb, nsl, t.sl_col,
                                                                                 t.sl_off, t.sl_ent);
         SBD_LAUNCH("slice_fill_kernel");
-        slice_order_kernel<<<blocks_for(4 * nsl, 32, 65535), 32, 0, c.stream>>>(t.s_ptr, nsl, t.sl_col, t.sl_off, t.sl_ent);
+        slice_order_kernel<<<blocks_for(4 * nsl, 1, 65535), 32, 0, c.stream>>>(t.s_ptr, nsl, t.sl_col, t.sl_off, t.sl_ent);
         SBD_LAUNCH("slice_order_kernel");
     }
     dfree(c, keys);
@@ -1077,7 +1322,7 @@ static void build_slices(Ctx &c, SpinTables &t)
     dfree(c, off);
 }
 
-void build_range_lists(Ctx &c, int spin)
+void build_range_lists(Ctx &c, int spin, bool beta)
 {
     SpinTables &t = c.sp[spin];
     RangeLists &r = t.rl;
@@ -1128,7 +1373,7 @@ void build_range_lists(Ctx &c, int spin)
         range_fill_kernel<2><<<fb, 256, 0, c.stream>>>(t.d_ptr, t.d_j, nullptr, t.d_v64, groups, c.norb, r);
         SBD_LAUNCH("range_fill_kernel(doubles)");
     }
-    build_slices(c, t);
+    build_slices(c, t, beta);
     const int npair = c.norb * (c.norb - 1) / 2;
     r.jg = dalloc_n<double>(c, (size_t)npair * n);
     if (npair) {

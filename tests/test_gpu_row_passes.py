@@ -1,4 +1,4 @@
-"""Row passes of the sigma product at the sizes where they can go wrong, against the oracle: one, just
+"""Sigma product at the sizes where its row passes can go wrong, against the oracle: one, just
 one, and several ranges of staged strings; row blocks (16 or 32 rows) with and without a remainder;
 groups of lists (8) and parts (16) that are empty, partial and full; the coefficient table in shared
 memory (norb <= 42) and in global memory."""
@@ -15,6 +15,7 @@ CASES = [
     (29, 10, 17, 2803),                      # three ranges on the other side
     (44, 3, 1809, 16), (44, 15, 47, 130),    # coefficients in global memory, one and two ranges
     (42, 4, 948, 15), (43, 4, 948, 15),      # last norb with the table staged, first without; two ranges, one
+    (64, 5, 40, 530), (58, 4, 33, 2500),     # orbital pairs of the alpha-beta pass in two parts
     (12, 4, 1, 129), (12, 4, 7, 128), (12, 4, 9, 32), (12, 4, 16, 1), (10, 3, 120, 17),
 ]
 
