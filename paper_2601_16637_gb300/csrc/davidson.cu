@@ -74,6 +74,30 @@ __device__ __forceinline__ T block_sum(T v, T *red)
     return s;  // valid in thread 0
 }
 
+// out[a] = block sum of value(a), a < k <= K, in the order block_sum adds: the warps' sums of all k go
+// through shared memory together, so k sums cost one barrier instead of 2k (32 dot products of a short
+// vector spent 28 us on them)
+template <int K, typename F>
+__device__ __forceinline__ void block_sums(int k, F &&value, double *out)
+{
+    __shared__ double red[K][kBlas / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < K; ++a)
+        if (a < k) {  // k is uniform over the block
+            double v = value(a);
+            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+            if (lane == 0) red[a][warp] = v;
+        }
+    __syncthreads();
+    if (threadIdx.x < k) {
+        double s = 0.0;
+        for (int w = 0; w < kBlas / 32; ++w) s += red[threadIdx.x][w];
+        out[threadIdx.x] = s;
+    }
+}
+
 // partial[b*kPart + a] = sum over block b's elements of X[a][i] y[i] (a < k <= kDotMax);
 // with NORM also partial[b*kPart + kDotMax] = sum y[i]^2
 template <bool NORM, int KB>
@@ -99,12 +123,7 @@ __global__ void __launch_bounds__(kBlas, KB <= 16 ? 4 : 2) mdot_partial(const do
             }
         }
     }
-#pragma unroll
-    for (int a = 0; a < KB; ++a)
-        if (a < k) {  // k is uniform over the block
-            const double s = block_sum(acc[a], red);
-            if (threadIdx.x == 0) partial[blockIdx.x * kPart + a] = s;
-        }
+    block_sums<KB>(k, [&](int a) { return acc[a]; }, partial + blockIdx.x * kPart);
     if (NORM) {
         const double s = block_sum(an, red);
         if (threadIdx.x == 0) partial[blockIdx.x * kPart + kDotMax] = s;
@@ -139,12 +158,7 @@ __global__ void __launch_bounds__(kBlas) mdot_pair_partial(const double *__restr
 #pragma unroll
         for (int u = 0; u < kPairChunk; ++u) f2_mac(acc[u], f2_split(x[u]), ys);
     }
-#pragma unroll
-    for (int a = 0; a < kPairChunk; ++a)
-        if (a < kc) {  // kc is uniform over the block
-            const double s = block_sum(f2_value(acc[a]), red);
-            if (threadIdx.x == 0) partial[blockIdx.x * kPart + a0 + a] = s;
-        }
+    block_sums<kPairChunk>(kc, [&](int a) { return f2_value(acc[a]); }, partial + blockIdx.x * kPart + a0);
     if (nrm) {
         const double s = block_sum(an, red);
         if (threadIdx.x == 0) partial[blockIdx.x * kPart + kDotMax] = s;
