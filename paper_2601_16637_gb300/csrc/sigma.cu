@@ -892,7 +892,9 @@ __global__ void __launch_bounds__(Threads<T>::value) ab_pass_kernel(const AbArgs
 // The element is hi_sum * 2^L + lo_sum exactly; the row is added to s(ia, :) in FP64 by the CTA
 // that owns the row.
 
-constexpr int kSrcThreads = 896;
+constexpr int kSrcThreads = 1024;  // packed dot products (896: 18.4 ms, 1,024: 18.1 at 1.0e8 determinants)
+template <bool PACKED>
+constexpr int kSrcThreadsOf = PACKED ? kSrcThreads : 896;  // one chain: more registers a thread
 
 struct AbSrcArgs {
     const float *C;  // [nA][nB] FP32 amplitudes
@@ -975,9 +977,6 @@ __device__ __forceinline__ void src_chunk(const AbSrcArgs &a, const float4 *__re
         const int64_t jb = info & kPackJMask;
         const int cnt = (int)(info >> kSrcPairShift);
         const uint32_t *ent = a.src_ent + (int64_t)sl * 32 * kSrcItem + lane;
-        uint32_t e[kSrcItem];
-#pragma unroll
-        for (int i = 0; i < kSrcItem; ++i) e[i] = i < cnt ? __ldg(ent + 32 * i) : 0u;
         if constexpr (PACKED) {
             // amplitudes of the chunk's alpha singles at column jb (consecutive lanes: consecutive or equal
             // columns), two to a word, then permuted so that register chunk s holds amplitude chunk s xor rot
@@ -1007,28 +1006,36 @@ __device__ __forceinline__ void src_chunk(const AbSrcArgs &a, const float4 *__re
                         }
                     }
             }
+            uint32_t n0 = cnt > 0 ? __ldg(ent) : 0u, n1 = cnt > 1 ? __ldg(ent + 32) : 0u;
 #pragma unroll
             for (int i = 0; i < kSrcItem; i += 2) {  // two singles per round for independent chains
+                const uint32_t e0 = n0, e1 = n1;
+                ent += 64;
+                n0 = i + 2 < cnt ? __ldg(ent) : 0u;
+                n1 = i + 3 < cnt ? __ldg(ent + 32) : 0u;
                 if (i < cnt) {
                     const bool two = i + 1 < cnt;
-                    const uint32_t o0 = ((e[i] >> kSrcPairShift) & 0x7ffu) * (RS * 16u) + first;
-                    const uint32_t o1 = ((e[i + 1] >> kSrcPairShift) & 0x7ffu) * (RS * 16u) + first;
+                    const uint32_t o0 = ((e0 >> kSrcPairShift) & 0x7ffu) * (RS * 16u) + first;
+                    const uint32_t o1 = ((e1 >> kSrcPairShift) & 0x7ffu) * (RS * 16u) + first;
                     uint64_t f0 = 0ull, f1 = 0ull;
 #pragma unroll
                     for (int s = 0; s < CPW; ++s) {  // chunk s xor rot of the row: 8 lanes, 8 bank groups
                         const ulonglong2 x0 = *reinterpret_cast<const ulonglong2 *>(Wb + (o0 ^ (s * 16u)));
-                        const ulonglong2 x1 = two ? *reinterpret_cast<const ulonglong2 *>(Wb + (o1 ^ (s * 16u)))
-                                                  : make_ulonglong2(0ull, 0ull);
+                        // where there is no second single, entry 0 reads the table's first row: unused
+                        const ulonglong2 x1 = *reinterpret_cast<const ulonglong2 *>(Wb + (o1 ^ (s * 16u)));
                         f0 = pk_fma(x0.x, cv[2 * s], f0);
                         f1 = pk_fma(x1.x, cv[2 * s], f1);
                         f0 = pk_fma(x0.y, cv[2 * s + 1], f0);
                         f1 = pk_fma(x1.y, cv[2 * s + 1], f1);
                     }
-                    src_add(acc_lo, acc_hi, e[i], pk_get(f0, 0) + pk_get(f0, 1), scale_hi, two_l, lbits);
-                    if (two) src_add(acc_lo, acc_hi, e[i + 1], pk_get(f1, 0) + pk_get(f1, 1), scale_hi, two_l, lbits);
+                    src_add(acc_lo, acc_hi, e0, pk_get(f0, 0) + pk_get(f0, 1), scale_hi, two_l, lbits);
+                    if (two) src_add(acc_lo, acc_hi, e1, pk_get(f1, 0) + pk_get(f1, 1), scale_hi, two_l, lbits);
                 }
             }
         } else {
+            uint32_t e[kSrcItem];
+#pragma unroll
+            for (int i = 0; i < kSrcItem; ++i) e[i] = i < cnt ? __ldg(ent + 32 * i) : 0u;
             // amplitudes of the chunk's alpha singles at column jb (consecutive lanes: consecutive or equal
             // columns), then rotated by `rot` chunks so that register chunk s holds amplitude chunk
             // (s + rot) mod CPW
@@ -1064,7 +1071,7 @@ __device__ __forceinline__ void src_chunk(const AbSrcArgs &a, const float4 *__re
                     for (int s = 0; s < CPW; ++s) {
                         const int q = (s + rot) & (CPW - 1);
                         const float4 x0 = w0[q];
-                        const float4 x1 = two ? w1[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float4 x1 = w1[q];  // where there is no second single: the first row, unused
                         f0 = fmaf(x0.x, cv[4 * s], f0);
                         f1 = fmaf(x1.x, cv[4 * s], f1);
                         f0 = fmaf(x0.y, cv[4 * s + 1], f0);
@@ -1762,7 +1769,7 @@ __global__ void __launch_bounds__(Threads<T>::value) ab_batch_kernel(const int *
 }
 
 template <bool PACKED>
-__global__ void __launch_bounds__(kSrcThreads, 1) ab_src_batch_kernel(const int *pn, const int64_t *off,
+__global__ void __launch_bounds__(kSrcThreadsOf<PACKED>, 1) ab_src_batch_kernel(const int *pn, const int64_t *off,
                                                                       const AbSrcArgs *args,
                                                                       unsigned long long *counter)
 {
@@ -1938,7 +1945,7 @@ void batch_attrs(SigmaBatch *b)
     if (b->src) {
         int occ_src = 0, optin = 0;
         SBD_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device));
-        b->src_threads = kSrcThreads / src_ctas(b->src_smem, optin, INT64_MAX, sms);
+        b->src_threads = (b->rows ? kSrcThreadsOf<false> : kSrcThreads) / src_ctas(b->src_smem, optin, INT64_MAX, sms);
         auto *kernel = b->rows ? ab_src_batch_kernel<false> : ab_src_batch_kernel<true>;
         SBD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->src_smem));
         SBD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_src, kernel, b->src_threads, b->src_smem));
