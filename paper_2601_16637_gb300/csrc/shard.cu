@@ -171,25 +171,32 @@ BlockPlan *block_plan_create(Ctx &c, int64_t r0, int64_t r1, int64_t j0, int64_t
     if (r0 < 0 || r1 <= r0 || r1 > c.nA || j0 < 0 || j1 <= j0 || j1 > c.nA)
         fail(SBD_ERR_INVALID_ARG, "block plan: row ranges must be non-empty and inside [0, nA)");
     // the lists that the plans restrict (and the beta pass of a block reads), made with the first plan
-    if (!c.sp[0].sig_d_ptr) build_sig_lists(c, c.sp[0]);
-    if (!c.sp[1].sig_d_ptr) {
-        if (c.sp[1].alias) {
-            SpinTables &a = c.sp[0], &b = c.sp[1];
-            b.sig_s_ptr = a.sig_s_ptr;
-            b.sig_ns = a.sig_ns;
-            b.s_pk_sig = a.s_pk_sig;
-            b.s_v64_sig = a.s_v64_sig;
-            b.s_pkv32 = a.s_pkv32;
-            b.s_vx2 = a.s_vx2;
-            b.sig_d_ptr = a.sig_d_ptr;
-            b.sig_nd = a.sig_nd;
-            b.d_j_sig = a.d_j_sig;
-            b.d_v64_sig = a.d_v64_sig;
-            b.d_jv32 = a.d_jv32;
-            b.d_vx2 = a.d_vx2;
-        } else {
-            build_sig_lists(c, c.sp[1]);
+    const size_t held = c.allocs.size();
+    try {
+        if (!c.sp[0].sig_d_ptr) build_sig_lists(c, c.sp[0]);
+        if (!c.sp[1].alias && !c.sp[1].sig_d_ptr) build_sig_lists(c, c.sp[1]);
+    } catch (...) {  // an allocation was refused: the handle is as it was
+        while (c.allocs.size() > held) dfree(c, c.allocs.back().first);
+        for (SpinTables &t : c.sp) {
+            t.sig_s_ptr = t.sig_d_ptr = nullptr;
+            t.sig_ns = t.sig_nd = 0;
         }
+        throw;
+    }
+    if (c.sp[1].alias) {
+        SpinTables &a = c.sp[0], &b = c.sp[1];
+        b.sig_s_ptr = a.sig_s_ptr;
+        b.sig_ns = a.sig_ns;
+        b.s_pk_sig = a.s_pk_sig;
+        b.s_v64_sig = a.s_v64_sig;
+        b.s_pkv32 = a.s_pkv32;
+        b.s_vx2 = a.s_vx2;
+        b.sig_d_ptr = a.sig_d_ptr;
+        b.sig_nd = a.sig_nd;
+        b.d_j_sig = a.d_j_sig;
+        b.d_v64_sig = a.d_v64_sig;
+        b.d_jv32 = a.d_jv32;
+        b.d_vx2 = a.d_vx2;
     }
     auto *p = new BlockPlan();
     p->c = &c;

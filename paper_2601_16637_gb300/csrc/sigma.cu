@@ -22,8 +22,8 @@
 // Every output element is owned by one thread group in each pass and each pass adds into it in
 // program order, so results are deterministic.
 //
-// Row-block products (alpha-row sharding) and the two-operand alpha-beta pass stage whole rows of C
-// in shared memory, R rows interleaved per column so one vector load fetches the same column of all
+// Row-block products (alpha-row sharding), the engine's mixed row passes and the two-operand alpha-beta
+// pass stage whole rows of C in shared memory, R rows interleaved per column so one vector load fetches the same column of all
 // R rows; each lane of an 8-lane group fetches 4 entries of the padded sigma copies of the lists with
 // 16-byte loads, and the next column's list bounds are prefetched.  The phase of a single is folded
 // into the shared-memory coefficient tables, which are indexed by 2*code + (phase<0).
