@@ -60,14 +60,15 @@ struct DevStatus {
 // other, and inside a part the lists descend in length and are taken kListGroup at a time.  Such a
 // group is what a warp walks side by side, so its lists are padded to the longest of them and stored
 // interleaved, block by block: a warp's load of one block of all its lists is one contiguous piece.
-// Padding entries have value zero and repeat the list's first target.
+// Padding entries have value zero and the target `pad`, a staged line of zeros: an amplitude that is no
+// number must not reach the sum of a string that it is not connected to (0 x inf is no zero).
 constexpr int kParts = 16;
 constexpr int kRangeDoubles = 4;  // entries of one list in a block of doubles
 constexpr int kRangeSingles = 2;  // and in a block of singles
 constexpr int kListGroup = 8;     // lists of a group
 constexpr int32_t kListHas = 1 << 30;  // the string's list has entries in this range
 struct RangeLists {
-    int w = 0, ng = 0;
+    int w = 0, ng = 0, pad = 0;
     int32_t *zi = nullptr;                     // [ng*groups*8] string | kListHas, or -1 (no string)
     uint32_t *qd = nullptr, *qs = nullptr;     // [ng*groups + 1] first block of a group's doubles, singles
     uint16_t *dt = nullptr;                    // doubles: target inside the range
@@ -129,8 +130,8 @@ struct SpinTables {
     // Singles for the two-operand alpha-beta pass, one lane per string: the strings in descending order
     // of their number of singles (ties ascending), cut into slices of 32; a slice holds as many steps as
     // its longest list, entry t of lane l at sl_ent[(sl_off[slice] + t)*32 + l].  An entry is the target
-    // (bits 0-17) and the coefficient row 2*pair + (phase < 0) at bits 18-29; padding repeats the list's
-    // first target with row 2*npair, which is zero.  Inside a list the entries are ordered so that the 8
+    // (bits 0-17) and the coefficient row 2*pair + (phase < 0) at bits 18-29; padding has the target n,
+    // a column of zeros, and the row 2*npair, which is zero too.  Inside a list the entries are ordered so that the 8
     // lanes of a 128-bit phase read distinct targets and rows modulo 8 where they can.
     int32_t *sl_col = nullptr;   // [slices*32] string, -1: none or no singles
     uint32_t *sl_off = nullptr;  // [slices + 1]

@@ -44,12 +44,14 @@ constexpr int kRangeRowBytes = 128;
 __host__ __device__ inline size_t range_j_bytes(int norb) { return (size_t)(norb * (norb - 1) / 2 + 1) * kRangeRowBytes; }
 __host__ __device__ inline size_t range_smem(int optin) { return ((size_t)optin - 1024) / kRangeRowBytes * kRangeRowBytes; }
 __host__ __device__ inline bool range_j_staged(int optin, int norb) { return 2 * range_j_bytes(norb) <= range_smem(optin); }
-// most strings of one range
+// most strings of one range (behind them: the table, whose last line is zero, or one line of zeros)
 inline int range_width_max(int optin, int norb)
 {
-    const size_t room = range_smem(optin) - (range_j_staged(optin, norb) ? range_j_bytes(norb) : 0);
+    const size_t room = range_smem(optin) - (range_j_staged(optin, norb) ? range_j_bytes(norb) : kRangeRowBytes);
     return (int)(room / kRangeRowBytes);
 }
+// the line of zeros that padding entries point to, for ranges of w strings
+inline int range_pad(int optin, int norb, int w) { return w + (range_j_staged(optin, norb) ? norb * (norb - 1) / 2 : 0); }
 
 // list value type of an arithmetic
 template <typename T>
@@ -329,7 +331,7 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
     constexpr int kWarps = kRangeThreads / 32;
     // the FP64-accurate arithmetics have no registers left for a second block (pairs: 7.3 -> 7.9 ms)
     constexpr int kAhead = sizeof(T) == 4 ? 2 : 1;
-    unsigned char *Js = smem + (size_t)a.w * kRangeRowBytes;  // [npair + 1] lines behind the w staged lines
+    unsigned char *Js = smem + (size_t)a.w * kRangeRowBytes;  // [npair + 1] lines, or a line of zeros, behind the w lines
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lst = lane >> 2, l = lane & 3;  // list of the group, lane of the list
     const int nr = (int)min((int64_t)ROWS, a.nrow - row0);
@@ -346,6 +348,8 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
         for (int p = warp * LPW + sub; p <= a.npair; p += kWarps * LPW)
             Acc::store(Js + (size_t)p * kRangeRowBytes, sr,
                        p < a.npair && srow ? __ldg(a.jg + (int64_t)p * a.nrow + row0 + sr) : 0.0);
+    } else if (threadIdx.x < kRangeRowBytes / 16) {
+        reinterpret_cast<float4 *>(Js)[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     const int64_t groups = part_group(a.n, kParts);
     // Groups are taken from a counter (their lengths differ, and the range ends with a barrier) in the

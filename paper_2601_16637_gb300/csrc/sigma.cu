@@ -760,7 +760,9 @@ __device__ __forceinline__ void ab_row(const AbArgs<T> &a, int64_t ia, unsigned 
 {
     constexpr int kThreads = Threads<T>::value, kWarps = kThreads / 32;
     const int n2 = a.norb * a.norb, nkey = a.norb * (a.norb - 1);
-    const size_t cs_bytes = STAGED ? round16((size_t)a.nB * R * sizeof(T)) : 0;
+    // column nB is zero (padding entries); it takes from the room that choose() leaves behind the nkey + 1
+    // coefficient rows (2 norb^2 - nkey - 1 more rows of R elements, at least 5 where there is a single)
+    const size_t cs_bytes = STAGED ? round16((size_t)(a.nB + 1) * R * sizeof(T)) : 0;
     T *Cs = reinterpret_cast<T *>(smem);
     T *Ws = reinterpret_cast<T *>(smem + cs_bytes);  // [nkey + 1][R]
     __shared__ int next_s;
@@ -783,10 +785,10 @@ __device__ __forceinline__ void ab_row(const AbArgs<T> &a, int64_t ia, unsigned 
         __syncthreads();
         if (tid == 0) next_s = kWarps;
         if (STAGED) {
-            for (int64_t c = tid; c < a.nB; c += kThreads) {
+            for (int64_t c = tid; c <= a.nB; c += kThreads) {
                 T v[R];
 #pragma unroll
-                for (int k = 0; k < R; ++k) v[k] = k < kr ? conv<T>(a.C[ja[k] * a.nB + c]) : T(0);
+                for (int k = 0; k < R; ++k) v[k] = k < kr && c < a.nB ? conv<T>(a.C[ja[k] * a.nB + c]) : T(0);
                 AbVec<T, R>::st(Cs + c * R, v);
             }
         }
@@ -834,7 +836,7 @@ __device__ __forceinline__ void ab_row(const AbArgs<T> &a, int64_t ia, unsigned 
                         if constexpr (STAGED) {
                             c.ld(Cs + (size_t)jb * R);
                         } else {
-                            c.v[0] = conv<T>(a.C[ja[0] * a.nB + jb]);
+                            c.v[0] = jb < a.nB ? conv<T>(a.C[ja[0] * a.nB + jb]) : T(0);
                         }
                         w.ld(Ws + (size_t)(e[i] >> kPackKeyShift) * R);
                         acc.mac(w, c);

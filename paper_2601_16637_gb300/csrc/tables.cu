@@ -747,7 +747,7 @@ __global__ void range_fill_kernel(const int64_t *__restrict__ ptr, const int32_t
         for (int x = lane; x < len; x += 32) {
             const int64_t e = lo + x, at = ((b0 + x / B) * kListGroup + o) * B + x % B;
             const bool real = e < hi;
-            const uint32_t t = hi > lo ? (uint32_t)(tgt[real ? e : lo] - g * r.w) : 0u;
+            const uint32_t t = real ? (uint32_t)(tgt[e] - g * r.w) : (uint32_t)r.pad;
             const double v = real ? val[e] : 0.0;
             if constexpr (KIND == 1) {
                 // padding: value 0 and pair index npair, whose row of the coefficient table is zero
@@ -813,16 +813,16 @@ __global__ void slice_col_kernel(const uint64_t *__restrict__ keys, int64_t n, i
     }
 }
 
-__global__ void slice_fill_kernel(const int64_t *__restrict__ ptr, const uint32_t *__restrict__ pk, int norb, int64_t nsl,
-                                  const int32_t *__restrict__ col, const uint32_t *__restrict__ off, uint32_t *ent)
+__global__ void slice_fill_kernel(const int64_t *__restrict__ ptr, const uint32_t *__restrict__ pk, int64_t n, int norb,
+                                  int64_t nsl, const int32_t *__restrict__ col, const uint32_t *__restrict__ off, uint32_t *ent)
 {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < 32 * nsl; x += (int64_t)gridDim.x * blockDim.x) {
         const int64_t s = x / 32;
         const int lane = (int)(x % 32), steps = (int)(off[s + 1] - off[s]);
         const int64_t b = col[x] >= 0 ? ptr[col[x]] : 0, e = col[x] >= 0 ? ptr[col[x] + 1] : 0;
-        const uint32_t zero = (uint32_t)(norb * (norb - 1)) << kPackKeyShift;
+        const uint32_t zero = (uint32_t)n | ((uint32_t)(norb * (norb - 1)) << kPackKeyShift);
         for (int t = 0; t < steps; ++t) {
-            uint32_t v = (b < e ? pk[b] & kPackJMask : 0u) | zero;
+            uint32_t v = zero;
             if (b + t < e) {
                 const uint32_t w = pk[b + t], key = w >> kPackKeyShift;
                 const int p = (int)(key >> 1) / norb, q = (int)(key >> 1) % norb;
@@ -1332,8 +1332,8 @@ static void build_slices(Ctx &c, SpinTables &t, bool entries)
     SBD_CUDA(cudaStreamSynchronize(c.stream));
     t.sl_ent = dalloc_n<uint32_t>(c, 32 * (size_t)steps);
     if (steps) {
-        slice_fill_kernel<<<blocks_for(32 * nsl, 128, 65535), 128, 0, c.stream>>>(t.s_ptr, t.s_pk, c.norb, nsl, t.sl_col,
-                                                                                t.sl_off, t.sl_ent);
+        slice_fill_kernel<<<blocks_for(32 * nsl, 128, 65535), 128, 0, c.stream>>>(t.s_ptr, t.s_pk, n, c.norb, nsl,
+                                                                                t.sl_col, t.sl_off, t.sl_ent);
         SBD_LAUNCH("slice_fill_kernel");
         slice_order_kernel<<<blocks_for(4 * nsl, 1, 65535), 32, 0, c.stream>>>(t.s_ptr, nsl, t.sl_col, t.sl_off, t.sl_ent);
         SBD_LAUNCH("slice_order_kernel");
@@ -1351,6 +1351,7 @@ void build_range_lists(Ctx &c, int spin, bool beta)
     const int wmax = range_width_max(c.smem_optin, c.norb);
     r.ng = (int)((n + wmax - 1) / wmax);
     r.w = (int)((n + r.ng - 1) / r.ng);
+    r.pad = range_pad(c.smem_optin, c.norb, r.w);
     const int64_t groups = part_group(n, kParts), nq = groups * r.ng;
     uint32_t *cd = dalloc_n<uint32_t>(c, (size_t)(n * r.ng)), *cs = dalloc_n<uint32_t>(c, (size_t)(n * r.ng));
     int64_t *cnt = dalloc_n<int64_t>(c, 2 * (size_t)nq);
