@@ -228,9 +228,11 @@ int sbd_davidson(sbd_handle handle, int nroots, double tol, sbd_precision prec, 
  * Per-kernel device time of the sigma kernels launched on this handle since
  * the last reset (only when sbd_options.timing was set), measured with CUDA
  * events recorded on the stream each kernel was launched on.  Slots:
- *   0 transpose of C, 1 beta gather pass (rows of C), 2 alpha gather pass
- *   (rows of C^T), 3 alpha-beta pass; FP64 kernels in 0..3, mixed in 4..7,
- *   SBD_F32X2 in 8..11.
+ *   0 transpose of C, 1 beta pass (lists of the beta strings, on the transpose of
+ *   C), 2 alpha pass (lists of the alpha strings, on C), 3 alpha-beta pass; FP64
+ *   kernels in 0..3, mixed in 4..7, SBD_F32X2 in 8..11.  Transposing the beta
+ *   pass' result back and adding the diagonal term counts to slot 1 for
+ *   SBD_MIXED and to slot 3 for the others, which add them last.
  * ms_host and launches_host: 12 entries each (either may be NULL).  Waits for
  * the recorded events; reset != 0 clears the counters afterwards.
  */
@@ -272,8 +274,8 @@ int sbd_sort_strings_noalloc(const uint64_t *keys_dev, int64_t n, int norb, int 
 
 /*
  * sbd_sigma_batched -- sigma = H c of n instances in one batched launch
- * sequence: a transpose and the beta, alpha and alpha-beta passes each run as
- * one persistent launch whose CTAs take (instance, row-group) work items from
+ * sequence: a transpose, the beta, alpha and alpha-beta passes and the transpose
+ * of the beta pass' result back each run as one persistent launch whose CTAs take (instance, row-group) work items from
  * a device counter (the batched engine's sigma; paper Sec. II-A/B Eq. 4).
  *   handles      n handles on the same device (distinct)
  *   c_dev[i]     device pointer, handle i's [nA][nB] vector (float for

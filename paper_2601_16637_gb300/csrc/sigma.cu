@@ -17,7 +17,8 @@
 // The second and third line are a gather inside row ia of C ("beta pass"), the next two the same
 // gather inside column ib ("alpha pass", same kernel: range_rows.cuh), and the last line is the
 // alpha-beta pass.  The beta pass runs on the transpose of C and leaves its result transposed; the
-// pass that transposes it back adds the diagonal term.
+// pass that transposes it back adds the diagonal term (in FP64 and pairs last of all: the sums of the other
+// passes are then rounded at their own size, error of an FP64 product 4.7e-16 -> 4.2e-16 at norb 29).
 //
 // Every output element is owned by one thread group in each pass and each pass adds into it in
 // program order, so results are deterministic.
@@ -683,7 +684,7 @@ struct AbSum {  // FP64: one chain per row k
 #pragma unroll
         for (int k = 0; k < R; ++k) s[k] = T(0);
     }
-    __device__ __forceinline__ void mac(const AbVec<T, R> &w, const AbVec<T, R> &c)
+    __device__ __forceinline__ void mac(int, const AbVec<T, R> &w, const AbVec<T, R> &c)
     {
 #pragma unroll
         for (int k = 0; k < R; ++k) s[k] = fma(w.v[k], c.v[k], s[k]);
@@ -701,7 +702,7 @@ template <int R>
 struct AbSum<float, R> {  // FP32: a short chain per block of entries
     float s, blk;
     __device__ __forceinline__ void zero() { s = blk = 0.f; }
-    __device__ __forceinline__ void mac(const AbVec<float, R> &w, const AbVec<float, R> &c)
+    __device__ __forceinline__ void mac(int, const AbVec<float, R> &w, const AbVec<float, R> &c)
     {
 #pragma unroll
         for (int k = 0; k < R; ++k) blk = fmaf(w.v[k], c.v[k], blk);
@@ -713,28 +714,30 @@ struct AbSum<float, R> {  // FP32: a short chain per block of entries
     }
     __device__ __forceinline__ double value() const { return (double)s; }
 };
+// pairs: a block of entries by itself, then added (as in the row passes)
 template <>
 struct AbSum<F2, 1> {
-    F2 s;
+    F2 s, blk;
     __device__ __forceinline__ void zero() { s = F2(0.f); }
-    __device__ __forceinline__ void mac(const AbVec<F2, 1> &w, const AbVec<F2, 1> &c) { f2_mac(s, w.v[0], c.v[0]); }
-    __device__ __forceinline__ void end_block()
+    __device__ __forceinline__ void mac(int i, const AbVec<F2, 1> &w, const AbVec<F2, 1> &c)
     {
-        const float h = __fadd_rn(s.hi, s.lo);
-        s.lo = __fsub_rn(s.lo, __fsub_rn(h, s.hi));
-        s.hi = h;
+        if (i == 0) blk = F2(0.f);
+        f2_mac(blk, w.v[0], c.v[0]);
     }
+    __device__ __forceinline__ void end_block() { s = f2_add(s, blk); }
     __device__ __forceinline__ double value() const { return f2_value(s); }
 };
 template <>
 struct AbSum<F2, 2> {
-    uint64_t hi, lo;
+    uint64_t bh, bl, hi, lo;
     __device__ __forceinline__ void zero() { hi = lo = 0ull; }
-    __device__ __forceinline__ void mac(const AbVec<F2, 2> &w, const AbVec<F2, 2> &c)
+    __device__ __forceinline__ void mac(int i, const AbVec<F2, 2> &w, const AbVec<F2, 2> &c)
     {
-        pk_f2_mac(hi, lo, w.v.x, pk_mul(w.v.x, pk_dup(-1.f)), w.v.y, c.v);
+        const uint64_t an = pk_mul(w.v.x, pk_dup(-1.f));
+        if (i == 0) pk_f2_mul(bh, bl, w.v.x, an, w.v.y, c.v);
+        else pk_f2_mac(bh, bl, w.v.x, an, w.v.y, c.v);
     }
-    __device__ __forceinline__ void end_block() { pk_f2_renorm(hi, lo); }
+    __device__ __forceinline__ void end_block() { pk_f2_add(hi, lo, bh, bl); }
     __device__ __forceinline__ double value() const
     {
         return ((double)pk_get(hi, 0) + (double)pk_get(lo, 0)) + ((double)pk_get(hi, 1) + (double)pk_get(lo, 1));
@@ -839,7 +842,7 @@ __device__ __forceinline__ void ab_row(const AbArgs<T> &a, int64_t ia, unsigned 
                             c.v[0] = jb < a.nB ? conv<T>(a.C[ja[0] * a.nB + jb]) : T(0);
                         }
                         w.ld(Ws + (size_t)(e[i] >> kPackKeyShift) * R);
-                        acc.mac(w, c);
+                        acc.mac(i, w, c);
                     }
                 acc.end_block();
             }
@@ -1258,9 +1261,10 @@ __global__ void transpose_kernel(const T *__restrict__ in, T *__restrict__ out, 
     }
 }
 
-// One 32 x 32 tile of sigma[r][c] = st[c][r] + hd[r][c] x[r][c]: the beta pass' transposed result
-// and the diagonal term (x: the FP64 amplitudes where the caller has them)
-template <typename E>
+// One 32 x 32 tile of sigma[r][c] (+)= st[c][r] + hd[r][c] x[r][c]: the beta pass' transposed result
+// and the diagonal term (x: the FP64 amplitudes where the caller has them).  The FP64-accurate products add it
+// last (ADD): the diagonal term is the largest, and every sum that comes after it is rounded at its size.
+template <typename E, bool ADD>
 __device__ __forceinline__ void untranspose_tile(double (&tile)[32][33], const double *__restrict__ st,
                                                  const double *__restrict__ hd, const E *__restrict__ x,
                                                  const double *__restrict__ x64, double *__restrict__ sigma,
@@ -1275,18 +1279,19 @@ __device__ __forceinline__ void untranspose_tile(double (&tile)[32][33], const d
         const int64_t r = by + j, c = bx + threadIdx.x;
         if (r < rows && c < cols) {
             const int64_t i = r * cols + c;
-            sigma[i] = tile[threadIdx.x][j] + hd[i] * (x64 ? x64[i] : (double)x[i]);
+            const double v = fma(hd[i], x64 ? x64[i] : (double)x[i], tile[threadIdx.x][j]);
+            sigma[i] = ADD ? sigma[i] + v : v;
         }
     }
 }
 
-template <typename E>
+template <typename E, bool ADD>
 __global__ void untranspose_kernel(const double *__restrict__ st, const double *__restrict__ hd,
                                    const E *__restrict__ x, const double *__restrict__ x64, double *__restrict__ sigma,
                                    int64_t rows, int64_t cols)
 {
     __shared__ double tile[32][33];
-    untranspose_tile<E>(tile, st, hd, x, x64, sigma, rows, cols, (int64_t)blockIdx.y * 32, (int64_t)blockIdx.x * 32);
+    untranspose_tile<E, ADD>(tile, st, hd, x, x64, sigma, rows, cols, (int64_t)blockIdx.y * 32, (int64_t)blockIdx.x * 32);
 }
 
 struct PassCfg {
@@ -1584,27 +1589,34 @@ void apply(Ctx &c, const typename In<T>::type *C, double *S, const double *c64, 
     const int base = kSlotBase<T>;
     E *Ct = reinterpret_cast<E *>(S);
     double *St = static_cast<double *>(c.work_t);
-    // the mixed alpha-beta pass takes the row maxima of C from the beta pass
-    const bool src = std::is_same<T, float>::value && src_fits(c);
     timed(c, base + 0, s, [&] { transpose<E>(C, Ct, c.nA, c.nB, s); });
-    RangeArgs<T> rb = range_args<T>(c, 1, Ct, St, 0), ra = range_args<T>(c, 0, C, S, 1);
+    constexpr bool kLast = !std::is_same<T, float>::value;  // beta part and diagonal added last (untranspose_tile)
+    RangeArgs<T> rb = range_args<T>(c, 1, Ct, St, 0), ra = range_args<T>(c, 0, C, S, !kLast);
+    const auto back = [&] {
+        const dim3 grid((unsigned)((c.nB + 31) / 32), (unsigned)((c.nA + 31) / 32));
+        untranspose_kernel<E, kLast><<<grid, dim3(32, 8), 0, s>>>(St, c.hd, C, c64, S, c.nA, c.nB);
+        SBD_LAUNCH("untranspose_kernel");
+    };
+    // the mixed alpha-beta pass takes the row maxima of C from the beta pass
+    const bool src = !kLast && src_fits(c);
     if (src) rb.rowmax = c.rowmax;
     timed(c, base + 1, s, [&] {
         launch_range<T>(c, rb, s);
-        const dim3 grid((unsigned)((c.nB + 31) / 32), (unsigned)((c.nA + 31) / 32));
-        untranspose_kernel<E><<<grid, dim3(32, 8), 0, s>>>(St, c.hd, C, c64, S, c.nA, c.nB);
-        SBD_LAUNCH("untranspose_kernel");
+        if (!kLast) back();
     });
     timed(c, base + 2, s, [&] { launch_range<T>(c, ra, s); });
-    if constexpr (std::is_same<T, float>::value) {
-        if (src) {
-            timed(c, base + 3, s, [&] { launch_ab_src(src_args(c, C, S, c.rowmax), c, s); });
-            return;
+    timed(c, base + 3, s, [&] {
+        if constexpr (!kLast) {
+            if (src) {
+                launch_ab_src(src_args(c, C, S, c.rowmax), c, s);
+                return;
+            }
         }
-    }
-    AbArgs<T> ab;
-    make_ab_args<T>(c, C, S, ab);
-    timed(c, base + 3, s, [&] { launch_ab<T>(ab, choose(c.nB, n2, sizeof(T), kRowsMax<T>, lim), s); });
+        AbArgs<T> ab;
+        make_ab_args<T>(c, C, S, ab);
+        launch_ab<T>(ab, choose(c.nB, n2, sizeof(T), kRowsMax<T>, lim), s);
+        if (kLast) back();
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -1664,7 +1676,7 @@ __device__ __forceinline__ int find_slot(const int64_t *off, int n, int64_t item
 }
 
 // BACK 0: the transposed amplitudes of every slot; 1: sigma = the beta pass' result transposed back
-// plus the diagonal term
+// plus the diagonal term (FP64-accurate products: added to sigma)
 template <typename T, bool BACK>
 __global__ void transpose_batch_kernel(const int *pn, const int64_t *off, const TDesc<T> *td)
 {
@@ -1678,7 +1690,7 @@ __global__ void transpose_batch_kernel(const int *pn, const int64_t *off, const 
         const int64_t by = (lt / tx) * 32, bx = (lt % tx) * 32;
         __syncthreads();
         if constexpr (BACK) {
-            untranspose_tile<T>(tile, d.st, d.hd, d.x, d.x64, d.y, d.rows, d.cols, by, bx);
+            untranspose_tile<T, sizeof(T) == 8>(tile, d.st, d.hd, d.x, d.x64, d.y, d.rows, d.cols, by, bx);
         } else {
             T *out = reinterpret_cast<T *>(d.y);
             for (int j = threadIdx.y; j < 32; j += 8) {
@@ -1842,7 +1854,7 @@ void batch_set(SigmaBatch *b, const SigmaSlot *slots, int n)
             oa[i + 1] = oa[i] + (c.nB + b->R - 1) / b->R;
         } else {
             rb[i] = range_args<T>(c, 1, reinterpret_cast<const E *>(sl.y), st, 0);
-            ra[i] = range_args<T>(c, 0, x, sl.y, 1);
+            ra[i] = range_args<T>(c, 0, x, sl.y, std::is_same<T, float>::value);
             rb[i].q = ra[i].q = q;
             rb[i].rowmax = rowmax;
         }
@@ -1887,8 +1899,10 @@ void batch_launch_r(SigmaBatch *b, cudaStream_t s)
         range_batch_kernel<T><<<b->grid_range, kRangeThreads, b->range_smem, s>>>(
             pn, off_b, reinterpret_cast<const RangeArgs<T> *>(d + L.rb), b->counters);
         SBD_LAUNCH("range_batch_kernel");
-        transpose_batch_kernel<E, true><<<b->grid_t, dim3(32, 8), 0, s>>>(pn, off_t, td);
-        SBD_LAUNCH("transpose_batch_kernel");
+        if (std::is_same<T, float>::value) {  // the other precisions add it last
+            transpose_batch_kernel<E, true><<<b->grid_t, dim3(32, 8), 0, s>>>(pn, off_t, td);
+            SBD_LAUNCH("transpose_batch_kernel");
+        }
         range_batch_kernel<T><<<b->grid_range, kRangeThreads, b->range_smem, s>>>(
             pn, off_a, reinterpret_cast<const RangeArgs<T> *>(d + L.ra), b->counters + 1);
         SBD_LAUNCH("range_batch_kernel");
@@ -1908,6 +1922,10 @@ void batch_launch_r(SigmaBatch *b, cudaStream_t s)
             pn, reinterpret_cast<const int64_t *>(d + L.off_ab), reinterpret_cast<const AbArgs<T> *>(d + L.ab),
             b->counters + 2);
         SBD_LAUNCH("ab_batch_kernel");
+    }
+    if (!std::is_same<T, float>::value) {
+        transpose_batch_kernel<E, true><<<b->grid_t, dim3(32, 8), 0, s>>>(pn, off_t, td);
+        SBD_LAUNCH("transpose_batch_kernel");
     }
 }
 
