@@ -697,6 +697,11 @@ struct AbSum {  // FP64: one chain per row k
         for (int k = 1; k < R; ++k) t += (double)s[k];
         return t;
     }
+    __device__ __forceinline__ void add_lane(int off)
+    {
+#pragma unroll
+        for (int k = 0; k < R; ++k) s[k] += __shfl_xor_sync(0xffffffffu, s[k], off);
+    }
 };
 template <int R>
 struct AbSum<float, R> {  // FP32: a short chain per block of entries
@@ -713,6 +718,7 @@ struct AbSum<float, R> {  // FP32: a short chain per block of entries
         blk = 0.f;
     }
     __device__ __forceinline__ double value() const { return (double)s; }
+    __device__ __forceinline__ void add_lane(int off) { s += __shfl_xor_sync(0xffffffffu, s, off); }
 };
 // pairs: a block of entries by itself, then added (as in the row passes)
 template <>
@@ -726,6 +732,11 @@ struct AbSum<F2, 1> {
     }
     __device__ __forceinline__ void end_block() { s = f2_add(s, blk); }
     __device__ __forceinline__ double value() const { return f2_value(s); }
+    __device__ __forceinline__ void add_lane(int off)
+    {
+        const F2 o(__shfl_xor_sync(0xffffffffu, s.hi, off), __shfl_xor_sync(0xffffffffu, s.lo, off));
+        s = f2_add(s, o);
+    }
 };
 template <>
 struct AbSum<F2, 2> {
@@ -738,9 +749,15 @@ struct AbSum<F2, 2> {
         else pk_f2_mac(bh, bl, w.v.x, an, w.v.y, c.v);
     }
     __device__ __forceinline__ void end_block() { pk_f2_add(hi, lo, bh, bl); }
+    __device__ __forceinline__ void add_lane(int off)
+    {
+        const uint64_t oh = __shfl_xor_sync(0xffffffffu, hi, off), ol = __shfl_xor_sync(0xffffffffu, lo, off);
+        pk_f2_add(hi, lo, oh, ol);
+    }
     __device__ __forceinline__ double value() const
     {
-        return ((double)pk_get(hi, 0) + (double)pk_get(lo, 0)) + ((double)pk_get(hi, 1) + (double)pk_get(lo, 1));
+        // (the halves added as pairs: an FP64 instruction takes 64 clocks, however few of its lanes work)
+        return f2_value(f2_add(F2(pk_get(hi, 0), pk_get(lo, 0)), F2(pk_get(hi, 1), pk_get(lo, 1))));
     }
 };
 
@@ -758,10 +775,18 @@ struct AbSum<F2, 2> {
 // against eight lanes per column (each column's list padded to 32 slots), 3.6e7 determinants, norb 29:
 // FP64 84.1 -> 33.7 ms, pairs 33.1 -> 18.9 ms; with the slices dealt out in a fixed pattern 36.6 and
 // 21.4 ms.
+// Pairs: where the longest slice is 3 (8) times a warp's share of all steps or more, it holds up the
+// barrier, and two (four) lanes walk a list: 2,000 rows x 150 columns at norb 24 839 -> 583 us, x 700
+// columns 1,753 -> 1,472; with equal lists (full space, 495 strings) one lane 397 us, two 451.  FP64 is bound by
+// its pipe even then (one lane 727 us, eight 1,686 at 300 columns).
+// Where a row of C does not fit shared memory its elements come from L2, and the bounds of the next slice are
+// loaded during this one (200 x 60,000 strings, norb 58: FP64 209 -> 111 ms, pairs 96 -> 76; for staged
+// FP64 the registers this takes cost a resident CTA: 61 -> 71 ms at 60,000 x 300, norb 40).
 template <typename T, int R, bool STAGED>
 __device__ __forceinline__ void ab_row(const AbArgs<T> &a, int64_t ia, unsigned char *smem)
 {
     constexpr int kThreads = Threads<T>::value, kWarps = kThreads / 32;
+    constexpr bool kAhead = !STAGED || kIsF2<T>;  // a slice's bounds loaded during the one before
     const int n2 = a.norb * a.norb, nkey = a.norb * (a.norb - 1);
     // column nB is zero (padding entries); it takes from the room that choose() leaves behind the nkey + 1
     // coefficient rows (2 norb^2 - nkey - 1 more rows of R elements, at least 5 where there is a single)
@@ -772,6 +797,7 @@ __device__ __forceinline__ void ab_row(const AbArgs<T> &a, int64_t ia, unsigned 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t e0 = a.as_ptr[ia], nsl = (a.nB + 31) / 32;
     const int K = (int)(a.as_ptr[ia + 1] - e0);
+    const unsigned longest = a.sl_off[1], steps = a.sl_off[nsl];  // of one slice, of all
     for (int k0 = 0; k0 < K; k0 += R) {
         const int kr = min(R, K - k0);
         int64_t ja[R];
@@ -809,45 +835,72 @@ __device__ __forceinline__ void ab_row(const AbArgs<T> &a, int64_t ia, unsigned 
             AbVec<T, R>::st(Ws + (size_t)key * R, v);
         }
         __syncthreads();
-        int64_t sl = warp;
-        while (sl < nsl) {
-            const uint32_t o0 = a.sl_off[sl];
-            const int len = (int)(a.sl_off[sl + 1] - o0);
-            if (len == 0) break;  // the lists descend: nothing follows
-            int nsl_next = 0;
-            if (lane == 0) nsl_next = atomicAdd(&next_s, 1);
-            nsl_next = __shfl_sync(0xffffffffu, nsl_next, 0);
-            const int col = a.sl_col[sl * 32 + lane];
-            const uint32_t *ent = a.sl_ent + (size_t)o0 * 32 + lane;
-            AbSum<T, R> acc;
-            acc.zero();
-            uint32_t nx[4];
+        // STEP lanes walk a column's list side by side, a warp 32 / STEP columns of a slice
+        const auto walk = [&](auto step) {
+            constexpr int STEP = decltype(step)::value;
+            const int64_t units = nsl * STEP;
+            const int sub = lane & (STEP - 1);
+            const auto unit_of = [&](int64_t un, int &len, int &col, const uint32_t *&ent) {
+                const int64_t sl = un / STEP;
+                const int l = (int)(un % STEP) * (32 / STEP) + lane / STEP;
+                const uint32_t o0 = a.sl_off[sl];
+                len = (int)(a.sl_off[sl + 1] - o0);
+                col = a.sl_col[sl * 32 + l];
+                ent = a.sl_ent + (size_t)o0 * 32 + l;
+            };
+            int64_t un = warp;
+            int len = 0, col = -1;
+            const uint32_t *ent = nullptr;
+            if (kAhead && un < units) unit_of(un, len, col, ent);
+            while (un < units) {
+                if (!kAhead) unit_of(un, len, col, ent);
+                if (len == 0) break;  // the lists descend: nothing follows
+                int next = 0;
+                if (lane == 0) next = atomicAdd(&next_s, 1);
+                next = __shfl_sync(0xffffffffu, next, 0);
+                int len_n = 0, col_n = -1;
+                const uint32_t *ent_n = nullptr;
+                if (kAhead && next < units) unit_of(next, len_n, col_n, ent_n);
+                AbSum<T, R> acc;
+                acc.zero();
+                uint32_t nx[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) nx[i] = i < len ? __ldg(ent + 32 * i) : 0u;
-            for (int t = 0; t < len; t += 4) {
-                uint32_t e[4];
+                for (int i = 0; i < 4; ++i) nx[i] = sub + STEP * i < len ? __ldg(ent + 32 * (sub + STEP * i)) : 0u;
+                for (int t = sub; t < len; t += 4 * STEP) {
+                    uint32_t e[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) e[i] = nx[i];
-                ent += 128;
+                    for (int i = 0; i < 4; ++i) e[i] = nx[i];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) nx[i] = t + 4 + i < len ? __ldg(ent + 32 * i) : 0u;
+                    for (int i = 0; i < 4; ++i)
+                        nx[i] = t + STEP * (4 + i) < len ? __ldg(ent + 32 * (t + STEP * (4 + i))) : 0u;
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (t + i < len) {
-                        AbVec<T, R> c, w;
-                        const int jb = pk_j(e[i]);
-                        if constexpr (STAGED) {
-                            c.ld(Cs + (size_t)jb * R);
-                        } else {
-                            c.v[0] = jb < a.nB ? conv<T>(a.C[ja[0] * a.nB + jb]) : T(0);
+                    for (int i = 0; i < 4; ++i)
+                        if (t + STEP * i < len) {
+                            AbVec<T, R> c, w;
+                            const int jb = pk_j(e[i]);
+                            if constexpr (STAGED) c.ld(Cs + (size_t)jb * R);
+                            else c.v[0] = jb < a.nB ? conv<T>(a.C[ja[0] * a.nB + jb]) : T(0);
+                            w.ld(Ws + (size_t)(e[i] >> kPackKeyShift) * R);
+                            acc.mac(i, w, c);
                         }
-                        w.ld(Ws + (size_t)(e[i] >> kPackKeyShift) * R);
-                        acc.mac(i, w, c);
-                    }
-                acc.end_block();
+                    acc.end_block();
+                }
+                if constexpr (STEP > 1) {
+                    __syncwarp();
+#pragma unroll
+                    for (int off = STEP / 2; off > 0; off >>= 1) acc.add_lane(off);
+                }
+                if (sub == 0 && col >= 0) atomicAdd(a.S + ia * a.nB + col, acc.value());
+                un = next;
+                if (kAhead) len = len_n, col = col_n, ent = ent_n;
             }
-            if (col >= 0) atomicAdd(a.S + ia * a.nB + col, acc.value());
-            sl = nsl_next;
+        };
+        if constexpr (STAGED && kIsF2<T>) {
+            if (longest * kWarps >= 8 * steps) walk(std::integral_constant<int, 4>());
+            else if (longest * kWarps >= 3 * steps) walk(std::integral_constant<int, 2>());
+            else walk(std::integral_constant<int, 1>());
+        } else {
+            walk(std::integral_constant<int, 1>());
         }
     }
 }
