@@ -165,21 +165,20 @@ __device__ __forceinline__ void pk_f2_add(uint64_t &hi, uint64_t &lo, uint64_t b
     lo = pk_sub(lo, pk_sub(hi, s));
 }
 
-// The sums of one lane: two chunks (h = 0, 1) of a staged line.  A chunk's 16 bytes are two words:
+// The sums of one lane: NH chunks of a staged line.  A chunk's 16 bytes are two words:
 // two packed pairs of rows (FP32), two FP64 rows, or the high and the low parts of two pair rows.
-template <typename T>
+template <typename T, int NH = 2>
 struct RangeAcc;
 
-template <>
-struct RangeAcc<float> {
+template <int NH>
+struct RangeAcc<float, NH> {
     static constexpr int kRowsPerChunk = 4;
     using Val = float;
-    uint64_t blk[4], acc[4], sum[4];
-    float v[4];
+    uint64_t blk[2 * NH], acc[2 * NH], sum[2 * NH];
     __device__ __forceinline__ void zero()
     {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] = sum[i] = 0ull;
+        for (int i = 0; i < 2 * NH; ++i) acc[i] = sum[i] = 0ull;
     }
     static __device__ __forceinline__ void load(const float *p, float (&v)[4])
     {
@@ -188,11 +187,11 @@ struct RangeAcc<float> {
     }
     // entry u of a block; the block's products are summed by themselves, and the blocks on two
     // levels (eight blocks, then all): short chains keep the rounding error of a long list down
-    __device__ __forceinline__ void mac(int u, float v, const ulonglong2 (&x)[2])
+    __device__ __forceinline__ void mac(int u, float v, const ulonglong2 (&x)[NH])
     {
         const uint64_t vv = pk_dup(v);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < NH; ++h) {
             blk[2 * h] = u == 0 ? pk_mul(vv, x[h].x) : pk_fma(vv, x[h].x, blk[2 * h]);
             blk[2 * h + 1] = u == 0 ? pk_mul(vv, x[h].y) : pk_fma(vv, x[h].y, blk[2 * h + 1]);
         }
@@ -200,19 +199,19 @@ struct RangeAcc<float> {
     __device__ __forceinline__ void end_block(unsigned count)
     {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] = pk_add(acc[i], blk[i]);
+        for (int i = 0; i < 2 * NH; ++i) acc[i] = pk_add(acc[i], blk[i]);
         if ((count & 7u) == 0u) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) sum[i] = pk_add(sum[i], acc[i]), acc[i] = 0ull;
+            for (int i = 0; i < 2 * NH; ++i) sum[i] = pk_add(sum[i], acc[i]), acc[i] = 0ull;
         }
     }
     // (v + sg*j) x, the entries of a block in two chains
-    __device__ __forceinline__ void single(int u, float v, float sg, const ulonglong2 (&j)[2], const ulonglong2 (&x)[2])
+    __device__ __forceinline__ void single(int u, float v, float sg, const ulonglong2 (&j)[NH], const ulonglong2 (&x)[NH])
     {
         const uint64_t vv = pk_dup(v), ss = pk_dup(sg);
-        uint64_t(&s)[4] = u == 0 ? acc : sum;
+        uint64_t(&s)[2 * NH] = u == 0 ? acc : sum;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < NH; ++h) {
             s[2 * h] = pk_fma(pk_fma(ss, j[h].x, vv), x[h].x, s[2 * h]);
             s[2 * h + 1] = pk_fma(pk_fma(ss, j[h].y, vv), x[h].y, s[2 * h + 1]);
         }
@@ -220,7 +219,7 @@ struct RangeAcc<float> {
     __device__ __forceinline__ void end_singles()
     {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) sum[i] = pk_add(sum[i], acc[i]), acc[i] = 0ull;
+        for (int i = 0; i < 2 * NH; ++i) sum[i] = pk_add(sum[i], acc[i]), acc[i] = 0ull;
     }
     __device__ __forceinline__ double value(int h, int i) const
     {
@@ -236,35 +235,35 @@ struct RangeAcc<float> {
     }
 };
 
-template <>
-struct RangeAcc<double> {
+template <int NH>
+struct RangeAcc<double, NH> {
     static constexpr int kRowsPerChunk = 2;
     using Val = double;
-    double acc[4];
+    double acc[2 * NH];
     __device__ __forceinline__ void zero()
     {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] = 0.0;
+        for (int i = 0; i < 2 * NH; ++i) acc[i] = 0.0;
     }
     static __device__ __forceinline__ void load(const double *p, double (&v)[4])
     {
         const double2 a = __ldg(reinterpret_cast<const double2 *>(p)), b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
         v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
     }
-    __device__ __forceinline__ void mac(int, double v, const ulonglong2 (&x)[2])
+    __device__ __forceinline__ void mac(int, double v, const ulonglong2 (&x)[NH])
     {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < NH; ++h) {
             acc[2 * h] = fma(v, __longlong_as_double((long long)x[h].x), acc[2 * h]);
             acc[2 * h + 1] = fma(v, __longlong_as_double((long long)x[h].y), acc[2 * h + 1]);
         }
     }
     __device__ __forceinline__ void end_block(unsigned) {}
-    __device__ __forceinline__ void single(int, double v, float sg, const ulonglong2 (&j)[2], const ulonglong2 (&x)[2])
+    __device__ __forceinline__ void single(int, double v, float sg, const ulonglong2 (&j)[NH], const ulonglong2 (&x)[NH])
     {
         const uint64_t flip = sg < 0.f ? 0x8000000000000000ull : 0ull;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < NH; ++h) {
             acc[2 * h] = fma(v + __longlong_as_double((long long)(j[h].x ^ flip)),
                              __longlong_as_double((long long)x[h].x), acc[2 * h]);
             acc[2 * h + 1] = fma(v + __longlong_as_double((long long)(j[h].y ^ flip)),
@@ -283,12 +282,16 @@ struct RangeAcc<double> {
     }
 };
 
-template <>
-struct RangeAcc<F2> {
+template <int NH>
+struct RangeAcc<F2, NH> {
     static constexpr int kRowsPerChunk = 2;
     using Val = float2;
-    uint64_t bh[2], bl[2], hi[2], lo[2];  // a block's sum, and the sum of the blocks
-    __device__ __forceinline__ void zero() { hi[0] = hi[1] = lo[0] = lo[1] = 0ull; }
+    uint64_t bh[NH], bl[NH], hi[NH], lo[NH];  // a block's sum, and the sum of the blocks
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int h = 0; h < NH; ++h) hi[h] = lo[h] = 0ull;
+    }
     static __device__ __forceinline__ void load(const float2 *p, float2 (&v)[4])
     {
         const float4 a = __ldg(reinterpret_cast<const float4 *>(p)), b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
@@ -300,26 +303,26 @@ struct RangeAcc<F2> {
         if (first) pk_f2_mul(bh[h], bl[h], ah, an, al, b);
         else pk_f2_mac(bh[h], bl[h], ah, an, al, b);
     }
-    __device__ __forceinline__ void mac(int u, float2 v, const ulonglong2 (&x)[2])
+    __device__ __forceinline__ void mac(int u, float2 v, const ulonglong2 (&x)[NH])
     {
         const uint64_t ah = pk_dup(v.x), an = pk_dup(-v.x), al = pk_dup(v.y);
-        mac2(u == 0, 0, ah, an, al, x[0]);
-        mac2(u == 0, 1, ah, an, al, x[1]);
+#pragma unroll
+        for (int h = 0; h < NH; ++h) mac2(u == 0, h, ah, an, al, x[h]);
     }
     // A block is summed by itself and then added: one chain over a list rounds its low part at the size of
     // the whole sum with every entry (error of products of 300 x 300 strings, norb 24: 1.10e-15, 0.93e-15 with
     // eight lanes to a list; this costs no more, the first product of a block needs no sum).
     __device__ __forceinline__ void end_block(unsigned)
     {
-        pk_f2_add(hi[0], lo[0], bh[0], bl[0]);
-        pk_f2_add(hi[1], lo[1], bh[1], bl[1]);
+#pragma unroll
+        for (int h = 0; h < NH; ++h) pk_f2_add(hi[h], lo[h], bh[h], bl[h]);
     }
-    __device__ __forceinline__ void single(int, float2 v, float sg, const ulonglong2 (&j)[2], const ulonglong2 (&x)[2])
+    __device__ __forceinline__ void single(int, float2 v, float sg, const ulonglong2 (&j)[NH], const ulonglong2 (&x)[NH])
     {
         const uint64_t ss = pk_dup(sg), sn = pk_dup(-sg);
         mac(0, v, x);
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int h = 0; h < NH; ++h)
             mac2(false, h, pk_mul(ss, j[h].x), pk_mul(sn, j[h].x), pk_mul(ss, j[h].y), x[h]);
         end_block(0);
     }
@@ -508,6 +511,150 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
                 }
             }
             zi = zi_n, db = db_n, de = de_n, sb = sb_n, se = se_n;
+        }
+    }
+    if constexpr (sizeof(T) == 4) {
+        if (a.rowmax && p0 == 0) {  // uniform over the CTA
+            atomicMax(rmax_s + sr, rmax);
+            __syncthreads();
+            if (threadIdx.x < nr) a.rowmax[row0 + threadIdx.x] = __uint_as_float(rmax_s[threadIdx.x]);
+        }
+    }
+}
+
+// The same sums for lists of one range and few strings: two warps share a group, each with one chunk of a line
+// per lane (half of the rows).  With one or two groups to a CTA a pass takes as long as one warp takes for its
+// lists (FP64 product of 100 x 100 strings, norb 12: 119 -> 99 us).
+// DIRECT: X and Y have the rows outside, [nrow][n], and the diagonal term hd x64 (null: hd X) is added.  The two
+// transposes of a small product cost more as launches (8 us) than the scattered accesses.
+template <typename T, bool DIRECT>
+__device__ __forceinline__ void range_small(const RangeArgs<T> &a, const double *__restrict__ hd,
+                                            const double *__restrict__ x64, int64_t row0, int p0, int p1,
+                                            unsigned char *smem)
+{
+    using Acc = RangeAcc<T, 1>;
+    using In = typename RangeIn<T>::type;
+    constexpr int ROWS = kRangeRows<T>, RPC = Acc::kRowsPerChunk, LPW = 32 / ROWS;
+    constexpr int kWarps = kRangeThreads / 32;
+    unsigned char *Js = smem + (size_t)a.w * kRangeRowBytes;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lst = lane >> 2, l = lane & 3;
+    const int nr = (int)min((int64_t)ROWS, a.nrow - row0);
+    const int sr = lane & (ROWS - 1), sub = lane / ROWS;
+    const bool srow = sr < nr;
+    unsigned rmax = 0u;
+    __shared__ unsigned rmax_s[ROWS];
+    __syncthreads();  // the previous rows are finished with shared memory
+    if (threadIdx.x < ROWS) rmax_s[threadIdx.x] = 0u;
+    if (a.jstaged) {
+        for (int p = warp * LPW + sub; p <= a.npair; p += kWarps * LPW)
+            Acc::store(Js + (size_t)p * kRangeRowBytes, sr,
+                       p < a.npair && srow ? __ldg(a.jg + (int64_t)p * a.nrow + row0 + sr) : 0.0);
+    } else if (threadIdx.x < kRangeRowBytes / 16) {
+        reinterpret_cast<float4 *>(Js)[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    const In *src = a.X + (DIRECT ? (row0 + sr) * a.n : row0 + sr);
+    const int64_t sj = DIRECT ? 1 : a.nrow;  // between the amplitudes of a row
+    for (int jb = warp * LPW + sub; jb < a.n; jb += 8 * kWarps * LPW) {
+        In v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int j = jb + u * kWarps * LPW;
+            v[u] = (j < a.n && srow) ? src[j * sj] : In(0);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int j = jb + u * kWarps * LPW;
+            if (j < a.n) Acc::store(smem + (size_t)j * kRangeRowBytes, sr, (double)v[u]);
+            if constexpr (sizeof(T) == 4) rmax = max(rmax, __float_as_uint(fabsf(v[u])));
+        }
+    }
+    __syncthreads();
+    const int q0 = (int)part_group(a.n, p0), q1 = (int)part_group(a.n, p1);
+    for (int task = warp; task < 2 * (q1 - q0); task += kWarps) {
+        const int q = q0 + (task >> 1);
+        const int c = (l + 4 * (lst & 1)) ^ (4 * (task & 1));
+        const unsigned char *x0 = smem + c * 16;
+        const int zi = a.zi[(int64_t)q * kListGroup + lst];
+        const uint32_t db = a.qd[q], de = a.qd[q + 1], sb = a.qs[q], se = a.qs[q + 1];
+        Acc acc;
+        acc.zero();
+        uint2 m_n = make_uint2(0u, 0u);  // the next block of singles
+        typename Acc::Val v_n[2] = {};
+        const auto load_singles = [&](uint32_t b) {
+            const size_t at = (size_t)b * kListGroup + lst;
+            m_n = __ldg(reinterpret_cast<const uint2 *>(a.sm) + at);
+            v_n[0] = __ldg(a.sv + at * 2), v_n[1] = __ldg(a.sv + at * 2 + 1);
+        };
+        if (sb < se) load_singles(sb);
+        for (uint32_t b = sb; b < se; ++b) {
+            const uint32_t m[2] = {m_n.x, m_n.y};
+            const typename Acc::Val v[2] = {v_n[0], v_n[1]};
+            if (b + 1 < se) load_singles(b + 1);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int pr = (int)((m[u] >> 16) & 0x7fffu);
+                const ulonglong2 x[1] = {*reinterpret_cast<const ulonglong2 *>(x0 + (m[u] & 0xffffu) * kRangeRowBytes)};
+                ulonglong2 j[1];
+                if (a.jstaged) {
+                    j[0] = *reinterpret_cast<const ulonglong2 *>(Js + pr * kRangeRowBytes + c * 16);
+                } else {
+                    double t[RPC];
+#pragma unroll
+                    for (int i = 0; i < RPC; ++i) {
+                        const int r = c + 8 * i;
+                        t[i] = pr < a.npair && r < nr ? __ldg(a.jg + (int64_t)pr * a.nrow + row0 + r) : 0.0;
+                    }
+                    j[0] = Acc::chunk(t);
+                }
+                acc.single(u, v[u], (m[u] >> 31) ? -1.f : 1.f, j, x);
+            }
+        }
+        acc.end_singles();
+        const uint2 *tp = reinterpret_cast<const uint2 *>(a.dt) + (size_t)db * kListGroup + lst;
+        const typename Acc::Val *vp = a.dv + ((size_t)db * kListGroup + lst) * 4;
+        const unsigned nb = de - db;
+        constexpr int kAhead = 2;
+        typename Acc::Val v[kAhead][4];
+        uint2 t4[kAhead];
+#pragma unroll
+        for (int s = 0; s < kAhead; ++s)
+            if (s < nb) {
+                t4[s] = __ldg(tp + s * kListGroup);
+                Acc::load(vp + s * kListGroup * 4, v[s]);
+            }
+        for (unsigned b = 0; b < nb; b += kAhead) {
+#pragma unroll
+            for (int s = 0; s < kAhead; ++s) {
+                if (b + s >= nb) break;
+                const uint2 t = t4[s];
+                const typename Acc::Val val[4] = {v[s][0], v[s][1], v[s][2], v[s][3]};
+                if (b + s + kAhead < nb) {
+                    t4[s] = __ldg(tp + (s + kAhead) * kListGroup);
+                    Acc::load(vp + (s + kAhead) * kListGroup * 4, v[s]);
+                }
+                const uint32_t j[4] = {t.x & 0xffffu, t.x >> 16, t.y & 0xffffu, t.y >> 16};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const ulonglong2 x[1] = {*reinterpret_cast<const ulonglong2 *>(x0 + j[u] * kRangeRowBytes)};
+                    acc.mac(u, val[u], x);
+                }
+                acc.end_block(b + s + 1);
+            }
+            tp += kAhead * kListGroup;
+            vp += kAhead * kListGroup * 4;
+        }
+        if (zi < 0) continue;
+        const bool has = zi & kListHas;
+        const int64_t i = zi & ~kListHas;
+#pragma unroll
+        for (int k = 0; k < RPC; ++k) {
+            const int r = c + 8 * k;
+            if (r >= nr) continue;
+            const int64_t at = DIRECT ? (row0 + r) * a.n + i : i * a.nrow + row0 + r;
+            double y = has ? acc.value(0, k) : 0.0;
+            if (DIRECT) y = fma(hd[at], x64 ? x64[at] : (double)a.X[at], y);
+            if (DIRECT || has || !a.accumulate) a.Y[at] = a.accumulate ? a.Y[at] + y : y;
         }
     }
     if constexpr (sizeof(T) == 4) {

@@ -645,6 +645,20 @@ __global__ void __launch_bounds__(kRangeThreads, 1) range_rows_kernel(const Rang
     }
 }
 
+template <typename T, bool DIRECT>
+__global__ void __launch_bounds__(kRangeThreads, 1) range_small_kernel(const RangeArgs<T> a, const double *hd,
+                                                                      const double *x64, int64_t units)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    int64_t u = units * blockIdx.x / gridDim.x;
+    const int64_t end = units * (blockIdx.x + 1) / gridDim.x;
+    while (u < end) {
+        const int p0 = (int)(u % kParts), p1 = (int)min((int64_t)kParts, p0 + (end - u));
+        range_small<T, DIRECT>(a, hd, x64, u / kParts * kRangeRows<T>, p0, p1, smem);
+        u += p1 - p0;
+    }
+}
+
 template <typename T>
 struct AbArgs {
     const typename In<T>::type *C;  // [nA][nB]
@@ -1435,6 +1449,8 @@ template <typename T>
 void set_attrs(int optin)
 {
     SBD_CUDA(cudaFuncSetAttribute(range_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
+    SBD_CUDA(cudaFuncSetAttribute(range_small_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
+    SBD_CUDA(cudaFuncSetAttribute(range_small_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
     if constexpr (sizeof(T) == 4) {
         SBD_CUDA(cudaFuncSetAttribute(row_pass_kernel<T, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
         SBD_CUDA(cudaFuncSetAttribute(ab_pass_kernel<T, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
@@ -1447,11 +1463,31 @@ void set_attrs(int optin)
     SBD_CUDA(cudaFuncSetAttribute(ab_pass_kernel<T, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
 }
 
+// Lists of few strings: range_small (at most six groups to a part, so that half of a CTA's warps would idle).
+// Products of n x n strings without and with it, pairs, norb 24: n = 300 211 -> 183 us, 800 811 -> 768,
+// 1,200 1,835 -> 1,882.
+constexpr int kSmallStrings = 768;
+bool small_range(int64_t n, int ng) { return ng == 1 && n <= kSmallStrings; }
+
+template <typename T>
+void launch_direct(const Ctx &c, const RangeArgs<T> &a, const double *x64, cudaStream_t s)
+{
+    const int64_t units = (a.nrow + kRangeRows<T> - 1) / kRangeRows<T> * kParts;
+    const int grid = (int)std::min<int64_t>(units, c.num_sms);
+    range_small_kernel<T, true><<<grid, kRangeThreads, range_smem(c.smem_optin), s>>>(a, c.hd, x64, units);
+    SBD_LAUNCH("range_small_kernel");
+}
+
 template <typename T>
 void launch_range(const Ctx &c, const RangeArgs<T> &a, cudaStream_t s)
 {
     const int64_t units = (a.nrow + kRangeRows<T> - 1) / kRangeRows<T> * kParts;
     const int grid = (int)std::min<int64_t>(units, c.num_sms);
+    if (small_range(a.n, a.ng)) {
+        range_small_kernel<T, false><<<grid, kRangeThreads, range_smem(c.smem_optin), s>>>(a, nullptr, nullptr, units);
+        SBD_LAUNCH("range_small_kernel");
+        return;
+    }
     range_rows_kernel<T><<<grid, kRangeThreads, range_smem(c.smem_optin), s>>>(a, units);
     SBD_LAUNCH("range_rows_kernel");
 }
@@ -1630,6 +1666,10 @@ RangeArgs<T> range_args(const Ctx &c, int ls, const typename In<T>::type *X, dou
     return a;
 }
 
+// Whether the beta pass takes the rows of C as they are (range_small, DIRECT).  Mixed products, norb 12: 100 x 100
+// strings 45 -> 36 us without the transposes, 495 x 200 87 -> 78, 495 x 495 the same; pairs 303 -> 298, 503 -> 509.
+bool direct_beta(const Ctx &c) { return small_range(c.nB, c.sp[1].rl.ng) && c.N <= (int64_t)1 << 17; }
+
 // The transposed copy of C is kept in the output buffer until the beta pass has read it, and the
 // beta pass' transposed result in the handle's work vector, so the row passes need no memory of
 // their own.
@@ -1642,21 +1682,29 @@ void apply(Ctx &c, const typename In<T>::type *C, double *S, const double *c64, 
     const int base = kSlotBase<T>;
     E *Ct = reinterpret_cast<E *>(S);
     double *St = static_cast<double *>(c.work_t);
-    timed(c, base + 0, s, [&] { transpose<E>(C, Ct, c.nA, c.nB, s); });
     constexpr bool kLast = !std::is_same<T, float>::value;  // beta part and diagonal added last (untranspose_tile)
-    RangeArgs<T> rb = range_args<T>(c, 1, Ct, St, 0), ra = range_args<T>(c, 0, C, S, !kLast);
+    const bool direct = direct_beta(c);
+    RangeArgs<T> rb = range_args<T>(c, 1, direct ? C : Ct, direct ? S : St, direct && kLast);
+    RangeArgs<T> ra = range_args<T>(c, 0, C, S, !kLast);
+    // the mixed alpha-beta pass takes the row maxima of C from the beta pass
+    const bool src = !kLast && src_fits(c);
+    if (src) rb.rowmax = c.rowmax;
     const auto back = [&] {
+        if (direct) {
+            launch_direct<T>(c, rb, c64, s);
+            return;
+        }
         const dim3 grid((unsigned)((c.nB + 31) / 32), (unsigned)((c.nA + 31) / 32));
         untranspose_kernel<E, kLast><<<grid, dim3(32, 8), 0, s>>>(St, c.hd, C, c64, S, c.nA, c.nB);
         SBD_LAUNCH("untranspose_kernel");
     };
-    // the mixed alpha-beta pass takes the row maxima of C from the beta pass
-    const bool src = !kLast && src_fits(c);
-    if (src) rb.rowmax = c.rowmax;
-    timed(c, base + 1, s, [&] {
-        launch_range<T>(c, rb, s);
-        if (!kLast) back();
-    });
+    if (!direct) timed(c, base + 0, s, [&] { transpose<E>(C, Ct, c.nA, c.nB, s); });
+    if (!direct || !kLast) {
+        timed(c, base + 1, s, [&] {
+            if (!direct) launch_range<T>(c, rb, s);
+            if (!kLast) back();
+        });
+    }
     timed(c, base + 2, s, [&] { launch_range<T>(c, ra, s); });
     timed(c, base + 3, s, [&] {
         if constexpr (!kLast) {
@@ -1668,8 +1716,9 @@ void apply(Ctx &c, const typename In<T>::type *C, double *S, const double *c64, 
         AbArgs<T> ab;
         make_ab_args<T>(c, C, S, ab);
         launch_ab<T>(ab, choose(c.nB, n2, sizeof(T), kRowsMax<T>, lim), s);
-        if (kLast) back();
+        if (kLast && !direct) back();
     });
+    if (kLast && direct) timed(c, base + 1, s, back);
 }
 
 // ---------------------------------------------------------------------------
