@@ -309,12 +309,11 @@ int sbd_create(sbd_handle *out, int norb, int nalpha, int nbeta, const double *h
         SBD_CUDA(cudaMemsetAsync(&c.dstat->nonfinite, 0, 2 * sizeof(int), c.stream));
         c.h64 = dalloc_n<double>(c, n2);
         c.eri64 = dalloc_n<double>(c, n2 * n2);
-        c.eri32 = dalloc_n<float>(c, n2 * n2);
         SBD_CUDA(cudaMemcpyAsync(c.h64, h, n2 * sizeof(double), cudaMemcpyDefault, c.stream));
         SBD_CUDA(cudaMemcpyAsync(c.eri64, eri, n2 * n2 * sizeof(double), cudaMemcpyDefault, c.stream));
         check_finite(c, c.h64, (int64_t)n2);
         check_finite(c, c.eri64, (int64_t)(n2 * n2));
-        to_float(c.eri64, c.eri32, (int64_t)(n2 * n2), c.stream);
+        pack_integrals(c);
         // strings: copy, validate, sort, look for duplicates
         const uint64_t *src[2] = {A, B};
         const int64_t cnt[2] = {nA, nB};

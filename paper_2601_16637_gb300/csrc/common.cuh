@@ -72,14 +72,15 @@ struct RangeLists {
     int32_t *zi = nullptr;                     // [ng*groups*8] string | kListHas, or -1 (no string)
     uint32_t *qd = nullptr, *qs = nullptr;     // [ng*groups + 1] first block of a group's doubles, singles
     uint16_t *dt = nullptr;                    // doubles: target inside the range
-    float *dv32 = nullptr;                     // and matrix element, in the three arithmetics
-    double *dv64 = nullptr;
-    float2 *dvx2 = nullptr;
-    uint32_t *sm = nullptr;  // singles: target inside the range | orbital pair << 16 | phase -1 << 31
-    float *sv32 = nullptr;
+    float *dhi = nullptr, *dlo = nullptr;      // and matrix element: its FP32 rounding, FP32 of the remainder,
+    double *dv64 = nullptr;                    // FP64 (mixed products read the first, pair products two)
+    uint32_t *sm = nullptr;  // singles: target inside the range | used pair << 16 | phase -1 << 31
+    float *shi = nullptr, *slo = nullptr;
     double *sv64 = nullptr;
-    float2 *svx2 = nullptr;
-    double *jg = nullptr;  // [npair][n] J_i[rs] = sum_{k in string i} (rs|kk), pair r(r-1)/2 + s
+    // the orbital pairs {r, s} that occur in the singles, and for the strings i of the other spin
+    // J_i[rs] = sum_{k in i} (rs|kk), [np][other n]
+    int np = 0;
+    double *jg = nullptr;
 };
 // first group of part p (p = kParts: groups of a range) for n strings
 __host__ __device__ __forceinline__ int64_t part_group(int64_t n, int p)
@@ -87,6 +88,13 @@ __host__ __device__ __forceinline__ int64_t part_group(int64_t n, int p)
     const int64_t a = n / kParts, rest = n % kParts;  // parts below `rest` hold a + 1 strings, the others a
     const int64_t big = a / kListGroup + 1, small = (a + kListGroup - 1) / kListGroup;
     return p < rest ? p * big : rest * big + (p - rest) * small;
+}
+
+// index of the unordered orbital pair {p, q}
+__host__ __device__ __forceinline__ int orbital_pair(int p, int q)
+{
+    const int r = p > q ? p : q, s = p > q ? q : p;
+    return r * (r - 1) / 2 + s;
 }
 
 struct SpinTables {
@@ -164,7 +172,7 @@ struct Ctx {
     int norb = 0, na = 0, nb = 0;
     int64_t nA = 0, nB = 0, N = 0;
     double *h64 = nullptr, *eri64 = nullptr;
-    float *eri32 = nullptr;
+    float *eri32 = nullptr;  // (pq|rs) of orbital pairs p > q, r > s, [npair][npair], pair p(p-1)/2 + q
     SpinTables sp[2];
     double *hd = nullptr;   // [N] Hamiltonian diagonal
     void *work_t = nullptr; // [N] doubles: transposed copy of one vector
@@ -264,6 +272,7 @@ void build_sig_lists(Ctx &c, SpinTables &t, bool fp32_only = false);
 // does not read
 void build_engine_lists(Ctx &c, int rows);
 void build_diagonal(Ctx &c);
+void pack_integrals(Ctx &c);  // eri32 from eri64
 void to_float(const double *in, float *out, int64_t n, cudaStream_t s);
 
 // sigma.cu

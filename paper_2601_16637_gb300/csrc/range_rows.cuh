@@ -50,17 +50,17 @@ inline int range_width_max(int optin, int norb)
     const size_t room = range_smem(optin) - (range_j_staged(optin, norb) ? range_j_bytes(norb) : kRangeRowBytes);
     return (int)(room / kRangeRowBytes);
 }
-// the line of zeros that padding entries point to, for ranges of w strings
-inline int range_pad(int optin, int norb, int w) { return w + (range_j_staged(optin, norb) ? norb * (norb - 1) / 2 : 0); }
+// the line of zeros that padding entries point to, for ranges of w strings and np pairs in the table
+inline int range_pad(int optin, int norb, int w, int np) { return w + (range_j_staged(optin, norb) ? np : 0); }
 
-// list value type of an arithmetic
+// list value type of an arithmetic (pairs: the high parts; the low parts are an array of their own)
 template <typename T>
 struct RangeVal {
     using type = T;
 };
 template <>
 struct RangeVal<F2> {
-    using type = float2;
+    using type = float;
 };
 // element type of the vectors (the pair arithmetic reads FP64 vectors)
 template <typename T>
@@ -79,7 +79,7 @@ struct RangeArgs {
     int64_t n, nrow;
     int accumulate;  // add to Y (0: the first range writes)
     float *rowmax;   // FP32 only, optional: [nrow] max_j |X[j][r]|
-    int npair, jstaged, w, ng;
+    int npair, jstaged, w, ng;  // npair: orbital pairs of the lists
     int q;             // batched launches: pieces a row block is cut into (a divisor of kParts)
     const double *jg;  // [npair][nrow]
     const int32_t *zi;
@@ -88,6 +88,7 @@ struct RangeArgs {
     const typename RangeVal<T>::type *dv;
     const uint32_t *sm;
     const typename RangeVal<T>::type *sv;
+    const float *dlo, *slo;  // pairs: low parts
 };
 
 template <typename T>
@@ -180,7 +181,8 @@ struct RangeAcc<float, NH> {
 #pragma unroll
         for (int i = 0; i < 2 * NH; ++i) acc[i] = sum[i] = 0ull;
     }
-    static __device__ __forceinline__ void load(const float *p, float (&v)[4])
+    static __device__ __forceinline__ Val val(const float *p, const float *) { return __ldg(p); }
+    static __device__ __forceinline__ void load(const float *p, const float *, float (&v)[4])
     {
         const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
         v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
@@ -245,7 +247,8 @@ struct RangeAcc<double, NH> {
 #pragma unroll
         for (int i = 0; i < 2 * NH; ++i) acc[i] = 0.0;
     }
-    static __device__ __forceinline__ void load(const double *p, double (&v)[4])
+    static __device__ __forceinline__ Val val(const double *p, const float *) { return __ldg(p); }
+    static __device__ __forceinline__ void load(const double *p, const float *, double (&v)[4])
     {
         const double2 a = __ldg(reinterpret_cast<const double2 *>(p)), b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
         v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
@@ -292,11 +295,12 @@ struct RangeAcc<F2, NH> {
 #pragma unroll
         for (int h = 0; h < NH; ++h) hi[h] = lo[h] = 0ull;
     }
-    static __device__ __forceinline__ void load(const float2 *p, float2 (&v)[4])
+    static __device__ __forceinline__ Val val(const float *hi, const float *lo) { return make_float2(__ldg(hi), __ldg(lo)); }
+    static __device__ __forceinline__ void load(const float *hi, const float *lo, float2 (&v)[4])
     {
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(p)), b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
-        v[0] = make_float2(a.x, a.y), v[1] = make_float2(a.z, a.w);
-        v[2] = make_float2(b.x, b.y), v[3] = make_float2(b.z, b.w);
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(hi)), b = __ldg(reinterpret_cast<const float4 *>(lo));
+        v[0] = make_float2(a.x, b.x), v[1] = make_float2(a.y, b.y);
+        v[2] = make_float2(a.z, b.z), v[3] = make_float2(a.w, b.w);
     }
     __device__ __forceinline__ void mac2(bool first, int h, uint64_t ah, uint64_t an, uint64_t al, ulonglong2 b)
     {
@@ -429,7 +433,7 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
                     const uint32_t m[2] = {m2.x, m2.y};
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
-                        const typename Acc::Val v = __ldg(a.sv + at * 2 + u);
+                        const typename Acc::Val v = Acc::val(a.sv + at * 2 + u, a.slo + at * 2 + u);
                         const uint32_t jo = (m[u] & 0xffffu) * kRangeRowBytes;
                         const int pr = (int)((m[u] >> 16) & 0x7fffu);
                         const ulonglong2 x[2] = {*reinterpret_cast<const ulonglong2 *>(x0 + jo),
@@ -459,13 +463,14 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
                     typename Acc::Val v[kAhead][4];
                     uint2 t4[kAhead];
                     const uint2 *tp = reinterpret_cast<const uint2 *>(a.dt) + (size_t)db * kListGroup + lst;
-                    const typename Acc::Val *vp = a.dv + ((size_t)db * kListGroup + lst) * 4;
+                    const typename RangeVal<T>::type *vp = a.dv + ((size_t)db * kListGroup + lst) * 4;
+                    const float *lp = a.dlo + ((size_t)db * kListGroup + lst) * 4;
                     const unsigned nb = de - db;
 #pragma unroll
                     for (int s = 0; s < kAhead; ++s)
                         if (s < nb) {
                             t4[s] = __ldg(tp + s * kListGroup);
-                            Acc::load(vp + s * kListGroup * 4, v[s]);
+                            Acc::load(vp + s * kListGroup * 4, lp + s * kListGroup * 4, v[s]);
                         }
                     for (unsigned b = 0; b < nb; b += kAhead) {
 #pragma unroll
@@ -475,7 +480,7 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
                             const typename Acc::Val c[4] = {v[s][0], v[s][1], v[s][2], v[s][3]};
                             if (b + s + kAhead < nb) {
                                 t4[s] = __ldg(tp + (s + kAhead) * kListGroup);
-                                Acc::load(vp + (s + kAhead) * kListGroup * 4, v[s]);
+                                Acc::load(vp + (s + kAhead) * kListGroup * 4, lp + (s + kAhead) * kListGroup * 4, v[s]);
                             }
                             const uint32_t j[4] = {t.x & 0xffffu, t.x >> 16, t.y & 0xffffu, t.y >> 16};
 #pragma unroll
@@ -489,6 +494,7 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
                         }
                         tp += kAhead * kListGroup;
                         vp += kAhead * kListGroup * 4;
+                        lp += kAhead * kListGroup * 4;
                     }
                 }
                 if (zi >= 0 && (!add || (zi & kListHas))) {  // the string's sum changes Y
@@ -584,7 +590,7 @@ __device__ __forceinline__ void range_small(const RangeArgs<T> &a, const double 
         const auto load_singles = [&](uint32_t b) {
             const size_t at = (size_t)b * kListGroup + lst;
             m_n = __ldg(reinterpret_cast<const uint2 *>(a.sm) + at);
-            v_n[0] = __ldg(a.sv + at * 2), v_n[1] = __ldg(a.sv + at * 2 + 1);
+            v_n[0] = Acc::val(a.sv + at * 2, a.slo + at * 2), v_n[1] = Acc::val(a.sv + at * 2 + 1, a.slo + at * 2 + 1);
         };
         if (sb < se) load_singles(sb);
         for (uint32_t b = sb; b < se; ++b) {
@@ -612,7 +618,8 @@ __device__ __forceinline__ void range_small(const RangeArgs<T> &a, const double 
         }
         acc.end_singles();
         const uint2 *tp = reinterpret_cast<const uint2 *>(a.dt) + (size_t)db * kListGroup + lst;
-        const typename Acc::Val *vp = a.dv + ((size_t)db * kListGroup + lst) * 4;
+        const typename RangeVal<T>::type *vp = a.dv + ((size_t)db * kListGroup + lst) * 4;
+        const float *lp = a.dlo + ((size_t)db * kListGroup + lst) * 4;
         const unsigned nb = de - db;
         constexpr int kAhead = 2;
         typename Acc::Val v[kAhead][4];
@@ -621,7 +628,7 @@ __device__ __forceinline__ void range_small(const RangeArgs<T> &a, const double 
         for (int s = 0; s < kAhead; ++s)
             if (s < nb) {
                 t4[s] = __ldg(tp + s * kListGroup);
-                Acc::load(vp + s * kListGroup * 4, v[s]);
+                Acc::load(vp + s * kListGroup * 4, lp + s * kListGroup * 4, v[s]);
             }
         for (unsigned b = 0; b < nb; b += kAhead) {
 #pragma unroll
@@ -631,7 +638,7 @@ __device__ __forceinline__ void range_small(const RangeArgs<T> &a, const double 
                 const typename Acc::Val val[4] = {v[s][0], v[s][1], v[s][2], v[s][3]};
                 if (b + s + kAhead < nb) {
                     t4[s] = __ldg(tp + (s + kAhead) * kListGroup);
-                    Acc::load(vp + (s + kAhead) * kListGroup * 4, v[s]);
+                    Acc::load(vp + (s + kAhead) * kListGroup * 4, lp + (s + kAhead) * kListGroup * 4, v[s]);
                 }
                 const uint32_t j[4] = {t.x & 0xffffu, t.x >> 16, t.y & 0xffffu, t.y >> 16};
 #pragma unroll
@@ -643,6 +650,7 @@ __device__ __forceinline__ void range_small(const RangeArgs<T> &a, const double 
             }
             tp += kAhead * kListGroup;
             vp += kAhead * kListGroup * 4;
+            lp += kAhead * kListGroup * 4;
         }
         if (zi < 0) continue;
         const bool has = zi & kListHas;

@@ -665,7 +665,7 @@ struct AbArgs {
     double *S;                       // [nA][nB], accumulated
     int64_t nA, nB;
     int norb;
-    const typename In<T>::type *eri;  // (pq|rs) as a [norb^2][norb^2] matrix
+    const typename In<T>::type *eri;  // (pq|rs): FP32 [npair][npair], else [norb^2][norb^2]
     const int64_t *as_ptr;
     const uint32_t *as_pk;
     const int32_t *sl_col;  // beta singles in slices (SpinTables::sl_*)
@@ -823,6 +823,7 @@ __device__ __forceinline__ void ab_row(const AbArgs<T> &a, int64_t ia, unsigned 
             const uint32_t pk = ok ? a.as_pk[e0 + k0 + k] : 0u;
             ja[k] = pk_j(pk);
             pq[k] = pk_code(pk);
+            if (std::is_same<T, float>::value) pq[k] = ok ? orbital_pair(pq[k] / a.norb, pq[k] % a.norb) : 0;
             u[k] = ok ? (pk_neg(pk) ? -1.0 : 1.0) : 0.0;
         }
         __syncthreads();
@@ -844,8 +845,10 @@ __device__ __forceinline__ void ab_row(const AbArgs<T> &a, int64_t ia, unsigned 
             const double sg = (key & 1) ? -1.0 : 1.0;
             T v[R];
 #pragma unroll
-            for (int k = 0; k < R; ++k)
-                v[k] = key < nkey ? conv<T>((typename In<T>::type)(sg * u[k]) * __ldg(a.eri + (size_t)pq[k] * n2 + rs)) : T(0);
+            for (int k = 0; k < R; ++k) {
+                const size_t at = std::is_same<T, float>::value ? (size_t)pq[k] * (nkey / 2) + pair : (size_t)pq[k] * n2 + rs;
+                v[k] = key < nkey ? conv<T>((typename In<T>::type)(sg * u[k]) * __ldg(a.eri + at)) : T(0);
+            }
             AbVec<T, R>::st(Ws + (size_t)key * R, v);
         }
         __syncthreads();
@@ -973,7 +976,7 @@ struct AbSrcArgs {
     double *S;       // [nA][nB], accumulated
     int64_t nA, nB;
     int norb, npair;
-    const float *eri;         // FP32 (pq|rs) as [norb^2][norb^2]
+    const float *eri;         // FP32 (pq|rs) as [npair][npair]
     const int64_t *as_ptr;    // alpha singles, canonical CSR
     const uint32_t *as_pk;
     const uint32_t *src_item; // beta singles, source-major items (string | entries << 18)
@@ -986,17 +989,14 @@ struct AbSrcArgs {
     const int32_t *row_order; // rows by descending number of alpha singles, -1 where there is none; may be null
 };
 
-// shared memory of one CTA: W [width][8] float4, accumulator [nB] u64, pair -> rs code
+// shared memory of one CTA: W [width][8] float4, accumulator [nB] u64
 __host__ __device__ constexpr size_t src_w_bytes(int width) { return (size_t)width * 128; }
-__host__ __device__ inline size_t src_smem(int npair, int width, int64_t nB)
-{
-    return src_w_bytes(width) + (size_t)nB * 8 + round16((size_t)npair * 2);
-}
+__host__ __device__ inline size_t src_smem(int width, int64_t nB) { return src_w_bytes(width) + (size_t)nB * 8; }
 // the fewest parts whose table fits `limit` bytes, 0 if kSrcParts do not
 inline int src_parts_for(int npair, int64_t nB, size_t limit)
 {
     for (int h = 1; h <= kSrcParts; ++h)
-        if (src_smem(npair, (npair + h - 1) / h, nB) <= limit) return h;
+        if (src_smem((npair + h - 1) / h, nB) <= limit) return h;
     return 0;
 }
 
@@ -1163,11 +1163,10 @@ __device__ __forceinline__ void src_chunk(const AbSrcArgs &a, const float4 *__re
 
 // W[x][position p] for the chunk's alpha singles, position p holding amplitude chunk p mod CPW
 template <int KC>
-__device__ __forceinline__ void src_build_w(const AbSrcArgs &a, float4 *Wt, const int16_t *rs_of, int width,
-                                            const int *pq_s, const float *u_s, int kc)
+__device__ __forceinline__ void src_build_w(const AbSrcArgs &a, float4 *Wt, int p0, int width, const int *pq_s,
+                                            const float *u_s, int kc)
 {
     constexpr int CPW = KC / 4, RS = 8;
-    const int n2 = a.norb * a.norb;
     const int p = threadIdx.x % RS, c = p & (CPW - 1);  // RS divides the block size
     float u[4];
     const float *row[4];
@@ -1175,14 +1174,12 @@ __device__ __forceinline__ void src_build_w(const AbSrcArgs &a, float4 *Wt, cons
     for (int i = 0; i < 4; ++i) {
         const int k = 4 * c + i;
         u[i] = k < kc ? u_s[k] : 0.f;
-        row[i] = a.eri + (size_t)(k < kc ? pq_s[k] : 0) * n2;
+        row[i] = a.eri + (size_t)(k < kc ? pq_s[k] : 0) * a.npair + p0;
     }
 #pragma unroll 4
-    for (int x = threadIdx.x / RS; x < width; x += blockDim.x / RS) {
-        const int rs = rs_of[x];
-        Wt[(size_t)x * RS + p] = make_float4(u[0] * __ldg(row[0] + rs), u[1] * __ldg(row[1] + rs),
-                                             u[2] * __ldg(row[2] + rs), u[3] * __ldg(row[3] + rs));
-    }
+    for (int x = threadIdx.x / RS; x < width; x += blockDim.x / RS)
+        Wt[(size_t)x * RS + p] = make_float4(u[0] * __ldg(row[0] + x), u[1] * __ldg(row[1] + x),
+                                             u[2] * __ldg(row[2] + x), u[3] * __ldg(row[3] + x));
 }
 
 template <bool PACKED>
@@ -1192,7 +1189,6 @@ __device__ __forceinline__ void src_row(const AbSrcArgs &a, int64_t ia, unsigned
     float4 *Wt = reinterpret_cast<float4 *>(smem);
     unsigned *acc_lo = reinterpret_cast<unsigned *>(smem + src_w_bytes(a.width));
     unsigned *acc_hi = acc_lo + a.nB;
-    const int16_t *rs_of = reinterpret_cast<const int16_t *>(smem + src_w_bytes(a.width) + (size_t)a.nB * 8);
     __shared__ __align__(16) int ja_s[32];
     __shared__ int pq_s[32];
     __shared__ float u_s[32];
@@ -1206,11 +1202,6 @@ __device__ __forceinline__ void src_row(const AbSrcArgs &a, int64_t ia, unsigned
     const int K = (int)(a.as_ptr[ia + 1] - e0);
     __syncthreads();  // the previous row is finished with shared memory
     for (int64_t ib = tid; ib < a.nB; ib += blockDim.x) acc_lo[ib] = acc_hi[ib] = 0u;
-    {
-        int16_t *rs_w = reinterpret_cast<int16_t *>(smem + src_w_bytes(a.width) + (size_t)a.nB * 8);
-        for (int r = 1; r < a.norb; ++r)
-            for (int s = tid; s < r; s += blockDim.x) rs_w[r * (r - 1) / 2 + s] = (int16_t)(r * a.norb + s);
-    }
     if (tid < 32) {
         float m = 0.f;
         for (int k = tid; k < K; k += 32) m += __ldg(a.rowmax + (a.as_pk[e0 + k] & kPackJMask));
@@ -1250,7 +1241,8 @@ __device__ __forceinline__ void src_row(const AbSrcArgs &a, int64_t ia, unsigned
         if (tid < kc) {
             const uint32_t pk = a.as_pk[e0 + k0 + tid];
             ja_s[tid] = (int)(pk & kPackJMask);
-            pq_s[tid] = (int)(pk >> (kPackKeyShift + 1));
+            const int code = (int)(pk >> (kPackKeyShift + 1));
+            pq_s[tid] = orbital_pair(code / a.norb, code % a.norb);
             u_s[tid] = ((pk >> kPackKeyShift) & 1u) ? -1.f : 1.f;
         }
         for (int h = 0; h < a.parts; ++h) {
@@ -1258,9 +1250,9 @@ __device__ __forceinline__ void src_row(const AbSrcArgs &a, int64_t ia, unsigned
             if (h) __syncthreads();  // the previous part is finished with W
             if (tid == 0) ctr = a.slice[h];
             __syncthreads();
-            if (kc <= 8) src_build_w<8>(a, Wt, rs_of + p0, width, pq_s, u_s, kc);
-            else if (kc <= 16) src_build_w<16>(a, Wt, rs_of + p0, width, pq_s, u_s, kc);
-            else src_build_w<32>(a, Wt, rs_of + p0, width, pq_s, u_s, kc);
+            if (kc <= 8) src_build_w<8>(a, Wt, p0, width, pq_s, u_s, kc);
+            else if (kc <= 16) src_build_w<16>(a, Wt, p0, width, pq_s, u_s, kc);
+            else src_build_w<32>(a, Wt, p0, width, pq_s, u_s, kc);
             __syncthreads();
             const int sl1 = a.slice[h + 1];
             if (kc <= 8) src_chunk<8, PACKED>(a, Wt, acc_lo, acc_hi, ja_s, kc, scale_hi, two_l, lbits, sl1, &ctr);
@@ -1387,12 +1379,12 @@ PassCfg choose(int64_t ncol, int n2, size_t elem, int rmax, size_t limit)
 
 size_t smem_limit(const Ctx &c) { return (size_t)c.smem_optin - 1024; }
 
-// max |x| over n floats, as the bit pattern of a non-negative float (out zeroed beforehand)
-__global__ void absmax_kernel(const float *__restrict__ x, int64_t n, unsigned *out)
+// max |FP32 of x| over n values, as the bit pattern of a non-negative float (out zeroed beforehand)
+__global__ void absmax_kernel(const double *__restrict__ x, int64_t n, unsigned *out)
 {
     unsigned m = 0u;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, __float_as_uint(fabsf(x[i])));
+        m = max(m, __float_as_uint(fabsf((float)x[i])));
     m = __reduce_max_sync(0xffffffffu, m);
     if ((threadIdx.x & 31) == 0) atomicMax(out, m);
 }
@@ -1438,7 +1430,7 @@ int src_ctas(size_t smem, int sm_bytes, int64_t rows, int num_sms)
 
 void launch_ab_src(const AbSrcArgs &a, const Ctx &c, cudaStream_t s)
 {
-    const size_t smem = src_smem(a.npair, a.width, a.nB);
+    const size_t smem = src_smem(a.width, a.nB);
     const int f = src_ctas(smem, c.smem_optin, a.nA, c.num_sms);
     const int grid = (int)std::min<int64_t>(a.nA, (int64_t)c.num_sms * f);
     ab_src_kernel<<<grid, kSrcThreads / f, smem, s>>>(a);
@@ -1630,11 +1622,10 @@ void make_row_args(const Ctx &c, const float *C, double *S, const double *c64, c
 }
 
 template <typename T>
-const typename RangeVal<T>::type *range_vals(const float *v32, const double *v64, const float2 *vx2)
+const typename RangeVal<T>::type *range_vals(const float *hi, const double *v64)
 {
-    if constexpr (kIsF2<T>) return vx2;
-    else if constexpr (sizeof(T) == 4) return v32;
-    else return v64;
+    if constexpr (std::is_same<T, double>::value) return v64;
+    else return hi;
 }
 
 // Row pass over the lists of spin `ls` of a handle: X and Y have that spin's strings as rows of
@@ -1650,19 +1641,21 @@ RangeArgs<T> range_args(const Ctx &c, int ls, const typename In<T>::type *X, dou
     a.n = t.n;
     a.nrow = o.n;
     a.accumulate = accumulate;
-    a.npair = npairs(c.norb);
+    a.npair = r.np;
     a.jstaged = range_j_staged(c.smem_optin, c.norb);
     a.w = r.w;
     a.ng = r.ng;
     a.q = 1;
-    a.jg = o.rl.jg;
+    a.jg = r.jg;
     a.zi = r.zi;
     a.qd = r.qd;
     a.qs = r.qs;
     a.dt = r.dt;
     a.sm = r.sm;
-    a.dv = range_vals<T>(r.dv32, r.dv64, r.dvx2);
-    a.sv = range_vals<T>(r.sv32, r.sv64, r.svx2);
+    a.dv = range_vals<T>(r.dhi, r.dv64);
+    a.sv = range_vals<T>(r.shi, r.sv64);
+    a.dlo = r.dlo;
+    a.slo = r.slo;
     return a;
 }
 
@@ -2095,7 +2088,7 @@ void sigma_prepare(Ctx &c)
     const int64_t n4 = (int64_t)c.norb * c.norb * c.norb * c.norb;
     unsigned *m = reinterpret_cast<unsigned *>(c.dstat);  // status words are free after create
     SBD_CUDA(cudaMemsetAsync(m, 0, sizeof(unsigned), c.stream));
-    absmax_kernel<<<(int)std::min<int64_t>((n4 + 255) / 256, 1024), 256, 0, c.stream>>>(c.eri32, n4, m);
+    absmax_kernel<<<(int)std::min<int64_t>((n4 + 255) / 256, 1024), 256, 0, c.stream>>>(c.eri64, n4, m);
     SBD_LAUNCH("absmax_kernel");
     unsigned bits = 0;
     SBD_CUDA(cudaMemcpyAsync(&bits, m, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream));
@@ -2152,7 +2145,7 @@ SigmaBatch *sigma_batch_create(int max_slots, sbd_precision prec, int R, int max
     const size_t lim = sigma_batch_smem_limit(device);
     const int mp = npairs(max_norb), h = max_norb >= 2 ? src_parts_for(mp, max_strings, lim) : 0;
     // one part for the largest instance is one part for all; else a smaller one may take up to the limit
-    b->src_smem = h == 1 ? src_smem(mp, mp, max_strings) : lim;
+    b->src_smem = h == 1 ? src_smem(mp, max_strings) : lim;
     b->src = prec == SBD_MIXED && h > 0;
     if (R == kHalfRows && !b->src) {
         delete b;

@@ -571,9 +571,8 @@ __global__ void padded_count_kernel(const int64_t *__restrict__ ptr, int64_t n, 
 // index of the unordered pair of the orbital code of a packed single
 __device__ __forceinline__ int single_pair(uint32_t pk, int norb)
 {
-    const int code = (int)(pk >> (kPackKeyShift + 1)), p = code / norb, q = code - p * norb;
-    const int r = max(p, q), s = min(p, q);
-    return r * (r - 1) / 2 + s;
+    const int code = (int)(pk >> (kPackKeyShift + 1)), p = code / norb;
+    return orbital_pair(p, code - p * norb);
 }
 
 __global__ void src_count_kernel(const int64_t *__restrict__ ptr, const uint32_t *__restrict__ pk, int64_t n, int norb,
@@ -776,7 +775,7 @@ __device__ __forceinline__ float2 split2(double x)
 template <int KIND>
 __global__ void range_fill_kernel(const int64_t *__restrict__ ptr, const int32_t *__restrict__ tgt,
                                   const uint32_t *__restrict__ pk, const double *__restrict__ val, int64_t groups,
-                                  int norb, RangeLists r)
+                                  int norb, const int *__restrict__ used, RangeLists r)
 {
     constexpr int B = KIND == 1 ? kRangeSingles : kRangeDoubles;
     const uint32_t *qp = KIND == 1 ? r.qs : r.qd;
@@ -800,47 +799,79 @@ __global__ void range_fill_kernel(const int64_t *__restrict__ ptr, const int32_t
             const uint32_t t = real ? (uint32_t)(tgt[e] - g * r.w) : (uint32_t)r.pad;
             const double v = real ? val[e] : 0.0;
             if constexpr (KIND == 1) {
-                // padding: value 0 and pair index npair, whose row of the coefficient table is zero
-                uint32_t m = t | ((uint32_t)(norb * (norb - 1) / 2) << 16);
-                if (real) {
-                    const uint32_t key = pk[e] >> kPackKeyShift;
-                    const int p = (int)(key >> 1) / norb, s = (int)(key >> 1) % norb;
-                    const int mx = max(p, s), mn = min(p, s);
-                    m = t | ((uint32_t)(mx * (mx - 1) / 2 + mn) << 16) | ((key & 1u) << 31);
-                }
-                r.sm[at] = m;
-                r.sv32[at] = __double2float_rn(v);
+                // padding: value 0 and pair index np, whose row of the coefficient table is zero
+                const uint32_t pair = real ? (uint32_t)used[single_pair(pk[e], norb)] : (uint32_t)r.np;
+                const uint32_t neg = real ? (pk[e] >> kPackKeyShift) & 1u : 0u;
+                r.sm[at] = t | (pair << 16) | (neg << 31);
+                const float2 x = split2(v);
+                r.shi[at] = x.x;
+                r.slo[at] = x.y;
                 r.sv64[at] = v;
-                r.svx2[at] = split2(v);
             } else {
+                const float2 x = split2(v);
                 r.dt[at] = (uint16_t)t;
-                r.dv32[at] = __double2float_rn(v);
+                r.dhi[at] = x.x;
+                r.dlo[at] = x.y;
                 r.dv64[at] = v;
-                r.dvx2[at] = split2(v);
             }
         }
     }
 }
 
-// jg[pair][i] = sum_{k in string i} (rs|kk)
-__global__ void pair_j_kernel(const uint64_t *__restrict__ S, int64_t n, int norb, const double *__restrict__ eri,
-                              double *jg)
+// flag[pair] = 1 for the pairs of the singles
+__global__ void pair_mark_kernel(const uint32_t *__restrict__ pk, int64_t ns, int norb, int *flag)
 {
-    const int npair = norb * (norb - 1) / 2;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ns; e += (int64_t)gridDim.x * blockDim.x) {
+        int *f = flag + single_pair(pk[e], norb);
+        if (*f == 0) *f = 1;
+    }
+}
+
+// used[pair] = index of a marked pair among them (in: its mark), list[index] = pair, *np = their number; one
+// CTA of 1024 threads, two pairs (of at most 2016) each
+__global__ void __launch_bounds__(1024) pair_list_kernel(int *used, int npair, int *list, int *np)
+{
+    const int x = 2 * threadIdx.x;
+    const int f0 = x < npair ? used[x] : 0, f1 = x + 1 < npair ? used[x + 1] : 0;
+    int64_t total;
+    const int at = (int)scan_block(f0 + f1, total);
+    if (f0) used[x] = at, list[at] = x;
+    if (f1) used[x + 1] = at + f0, list[at + f0] = x + 1;
+    if (threadIdx.x == 0) *np = (int)total;
+}
+
+// jg[x][i] = sum_{k in string i} (rs|kk), rs = pair list[x]
+__global__ void pair_j_kernel(const uint64_t *__restrict__ S, int64_t n, int norb, const double *__restrict__ eri,
+                              const int *__restrict__ list, int np, double *jg)
+{
     const int64_t n2 = (int64_t)norb * norb;
-    int r = 1, s = 0;
-    for (int x = 0; x < (int)blockIdx.y; ++x)
-        if (++s == r) ++r, s = 0;
-    for (int x = blockIdx.y; x < npair; x += gridDim.y) {
-        const double *row = eri + ((int64_t)r * norb + s) * n2;
+    for (int x = blockIdx.y; x < np; x += gridDim.y) {
+        const int pair = list[x];
+        int r = (int)((1.f + sqrtf(8.f * (float)pair + 1.f)) * 0.5f);
+        if (r * (r - 1) / 2 > pair) --r;
+        if (r * (r + 1) / 2 <= pair) ++r;
+        const double *row = eri + ((int64_t)r * norb + (pair - r * (r - 1) / 2)) * n2;
         for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
             double v = 0.0;
             for (uint64_t m = S[i]; m; m &= m - 1ull) v += __ldg(row + (int64_t)(__ffsll((long long)m) - 1) * (norb + 1));
             jg[(int64_t)x * n + i] = v;
         }
-        for (int k = 0; k < (int)gridDim.y; ++k)
-            if (++s == r) ++r, s = 0;
     }
+}
+
+// out[pq][rs] = FP32 of (pq|rs), p > q, r > s
+__global__ void pack_integrals_kernel(const double *__restrict__ eri, int norb, float *out)
+{
+    const int npair = norb * (norb - 1) / 2;
+    for (int r = 1; r < norb; ++r)
+        for (int x = blockIdx.x; x < npair; x += gridDim.x) {
+            int p = (int)((1.f + sqrtf(8.f * (float)x + 1.f)) * 0.5f);
+            if (p * (p - 1) / 2 > x) --p;
+            if (p * (p + 1) / 2 <= x) ++p;
+            const int q = x - p * (p - 1) / 2;
+            for (int s = threadIdx.x; s < r; s += blockDim.x)
+                out[(size_t)x * npair + r * (r - 1) / 2 + s] = (float)eri_at(eri, norb, p, q, r, s);
+        }
 }
 
 // ---- slices of the two-operand alpha-beta pass -----------------------------------
@@ -1311,9 +1342,9 @@ void build_engine_lists(Ctx &c, int rows)
             std::copy(slice, slice + kSrcParts + 1, t.src_slice);
             continue;
         }
-        // the FP32 and FP64 elements of the range lists: the engine's products are these lists' and pairs
-        for (void *q : {(void *)t.rl.dv32, (void *)t.rl.dv64, (void *)t.rl.sv32, (void *)t.rl.sv64}) dfree(c, q);
-        t.rl.dv32 = t.rl.sv32 = nullptr;
+        // the FP64 elements of the range lists: the engine's products are mixed and pairs
+        dfree(c, t.rl.dv64);
+        dfree(c, t.rl.sv64);
         t.rl.dv64 = t.rl.sv64 = nullptr;
         if (rows == 0 || rows == 8) build_half_lists(c, t);
         if (rows != 8) build_sig_lists(c, t, true);
@@ -1416,7 +1447,6 @@ void build_range_lists(Ctx &c, int spin, bool beta)
     const int wmax = range_width_max(c.smem_optin, c.norb);
     r.ng = (int)((n + wmax - 1) / wmax);
     r.w = (int)((n + r.ng - 1) / r.ng);
-    r.pad = range_pad(c.smem_optin, c.norb, r.w);
     const int64_t groups = part_group(n, kParts), nq = groups * r.ng;
     uint32_t *cd = dalloc_n<uint32_t>(c, (size_t)(n * r.ng)), *cs = dalloc_n<uint32_t>(c, (size_t)(n * r.ng));
     int64_t *cnt = dalloc_n<int64_t>(c, 2 * (size_t)nq);
@@ -1439,38 +1469,59 @@ void build_range_lists(Ctx &c, int spin, bool beta)
         SBD_LAUNCH("narrow_kernel");
         SBD_CUDA(cudaMemcpyAsync(&total[kind], sum + nq, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
     }
+    // the orbital pairs that the singles need J of (few of them in a sparse set of many orbitals)
+    const int npair = c.norb * (c.norb - 1) / 2;
+    int *used = dalloc_n<int>(c, (size_t)npair), *list = dalloc_n<int>(c, (size_t)npair + 1);
+    SBD_CUDA(cudaMemsetAsync(used, 0, sizeof(int) * (size_t)npair, c.stream));
+    pair_mark_kernel<<<blocks_for(t.ns, 256, 2048), 256, 0, c.stream>>>(t.s_pk, t.ns, c.norb, used);
+    SBD_LAUNCH("pair_mark_kernel");
+    pair_list_kernel<<<1, 1024, 0, c.stream>>>(used, npair, list, list + npair);
+    SBD_LAUNCH("pair_list_kernel");
+    SBD_CUDA(cudaMemcpyAsync(&r.np, list + npair, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
     SBD_CUDA(cudaStreamSynchronize(c.stream));
+    r.pad = range_pad(c.smem_optin, c.norb, r.w, r.np);
     const size_t ms = (size_t)total[0] * kListGroup * kRangeSingles, md = (size_t)total[1] * kListGroup * kRangeDoubles;
     if (total[0] > 0xffffffffLL || total[1] > 0xffffffffLL) fail(SBD_ERR_UNSUPPORTED, "excitation lists too large");
     r.sm = dalloc_n<uint32_t>(c, ms);
-    r.sv32 = dalloc_n<float>(c, ms);
+    r.shi = dalloc_n<float>(c, ms);
+    r.slo = dalloc_n<float>(c, ms);
     r.sv64 = dalloc_n<double>(c, ms);
-    r.svx2 = dalloc_n<float2>(c, ms);
     r.dt = dalloc_n<uint16_t>(c, md);
-    r.dv32 = dalloc_n<float>(c, md);
+    r.dhi = dalloc_n<float>(c, md);
+    r.dlo = dalloc_n<float>(c, md);
     r.dv64 = dalloc_n<double>(c, md);
-    r.dvx2 = dalloc_n<float2>(c, md);
     const int fb = blocks_for(nq * kListGroup * 32, 256, 16384);
     if (ms) {
-        range_fill_kernel<1><<<fb, 256, 0, c.stream>>>(t.s_ptr, t.s_j, t.s_pk, t.s_v64, groups, c.norb, r);
+        range_fill_kernel<1><<<fb, 256, 0, c.stream>>>(t.s_ptr, t.s_j, t.s_pk, t.s_v64, groups, c.norb, used, r);
         SBD_LAUNCH("range_fill_kernel(singles)");
     }
     if (md) {
-        range_fill_kernel<2><<<fb, 256, 0, c.stream>>>(t.d_ptr, t.d_j, nullptr, t.d_v64, groups, c.norb, r);
+        range_fill_kernel<2><<<fb, 256, 0, c.stream>>>(t.d_ptr, t.d_j, nullptr, t.d_v64, groups, c.norb, nullptr, r);
         SBD_LAUNCH("range_fill_kernel(doubles)");
     }
     build_slices(c, t, beta);
-    const int npair = c.norb * (c.norb - 1) / 2;
-    r.jg = dalloc_n<double>(c, (size_t)npair * n);
-    if (npair) {
-        const dim3 jb((unsigned)blocks_for(n, 256, 1024), (unsigned)std::min(npair, 256));
-        pair_j_kernel<<<jb, 256, 0, c.stream>>>(t.strings, n, c.norb, c.eri64, r.jg);
+    const SpinTables &o = c.sp[1 - spin];
+    r.jg = dalloc_n<double>(c, (size_t)r.np * o.n);
+    if (r.np) {
+        const dim3 jb((unsigned)blocks_for(o.n, 256, 1024), (unsigned)std::min(r.np, 256));
+        pair_j_kernel<<<jb, 256, 0, c.stream>>>(o.strings, o.n, c.norb, c.eri64, list, r.np, r.jg);
         SBD_LAUNCH("pair_j_kernel");
     }
+    dfree(c, used);
+    dfree(c, list);
     dfree(c, cd);
     dfree(c, cs);
     dfree(c, cnt);
     dfree(c, sum);
+}
+
+void pack_integrals(Ctx &c)
+{
+    const int npair = c.norb * (c.norb - 1) / 2;
+    c.eri32 = dalloc_n<float>(c, (size_t)npair * npair);
+    if (!npair) return;
+    pack_integrals_kernel<<<npair, 64, 0, c.stream>>>(c.eri64, c.norb, c.eri32);
+    SBD_LAUNCH("pack_integrals_kernel");
 }
 
 void build_diagonal(Ctx &c)

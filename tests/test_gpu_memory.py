@@ -1,0 +1,49 @@
+"""Device memory that handles, block plans and engine jobs hold: instances that fit a byte budget keep fitting it."""
+import numpy as np
+import pytest
+
+from paper_2601_16637_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2601_16637_gb300 import binding
+
+    binding.load()
+    return binding
+
+
+def test_sparse_set_of_many_orbitals_holds_no_dense_tables(B):
+    # no two of these strings are a single excitation apart: besides the integrals (8 bytes each, and 4 for
+    # each two pairs of orbitals) and two vectors, only lists proportional to the strings
+    rng = np.random.default_rng(1)
+    norb, n, m = 64, 20000, 64
+    h, eri, _ = _integrals(norb)
+
+    def strings(k):
+        occ = np.argsort(rng.random((k, norb)), axis=1)[:, :32].astype(np.uint64)
+        return np.unique((np.uint64(1) << occ).sum(1, dtype=np.uint64))
+
+    A, Bs = strings(n), strings(m)
+    with B.SBD(norb, 32, 32, h, eri, A, Bs) as g:
+        assert all(B.sbd_table_size(g.handle, s, 1) == 0 for s in (0, 1))
+        npair = norb * (norb - 1) // 2
+        assert g.memory() <= 8 * norb**4 + 4 * npair**2 + 16 * A.size * Bs.size + 400 * (A.size + Bs.size)
+
+
+def _integrals(norb):
+    rng = np.random.default_rng(3)
+    b = rng.standard_normal((4, norb, norb)) * 0.1
+    b = b + b.transpose(0, 2, 1)
+    h = b[0] + np.diag(-2.0 + 0.1 * np.arange(norb))
+    return h, np.einsum("kpq,krs->pqrs", b, b), rng
+
+
+def test_handle_fits_the_budget_it_used_to(B):
+    # 2,000 x 2,000 strings at norb 58: 2.68e8 bytes with lists padded per string, a third copy of
+    # their values and FP32 integrals of all index quadruples
+    wl = W.make("budget", 58, 19, 19, 2000, 2000, 0.35, 5)
+    with B.SBD.from_workload(wl, hbm_budget_bytes=270_000_000) as g:
+        assert g.memory() <= 270_000_000
