@@ -303,8 +303,8 @@ int sbd_sigma_batched(int n, const sbd_handle *handles, const void *const *c_dev
  * rounding order of the partial sums).  c_block: device pointer, (j1-j0)*nB elements (float for
  * SBD_MIXED, double otherwise); sigma_rows: device pointer, (r1-r0)*nB doubles, accumulated (zero
  * it before the first block).  A plan holds device memory through the handle's allocator and
- * budget and must be destroyed before the handle (the handle's first plan also makes copies of its
- * lists, which the handle keeps); calls on one plan must not overlap.  Errors of
+ * budget and must be destroyed before the handle (the first plan whose output rows lie partly in its
+ * block also makes copies of the beta lists, which the handle keeps); calls on one plan must not overlap.  Errors of
  * sbd_block_plan_create are reported on the handle, those of the other two on the calling thread
  * (sbd_last_error(NULL)).
  */

@@ -233,7 +233,7 @@ int sbd_block_plan_create(sbd_handle h, int64_t r0, int64_t r1, int64_t j0, int6
     if (!h || !out) return SBD_ERR_INVALID_ARG;
     *out = nullptr;
     return guarded(h, [&]() -> int {
-        BlockPlan *p = block_plan_create(h->c, r0, r1, j0, j1);
+        BlockPlan *p = block_plan_create(h->c, r0, r1, j0, j1, kValHi | kValLo | kValF64);
         auto *bp = new (std::nothrow) sbd_block_plan_s{h, p};
         if (!bp) {
             block_plan_destroy(p);
@@ -540,9 +540,13 @@ int sbd_davidson_sharded(sbd_handle h, const int64_t *bounds, const sbd_comm *co
                     q = nullptr;
                 }
         };
+        // the products of the solve: its precision, and for mixed solves that of the defect correction
+        const int mask = value_mask(prec) |
+                         (prec == SBD_MIXED ? value_mask(c.opt.refine_precision == SBD_F32X2 ? SBD_F32X2 : SBD_FP64) : 0);
         try {
             for (int b = 0; b < sh.world; ++b)
-                sh.plans.push_back(block_plan_create(c, sh.row0(), sh.row0() + sh.rows(), sh.bounds[b], sh.bounds[b + 1]));
+                sh.plans.push_back(
+                    block_plan_create(c, sh.row0(), sh.row0() + sh.rows(), sh.bounds[b], sh.bounds[b + 1], mask));
             if (sh.world > 1)
                 for (void *&q : sh.ring) q = dalloc(c, sizeof(double) * (size_t)maxrows * (size_t)c.nB);
             const int rc = davidson(c, nroots, tol, prec, energies_host, vecs_rows, residuals_host, report, &sh);

@@ -90,6 +90,21 @@ __host__ __device__ __forceinline__ int64_t part_group(int64_t n, int p)
     return p < rest ? p * big : rest * big + (p - rest) * small;
 }
 
+// Copies of the same-spin lists in the order that the passes over whole staged rows read them (row-block
+// products, engine jobs): each list is padded with zero entries to a multiple of kListPad and
+// reordered so that the 8 entries one 128-bit shared-memory phase gathers have distinct targets modulo 8
+// where possible (kBankGroups).  Values are held as `mask` says.
+enum { kValHi = 1, kValLo = 2, kValF64 = 4 };  // FP32 rounding, FP32 of the remainder, FP64
+struct SigLists {
+    int mask = 0;                                // 0: not built
+    int64_t *s_ptr = nullptr, *d_ptr = nullptr;  // [rows + 1], padded CSR offsets
+    int64_t ns = 0, nd = 0;
+    uint32_t *s_pk = nullptr;  // packed single (SpinTables::s_pk)
+    int32_t *d_j = nullptr;    // target of a double
+    float *s_hi = nullptr, *s_lo = nullptr, *d_hi = nullptr, *d_lo = nullptr;
+    double *s_v = nullptr, *d_v = nullptr;
+};
+
 // index of the unordered orbital pair {p, q}
 __host__ __device__ __forceinline__ int orbital_pair(int p, int q)
 {
@@ -110,21 +125,7 @@ struct SpinTables {
     // packed single: target j (bits 0-17) | code p*norb+q (bits 18-29) | phase -1 (bit 30)
     uint32_t *s_pk = nullptr;
     double *s_v64 = nullptr, *d_v64 = nullptr;   // same-spin matrix elements
-    // Sigma copies of the lists, made with the first block plan (which restricts them) or for an engine
-    // job (the FP32 ones): the same
-    // entries per source, each list padded with zero entries to a multiple of kListPad and reordered so
-    // that the 8 entries one 128-bit shared-memory phase gathers have distinct targets modulo 8 where
-    // possible (kBankGroups).
-    int64_t *sig_s_ptr = nullptr, *sig_d_ptr = nullptr;  // [n+1], padded CSR offsets
-    int64_t sig_ns = 0, sig_nd = 0;
-    uint32_t *s_pk_sig = nullptr;
-    double *s_v64_sig = nullptr;
-    int32_t *d_j_sig = nullptr;
-    double *d_v64_sig = nullptr;
-    uint2 *s_pkv32 = nullptr;  // (s_pk_sig, FP32 value bits), for the mixed sigma
-    uint2 *d_jv32 = nullptr;   // (d_j_sig, FP32 value bits), for the mixed sigma
-    float2 *s_vx2 = nullptr;   // s_v64_sig as FP32 pairs (hi, lo), for the FP32-pair sigma
-    float2 *d_vx2 = nullptr;   // d_v64_sig as FP32 pairs
+    SigLists sig;  // of the whole set: for engine jobs, and of the beta spin for block plans
     // Engine jobs: the mixed row passes' lists split at the middle of the string set (half = (n + 1) / 2):
     // virtual list 2i holds the entries of source i with target < half, list 2i + 1 those with target
     // >= half, each padded to kListPad and in sigma order.
@@ -266,8 +267,9 @@ void sort_validate_into(const uint64_t *in, int64_t n, int norb, int nel, uint64
 void build_tables(Ctx &c, int spin);
 // beta: also what the alpha-beta passes read of their beta spin
 void build_range_lists(Ctx &c, int spin, bool beta);
-// sigma copies of one spin's lists, for block plans and (only the FP32 ones) engine jobs
-void build_sig_lists(Ctx &c, SpinTables &t, bool fp32_only = false);
+// copies of the lists of rows [r0, r0 + nr) with targets in [j0, j1), renumbered from j0; where `out` is built
+// already, the values of `mask` that it lacks
+void build_sig_lists(Ctx &c, const SpinTables &t, int64_t r0, int64_t nr, int64_t j0, int64_t j1, int mask, SigLists &out);
 // lists of the engine's mixed row passes with `rows` rows per item (0: any); drops what such a job
 // does not read
 void build_engine_lists(Ctx &c, int rows);
@@ -286,26 +288,20 @@ void build_src_lists(Ctx &c, int spin);
 // row-block sigma for alpha-row sharding (shard.cu, sigma.cu)
 
 // The alpha lists of output rows [r0, r1) restricted to sources in [j0, j1), targets renumbered
-// from j0, in the layouts of SpinTables (canonical singles; padded sigma singles and doubles).
+// from j0: canonical singles, and padded singles and doubles in the arithmetics of sig.mask.
 struct BlockPlan {
     Ctx *c = nullptr;
     int64_t r0 = 0, r1 = 0, j0 = 0, j1 = 0;
     int64_t *s_ptr = nullptr;
     uint32_t *s_pk = nullptr;
-    int64_t *sig_s_ptr = nullptr, *sig_d_ptr = nullptr;
-    uint32_t *s_pk_sig = nullptr;
-    double *s_v64_sig = nullptr;
-    uint2 *s_pkv32 = nullptr;
-    float2 *s_vx2 = nullptr;
-    int32_t *d_j_sig = nullptr;
-    double *d_v64_sig = nullptr;
-    uint2 *d_jv32 = nullptr;
-    float2 *d_vx2 = nullptr;
+    SigLists sig;
     void *work_t = nullptr;  // [nB][j1 - j0] doubles: the transposed source block
     float *rowmax = nullptr; // [j1 - j0] max |c| of each source row (mixed alpha-beta pass)
     std::vector<void *> allocs;
 };
-BlockPlan *block_plan_create(Ctx &c, int64_t r0, int64_t r1, int64_t j0, int64_t j1);
+// mask: values of the arithmetics that the plan is for (value_mask)
+BlockPlan *block_plan_create(Ctx &c, int64_t r0, int64_t r1, int64_t j0, int64_t j1, int mask);
+inline int value_mask(sbd_precision p) { return p == SBD_MIXED ? kValHi : p == SBD_F32X2 ? kValHi | kValLo : kValF64; }
 void block_plan_destroy(BlockPlan *p);
 // sigma_rows[(ia - r0)*nB + ib] += sum over (ja, jb), ja in [j0, j1), of H[(ia,ib),(ja,jb)] cblock[(ja - j0)*nB + jb]
 // x64_rows (optional, mixed precision): FP64 amplitudes of the output rows, for the diagonal term

@@ -179,90 +179,54 @@ __device__ __forceinline__ int pk_key(uint32_t pk) { return (int)(pk >> kPackKey
 __device__ __forceinline__ int pk_code(uint32_t pk) { return (int)(pk >> (kPackKeyShift + 1)); }
 __device__ __forceinline__ bool pk_neg(uint32_t pk) { return ((pk >> kPackKeyShift) & 1u) != 0u; }
 
-// Excitation lists of the column spin (padded sigma copies), in the layout each precision
-// reads.  Every list starts at a multiple of kListPad entries.  The 8 lanes of a group read a
-// list in chunks of up to 32 slots: in a chunk, lane l takes slots 4l..4l+3 (two 2-entry loads),
-// and entry u of the lane is the slot the u-th 128-bit shared-memory phase of the pass gathers
-// for that lane.  (Taking the two halves of a chunk as two contiguous runs instead halves the
-// sectors each load touches but loses the L1 hits of the second load, and was slower at 1.0e8
-// determinants.)
-__device__ __forceinline__ void list_slots(int64_t s0, int cb, int lc, int lig, int64_t &e0, int64_t &e1)
+// Excitation lists of the column spin (SigLists), as each precision reads them.  Every list starts at a
+// multiple of kListPad entries.  The 8 lanes of a group read a list in chunks of up to 32 slots: in a
+// chunk, lane l takes slots 4l..4l+3, and entry u of the lane is the slot the u-th 128-bit shared-memory
+// phase of the pass gathers for that lane.
+__device__ __forceinline__ void load4(const uint32_t *p, uint32_t (&v)[4])
 {
-    (void)lc;
-    e0 = s0 + cb + 4 * lig;
-    e1 = e0 + 2;
+    const uint4 a = __ldg(reinterpret_cast<const uint4 *>(p));
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+}
+__device__ __forceinline__ void load4(const int32_t *p, int (&v)[4])
+{
+    const int4 a = __ldg(reinterpret_cast<const int4 *>(p));
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+}
+__device__ __forceinline__ void load4(const float *p, const float *, float (&v)[4])
+{
+    const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+}
+__device__ __forceinline__ void load4(const double *p, const float *, double (&v)[4])
+{
+    const double2 a = __ldg(reinterpret_cast<const double2 *>(p)), b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
+    v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+}
+__device__ __forceinline__ void load4(const float *p, const float *q, F2 (&v)[4])
+{
+    const float4 a = __ldg(reinterpret_cast<const float4 *>(p)), b = __ldg(reinterpret_cast<const float4 *>(q));
+    v[0] = F2(a.x, b.x), v[1] = F2(a.y, b.y), v[2] = F2(a.z, b.z), v[3] = F2(a.w, b.w);
 }
 
 template <typename T>
-struct Lists;
-template <>
-struct Lists<float> {
-    const uint2 *s;  // (packed single, value bits)
-    const uint2 *d;  // (target, value bits)
-    __device__ void singles4(int64_t e0, int64_t e1, uint32_t (&pk)[4], float (&v)[4]) const
-    {
-        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(s + e0));
-        const uint4 b = __ldg(reinterpret_cast<const uint4 *>(s + e1));
-        pk[0] = a.x, v[0] = __uint_as_float(a.y), pk[1] = a.z, v[1] = __uint_as_float(a.w);
-        pk[2] = b.x, v[2] = __uint_as_float(b.y), pk[3] = b.z, v[3] = __uint_as_float(b.w);
-    }
-    __device__ void doubles4(int64_t e0, int64_t e1, int (&j)[4], float (&v)[4]) const
-    {
-        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(d + e0));
-        const uint4 b = __ldg(reinterpret_cast<const uint4 *>(d + e1));
-        j[0] = (int)a.x, v[0] = __uint_as_float(a.y), j[1] = (int)a.z, v[1] = __uint_as_float(a.w);
-        j[2] = (int)b.x, v[2] = __uint_as_float(b.y), j[3] = (int)b.z, v[3] = __uint_as_float(b.w);
-    }
-};
-template <>
-struct Lists<double> {
+struct Lists {
+    using V = typename RangeVal<T>::type;
     const uint32_t *spk;
-    const double *sv;
+    const V *sv;
+    const float *slo;
     const int32_t *dj;
-    const double *dv;
-    __device__ void singles4(int64_t e0, int64_t e1, uint32_t (&pk)[4], double (&v)[4]) const
+    const V *dv;
+    const float *dlo;
+    __device__ void singles4(int64_t e, uint32_t (&pk)[4], T (&v)[4]) const
     {
-        const uint2 a = __ldg(reinterpret_cast<const uint2 *>(spk + e0));
-        const uint2 a1 = __ldg(reinterpret_cast<const uint2 *>(spk + e1));
-        const double2 b = __ldg(reinterpret_cast<const double2 *>(sv + e0));
-        const double2 c = __ldg(reinterpret_cast<const double2 *>(sv + e1));
-        pk[0] = a.x, pk[1] = a.y, pk[2] = a1.x, pk[3] = a1.y;
-        v[0] = b.x, v[1] = b.y, v[2] = c.x, v[3] = c.y;
+        load4(spk + e, pk);
+        load4(sv + e, slo + e, v);
     }
-    __device__ void doubles4(int64_t e0, int64_t e1, int (&j)[4], double (&v)[4]) const
+    __device__ void doubles4(int64_t e, int (&j)[4], T (&v)[4]) const
     {
-        const int2 a = __ldg(reinterpret_cast<const int2 *>(dj + e0));
-        const int2 a1 = __ldg(reinterpret_cast<const int2 *>(dj + e1));
-        const double2 b = __ldg(reinterpret_cast<const double2 *>(dv + e0));
-        const double2 c = __ldg(reinterpret_cast<const double2 *>(dv + e1));
-        j[0] = a.x, j[1] = a.y, j[2] = a1.x, j[3] = a1.y;
-        v[0] = b.x, v[1] = b.y, v[2] = c.x, v[3] = c.y;
-    }
-};
-
-template <>
-struct Lists<F2> {
-    const uint32_t *spk;
-    const float2 *sv;
-    const int32_t *dj;
-    const float2 *dv;
-    __device__ void singles4(int64_t e0, int64_t e1, uint32_t (&pk)[4], F2 (&v)[4]) const
-    {
-        const uint2 a = __ldg(reinterpret_cast<const uint2 *>(spk + e0));
-        const uint2 a1 = __ldg(reinterpret_cast<const uint2 *>(spk + e1));
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(sv + e0));
-        const float4 c = __ldg(reinterpret_cast<const float4 *>(sv + e1));
-        pk[0] = a.x, pk[1] = a.y, pk[2] = a1.x, pk[3] = a1.y;
-        v[0] = F2(b.x, b.y), v[1] = F2(b.z, b.w), v[2] = F2(c.x, c.y), v[3] = F2(c.z, c.w);
-    }
-    __device__ void doubles4(int64_t e0, int64_t e1, int (&j)[4], F2 (&v)[4]) const
-    {
-        const int2 a = __ldg(reinterpret_cast<const int2 *>(dj + e0));
-        const int2 a1 = __ldg(reinterpret_cast<const int2 *>(dj + e1));
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(dv + e0));
-        const float4 c = __ldg(reinterpret_cast<const float4 *>(dv + e1));
-        j[0] = a.x, j[1] = a.y, j[2] = a1.x, j[3] = a1.y;
-        v[0] = F2(b.x, b.y), v[1] = F2(b.z, b.w), v[2] = F2(c.x, c.y), v[3] = F2(c.z, c.w);
+        load4(dj + e, j);
+        load4(dv + e, dlo + e, v);
     }
 };
 
@@ -392,11 +356,9 @@ __device__ __forceinline__ void row_group(const RowArgs<T> &a, int64_t r0, unsig
                 for (int cb = 0; cb < ls; cb += kGroup * kListPad) {
                     const int lc = min(kGroup * kListPad, ls - cb);
                     if (kListPad * lig >= lc) break;
-                    int64_t e0, e1;
-                    list_slots(s0, cb, lc, lig, e0, e1);
                     uint32_t pk[4];
                     T v[4];
-                    a.lists.singles4(e0, e1, pk, v);
+                    a.lists.singles4(s0 + cb + kListPad * lig, pk, v);
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         T xj[R], jv[R];
@@ -417,11 +379,9 @@ __device__ __forceinline__ void row_group(const RowArgs<T> &a, int64_t r0, unsig
                 for (int cb = 0; cb < ld; cb += kGroup * kListPad) {
                     const int lc = min(kGroup * kListPad, ld - cb);
                     if (kListPad * lig >= lc) break;
-                    int64_t e0, e1;
-                    list_slots(d0, cb, lc, lig, e0, e1);
                     int jj[4];
                     T v[4];
-                    a.lists.doubles4(e0, e1, jj, v);
+                    a.lists.doubles4(d0 + cb + kListPad * lig, jj, v);
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         T xj[R];
@@ -548,10 +508,9 @@ __device__ __forceinline__ void row_halves(const RowArgs<float> &a, int64_t r0, 
                 for (int cb2 = 0; cb2 < ls; cb2 += kGroup * kListPad) {
                     const int lc = min(kGroup * kListPad, ls - cb2);
                     if (kListPad * lig >= lc) break;
-                    int64_t e0, e1;
-                    list_slots(s0, cb2, lc, lig, e0, e1);
+                    const int64_t e0 = s0 + cb2 + kListPad * lig;
                     const uint4 p0 = __ldg(reinterpret_cast<const uint4 *>(a.hls + e0));
-                    const uint4 p1 = __ldg(reinterpret_cast<const uint4 *>(a.hls + e1));
+                    const uint4 p1 = __ldg(reinterpret_cast<const uint4 *>(a.hls + e0 + 2));
                     const uint32_t pk[4] = {p0.x, p0.z, p1.x, p1.z};
                     const float vv[4] = {__uint_as_float(p0.y), __uint_as_float(p0.w), __uint_as_float(p1.y),
                                          __uint_as_float(p1.w)};
@@ -575,8 +534,7 @@ __device__ __forceinline__ void row_halves(const RowArgs<float> &a, int64_t r0, 
                 for (int cb2 = 0; cb2 < ld; cb2 += kGroup * kListPad) {
                     const int lc = min(kGroup * kListPad, ld - cb2);
                     if (kListPad * lig >= lc) break;
-                    int64_t e0, e1;
-                    list_slots(d0, cb2, lc, lig, e0, e1);
+                    const int64_t e0 = d0 + cb2 + kListPad * lig;
                     // entries e0 .. e0 + 3: four values (16 bytes) and four 16-bit targets (8 bytes)
                     const float4 v4 = __ldg(reinterpret_cast<const float4 *>(a.hldv + e0));
                     const uint2 t4 = __ldg(reinterpret_cast<const uint2 *>(a.hldt + e0));
@@ -1521,21 +1479,10 @@ void transpose(const T *in, T *out, int64_t rows, int64_t cols, cudaStream_t s, 
 }
 
 template <typename T>
-Lists<T> lists_of(const SpinTables &t);
-template <>
-Lists<float> lists_of<float>(const SpinTables &t)
+Lists<T> lists_of(const SigLists &l)
 {
-    return Lists<float>{t.s_pkv32, t.d_jv32};
-}
-template <>
-Lists<double> lists_of<double>(const SpinTables &t)
-{
-    return Lists<double>{t.s_pk_sig, t.s_v64_sig, t.d_j_sig, t.d_v64_sig};
-}
-template <>
-Lists<F2> lists_of<F2>(const SpinTables &t)
-{
-    return Lists<F2>{t.s_pk_sig, t.s_vx2, t.d_j_sig, t.d_vx2};
+    if constexpr (std::is_same<T, double>::value) return Lists<double>{l.s_pk, l.s_v, nullptr, l.d_j, l.d_v, nullptr};
+    else return Lists<T>{l.s_pk, l.s_hi, l.s_lo, l.d_j, l.d_hi, l.d_lo};
 }
 
 // timing slot of the first sigma kernel of a precision (transpose, beta, alpha, alpha-beta follow)
@@ -1586,9 +1533,9 @@ void make_row_args(const Ctx &c, const float *C, double *S, const double *c64, c
 {
     const SpinTables &ta = c.sp[0], &tb = c.sp[1];
     auto lists = [](RowArgs<float> &r, const SpinTables &t) {
-        r.s_ptr = t.sig_s_ptr;
-        r.d_ptr = t.sig_d_ptr;
-        r.lists = lists_of<float>(t);
+        r.s_ptr = t.sig.s_ptr;
+        r.d_ptr = t.sig.d_ptr;
+        r.lists = lists_of<float>(t.sig);
         r.hls_ptr = t.hs_ptr;
         r.hld_ptr = t.hd_ptr;
         r.hls = t.hs;
@@ -2254,9 +2201,9 @@ void apply_block(BlockPlan &p, const typename In<T>::type *Cb, double *S, cudaSt
         b.hd = c.hd + lo * c.nB;
         b.xd64 = x64 ? x64 + (lo - p.r0) * c.nB : nullptr;
         b.row_strings = ta.strings + lo;
-        b.s_ptr = tb.sig_s_ptr;
-        b.d_ptr = tb.sig_d_ptr;
-        b.lists = lists_of<T>(tb);
+        b.s_ptr = tb.sig.s_ptr;
+        b.d_ptr = tb.sig.d_ptr;
+        b.lists = lists_of<T>(tb.sig);
         launch_row<T>(b, choose(c.nB, n2, sizeof(T), rmax, lim), s);
     }
     // alpha pass: rows of the transposed block, output columns r0..r1, lists restricted to the block
@@ -2269,11 +2216,9 @@ void apply_block(BlockPlan &p, const typename In<T>::type *Cb, double *S, cudaSt
     ra.y_rs = 1;
     ra.y_cs = c.nB;
     ra.row_strings = tb.strings;
-    ra.s_ptr = p.sig_s_ptr;
-    ra.d_ptr = p.sig_d_ptr;
-    if constexpr (kIsF2<T>) ra.lists = Lists<F2>{p.s_pk_sig, p.s_vx2, p.d_j_sig, p.d_vx2};
-    else if constexpr (sizeof(T) == 4) ra.lists = Lists<float>{p.s_pkv32, p.d_jv32};
-    else ra.lists = Lists<double>{p.s_pk_sig, p.s_v64_sig, p.d_j_sig, p.d_v64_sig};
+    ra.s_ptr = p.sig.s_ptr;
+    ra.d_ptr = p.sig.d_ptr;
+    ra.lists = lists_of<T>(p.sig);
     launch_row<T>(ra, choose(nj, n2, sizeof(T), rmax, lim), s);
     // alpha-beta pass: output rows r0..r1, their alpha singles inside the block
     if constexpr (std::is_same<T, float>::value) {
@@ -2300,6 +2245,7 @@ void apply_block(BlockPlan &p, const typename In<T>::type *Cb, double *S, cudaSt
 void sigma_block_apply(BlockPlan &p, const void *cblock, double *sigma_rows, sbd_precision prec, cudaStream_t s,
                        const double *x64_rows)
 {
+    if (value_mask(prec) & ~p.sig.mask) fail(SBD_ERR_INVALID_ARG, "block plan: not made for this precision");
     if (prec == SBD_FP64) apply_block<double>(p, static_cast<const double *>(cblock), sigma_rows, s, nullptr);
     else if (prec == SBD_F32X2) apply_block<F2>(p, static_cast<const double *>(cblock), sigma_rows, s, nullptr);
     else apply_block<float>(p, static_cast<const float *>(cblock), sigma_rows, s, x64_rows);

@@ -469,13 +469,14 @@ __device__ __forceinline__ int slot_of(int q, int Lp)
 // The picks follow one another; a warp scores a list's entries at once (one thread per list: up to 1.3 ms
 // for a few thousand strings).
 constexpr int kJointMax = 1024;
-__global__ void joint_order_kernel(const int64_t *__restrict__ ptr, const int64_t *__restrict__ sig_ptr, int64_t n,
-                                   const int32_t *__restrict__ j_src, const uint32_t *__restrict__ pk, int64_t *perm)
+__global__ void joint_order_kernel(const int64_t *__restrict__ beg, const int64_t *__restrict__ end,
+                                   const int64_t *__restrict__ sig_ptr, int64_t n, const int32_t *__restrict__ j_src,
+                                   const uint32_t *__restrict__ pk, int32_t *perm)
 {
     const int lane = threadIdx.x & 31;
     for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; i < n;
          i += (int64_t)gridDim.x * blockDim.x / 32) {
-        const int64_t b = ptr[i], e = ptr[i + 1], sb = sig_ptr[i];
+        const int64_t b = beg[i], e = end[i], sb = sig_ptr[i];
         const int L = (int)(e - b), Lp = (int)(sig_ptr[i + 1] - sb);
         if (L > kJointMax) continue;  // sigma_order_kernel orders these
         for (int q = lane; q < Lp; q += 32) perm[sb + q] = -1;  // slots no entry lands on stay padding
@@ -518,19 +519,21 @@ __global__ void joint_order_kernel(const int64_t *__restrict__ ptr, const int64_
                 if (lane == rj || lane == 8 + rk) --count;
                 used_j |= 1u << rj;
                 used_k |= 1u << rk;
-                if (lane == 0) perm[sb + slot_of(q, Lp)] = b + x;
+                if (lane == 0) perm[sb + slot_of(q, Lp)] = (int32_t)(b + x);
             }
         }
     }
 }
 
-// perm[sig_ptr[i] + slot] = index of the canonical entry, or -1 for padding.  One thread per source.
+// perm[sig_ptr[i] + slot] = index of the canonical entry (of [beg[i], end[i])), or -1 for padding.  One thread per
+// source.
 // joint: lists of at most kJointMax entries are joint_order_kernel's.
-__global__ void sigma_order_kernel(const int64_t *__restrict__ ptr, const int64_t *__restrict__ sig_ptr, int64_t n,
-                                   const int32_t *__restrict__ j_src, bool joint, int64_t *perm)
+__global__ void sigma_order_kernel(const int64_t *__restrict__ beg, const int64_t *__restrict__ end,
+                                   const int64_t *__restrict__ sig_ptr, int64_t n, const int32_t *__restrict__ j_src,
+                                   bool joint, int32_t *perm)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = ptr[i], e = ptr[i + 1], sb = sig_ptr[i], se = sig_ptr[i + 1];
+        const int64_t b = beg[i], e = end[i], sb = sig_ptr[i], se = sig_ptr[i + 1];
         const int Lp = (int)(se - sb);
         if (joint && e - b <= kJointMax) continue;
         for (int q = 0; q < Lp; ++q) perm[sb + q] = -1;  // slots no entry lands on stay padding
@@ -543,25 +546,61 @@ __global__ void sigma_order_kernel(const int64_t *__restrict__ ptr, const int64_
             int q = 0;  // position in round order
 #pragma unroll
             for (int w = 0; w < kBankGroups; ++w) q += min(count[w], t) + ((w < r && count[w] > t) ? 1 : 0);
-            perm[sb + slot_of(q, Lp)] = x;
+            perm[sb + slot_of(q, Lp)] = (int32_t)x;
         }
     }
 }
 
-template <typename V>
-__global__ void gather_kernel(const V *__restrict__ src, const int64_t *__restrict__ perm, V *dst, int64_t n)
+// first entry of [lo, hi) with target >= key (targets ascend)
+__device__ __forceinline__ int64_t first_at_least(const int32_t *__restrict__ tgt, int64_t lo, int64_t hi, int64_t key)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = perm[i];
-        dst[i] = p >= 0 ? src[p] : V(0);
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) / 2;
+        if (tgt[mid] < key) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// x = hi + lo with hi the FP32 rounding of x and lo the FP32 rounding of the remainder
+__device__ __forceinline__ float2 split2(double x)
+{
+    const float hi = __double2float_rn(x);
+    return make_float2(hi, __double2float_rn(x - (double)hi));
+}
+
+// entries of list r0 + i with targets in [j0, j1): [beg[i], end[i])
+__global__ void row_bounds_kernel(const int64_t *__restrict__ ptr, const int32_t *__restrict__ tgt, int64_t r0, int64_t nr,
+                                  int64_t j0, int64_t j1, int64_t *beg, int64_t *end)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nr; i += (int64_t)gridDim.x * blockDim.x) {
+        beg[i] = first_at_least(tgt, ptr[r0 + i], ptr[r0 + i + 1], j0);
+        end[i] = first_at_least(tgt, beg[i], ptr[r0 + i + 1], j1);
     }
 }
 
-// padded counts: cnt[i] = ceil((ptr[i+1]-ptr[i]) / kListPad) * kListPad
-__global__ void padded_count_kernel(const int64_t *__restrict__ ptr, int64_t n, int64_t *cnt)
+// The entries perm names, zeros for padding: key (a packed single or, pk null, a target; from j0) and values; a
+// null output is left out
+__global__ void sig_gather_kernel(const int32_t *__restrict__ perm, int64_t m, const int32_t *__restrict__ j,
+                                  const uint32_t *__restrict__ pk, const double *__restrict__ val, int64_t j0, uint32_t *key,
+                                  float *hi, float *lo, double *v64)
+{
+    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < m; o += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t e = perm[o];
+        const double v = e >= 0 ? val[e] : 0.0;
+        if (key) key[o] = e >= 0 ? (uint32_t)(j[e] - j0) | (pk ? pk[e] & ~kPackJMask : 0u) : 0u;
+        const float2 x = split2(v);
+        if (hi) hi[o] = x.x;
+        if (lo) lo[o] = x.y;
+        if (v64) v64[o] = v;
+    }
+}
+
+// padded counts: cnt[i] = ceil((end[i]-beg[i]) / kListPad) * kListPad
+__global__ void padded_count_kernel(const int64_t *__restrict__ beg, const int64_t *__restrict__ end, int64_t n, int64_t *cnt)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t L = ptr[i + 1] - ptr[i];
+        const int64_t L = end[i] - beg[i];
         cnt[i] = (L + kListPad - 1) / kListPad * kListPad;
     }
 }
@@ -656,7 +695,7 @@ __global__ void half_split_kernel(const int64_t *__restrict__ ptr, const int32_t
 
 // Doubles of the half-split lists: val[o] = FP32 of v[perm[o]], tgt[o] = its target relative to
 // the column half it lies in (target - half for targets >= half); zeros for padding
-__global__ void gather_half_doubles_kernel(const int64_t *__restrict__ perm, int64_t m,
+__global__ void gather_half_doubles_kernel(const int32_t *__restrict__ perm, int64_t m,
                                            const int32_t *__restrict__ j, const double *__restrict__ v,
                                            int64_t half, float *val, uint16_t *tgt)
 {
@@ -669,7 +708,7 @@ __global__ void gather_half_doubles_kernel(const int64_t *__restrict__ perm, int
 }
 
 // out[o] = (key[perm[o]], FP32 of val[perm[o]]), zeros for padding
-__global__ void gather_pair_kernel(const int64_t *__restrict__ perm, int64_t m, const uint32_t *__restrict__ key,
+__global__ void gather_pair_kernel(const int32_t *__restrict__ perm, int64_t m, const uint32_t *__restrict__ key,
                                    const double *__restrict__ val, uint2 *out)
 {
     for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < m; o += (int64_t)gridDim.x * blockDim.x) {
@@ -679,17 +718,6 @@ __global__ void gather_pair_kernel(const int64_t *__restrict__ perm, int64_t m, 
 }
 
 // ---- range lists of the row passes (RangeLists) --------------------------------
-
-// first entry of [lo, hi) with target >= key (targets ascend)
-__device__ __forceinline__ int64_t first_at_least(const int32_t *__restrict__ tgt, int64_t lo, int64_t hi, int64_t key)
-{
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) / 2;
-        if (tgt[mid] < key) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
 
 // cnt[g*n + i] = blocks of `pad` entries that string i's list needs for the targets of range g
 __global__ void range_count_kernel(const int64_t *__restrict__ ptr, const int32_t *__restrict__ tgt, int64_t n, int w,
@@ -762,13 +790,6 @@ __global__ void range_group_kernel(int64_t n, int64_t groups, int64_t total, con
         nd[q] = md;
         ns[q] = ms;
     }
-}
-
-// x = hi + lo with hi the FP32 rounding of x and lo the FP32 rounding of the remainder
-__device__ __forceinline__ float2 split2(double x)
-{
-    const float hi = __double2float_rn(x);
-    return make_float2(hi, __double2float_rn(x - (double)hi));
 }
 
 // One warp per list (group q, place o): copies its entries (KIND 1 singles, 2 doubles) to their blocks.
@@ -1029,23 +1050,6 @@ __global__ void src_entry_order_kernel(const uint32_t *__restrict__ item, uint32
     }
 }
 
-// (key, FP32 value) pairs for single 8-byte loads in the mixed sigma
-__global__ void pair_kernel(const uint32_t *__restrict__ key, const double *__restrict__ val, uint2 *out, int64_t n)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = make_uint2(key[i], __float_as_uint(__double2float_rn(val[i])));
-}
-
-// x = hi + lo with hi the FP32 rounding of x and lo the FP32 rounding of the remainder
-__global__ void split_kernel(const double *__restrict__ in, float2 *out, int64_t n)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double x = in[i];
-        const float hi = __double2float_rn(x);
-        out[i] = make_float2(hi, __double2float_rn(x - (double)hi));
-    }
-}
-
 __global__ void to_float_kernel(const double *in, float *out, int64_t n)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -1199,77 +1203,64 @@ void build_tables(Ctx &c, int spin)
 }
 
 // sigma order of n lists; pk (singles only): packed entries, for the joint target/row order
-static void order_lists(Ctx &c, const int64_t *ptr, const int64_t *sig_ptr, int64_t n, const int32_t *j,
-                        const uint32_t *pk, int64_t *perm)
+static void order_lists(Ctx &c, const int64_t *beg, const int64_t *end, const int64_t *sig_ptr, int64_t n, const int32_t *j,
+                        const uint32_t *pk, int32_t *perm)
 {
     if (pk) {
-        joint_order_kernel<<<blocks_for(n, 4, 65535), 128, 0, c.stream>>>(ptr, sig_ptr, n, j, pk, perm);
+        joint_order_kernel<<<blocks_for(n, 4, 65535), 128, 0, c.stream>>>(beg, end, sig_ptr, n, j, pk, perm);
         SBD_LAUNCH("joint_order_kernel");
     }
-    sigma_order_kernel<<<blocks_for(n, 128), 128, 0, c.stream>>>(ptr, sig_ptr, n, j, pk != nullptr, perm);
+    sigma_order_kernel<<<blocks_for(n, 128), 128, 0, c.stream>>>(beg, end, sig_ptr, n, j, pk != nullptr, perm);
     SBD_LAUNCH("sigma_order_kernel");
 }
 
-void build_sig_lists(Ctx &c, SpinTables &t, bool fp32_only)
+void build_sig_lists(Ctx &c, const SpinTables &t, int64_t r0, int64_t nr, int64_t j0, int64_t j1, int mask, SigLists &out)
 {
-    const int64_t n = t.n;
-    int64_t *cnt = dalloc_n<int64_t>(c, 2 * (size_t)n);
-    t.sig_s_ptr = dalloc_n<int64_t>(c, n + 1);
-    int64_t *d_ptr = dalloc_n<int64_t>(c, n + 1);
-    padded_count_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(t.s_ptr, n, cnt);
-    padded_count_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(t.d_ptr, n, cnt + n);
-    SBD_LAUNCH("padded_count_kernel");
-    scan(c, cnt, n, t.sig_s_ptr);
-    scan(c, cnt + n, n, d_ptr);
-    SBD_CUDA(cudaMemcpyAsync(&t.sig_ns, t.sig_s_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
-    SBD_CUDA(cudaMemcpyAsync(&t.sig_nd, d_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
-    SBD_CUDA(cudaStreamSynchronize(c.stream));
-    t.s_pk_sig = dalloc_n<uint32_t>(c, t.sig_ns);
-    t.s_v64_sig = dalloc_n<double>(c, t.sig_ns);
-    t.s_pkv32 = dalloc_n<uint2>(c, t.sig_ns);
-    t.s_vx2 = dalloc_n<float2>(c, t.sig_ns);
-    t.d_j_sig = dalloc_n<int32_t>(c, t.sig_nd);
-    t.d_v64_sig = dalloc_n<double>(c, t.sig_nd);
-    t.d_jv32 = dalloc_n<uint2>(c, t.sig_nd);
-    t.d_vx2 = dalloc_n<float2>(c, t.sig_nd);
-    int64_t *perm = dalloc_n<int64_t>(c, (size_t)std::max<int64_t>(std::max(t.sig_ns, t.sig_nd), 1));
-    if (t.sig_ns) {
-        order_lists(c, t.s_ptr, t.sig_s_ptr, n, t.s_j, t.s_pk, perm);
-        SBD_LAUNCH("sigma_order_kernel(singles)");
-        const int gb = blocks_for(t.sig_ns, 256, 16384);
-        gather_kernel<uint32_t><<<gb, 256, 0, c.stream>>>(t.s_pk, perm, t.s_pk_sig, t.sig_ns);
-        gather_kernel<double><<<gb, 256, 0, c.stream>>>(t.s_v64, perm, t.s_v64_sig, t.sig_ns);
-        SBD_LAUNCH("gather_kernel(singles)");
-        pair_kernel<<<gb, 256, 0, c.stream>>>(t.s_pk_sig, t.s_v64_sig, t.s_pkv32, t.sig_ns);
-        SBD_LAUNCH("pair_kernel(singles)");
-        split_kernel<<<gb, 256, 0, c.stream>>>(t.s_v64_sig, t.s_vx2, t.sig_ns);
-        SBD_LAUNCH("split_kernel(singles)");
+    const int add = mask & ~out.mask;
+    if (!add) return;
+    int64_t *beg = dalloc_n<int64_t>(c, (size_t)nr), *end = dalloc_n<int64_t>(c, (size_t)nr);
+    for (int kind = 1; kind <= 2; ++kind) {
+        const bool singles = kind == 1;
+        const int32_t *j = singles ? t.s_j : t.d_j;
+        const uint32_t *pk = singles ? t.s_pk : nullptr;
+        int64_t *&ptr = singles ? out.s_ptr : out.d_ptr;
+        int64_t &m = singles ? out.ns : out.nd;
+        row_bounds_kernel<<<blocks_for(nr, 256), 256, 0, c.stream>>>(singles ? t.s_ptr : t.d_ptr, j, r0, nr, j0, j1, beg, end);
+        SBD_LAUNCH("row_bounds_kernel");
+        if (!out.mask) {
+            int64_t *cnt = dalloc_n<int64_t>(c, (size_t)nr);
+            ptr = dalloc_n<int64_t>(c, (size_t)nr + 1);
+            padded_count_kernel<<<blocks_for(nr, 256), 256, 0, c.stream>>>(beg, end, nr, cnt);
+            SBD_LAUNCH("padded_count_kernel");
+            scan(c, cnt, nr, ptr);
+            SBD_CUDA(cudaMemcpyAsync(&m, ptr + nr, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream));
+            SBD_CUDA(cudaStreamSynchronize(c.stream));
+            dfree(c, cnt);
+        }
+        uint32_t *key = nullptr;
+        if (!out.mask) {
+            key = dalloc_n<uint32_t>(c, (size_t)m);
+            if (singles) out.s_pk = key;
+            else out.d_j = reinterpret_cast<int32_t *>(key);
+        }
+        float *hi = add & kValHi ? dalloc_n<float>(c, (size_t)m) : nullptr;
+        float *lo = add & kValLo ? dalloc_n<float>(c, (size_t)m) : nullptr;
+        double *v = add & kValF64 ? dalloc_n<double>(c, (size_t)m) : nullptr;
+        if (hi) (singles ? out.s_hi : out.d_hi) = hi;
+        if (lo) (singles ? out.s_lo : out.d_lo) = lo;
+        if (v) (singles ? out.s_v : out.d_v) = v;
+        if (m) {
+            int32_t *perm = dalloc_n<int32_t>(c, (size_t)m);
+            order_lists(c, beg, end, ptr, nr, j, pk, perm);
+            sig_gather_kernel<<<blocks_for(m, 256, 16384), 256, 0, c.stream>>>(perm, m, j, pk, singles ? t.s_v64 : t.d_v64, j0,
+                                                                              key, hi, lo, v);
+            SBD_LAUNCH("sig_gather_kernel");
+            dfree(c, perm);
+        }
     }
-    if (t.sig_nd) {
-        order_lists(c, t.d_ptr, d_ptr, n, t.d_j, nullptr, perm);
-        SBD_LAUNCH("sigma_order_kernel(doubles)");
-        const int gb = blocks_for(t.sig_nd, 256, 16384);
-        gather_kernel<int32_t><<<gb, 256, 0, c.stream>>>(t.d_j, perm, t.d_j_sig, t.sig_nd);
-        gather_kernel<double><<<gb, 256, 0, c.stream>>>(t.d_v64, perm, t.d_v64_sig, t.sig_nd);
-        SBD_LAUNCH("gather_kernel(doubles)");
-        pair_kernel<<<gb, 256, 0, c.stream>>>(reinterpret_cast<const uint32_t *>(t.d_j_sig), t.d_v64_sig, t.d_jv32,
-                                               t.sig_nd);
-        SBD_LAUNCH("pair_kernel(doubles)");
-        split_kernel<<<gb, 256, 0, c.stream>>>(t.d_v64_sig, t.d_vx2, t.sig_nd);
-        SBD_LAUNCH("split_kernel(doubles)");
-    }
-    dfree(c, perm);
-    dfree(c, cnt);
-    if (fp32_only) {
-        for (void *q : {(void *)t.s_pk_sig, (void *)t.s_v64_sig, (void *)t.s_vx2, (void *)t.d_j_sig, (void *)t.d_v64_sig,
-                        (void *)t.d_vx2})
-            dfree(c, q);
-        t.s_pk_sig = nullptr;
-        t.s_v64_sig = t.d_v64_sig = nullptr;
-        t.s_vx2 = t.d_vx2 = nullptr;
-        t.d_j_sig = nullptr;
-    }
-    t.sig_d_ptr = d_ptr;  // set last: marks the copies as complete
+    dfree(c, beg);
+    dfree(c, end);
+    out.mask |= add;
 }
 
 // Lists split at the middle of the string set
@@ -1289,7 +1280,7 @@ static void build_half_lists(Ctx &c, SpinTables &t)
             half_split_kernel<<<blocks_for(n, 256), 256, 0, c.stream>>>(ptr, tgt, n, t.half, ptr2);
             SBD_LAUNCH("half_split_kernel");
             hptr = dalloc_n<int64_t>(c, 2 * (size_t)n + 1);
-            padded_count_kernel<<<blocks_for(2 * n, 256), 256, 0, c.stream>>>(ptr2, 2 * n, cnt2);
+            padded_count_kernel<<<blocks_for(2 * n, 256), 256, 0, c.stream>>>(ptr2, ptr2 + 1, 2 * n, cnt2);
             SBD_LAUNCH("padded_count_kernel(halves)");
             scan(c, cnt2, 2 * n, hptr);
             int64_t m = 0;
@@ -1303,8 +1294,8 @@ static void build_half_lists(Ctx &c, SpinTables &t)
                 t.hdt = dalloc_n<uint16_t>(c, mm);
             }
             if (m) {
-                int64_t *hperm = dalloc_n<int64_t>(c, (size_t)m);
-                order_lists(c, ptr2, hptr, 2 * n, tgt, kind == 0 ? t.s_pk : nullptr, hperm);
+                int32_t *hperm = dalloc_n<int32_t>(c, (size_t)m);
+                order_lists(c, ptr2, ptr2 + 1, hptr, 2 * n, tgt, kind == 0 ? t.s_pk : nullptr, hperm);
                 SBD_LAUNCH("sigma_order_kernel(halves)");
                 if (kind == 0) {
                     gather_pair_kernel<<<blocks_for(m, 256, 16384), 256, 0, c.stream>>>(hperm, m, t.s_pk, t.s_v64,
@@ -1347,7 +1338,7 @@ void build_engine_lists(Ctx &c, int rows)
         dfree(c, t.rl.sv64);
         t.rl.dv64 = t.rl.sv64 = nullptr;
         if (rows == 0 || rows == 8) build_half_lists(c, t);
-        if (rows != 8) build_sig_lists(c, t, true);
+        if (rows != 8) build_sig_lists(c, t, 0, t.n, 0, t.n, kValHi, t.sig);
     }
     SBD_CUDA(cudaStreamSynchronize(c.stream));
 }

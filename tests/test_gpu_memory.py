@@ -47,3 +47,56 @@ def test_handle_fits_the_budget_it_used_to(B):
     wl = W.make("budget", 58, 19, 19, 2000, 2000, 0.35, 5)
     with B.SBD.from_workload(wl, hbm_budget_bytes=270_000_000) as g:
         assert g.memory() <= 270_000_000
+
+
+def test_refused_allocation_of_a_block_plan_leaves_the_handle_as_it_was(B):
+    import torch
+
+    wl = W.make("plan", 14, 4, 4, 120, 90, 0.3, 8)
+    state = {"left": None}
+
+    def alloc(ctx, nbytes, stream):
+        if state["left"] is not None:
+            state["left"] -= 1
+            if state["left"] < 0:
+                return None
+        return torch.cuda.caching_allocator_alloc(int(nbytes), stream=int(stream or 0))
+
+    def free(ctx, ptr, stream):
+        torch.cuda.caching_allocator_delete(int(ptr))
+
+    opts = B.sbd_default_options()
+    fa, ff = B.ALLOC_FN(alloc), B.FREE_FN(free)
+    opts.alloc, opts.free = fa, ff
+    h = B.sbd_create(wl.norb, 4, 4, wl.h, wl.eri, wl.A, wl.B, opts, 0)
+    try:
+        nA, nB = B.sbd_dims(h)
+        x = torch.from_numpy(W.random_vector(nA * nB, 2)[0]).cuda()
+        ref, out = torch.empty_like(x), torch.empty_like(x)
+        B.sbd_sigma(h, x, ref, 1, "fp64", 0)
+        torch.cuda.synchronize()
+        held, refused = B.sbd_memory(h), 0
+        while True:
+            state["left"] = refused
+            try:
+                plan = B.sbd_block_plan_create(h, 0, nA, 0, nA)
+                break
+            except B.SbdError as e:
+                assert e.code == -5
+                refused += 1
+                state["left"] = None
+                assert B.sbd_memory(h) == held
+                B.sbd_sigma(h, x, out, 1, "fp64", 0)
+                torch.cuda.synchronize()
+                assert torch.equal(out, ref)
+        state["left"] = None
+        assert refused >= 10
+        out.zero_()
+        B.sbd_sigma_block(plan, x, out, "fp64", 0)
+        torch.cuda.synchronize()
+        assert float((out - ref).abs().max()) <= 1e-14 * float(ref.abs().max())
+        B.sbd_block_plan_destroy(plan)
+    finally:
+        state["left"] = None
+        B.sbd_destroy(h)
+        torch.cuda.synchronize()
