@@ -270,6 +270,14 @@ const char *sbd_last_error(sbd_handle h) { return h ? h->c.last_error.c_str() : 
 int sbd_create(sbd_handle *out, int norb, int nalpha, int nbeta, const double *h, const double *eri,
                const uint64_t *A, int64_t nA, const uint64_t *B, int64_t nB, const sbd_options *opt, void *stream)
 {
+    return create_handle(out, norb, nalpha, nbeta, h, eri, A, nA, B, nB, opt, stream, false);
+}
+
+}  // extern "C"
+
+int sbd::create_handle(sbd_handle *out, int norb, int nalpha, int nbeta, const double *h, const double *eri, const uint64_t *A,
+                       int64_t nA, const uint64_t *B, int64_t nB, const sbd_options *opt, void *stream, bool job)
+{
     if (!out) {
         g_last_error = "out is NULL";
         return SBD_ERR_INVALID_ARG;
@@ -292,6 +300,7 @@ int sbd_create(sbd_handle *out, int norb, int nalpha, int nbeta, const double *h
     Ctx &c = hd->c;
     if (opt) c.opt = *opt;
     else sbd_default_options(&c.opt);
+    c.job = job;
     c.stream = (cudaStream_t)stream;
     c.norb = norb;
     c.na = nalpha;
@@ -383,6 +392,8 @@ int sbd_create(sbd_handle *out, int norb, int nalpha, int nbeta, const double *h
     return SBD_OK;
 }
 
+extern "C" {
+
 int sbd_destroy(sbd_handle h)
 {
     if (!h) return SBD_ERR_INVALID_ARG;
@@ -444,10 +455,7 @@ int sbd_tables(sbd_handle h, int spin, int kind, int64_t *ptr_host, int32_t *tar
         if (target_host && m)
             SBD_CUDA(cudaMemcpyAsync(target_host, kind == 1 ? t.s_j : t.d_j, (size_t)m * sizeof(int32_t),
                                      cudaMemcpyDeviceToHost, s));
-        if (orbs_host && m)
-            SBD_CUDA(cudaMemcpyAsync(orbs_host, kind == 1 ? t.s_orb : t.d_orb, (size_t)m * 4, cudaMemcpyDeviceToHost, s));
-        if (sign_host && m)
-            SBD_CUDA(cudaMemcpyAsync(sign_host, kind == 1 ? t.s_sign : t.d_sign, (size_t)m, cudaMemcpyDeviceToHost, s));
+        table_moves(h->c, spin, kind == 1, orbs_host, sign_host);
         SBD_CUDA(cudaStreamSynchronize(s));
         return SBD_OK;
     });

@@ -120,8 +120,6 @@ struct SpinTables {
     int64_t *s_ptr = nullptr, *d_ptr = nullptr;  // [n+1]
     int64_t ns = 0, nd = 0;                      // total entries
     int32_t *s_j = nullptr, *d_j = nullptr;      // target index
-    uint8_t *s_orb = nullptr, *d_orb = nullptr;  // p1,p2,q1,q2 per entry
-    int8_t *s_sign = nullptr, *d_sign = nullptr; // fermionic phase
     // packed single: target j (bits 0-17) | code p*norb+q (bits 18-29) | phase -1 (bit 30)
     uint32_t *s_pk = nullptr;
     double *s_v64 = nullptr, *d_v64 = nullptr;   // same-spin matrix elements
@@ -170,6 +168,7 @@ struct Ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
     sbd_options opt{};
+    bool job = false;  // an engine job: mixed products over whole staged rows, pair products for the check
     int norb = 0, na = 0, nb = 0;
     int64_t nA = 0, nB = 0, N = 0;
     double *h64 = nullptr, *eri64 = nullptr;
@@ -198,6 +197,9 @@ struct Ctx {
 
 // the context inside a C-ABI handle (api.cu)
 Ctx &ctx_of(sbd_handle h);
+// sbd_create; job: see Ctx
+int create_handle(sbd_handle *out, int norb, int nalpha, int nbeta, const double *h, const double *eri, const uint64_t *A,
+                  int64_t nA, const uint64_t *B, int64_t nB, const sbd_options *opt, void *stream, bool job);
 
 // kernel timing helpers (api.cu)
 cudaEvent_t take_event(Ctx &c);
@@ -270,10 +272,11 @@ void build_range_lists(Ctx &c, int spin, bool beta);
 // copies of the lists of rows [r0, r0 + nr) with targets in [j0, j1), renumbered from j0; where `out` is built
 // already, the values of `mask` that it lacks
 void build_sig_lists(Ctx &c, const SpinTables &t, int64_t r0, int64_t nr, int64_t j0, int64_t j1, int mask, SigLists &out);
-// lists of the engine's mixed row passes with `rows` rows per item (0: any); drops what such a job
-// does not read
+// lists of the engine's mixed row passes with `rows` rows per item (0: any)
 void build_engine_lists(Ctx &c, int rows);
 void build_diagonal(Ctx &c);
+// orbitals (4 per entry) and phases of a spin's singles or doubles, worked out from the strings into host memory
+void table_moves(const Ctx &c, int spin, bool singles, uint8_t *orbs_host, int8_t *sign_host);
 void pack_integrals(Ctx &c);  // eri32 from eri64
 void to_float(const double *in, float *out, int64_t n, cudaStream_t s);
 

@@ -815,8 +815,8 @@ bool sbd_engine_s::admit_one()
         // the tables, diagonal and work vectors of the handle (and whatever sbd_create holds while it
         // runs) must fit what the budget leaves after the jobs in use and this job's basis
         if (opt.hbm_budget_bytes) o.hbm_budget_bytes = opt.hbm_budget_bytes - bytes_in_use - basis_bytes(N);
-        int rc = sbd_create(&s.handle, j->norb, j->na, j->nb, j->h.data(), j->eri.data(), j->A.data(), nA,
-                            j->B.data(), nB, &o, (void *)stream);
+        int rc = create_handle(&s.handle, j->norb, j->na, j->nb, j->h.data(), j->eri.data(), j->A.data(), nA,
+                               j->B.data(), nB, &o, (void *)stream, true);
         if (rc == SBD_OK) {
             try {
                 build_engine_lists(ctx_of(s.handle), rows_per_item);

@@ -22,6 +22,8 @@
 //   diagonal  sum_{i in S} h_ii + 1/2 sum_{i,j in S} [(ii|jj) - (ij|ji)]
 //   single    phase * [h_pq + sum_{k in S_j} ((pq|kk) - (pk|kq))]
 //   double    phase * [(p1 q1|p2 q2) - (p1 q2|p2 q1)]
+#include <string.h>
+
 #include <algorithm>
 
 #include "common.cuh"
@@ -50,62 +52,82 @@ __device__ __forceinline__ int move_phase(uint64_t ket, int from, int to)
     return (__popcll(ket & between_mask(from, to)) & 1) ? -1 : 1;
 }
 
-struct Entry {
-    int32_t j;
+// p1, p2 (occupied in si only), q1, q2 (in sj only), each ascending, 255 where there is none; and the phase
+struct Move {
     uint8_t orb[4];
     int8_t sign;
+};
+struct Entry : Move {
+    int32_t j;
     double val;
 };
+
+__device__ __forceinline__ Move single_move(uint64_t si, uint64_t sj)
+{
+    const uint64_t x = si ^ sj;
+    const int p = __ffsll((long long)(x & si)) - 1, q = __ffsll((long long)(x & sj)) - 1;
+    return Move{{(uint8_t)p, 255, (uint8_t)q, 255}, (int8_t)move_phase(sj, q, p)};
+}
+
+__device__ __forceinline__ Move double_move(uint64_t si, uint64_t sj)
+{
+    const uint64_t x = si ^ sj, pb = x & si, qb = x & sj;
+    const int p1 = __ffsll((long long)pb) - 1, p2 = 63 - __clzll((long long)pb);
+    const int q1 = __ffsll((long long)qb) - 1, q2 = 63 - __clzll((long long)qb);
+    const uint64_t sj2 = sj ^ (1ull << q2) ^ (1ull << p2);
+    return Move{{(uint8_t)p1, (uint8_t)p2, (uint8_t)q1, (uint8_t)q2},
+                (int8_t)(move_phase(sj, q2, p2) * move_phase(sj2, q1, p1))};
+}
 
 __device__ Entry make_single(uint64_t si, uint64_t sj, int32_t j, int norb, const double *__restrict__ h,
                              const double *__restrict__ eri)
 {
     Entry e;
-    const uint64_t x = si ^ sj;
-    const int p = __ffsll((long long)(x & si)) - 1;
-    const int q = __ffsll((long long)(x & sj)) - 1;
-    const int sg = move_phase(sj, q, p);
+    static_cast<Move &>(e) = single_move(si, sj);
+    const int p = e.orb[0], q = e.orb[2];
     double v = __ldg(h + (size_t)p * norb + q);
     for (uint64_t m = sj; m; m &= m - 1ull) {
         const int k = __ffsll((long long)m) - 1;
         v += eri_at(eri, norb, p, q, k, k) - eri_at(eri, norb, p, k, k, q);
     }
     e.j = j;
-    e.orb[0] = (uint8_t)p;
-    e.orb[1] = 255;
-    e.orb[2] = (uint8_t)q;
-    e.orb[3] = 255;
-    e.sign = (int8_t)sg;
-    e.val = sg * v;
+    e.val = e.sign * v;
     return e;
 }
 
 __device__ Entry make_double(uint64_t si, uint64_t sj, int32_t j, int norb, const double *__restrict__ eri)
 {
     Entry e;
-    const uint64_t x = si ^ sj, pb = x & si, qb = x & sj;
-    const int p1 = __ffsll((long long)pb) - 1, p2 = 63 - __clzll((long long)pb);
-    const int q1 = __ffsll((long long)qb) - 1, q2 = 63 - __clzll((long long)qb);
-    const int s2 = move_phase(sj, q2, p2);
-    const uint64_t sj2 = sj ^ (1ull << q2) ^ (1ull << p2);
-    const int s1 = move_phase(sj2, q1, p1);
-    const int sg = s1 * s2;
+    static_cast<Move &>(e) = double_move(si, sj);
+    const int p1 = e.orb[0], p2 = e.orb[1], q1 = e.orb[2], q2 = e.orb[3];
     const double v = eri_at(eri, norb, p1, q1, p2, q2) - eri_at(eri, norb, p1, q2, p2, q1);
     e.j = j;
-    e.orb[0] = (uint8_t)p1;
-    e.orb[1] = (uint8_t)p2;
-    e.orb[2] = (uint8_t)q1;
-    e.orb[3] = (uint8_t)q2;
-    e.sign = (int8_t)sg;
-    e.val = sg * v;
+    e.val = e.sign * v;
     return e;
+}
+
+// orbitals and phases of `m` entries of a table from entry e0 on (either output may be null)
+__global__ void moves_kernel(const uint64_t *__restrict__ S, int64_t n, const int64_t *__restrict__ ptr,
+                             const int32_t *__restrict__ tgt, bool singles, int64_t e0, int64_t m, uint32_t *orbs, int8_t *sign)
+{
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < m; x += (int64_t)gridDim.x * blockDim.x) {
+        int64_t lo = 0, hi = n;  // the row: ptr[lo] <= e0 + x < ptr[hi]
+        while (hi - lo > 1) {
+            const int64_t mid = (lo + hi) / 2;
+            if (ptr[mid] <= e0 + x) lo = mid;
+            else hi = mid;
+        }
+        const uint64_t si = S[lo], sj = S[tgt[e0 + x]];
+        const Move v = singles ? single_move(si, sj) : double_move(si, sj);
+        if (orbs)
+            orbs[x] = (uint32_t)v.orb[0] | (uint32_t)v.orb[1] << 8 | (uint32_t)v.orb[2] << 16 | (uint32_t)v.orb[3] << 24;
+        if (sign) sign[x] = v.sign;
+    }
 }
 
 struct TableOut {
     const int64_t *s_ptr, *d_ptr;
     int32_t *s_j, *d_j;
-    uint8_t *s_orb, *d_orb;
-    int8_t *s_sign, *d_sign;
     uint32_t *s_pk;
     double *s_v, *d_v;
 };
@@ -113,11 +135,6 @@ struct TableOut {
 __device__ __forceinline__ void store_single(const TableOut &o, int64_t pos, const Entry &e, int norb)
 {
     o.s_j[pos] = e.j;
-    o.s_orb[4 * pos + 0] = e.orb[0];
-    o.s_orb[4 * pos + 1] = e.orb[1];
-    o.s_orb[4 * pos + 2] = e.orb[2];
-    o.s_orb[4 * pos + 3] = e.orb[3];
-    o.s_sign[pos] = e.sign;
     o.s_v[pos] = e.val;
     const uint32_t key = 2u * (uint32_t)(e.orb[0] * norb + e.orb[2]) + (e.sign < 0 ? 1u : 0u);
     o.s_pk[pos] = (uint32_t)e.j | (key << kPackKeyShift);
@@ -126,11 +143,6 @@ __device__ __forceinline__ void store_single(const TableOut &o, int64_t pos, con
 __device__ __forceinline__ void store_double(const TableOut &o, int64_t pos, const Entry &e)
 {
     o.d_j[pos] = e.j;
-    o.d_orb[4 * pos + 0] = e.orb[0];
-    o.d_orb[4 * pos + 1] = e.orb[1];
-    o.d_orb[4 * pos + 2] = e.orb[2];
-    o.d_orb[4 * pos + 3] = e.orb[3];
-    o.d_sign[pos] = e.sign;
     o.d_v[pos] = e.val;
 }
 
@@ -827,13 +839,13 @@ __global__ void range_fill_kernel(const int64_t *__restrict__ ptr, const int32_t
                 const float2 x = split2(v);
                 r.shi[at] = x.x;
                 r.slo[at] = x.y;
-                r.sv64[at] = v;
+                if (r.sv64) r.sv64[at] = v;
             } else {
                 const float2 x = split2(v);
                 r.dt[at] = (uint16_t)t;
                 r.dhi[at] = x.x;
                 r.dlo[at] = x.y;
-                r.dv64[at] = v;
+                if (r.dv64) r.dv64[at] = v;
             }
         }
     }
@@ -1097,6 +1109,34 @@ int blocks_for(int64_t n, int threads, int cap = 65535)
 
 }  // namespace
 
+void table_moves(const Ctx &c, int spin, bool singles, uint8_t *orbs_host, int8_t *sign_host)
+{
+    constexpr int64_t kPiece = 1 << 20;
+    const SpinTables &t = c.sp[spin];
+    const int64_t total = singles ? t.ns : t.nd;
+    if (!total || (!orbs_host && !sign_host)) return;
+    struct Staging {  // pinned: the kernel writes to it
+        unsigned char *p = nullptr;
+        ~Staging() { (void)cudaFreeHost(p); }
+    } st;
+    const int64_t piece = std::min(total, kPiece);
+    if (cudaHostAlloc((void **)&st.p, (size_t)piece * 5, cudaHostAllocMapped) != cudaSuccess) {
+        (void)cudaGetLastError();
+        fail(SBD_ERR_OUT_OF_MEMORY, "pinned staging for the tables");
+    }
+    uint32_t *orbs = orbs_host ? reinterpret_cast<uint32_t *>(st.p) : nullptr;
+    int8_t *sign = sign_host ? reinterpret_cast<int8_t *>(st.p + 4 * piece) : nullptr;
+    for (int64_t e = 0; e < total; e += piece) {
+        const int64_t m = std::min(piece, total - e);
+        moves_kernel<<<blocks_for(m, 256), 256, 0, c.stream>>>(t.strings, t.n, singles ? t.s_ptr : t.d_ptr,
+                                                               singles ? t.s_j : t.d_j, singles, e, m, orbs, sign);
+        SBD_LAUNCH("moves_kernel");
+        SBD_CUDA(cudaStreamSynchronize(c.stream));
+        if (orbs) memcpy(orbs_host + 4 * e, orbs, (size_t)m * 4);
+        if (sign) memcpy(sign_host + e, sign, (size_t)m);
+    }
+}
+
 // One CTA up to kScanOne elements (its time grows with them: 0.12 ms at 60,000, 11 ms at 5.6e6 list groups)
 constexpr int64_t kScanOne = 1 << 14;
 static void scan(Ctx &c, const int64_t *cnt, int64_t n, int64_t *ptr)
@@ -1168,22 +1208,14 @@ void build_tables(Ctx &c, int spin)
     if (t.ns > 0x7fffffffLL || t.nd > 0x7fffffffLL) fail(SBD_ERR_UNSUPPORTED, "excitation table too large");
 
     t.s_j = dalloc_n<int32_t>(c, t.ns);
-    t.s_orb = dalloc_n<uint8_t>(c, 4 * t.ns);
-    t.s_sign = dalloc_n<int8_t>(c, t.ns);
     t.s_pk = dalloc_n<uint32_t>(c, t.ns);
     t.s_v64 = dalloc_n<double>(c, t.ns);
     t.d_j = dalloc_n<int32_t>(c, t.nd);
-    t.d_orb = dalloc_n<uint8_t>(c, 4 * t.nd);
-    t.d_sign = dalloc_n<int8_t>(c, t.nd);
     t.d_v64 = dalloc_n<double>(c, t.nd);
     o.s_ptr = t.s_ptr;
     o.d_ptr = t.d_ptr;
     o.s_j = t.s_j;
     o.d_j = t.d_j;
-    o.s_orb = t.s_orb;
-    o.d_orb = t.d_orb;
-    o.s_sign = t.s_sign;
-    o.d_sign = t.d_sign;
     o.s_pk = t.s_pk;
     o.s_v = t.s_v64;
     o.d_v = t.d_v64;
@@ -1333,10 +1365,6 @@ void build_engine_lists(Ctx &c, int rows)
             std::copy(slice, slice + kSrcParts + 1, t.src_slice);
             continue;
         }
-        // the FP64 elements of the range lists: the engine's products are mixed and pairs
-        dfree(c, t.rl.dv64);
-        dfree(c, t.rl.sv64);
-        t.rl.dv64 = t.rl.sv64 = nullptr;
         if (rows == 0 || rows == 8) build_half_lists(c, t);
         if (rows != 8) build_sig_lists(c, t, 0, t.n, 0, t.n, kValHi, t.sig);
     }
@@ -1476,11 +1504,11 @@ void build_range_lists(Ctx &c, int spin, bool beta)
     r.sm = dalloc_n<uint32_t>(c, ms);
     r.shi = dalloc_n<float>(c, ms);
     r.slo = dalloc_n<float>(c, ms);
-    r.sv64 = dalloc_n<double>(c, ms);
+    r.sv64 = c.job ? nullptr : dalloc_n<double>(c, ms);
     r.dt = dalloc_n<uint16_t>(c, md);
     r.dhi = dalloc_n<float>(c, md);
     r.dlo = dalloc_n<float>(c, md);
-    r.dv64 = dalloc_n<double>(c, md);
+    r.dv64 = c.job ? nullptr : dalloc_n<double>(c, md);
     const int fb = blocks_for(nq * kListGroup * 32, 256, 16384);
     if (ms) {
         range_fill_kernel<1><<<fb, 256, 0, c.stream>>>(t.s_ptr, t.s_j, t.s_pk, t.s_v64, groups, c.norb, used, r);

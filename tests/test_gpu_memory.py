@@ -100,3 +100,26 @@ def test_refused_allocation_of_a_block_plan_leaves_the_handle_as_it_was(B):
         state["left"] = None
         B.sbd_destroy(h)
         torch.cuda.synchronize()
+
+
+def test_block_plans_fit_the_budget_they_used_to(B):
+    # 3,001 x 4,003 strings at norb 40, the two plans of one of two ranks: 4.96e8 bytes when the handle kept ordered
+    # lists of both spins and no range lists
+    wl = W.make("plans", 40, 13, 13, 3001, 4003, 0.35, 5)
+    with B.SBD.from_workload(wl, hbm_budget_bytes=500_000_000) as g:
+        plans = [B.sbd_block_plan_create(g.handle, 0, 1500, *j) for j in ((0, 1500), (1500, 3001))]
+        assert g.memory() <= 496_000_000
+        for p in plans:
+            B.sbd_block_plan_destroy(p)
+
+
+def test_engine_jobs_fit_the_budget_they_used_to(B):
+    # two jobs of 1,500 x 2,000 strings at norb 58 held 1.225e9 bytes before the range lists
+    wl = W.make("jobs", 58, 19, 19, 1500, 2000, 0.35, 5)
+    with B.Engine(max_slots=2, max_subspace=6, max_iter=4, max_norb=58, max_strings=2000, rows_per_item=4,
+                  hbm_budget_bytes=1_235_000_000) as e:
+        for _ in range(2):
+            e.submit(wl, tol=1e-8)
+        e.step()
+        st = e.stats()
+        assert st["active"] == 2 and st["requeued"] == 0, st
