@@ -175,7 +175,7 @@ struct Ctx {
     float *eri32 = nullptr;  // (pq|rs) of orbital pairs p > q, r > s, [npair][npair], pair p(p-1)/2 + q
     SpinTables sp[2];
     double *hd = nullptr;   // [N] Hamiltonian diagonal
-    void *work_t = nullptr; // [N] doubles: transposed copy of one vector
+    void *work_t = nullptr; // [N] doubles: the beta pass' transposed result
     float *rowmax = nullptr; // [nA] max |c(ia, :)| of the last mixed-precision vector (written by its beta pass)
     float eri_absmax = 0.f;  // max |(pq|rs)| of the FP32 integrals
     size_t bytes_held = 0;
@@ -318,9 +318,10 @@ void sigma_block_apply(BlockPlan &p, const void *cblock, double *sigma_rows, sbd
 struct SigmaSlot {
     const Ctx *c;
     const void *x;       // amplitudes [nA][nB]: float (mixed) or double (FP64)
-    double *y;           // sigma [nA][nB], overwritten
+    double *y;           // sigma [nA][nB], overwritten; scratch until the last pass, must not overlap x or x64
     const double *x64;   // mixed only: FP64 amplitudes for the diagonal term, or null
-    void *xt;            // [nA*nB] elements of the precision: transposed copy of x
+    void *xt;            // work space of nA*nB doubles: the beta pass' transposed result, or (passes over whole
+                         // staged rows) the transposed amplitudes
 };
 struct SigmaBatch;
 // Device descriptors for up to max_slots instances whose string sets have at most max_strings
@@ -342,7 +343,6 @@ void sigma_batch_set(SigmaBatch *b, const SigmaSlot *slots, int n);
 // captured in a CUDA graph once and replayed after each sigma_batch_set.
 void sigma_batch_launch(SigmaBatch *b, cudaStream_t s);
 void sigma_batch_destroy(SigmaBatch *b);
-int64_t sigma_batch_launches(const SigmaBatch *b);  // kernel launches per sigma_batch_launch
 // c64 (mixed only, may be NULL): the FP64 amplitudes, used for the diagonal term
 void sigma_apply(Ctx &c, const void *cvec, double *svec, sbd_precision prec, cudaStream_t s,
                  const double *c64 = nullptr);

@@ -39,7 +39,7 @@ constexpr int kRangeThreads = 768;
 constexpr int kRangeRowBytes = 128;
 
 // The table of J_r[rs] of the staged rows sits in shared memory while it leaves at least half of it
-// to the ranges (norb <= 42); above that the few singles read J from global memory, because shorter
+// to the ranges (norb <= 43); above that the few singles read J from global memory, because shorter
 // ranges would mean more passes over Y.
 __host__ __device__ inline size_t range_j_bytes(int norb) { return (size_t)(norb * (norb - 1) / 2 + 1) * kRangeRowBytes; }
 __host__ __device__ inline size_t range_smem(int optin) { return ((size_t)optin - 1024) / kRangeRowBytes * kRangeRowBytes; }

@@ -2054,7 +2054,7 @@ bool sigma_batch_fits(sbd_precision prec, int R, int max_strings, int max_norb, 
     const size_t lim = sigma_batch_smem_limit(device);
     if (R == kHalfRows)
         return prec == SBD_MIXED && max_norb >= 2 && sigma_batch_smem(prec, R, max_strings, max_norb) <= lim &&
-               (size_t)64 * npairs(max_norb) + (size_t)8 * max_strings + round16((size_t)2 * npairs(max_norb)) <= lim;
+               src_parts_for(npairs(max_norb), max_strings, lim) > 0;
     if (R == 4 && prec != SBD_MIXED) return false;
     return sigma_batch_smem(prec, R, max_strings, max_norb) <= lim;
 }
@@ -2155,8 +2155,6 @@ void sigma_batch_launch(SigmaBatch *b, cudaStream_t s)
         else batch_launch_r<float, 1>(b, s);
     }
 }
-
-int64_t sigma_batch_launches(const SigmaBatch *) { return 5; }
 
 void sigma_batch_destroy(SigmaBatch *b)
 {

@@ -1376,8 +1376,9 @@ void build_src_lists(Ctx &c, int spin)
     SpinTables &t = c.sp[spin];
     const int64_t n = t.n;
     const int norb = c.norb, npair = norb * (norb - 1) / 2;
-    t.src_parts = src_parts(norb, n, c.smem_optin);
-    const int parts = std::max(t.src_parts, 1);
+    const int parts = t.src_parts = src_parts(norb, n, c.smem_optin);
+    t.src_width = 1;
+    if (!parts) return;  // the two-operand pass runs instead
     t.src_width = std::max(1, (npair + parts - 1) / parts);
     int64_t *cnt = dalloc_n<int64_t>(c, (size_t)n);
     int64_t *ioff = dalloc_n<int64_t>(c, (size_t)parts * (n + 1));
