@@ -232,7 +232,8 @@ int sbd_davidson(sbd_handle handle, int nroots, double tol, sbd_precision prec, 
  *   C), 2 alpha pass (lists of the alpha strings, on C), 3 alpha-beta pass; FP64
  *   kernels in 0..3, mixed in 4..7, SBD_F32X2 in 8..11.  Transposing the beta
  *   pass' result back and adding the diagonal term counts to slot 1 for
- *   SBD_MIXED and to slot 3 for the others, which add them last.
+ *   SBD_MIXED and to slot 3 for the others, which add them last; small products
+ *   (up to 2^17 determinants) have no transposes.
  * ms_host and launches_host: 12 entries each (either may be NULL).  Waits for
  * the recorded events; reset != 0 clears the counters afterwards.
  */

@@ -22,7 +22,7 @@
 //
 // Measured, beta + alpha pass of one product (CUDA events, before: whole rows of C staged, one list
 // per eight lanes and one entry per lane): 1.0e8 determinants, FP32 25.1 -> 17.6 ms; 3.6e7
-// determinants (norb 29), FP32 7.0 -> 5.0, FP64 64.2 -> 49.8, FP32 pairs 20.8 -> 14.5 ms; 2.5e7
+// determinants (norb 29), FP32 7.0 -> 5.0, FP64 64.2 -> 49.6, FP32 pairs 20.8 -> 15.5 ms; 2.5e7
 // determinants at norb 58, FP32 about 12 -> 6.4 ms.
 // Steps on the way (FP32, 3.6e7 determinants): an octet per list with separate lists 6.0 ms, with
 // interleaved lists 6.2 (padding costs more than the contiguous loads save while every octet still
@@ -357,7 +357,7 @@ __device__ __forceinline__ void range_rows(const RangeArgs<T> &a, int64_t row0, 
     using In = typename RangeIn<T>::type;
     constexpr int ROWS = kRangeRows<T>, RPC = Acc::kRowsPerChunk, LPW = 32 / ROWS;  // LPW: lines a warp stages at once
     constexpr int kWarps = kRangeThreads / 32;
-    // the FP64-accurate arithmetics have no registers left for a second block (pairs: 7.3 -> 7.9 ms)
+    // the FP64-accurate arithmetics have no registers left for a second block (pairs: 7.8 -> 7.9 ms)
     constexpr int kAhead = sizeof(T) == 4 ? 2 : 1;
     unsigned char *Js = smem + (size_t)a.w * kRangeRowBytes;  // [npair + 1] lines, or a line of zeros, behind the w lines
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

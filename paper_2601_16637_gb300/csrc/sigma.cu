@@ -742,14 +742,14 @@ struct AbSum<F2, 2> {
 // a fixed pattern, the warp with the longest list held up the barrier of every group).  A column is
 // added to once per group, and the groups are separated by a barrier, so its adds land in order.
 //
-// Bound by the FP64 pipe (FP64) or by the two 16-byte gathers per entry (pairs: L1/shared pipe 72 %,
-// 45 % of the gather wavefronts are bank conflicts left by the ordering of the entries).  Measured
+// Bound by the FP64 pipe (FP64) or by the two 16-byte gathers per entry (pairs: L1/shared pipe 84 %,
+// 43 % of the wavefronts are bank conflicts left by the ordering of the entries).  Measured
 // against eight lanes per column (each column's list padded to 32 slots), 3.6e7 determinants, norb 29:
-// FP64 84.1 -> 33.7 ms, pairs 33.1 -> 18.9 ms; with the slices dealt out in a fixed pattern 36.6 and
+// FP64 84.1 -> 34 ms, pairs 33.1 -> 19.1 ms; with the slices dealt out in a fixed pattern 36.6 and
 // 21.4 ms.
 // Pairs: where the longest slice is 3 (8) times a warp's share of all steps or more, it holds up the
-// barrier, and two (four) lanes walk a list: 2,000 rows x 150 columns at norb 24 839 -> 583 us, x 700
-// columns 1,753 -> 1,472; with equal lists (full space, 495 strings) one lane 397 us, two 451.  FP64 is bound by
+// barrier, and two (four) lanes walk a list: 2,000 rows x 150 columns at norb 24 839 -> 569 us, x 700
+// columns 1,663 -> 1,430; with equal lists (full space, 495 strings) one lane 397 us, two 451.  FP64 is bound by
 // its pipe even then (one lane 727 us, eight 1,686 at 300 columns).
 // Where a row of C does not fit shared memory its elements come from L2, and the bounds of the next slice are
 // loaded during this one (200 x 60,000 strings, norb 58: FP64 209 -> 111 ms, pairs 96 -> 76; for staged
